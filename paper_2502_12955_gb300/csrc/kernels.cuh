@@ -1,9 +1,10 @@
 // kernels.cuh -- sm_103a kernels of the reactive multi-component LBM step.
 //
-// Storage: structure of arrays, one plane per direction, pop[i * pitch + slot[n]], node
-// n = x + nx*(y + ny*z).  The slot map puts the fluid nodes first, in list order, so a warp's
-// lanes touch consecutive slots in every plane and no cache line carries solid-node bytes; the
-// cells named (n, i) below are pop[i * pitch + slot[n]].
+// Storage: tiles of 32 slots (see Rec).  A tile holds one row of 32 elements per population of
+// every lattice, the flow components first, so all populations of a warp's 32 slots are one
+// contiguous record.  Node n = x + nx*(y + ny*z) sits at slot[n]; the slot map puts the fluid nodes
+// first, in list order, so a warp's lanes touch consecutive elements of every row and no cache
+// line carries solid-node bytes.  The cells named (n, i) below are row i at slot[n].
 // Every lattice keeps ONE copy of its populations and streams in place with the A-A pattern:
 //   even steps (parity 0) read f_i(n) from slot (n, i) and write the post-collision f*_i to
 //   slot (n, opp i); odd steps (parity 1) read f_i(n) from (n - c_i, opp i) and write f*_i to
@@ -121,21 +122,24 @@ __host__ __device__ __forceinline__ unsigned int fast_div(unsigned int n, FastDi
 
 // Everything a kernel needs, in double; kernels convert to their compute type.
 struct Args {
-  void* f[2];
-  void* h[3];                // scalar lattices: the given scalars, then the reaction product (if any)
-  void* fplane[2][19];       // base pointer of every population plane (host-computed)
-  void* hplane[3][7];
+  unsigned char* pop;        // every population, in tiles of 32 slots (see Rec): the flow components,
+                             // the given scalars, then the reaction product (if any)
+  long long pop_bytes;
   void* psi[2];              // compute-type psi per component (Shan-Chen only)
   uint8_t* flags;
   uint32_t* mask;
   double* acc;               // consumed (reactive solid) / deposited (fluid) per node
-  uint32_t* fluid_list;       // fluid node indices (sorted at each rebuild, appended by flips)
+  uint32_t* fluid_list;       // fluid nodes (sorted at each rebuild, appended by flips): the node index,
+                              // with kEdgeBit set where a neighbour may lie across a domain face
   unsigned int* fluid_count;  // [0] list length, [1] length at the last rebuild (see slot)
-  // Storage slot of every node: populations of node n live at plane * pitch + slot[n].  Each
+  // Storage slot of every node.  Each
   // rebuild renumbers the fluid nodes to slots 0 .. F-1 in list order (so list entry e < F has
   // slot e) and the solid nodes to F .. N-1; nodes that become fluid later keep their slot.
   uint32_t* slot;
   uint32_t* slot_new;         // rebuild scratch
+  // Byte offset of every node's first cell in pop, plus kOffBias rows (see wall_offsets); kept
+  // beside slot when pop fits in 32 bits (off_ok), for the plain step kernels
+  uint32_t* off;
   unsigned int* block_counts; // ordered-compaction scratch [chunks + 1]
   unsigned int* block_counts_v;   // the same for the in-domain positions of the fluid-list order
   double* wallx_slot;        // [NBANKS][WALLX_SLOTS] wall-exchange accumulators
@@ -156,7 +160,7 @@ struct Args {
   double* d_u;               // [3][N]
   double* d_C;               // [n_scal][N]
   void* snap;                // compute-type residual snapshots [4][pitch] by slot: u_x, u_y, u_z, C
-  long long pitch;           // elements per population plane (>= N, multiple of 32)
+  long long pitch;           // slots (>= N, multiple of 32)
   long long N;
   int nx, ny, nz;
   int n_comp, n_scal;        // n_scal: scalar lattices, the product included
@@ -176,7 +180,7 @@ struct Args {
   int moving_wall;           // the top plate moves (closed y axis)
   int flow_open_x;           // flow velocity inlet at x = 0, zero-gradient outlet at x = nx - 1
   double* u_in_row;          // [ny] inlet velocity u_x(y)
-  int voff_ok;               // 3 * pitch < 2^31: wall links can be addressed by 32-bit offsets
+  int off_ok;                // pop fits in 32-bit byte offsets: the plain step kernels apply
   int arrhenius;             // scalar 1 is the temperature: rate k(T_b), reaction heat into T
   int n_it;                  // fixed-point iterations of the C_b - T_b coupling per link
   double arr_A, arr_Ta, heat_release;
@@ -188,6 +192,10 @@ struct Args {
   void* kb;                  // compute-type [QC - 1][N]: k(T_b) of the link arriving in
                              // direction j at node n from the last exchange; NaN before one
 };
+
+// Fused multiply-add of the compute types.
+__device__ __forceinline__ float fmad(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fmad(double a, double b, double c) { return fma(a, b, c); }
 
 // Index guard of the bounds-checked build (-DLBM_BOUNDS_CHECK): an index outside [0, bound)
 // sets ERR_BOUNDS and is replaced by 0, so the access stays inside its buffer.  In normal
@@ -209,6 +217,8 @@ __device__ __forceinline__ long long chk_index(int* err, long long i, long long 
 template <class T>
 struct Coef {
   T om[2];          // 1 / tau
+  T hom[2];         // (1 - 1 / tau) / 2
+  T oq, omm;        // s_q / 8, s_m / 8: odd D3Q19 MRT groups
   T tau[2];
   T G[2][2], G_ads[2], psi_wall, rho0, g[3];
   T mrt_g[10];      // (s_k - 1/tau) / |R_k|^2 of the MRT rows (one component)
@@ -216,6 +226,7 @@ struct Coef {
   T wc0, wca;       // scalar weights: rest, axis
   T ics2c;          // 1 / c_s^2 of the scalar lattice
   T icb;            // 1 / (2 w_a + K), K = k tau_c / (tau_c - 1/2): wet-node closure
+  T cl1, cl2;       // 4 w_a icb - 1, 2 k icb: closed population and reaction rate per gathered one
   T kr;             // k
   T C_in[3];
   T DP, keep;       // deposition probability, 1 - DP
@@ -273,81 +284,108 @@ __device__ __forceinline__ Nbr make_nbr(const Args& a, int x, int y, int z) {
 template <class L>
 __device__ __forceinline__ bool flow_wall(uint32_t m, int i) { return (m >> i) & 1u; }
 
-// ------------------------------------------------------------- gathers
+// Fluid-list entries: node index, and a bit for nodes on the faces of the box.  Away from the faces a
+// neighbour's index is a constant away, so the coordinates (two divisions) and the periodic wrap
+// are worked out for edge nodes only.
+constexpr uint32_t kEdgeBit = 0x80000000u;
 
-// Pre-collision flow populations of node n (as stored; shift added for 16-bit storage).
-// Stored (deviation) values of the pre-collision flow populations of node n.
-// sn is the node's storage slot; neighbour slots come from the slot map.
-template <class L, class S>
-__device__ __forceinline__ void gather_flow(const S* __restrict__ f, long long pitch, long long sn,
-                                            const uint32_t* __restrict__ slot, uint32_t m,
-                                            const Nbr& nb, int parity, typename Store<S>::T* out) {
-#pragma unroll
-  for (int i = 0; i < L::Q; ++i) {
-    const S* p;
-    if (parity == 0 || i == 0 || flow_wall<L>(m, L::opp(i))) {
-      p = f + (long long)i * pitch + sn;
-    } else {
-      p = f + (long long)L::opp(i) * pitch + __ldg(slot + nb.at(-L::cx(i), -L::cy(i), -L::cz(i)));
-    }
-    out[i] = Store<S>::ld(p);
-  }
+template <class L>
+__device__ __forceinline__ uint32_t list_entry(const Args& a, int n, int x, int y, int z) {
+  const bool edge = x == 0 || x == a.nx - 1 || y == 0 || y == a.ny - 1 || (L::D == 3 && (z == 0 || z == a.nz - 1));
+  return uint32_t(n) | (edge ? kEdgeBit : 0u);
+}
+__device__ __forceinline__ int list_node(const Args& a, uint32_t entry) {
+  return int(LBM_CHK(a.err, entry & ~kEdgeBit, a.N));
 }
 
-// Same as gather_flow, addressing through per-plane base pointers with 64-bit node offsets
-// (no multiply by the plane pitch in the kernel).
-template <class L, class S>
-__device__ __forceinline__ void gather_flow_pl(void* const* planes, long long sn,
-                                               const uint32_t* __restrict__ slot, uint32_t m,
-                                               const Nbr& nb, int parity, typename Store<S>::T* out,
-                                               int* err, long long n_nodes, long long pitch) {
+// Neighbour offsets of fluid node n from its coordinates (fast divisions by nx and ny).
+__device__ __forceinline__ Nbr nbr_of(const Args& a, int n) {
+  const unsigned int q = fast_div(unsigned(n), a.div_x);
+  const unsigned int z = fast_div(q, a.div_y);
+  return make_nbr(a, n - int(q) * a.nx, int(q - z * unsigned(a.ny)), int(z));
+}
+// the same for a fluid-list entry of node n
+__device__ __forceinline__ Nbr nbr_entry(const Args& a, int n, uint32_t entry) {
+  if (entry & kEdgeBit) return nbr_of(a, n);
+  const int sy = a.nx, sz = a.nx * a.ny;
+  return Nbr{n, -1, 1, -sy, sy, -sz, sz};
+}
+
+// ------------------------------------------------------------- population tiles
+
+// Record of one tile of 32 slots: NC * Q rows of 32 flow elements, then NS * QC rows of 32 scalar
+// elements.  One record is a contiguous stretch (3.3 KB for D3Q19 + D3Q7 in FP32), so an even step
+// reads and writes each of a warp's rows from one base address with constant offsets and within
+// a few DRAM pages, where planes of the whole domain put every population in a page of its own.
+template <class L, class S, int NC, int NS>
+struct Rec {
+  using SC = typename ScalarOf<S>::type;
+  static constexpr int FROW = 32 * (int)sizeof(S), HROW = 32 * (int)sizeof(SC);
+  static constexpr int H0 = NC * L::Q * FROW;
+  static constexpr int BYTES = H0 + NS * L::QC * HROW;
+  static constexpr bool kSameElem = sizeof(S) == sizeof(SC);
+  __host__ __device__ static constexpr int frow(int s, int i) { return (s * L::Q + i) * FROW; }
+  __host__ __device__ static constexpr int hrow(int s, int j) { return H0 + (s * L::QC + j) * HROW; }
+  // byte offset of the first flow cell of a slot, and of its first scalar cell less H0
+  __device__ __forceinline__ static long long cell(long long sn) {
+    return (sn >> 5) * BYTES + (sn & 31) * (long long)sizeof(S);
+  }
+  template <class O>
+  __device__ __forceinline__ static O scell(O c) {
+    if (kSameElem) return c;
+    return c + ((c / O(sizeof(S))) & O(31)) * O(sizeof(SC) - sizeof(S));
+  }
+  __device__ __forceinline__ static S* f(const Args& a, long long c, int s, int i) {
+    return reinterpret_cast<S*>(a.pop + LBM_CHK(a.err, c + frow(s, i), a.pop_bytes));
+  }
+  __device__ __forceinline__ static SC* h(const Args& a, long long c, int s, int j) {
+    return reinterpret_cast<SC*>(a.pop + LBM_CHK(a.err, scell(c) + hrow(s, j), a.pop_bytes));
+  }
+};
+
+// ------------------------------------------------------------- gathers
+
+// cell offset of node n
+template <class R>
+__device__ __forceinline__ long long cell_of(const Args& a, long long n) {
+  return R::cell((long long)LBM_CHK(a.err, __ldg(a.slot + LBM_CHK(a.err, n, a.N)), a.pitch));
+}
+
+// Stored (deviation) values of the pre-collision flow populations of the node whose cells start at
+// offset c; neighbour cells come from the slot map.
+template <class L, class S, int NC, int NS>
+__device__ __forceinline__ void gather_flow(const Args& a, int s, long long c, uint32_t m, const Nbr& nb, int parity,
+                                            typename Store<S>::T* out) {
+  using R = Rec<L, S, NC, NS>;
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) {
     const S* p;
     if (parity == 0 || i == 0 || flow_wall<L>(m, L::opp(i)))
-      p = reinterpret_cast<const S*>(planes[i]) + LBM_CHK(err, sn, pitch);
+      p = R::f(a, c, s, i);
     else
-      p = reinterpret_cast<const S*>(planes[L::opp(i)]) +
-          (long long)LBM_CHK(err, __ldg(slot + LBM_CHK(err, nb.at(-L::cx(i), -L::cy(i), -L::cz(i)), n_nodes)), pitch);
+      p = R::f(a, cell_of<R>(a, nb.at(-L::cx(i), -L::cy(i), -L::cz(i))), s, L::opp(i));
     out[i] = Store<S>::ld(p);
   }
 }
 
-template <class L, class S>
-__device__ __forceinline__ void gather_scal_pl(void* const* planes, long long sn,
-                                               const uint32_t* __restrict__ slot, uint32_t m,
-                                               const Nbr& nb, int parity, typename Store<S>::T* out,
-                                               int* err, long long n_nodes, long long pitch) {
+template <class L, class S, int NC, int NS>
+__device__ __forceinline__ void gather_scal(const Args& a, int s, long long c, uint32_t m, const Nbr& nb, int parity,
+                                            typename Store<S>::T* out) {
+  using R = Rec<L, S, NC, NS>;
+  using SC = typename R::SC;
 #pragma unroll
   for (int j = 0; j < L::QC; ++j) {
-    const S* p;
+    const SC* p;
     if (parity == 0 || j == 0 || MaskBits<L>::code(m, L::opp(j)) != 0)
-      p = reinterpret_cast<const S*>(planes[j]) + LBM_CHK(err, sn, pitch);
+      p = R::h(a, c, s, j);
     else
-      p = reinterpret_cast<const S*>(planes[L::opp(j)]) +
-          (long long)LBM_CHK(err, __ldg(slot + LBM_CHK(err, nb.at(-L::cx(j), -L::cy(j), -L::cz(j)), n_nodes)), pitch);
-    out[j] = Store<S>::ld(p);
+      p = R::h(a, cell_of<R>(a, nb.at(-L::cx(j), -L::cy(j), -L::cz(j))), s, L::opp(j));
+    out[j] = Store<SC>::ld(p);
   }
 }
 
 template <class T>
 __device__ __forceinline__ T scal_w(int j, const Coef<T>& k) { return j == 0 ? k.wc0 : k.wca; }
-
-template <class L, class S>
-__device__ __forceinline__ void gather_scal(const S* __restrict__ h, long long pitch, long long sn,
-                                            const uint32_t* __restrict__ slot, uint32_t m,
-                                            const Nbr& nb, int parity, typename Store<S>::T* out) {
-#pragma unroll
-  for (int j = 0; j < L::QC; ++j) {
-    const S* p;
-    if (parity == 0 || j == 0 || MaskBits<L>::code(m, L::opp(j)) != 0) {
-      p = h + (long long)j * pitch + sn;
-    } else {
-      p = h + (long long)L::opp(j) * pitch + __ldg(slot + nb.at(-L::cx(j), -L::cy(j), -L::cz(j)));
-    }
-    out[j] = Store<S>::ld(p);
-  }
-}
 
 // Wet-node closure (Eq. wetnode9 per link).  For direction j whose source n - c_j is a
 // reactive solid: C_b = 2 hb / (2 w + K), h_j = 2 w C_b - hb, hb = gathered h_{opp j}.
@@ -368,6 +406,24 @@ __device__ __forceinline__ void close_scalar(T* h, uint32_t m, const Coef<T>& k,
       const T hn = T(2) * k.wca * Cb - hb - sh;
       h[j] = hn;
       on_link(j, Cb, old[j] - hn);
+    }
+  }
+}
+
+// The same closure with its constants folded (h_j = cl1 hb, rate = cl2 hb), for the step kernels:
+// on_link(j, rate, exchange).
+template <class L, class T, class OnLink>
+__device__ __forceinline__ void close_rate(T* h, uint32_t m, const Coef<T>& k, OnLink on_link) {
+  T old[L::QC];
+#pragma unroll
+  for (int j = 0; j < L::QC; ++j) old[j] = h[j];
+  const T sh = k.wca * k.cref[0];
+#pragma unroll
+  for (int j = 1; j < L::QC; ++j) {
+    if (MaskBits<L>::code(m, L::opp(j)) == 2u) {
+      const T hb = old[L::opp(j)] + sh;
+      h[j] = fmad(k.cl1, hb, -sh);
+      on_link(j, k.cl2 * hb, old[j] - h[j]);
     }
   }
 }
@@ -556,44 +612,18 @@ __device__ __forceinline__ T warp_sum(T v) {
 #define LBM_TILES_MIN_BLOCKS_ODD 3  // k_step_tiles: odd parity, slots prefetched a tile ahead (as k_step)
 #endif
 
-// Neighbour offsets of fluid node n from its coordinates (fast divisions by nx and ny).
-__device__ __forceinline__ Nbr nbr_of(const Args& a, int n) {
-  const unsigned int q = fast_div(unsigned(n), a.div_x);
-  const unsigned int z = fast_div(q, a.div_y);
-  return make_nbr(a, n - int(q) * a.nx, int(q - z * unsigned(a.ny)), int(z));
-}
-
-// Stored populations of list entry e (node n, link mask m) as the node gathers them.
-template <class L, class S, int NC, int NS, int parity>
-__device__ __forceinline__ void gather_entry(const Args& a, unsigned int e, unsigned int base, int n,
-                                             uint32_t m, typename Store<S>::T (&f)[NC][L::Q],
-                                             typename Store<S>::T (&h)[NS > 0 ? NS : 1][L::QC]) {
-  const long long sn = e < base ? (long long)e : (long long)__ldg(a.slot + n);
-  const Nbr nb = parity ? nbr_of(a, n) : Nbr{};
-#pragma unroll
-  for (int s = 0; s < NC; ++s) gather_flow_pl<L, S>(a.fplane[s], sn, a.slot, m, nb, parity, f[s], a.err, a.N, a.pitch);
-#pragma unroll
-  for (int s = 0; s < NS; ++s)
-    gather_scal_pl<L, typename ScalarOf<S>::type>(a.hplane[s], sn, a.slot, m, nb, parity, h[s], a.err, a.N, a.pitch);
-}
-
-// Neighbour-slot cache of the odd step.  An odd step reads cell (n - c_i, opp i) and writes
-// cell (n + c_i, i): every neighbour slot it needs on the way in, it needs again on the way out,
-// and the scalar lattice's axis links use the flow lattice's neighbours.  The gather of the first
-// flow component looks each slot up once and keeps it in shared memory, entry i - 1 for the
-// neighbour n + c_i; the later gathers and the scatters read it back.  A scalar link to a fluid
-// neighbour is always a fluid flow link too, so every entry they read was written.
-#ifndef LBM_ODD_SLOT_CACHE
-#define LBM_ODD_SLOT_CACHE 1
-#endif
+// Neighbour cache of the odd step.  An odd step reads cell (n - c_i, opp i) and writes cell
+// (n + c_i, i): every neighbour it needs on the way in, it needs again on the way out, and the
+// scalar lattices' axis links use the flow lattice's neighbours.  One shared-memory entry per
+// direction k (entry k - 1, for the neighbour n + c_k) serves all of them.  The entries are copied
+// in asynchronously (cp.async) while the previous node of the thread computes: the byte offset of the
+// neighbour's cells (Args::off) for the plain kernels, its slot for the full ones.
+//
 // k_step keeps the cache as rows of LBM_STEP_CACHE_STRIDE threads per direction (consecutive
 // threads in consecutive words; its blocks have at most that many threads); the ensemble's
 // tile kernel gives each thread Q consecutive words of dynamic shared memory instead, sized
 // to its block (Q - 1 used; the odd stride puts the threads of a warp on distinct banks).
 #define LBM_STEP_CACHE_STRIDE 256
-#ifndef LBM_ODD_SLOT_PREFETCH
-#define LBM_ODD_SLOT_PREFETCH 1   // k_step: the slots of the next node are copied in while this one runs
-#endif
 // Asynchronous copies (cp.async, sm_80 and later) of one 4-byte word from global to shared
 // memory; a thread waits for its own groups with cp_async_wait.
 __device__ __forceinline__ void cp_async4(uint32_t* smem, const uint32_t* gmem) {
@@ -604,84 +634,92 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// Start copying the slots of all Q - 1 neighbours n + c_i of node n into the cache rows (row i
-// for n + c_i), one step of the grid-stride loop ahead of their use.  Links into walls copy a
-// slot that is never read (the periodic image is always a valid node).
+// Start copying the map's values of all Q - 1 neighbours n + c_i of a list entry's node into the
+// cache.  Links into walls copy a value that is never read (the periodic image is a valid node).
 template <class L, int CS>
-__device__ __forceinline__ void prefetch_slots(const Args& a, int n, uint32_t* cache) {
-  const Nbr nb = nbr_of(a, n);
+__device__ __forceinline__ void prefetch_nbrs(const Args& a, const uint32_t* map, uint32_t entry, uint32_t* cache) {
+  const int n = list_node(a, entry);
+  const Nbr nb = nbr_entry(a, n, entry);
 #pragma unroll
   for (int i = 1; i < L::Q; ++i)
-    cp_async4(cache + (i - 1) * CS, a.slot + LBM_CHK(a.err, nb.at(L::cx(i), L::cy(i), L::cz(i)), a.N));
+    cp_async4(cache + (i - 1) * CS, map + LBM_CHK(a.err, nb.at(L::cx(i), L::cy(i), L::cz(i)), a.N));
 }
 
-// Flow links into walls read and write the node's own cell: (n, i) for the population arriving
-// in direction i, which sits in plane i while a fluid link's cell sits in plane opp(i).  Writing
-// into a wall link's cache entry the offset of that own cell relative to the neighbour's plane,
-// slot + (opp(k) - k) * pitch, lets every flow access take plane + entry without testing the
-// link (signed 32-bit: needs 3 * pitch < 2^31, checked on the host).
-template <class L, int CS>
-__device__ __forceinline__ void wall_offsets(const Args& a, long long sn, uint32_t m, uint32_t* cache) {
+// Byte offsets in the cache are biased by kOffBias rows.  Flow links into walls read and write the
+// node's own cell: (n, i) for the population arriving in direction i, which sits in row i while
+// a fluid link's cell sits in row opp(i).  Writing into a wall link's cache entry the own offset moved
+// by opp(k) - k rows (at most two rows down, so the biased offset stays positive) lets every flow
+// access take row + entry without testing the link.
+constexpr int kOffBias = 4;
+template <class L, class R, int CS>
+__device__ __forceinline__ void wall_offsets(uint32_t own, uint32_t m, uint32_t* cache) {
 #pragma unroll
   for (int k = 1; k < L::Q; ++k)
-    if (flow_wall<L>(m, k)) cache[(k - 1) * CS] = (uint32_t)(int)(sn + (long long)(L::opp(k) - k) * a.pitch);
+    if (flow_wall<L>(m, k)) cache[(k - 1) * CS] = own + uint32_t((L::opp(k) - k) * R::FROW);
 }
 
-template <class L, class S, int NC, int NS, int CS, bool PREFETCHED = false, bool VOFF = false>
-__device__ __forceinline__ void gather_entry_odd_cached(const Args& a, long long sn, int n, uint32_t m,
-                                                        uint32_t* cache, typename Store<S>::T (&f)[NC][L::Q],
-                                                        typename Store<S>::T (&h)[NS > 0 ? NS : 1][L::QC]) {
-  const Nbr nb = PREFETCHED ? Nbr{} : nbr_of(a, n);
+// The cells an odd step reads and writes through cache entry k: flow row (s, k) and scalar row (s, k)
+// of the neighbour n + c_k, or of the own node behind a wall (rows opp(k)).
+template <class L, class S, int NC, int NS, int CS, bool BND>
+struct OddCells {
+  using R = Rec<L, S, NC, NS>;
+  using SC = typename R::SC;
+  static constexpr long long kBias = (long long)kOffBias * R::FROW;
+  const Args& a;
+  long long c;      // the node's own cells
+  uint32_t m;
+  const uint32_t* cache;
+  __device__ __forceinline__ S* flow(int s, int k) const {
+    if (!BND) return reinterpret_cast<S*>(a.pop + LBM_CHK(a.err, (long long)cache[(k - 1) * CS] + (R::frow(s, k) - kBias), a.pop_bytes));
+    if (flow_wall<L>(m, k)) return R::f(a, c, s, L::opp(k));
+    return R::f(a, R::cell((long long)LBM_CHK(a.err, cache[(k - 1) * CS], a.pitch)), s, k);
+  }
+  // A scalar link to a fluid neighbour is a fluid flow link and a wall or reactive link a flow wall,
+  // so the entry serves both; only an open face (x links) may be a fluid link of a periodic flow.
+  __device__ __forceinline__ SC* scal(int s, int k) const {
+    if (!BND && R::kSameElem) {
+      if (L::cx(k) != 0 && MaskBits<L>::code(m, k) == 3u) return R::h(a, c, s, L::opp(k));
+      return reinterpret_cast<SC*>(a.pop + LBM_CHK(a.err, (long long)cache[(k - 1) * CS] + (R::hrow(s, k) - kBias), a.pop_bytes));
+    }
+    if (MaskBits<L>::code(m, k) != 0u) return R::h(a, c, s, L::opp(k));
+    if (!BND) return R::h(a, (long long)cache[(k - 1) * CS] - kBias, s, k);
+    return R::h(a, R::cell((long long)LBM_CHK(a.err, cache[(k - 1) * CS], a.pitch)), s, k);
+  }
+};
+
+template <class L, class S, int NC, int NS, int CS, bool BND>
+__device__ __forceinline__ void gather_odd(const OddCells<L, S, NC, NS, CS, BND>& o, typename Store<S>::T (&f)[NC][L::Q],
+                                           typename Store<S>::T (&h)[NS > 0 ? NS : 1][L::QC]) {
+  using R = Rec<L, S, NC, NS>;
 #pragma unroll
   for (int s = 0; s < NC; ++s) {
+    f[s][0] = Store<S>::ld(R::f(o.a, o.c, s, 0));
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-      const S* p;
-      if (VOFF && i != 0) {
-        // the entry holds the plane-relative offset of the cell, own or neighbour (see
-        // wall_offsets)
-        const long long off = (long long)(int)cache[(L::opp(i) - 1) * CS];
-        const long long base_k = (long long)L::opp(i) * a.pitch;   // the plane's start in the array
-        p = reinterpret_cast<const S*>(a.fplane[s][L::opp(i)]) +
-            (LBM_CHK(a.err, off + base_k, (long long)L::Q * a.pitch) - base_k);
-      } else if (i == 0 || flow_wall<L>(m, L::opp(i))) {
-        p = reinterpret_cast<const S*>(a.fplane[s][i]) + LBM_CHK(a.err, sn, a.pitch);
-      } else {
-        uint32_t q;
-        if (s == 0 && PREFETCHED) {
-          q = (uint32_t)LBM_CHK(a.err, cache[(L::opp(i) - 1) * CS], a.pitch);
-        } else if (s == 0) {
-          q = (uint32_t)LBM_CHK(a.err, __ldg(a.slot + LBM_CHK(a.err, nb.at(-L::cx(i), -L::cy(i), -L::cz(i)), a.N)),
-                                a.pitch);
-          cache[(L::opp(i) - 1) * CS] = q;
-        } else {
-          q = cache[(L::opp(i) - 1) * CS];
-        }
-        p = reinterpret_cast<const S*>(a.fplane[s][L::opp(i)]) + q;
-      }
-      f[s][i] = Store<S>::ld(p);
-    }
+    for (int i = 1; i < L::Q; ++i) f[s][i] = Store<S>::ld(o.flow(s, L::opp(i)));
   }
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
+    h[s][0] = Store<typename R::SC>::ld(R::h(o.a, o.c, s, 0));
 #pragma unroll
-    for (int j = 0; j < L::QC; ++j) {
-      using SC = typename ScalarOf<S>::type;
-      const SC* p;
-      if (j == 0 || MaskBits<L>::code(m, L::opp(j)) != 0)
-        p = reinterpret_cast<const SC*>(a.hplane[s][j]) + LBM_CHK(a.err, sn, a.pitch);
-      else
-        p = reinterpret_cast<const SC*>(a.hplane[s][L::opp(j)]) + cache[(L::opp(j) - 1) * CS];
-      h[s][j] = Store<SC>::ld(p);
-    }
+    for (int j = 1; j < L::QC; ++j) h[s][j] = Store<typename R::SC>::ld(o.scal(s, L::opp(j)));
   }
 }
 
-// ------------------------------------------------------------- collision helpers
+template <class L, class S, int NC, int NS>
+__device__ __forceinline__ void gather_even(const Args& a, long long c, typename Store<S>::T (&f)[NC][L::Q],
+                                            typename Store<S>::T (&h)[NS > 0 ? NS : 1][L::QC]) {
+  using R = Rec<L, S, NC, NS>;
+#pragma unroll
+  for (int s = 0; s < NC; ++s)
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) f[s][i] = Store<S>::ld(R::f(a, c, s, i));
+#pragma unroll
+  for (int s = 0; s < NS; ++s)
+#pragma unroll
+    for (int j = 0; j < L::QC; ++j) h[s][j] = Store<typename R::SC>::ld(R::h(a, c, s, j));
+}
 
-// Fused multiply-add of the compute types.
-__device__ __forceinline__ float fmad(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fmad(double a, double b, double c) { return fma(a, b, c); }
+// ------------------------------------------------------------- collision helpers
 
 // MRT correction on top of the BGK update: with n = f - f_eq + F_i / 2 split into pair sums sp
 // and differences dp (indexed by the first member of each opposite pair, sp[0] = n_0),
@@ -730,80 +768,189 @@ __device__ __forceinline__ void mrt_correct_rows(T* f, const T* sp, const T* dp,
   }
 }
 
-// D3Q19: the same rows (d'Humieres et al. 2002) evaluated through the sums their polynomials
-// share: axis pairs 1, 3, 5 (x, y, z), diagonal classes xy {7, 13}, xz {9, 15}, yz {11, 17}.
-template <class T, class G>
-__device__ __forceinline__ void mrt_correct_d3q19(T* f, const T* sp, const T* dp, const G* g) {
-  // even moments (e, eps, 3 pi_xx, pi_ww) from pair sums
-  const T A = sp[1] + sp[3] + sp[5];
-  const T Dxy = sp[7] + sp[13], Dxz = sp[9] + sp[15], Dyz = sp[11] + sp[17];
-  const T D = Dxy + Dxz + Dyz;
-  const T m_e = fmad(T(-30), sp[0], fmad(T(-11), A, T(8) * D));
-  const T m_eps = fmad(T(12), sp[0], fmad(T(-4), A, D));
-  const T m_pxx = fmad(T(-4), sp[1], fmad(T(2), sp[3] + sp[5], fmad(T(-2), Dyz, Dxy + Dxz)));
-  const T m_pww = fmad(T(2), sp[5] - sp[3], Dxy - Dxz);
-  // odd moments (q, m) from pair differences
-  const T P = dp[7] + dp[13], Mxy = dp[7] - dp[13];
-  const T R = dp[9] + dp[15], Mxz = dp[9] - dp[15];
-  const T S = dp[11] + dp[17], Myz = dp[11] - dp[17];
-  const T m_qx = fmad(T(-4), dp[1], P + R), m_mx = P - R;
-  const T m_qy = fmad(T(-4), dp[3], Mxy + S), m_my = S - Mxy;
-  const T m_qz = fmad(T(-4), dp[5], Mxz + Myz), m_mz = Mxz - Myz;
-  // row order of g: e, eps, q_x, q_y, q_z, 3 pi_xx, pi_ww, m_x, m_y, m_z
-  const T ce = T(g[0]) * m_e, cs = T(g[1]) * m_eps;
-  const T cqx = T(g[2]) * m_qx, cqy = T(g[3]) * m_qy, cqz = T(g[4]) * m_qz;
-  const T cpx = T(g[5]) * m_pxx, cpw = T(g[6]) * m_pww;
-  const T cmx = T(g[7]) * m_mx, cmy = T(g[8]) * m_my, cmz = T(g[9]) * m_mz;
-  // redistribution: even part E of each pair, odd part O; f_i -= E + O, f_opp -= E - O
-  f[0] = fmad(T(30), ce, fmad(T(-12), cs, f[0]));
-  const T a0 = fmad(T(-11), ce, T(-4) * cs);
-  const T Ex = fmad(T(-4), cpx, a0);
-  const T t = fmad(T(2), cpx, a0);
-  const T Ey = fmad(T(-2), cpw, t), Ez = fmad(T(2), cpw, t);
-  f[1] = fmad(T(4), cqx, f[1] - Ex);
-  f[2] = fmad(T(-4), cqx, f[2] - Ex);
-  f[3] = fmad(T(4), cqy, f[3] - Ey);
-  f[4] = fmad(T(-4), cqy, f[4] - Ey);
-  f[5] = fmad(T(4), cqz, f[5] - Ez);
-  f[6] = fmad(T(-4), cqz, f[6] - Ez);
-  const T d0 = fmad(T(8), ce, cs);
-  const T Exy = d0 + (cpx + cpw), Exz = d0 + (cpx - cpw), Eyz = fmad(T(-2), cpx, d0);
-  const T u1 = cqx + cmx, v1 = cqy - cmy;   // pairs 7 (+x+y): u1 + v1, 13 (+x-y): u1 - v1
-  const T u2 = cqx - cmx, v2 = cqz + cmz;   // pairs 9 (+x+z): u2 + v2, 15 (+x-z): u2 - v2
-  const T u3 = cqy + cmy, v3 = cqz - cmz;   // pairs 11 (+y+z): u3 + v3, 17 (+y-z): u3 - v3
-  const T O7 = u1 + v1, O13 = u1 - v1, O9 = u2 + v2, O15 = u2 - v2, O11 = u3 + v3, O17 = u3 - v3;
-  f[7] = (f[7] - Exy) - O7;
-  f[8] = (f[8] - Exy) + O7;
-  f[13] = (f[13] - Exy) - O13;
-  f[14] = (f[14] - Exy) + O13;
-  f[9] = (f[9] - Exz) - O9;
-  f[10] = (f[10] - Exz) + O9;
-  f[15] = (f[15] - Exz) - O15;
-  f[16] = (f[16] - Exz) + O15;
-  f[11] = (f[11] - Eyz) - O11;
-  f[12] = (f[12] - Eyz) + O11;
-  f[17] = (f[17] - Eyz) - O17;
-  f[18] = (f[18] - Eyz) + O17;
+// The collision works on opposite pairs: for the first member i of a pair (i < opp i) f[i] holds
+// the sum f_i + f_opp and f[opp i] the difference f_i - f_opp (to_pairs).  Even moments, the
+// equilibrium's and the force's even parts touch only sums, odd ones only differences, and the
+// post-collision pair is E + O, E - O.
+template <class L, class T>
+__device__ __forceinline__ void to_pairs(T* f) {
+#pragma unroll
+  for (int i = 1; i < L::Q; ++i) {
+    const int o = L::opp(i);
+    if (i > o) continue;
+    const T x = f[i], y = f[o];
+    f[i] = x + y;
+    f[o] = x - y;
+  }
 }
-template <class L, class T, class G>
-__device__ __forceinline__ void mrt_correct(T* f, const T* sp, const T* dp, const G* g) {
-  if constexpr (L::Q == 19) mrt_correct_d3q19<T, G>(f, sp, dp, g);
-  else mrt_correct_rows<L, T, G>(f, sp, dp, g);
+template <class L, class T>
+__device__ __forceinline__ T cdot(int i, T x, T y, T z) {
+  T r = T(0);
+  bool first = true;
+  const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
+  const T v[3] = {x, y, z};
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (c[q] == 0) continue;
+    if (first) r = c[q] > 0 ? v[q] : -v[q];
+    else r = c[q] > 0 ? r + v[q] : r - v[q];
+    first = false;
+  }
+  return r;
+}
+
+// BGK of one component on pairs (Eq. 1.16, 1.21), f* = (1 - om) f + om f_eq + (1 - om/2) F.  With
+// b = (1 - om/2) F the odd part of the last two is 3 w c.o, o = om rho u + b, and the even part
+// w (om drho + 4.5 (c.u)(c.e) - 1.5 u.e), e = o + b: about 7 operations per pair.  Velocity-shift
+// forcing (Eq. 1.17, 1.18) is the same with b = 0 and its own u.  The factor 3 is applied to the
+// vector and not folded into the weights: 1/18, 1/36 and 1/9 round to FP32 within 7e-9, 1/6, 1/12 and
+// 1/3 only within 3e-8, which would change the momentum by that factor every step.
+template <class L, class T>
+__device__ __forceinline__ void bgk_pairs(T* f, T om, T hom, T drho, T rho, T ux, T uy, T uz, T bx, T by, T bz) {
+  const T wa = T(L::w(1)), wd = T(L::w(L::Q - 1));
+  const T ro = om * rho;
+  const T ox = fmad(ro, ux, bx), oy = fmad(ro, uy, by), oz = fmad(ro, uz, bz);
+  const T ex = ox + bx, ey = oy + by, ez = oz + bz;
+  const T K = fmad(om, drho, T(-1.5) * fmad(ux, ex, fmad(uy, ey, uz * ez)));
+  f[0] = fmad(T(2) * hom, f[0], T(L::w(0)) * K);
+  const T Ka = wa * K, Kd = wd * K;
+  const T a45 = T(4.5 * L::w(1)), d45 = T(4.5 * L::w(L::Q - 1));
+  const T o3x = T(3) * ox, o3y = T(3) * oy, o3z = T(3) * oz;
+#pragma unroll
+  for (int i = 1; i < L::Q; ++i) {
+    const int o = L::opp(i);
+    if (i > o) continue;
+    const bool axis = L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i) + L::cz(i) * L::cz(i) == 1;
+    const T cu = axis ? cdot<L>(i, a45 * ux, a45 * uy, a45 * uz) : cdot<L>(i, d45 * ux, d45 * uy, d45 * uz);
+    const T Ee = fmad(cu, cdot<L>(i, ex, ey, ez), axis ? Ka : Kd);
+    const T Eo = axis ? cdot<L>(i, wa * o3x, wa * o3y, wa * o3z) : cdot<L>(i, wd * o3x, wd * o3y, wd * o3z);
+    const T E = fmad(hom, f[i], Ee), O = fmad(hom, f[o], Eo);
+    f[i] = E + O;
+    f[o] = E - O;
+  }
+}
+
+// MRT with Guo forcing on pairs, generic rows: with G = f_eq - F/2 and H = f_eq + F/2, n = f - G
+// relaxes to f* = H + (1 - om) n - sum_k R_k g_k (R_k.n).  rho u = j + F/2 (one component).
+template <class L, class T, class K>
+__device__ __forceinline__ void mrt_pairs_rows(T* f, const K& k, T drho, T jx, T jy, T jz, T ux, T uy, T uz, T Fx, T Fy,
+                                               T Fz) {
+  const T ax = fmad(T(-0.5), Fx, jx), ay = fmad(T(-0.5), Fy, jy), az = fmad(T(-0.5), Fz, jz);   // rho u - F
+  const T bx = fmad(T(1.5), Fx, jx), by = fmad(T(1.5), Fy, jy), bz = fmad(T(1.5), Fz, jz);      // rho u + F
+  const T KG = fmad(T(-1.5), fmad(ux, ax, fmad(uy, ay, uz * az)), drho);
+  const T KH = fmad(T(-1.5), fmad(ux, bx, fmad(uy, by, uz * bz)), drho);
+  const T hom = k.hom[0];
+  T sp[L::Q], dp[L::Q];
+  sp[0] = f[0] - T(L::w(0)) * KG;
+  f[0] = fmad(T(2) * hom, sp[0], T(L::w(0)) * KH);
+#pragma unroll
+  for (int i = 1; i < L::Q; ++i) {
+    const int o = L::opp(i);
+    if (i > o) continue;
+    const T w = T(L::w(i));
+    const T cu = T(4.5) * cdot<L>(i, ux, uy, uz);
+    const T Ge = w * fmad(cu, cdot<L>(i, ax, ay, az), KG), He = w * fmad(cu, cdot<L>(i, bx, by, bz), KH);
+    const T Go = w * cdot<L>(i, T(3) * jx, T(3) * jy, T(3) * jz);
+    const T Ho = w * cdot<L>(i, T(3) * (jx + Fx), T(3) * (jy + Fy), T(3) * (jz + Fz));
+    sp[i] = fmad(T(-2), Ge, f[i]);
+    dp[i] = fmad(T(-2), Go, f[o]);
+    const T E = fmad(hom, sp[i], He), O = fmad(hom, dp[i], Ho);
+    f[i] = E + O;
+    f[o] = E - O;
+  }
+  mrt_correct_rows<L, T>(f, sp, dp, k.mrt_g);
+}
+
+// D3Q19 MRT (rows of d'Humieres et al. 2002) on pairs.  n has no momentum, and the nine odd moments are
+// j, q, m, so its odd part is the q and m projections alone: f*_o = f_o + 3 w c.F - s_q, s_m times
+// them, with q_x(n) = 5 (j_x / 3 - d_x), m_x(n) = P - R and the row norms 40 and 8.  The momentum stays in
+// f_o and is not rebuilt from j with rounded weights.  The even rows are
+// evaluated through the sums their polynomials share: axis pairs x, y, z and the diagonal classes.
+// About 240 operations in place of 460 for the BGK update of single populations with a correction.
+template <class T, class K>
+__device__ __forceinline__ void mrt_pairs_d3q19(T* f, const K& k, T drho, T jx, T jy, T jz, T ux, T uy, T uz, T Fx, T Fy,
+                                                T Fz) {
+  // odd part: row classes of the differences (directions 7 +x+y, 9 +x+z, 11 +y+z, 13 +x-y, 15 +x-z, 17 +y-z)
+  const T P = f[8] + f[14], Mxy = f[8] - f[14], R = f[10] + f[16], Mxz = f[10] - f[16], S = f[12] + f[18],
+          Myz = f[12] - f[18];
+  const T third = T(1.0 / 3.0), sixth = T(1.0 / 6.0), half6 = T(1.0 / 12.0), half = T(0.5);
+  const T cqx = k.oq * fmad(third, jx, -f[2]), cqy = k.oq * fmad(third, jy, -f[4]), cqz = k.oq * fmad(third, jz, -f[6]);
+  const T cmx = k.omm * (P - R), cmy = k.omm * (S - Mxy), cmz = k.omm * (Mxz - Myz);
+  const T Ox = fmad(half, f[2], fmad(T(4), cqx, sixth * Fx)), Oy = fmad(half, f[4], fmad(T(4), cqy, sixth * Fy)),
+          Oz = fmad(half, f[6], fmad(T(4), cqz, sixth * Fz));
+  const T qx = fmad(half6, Fx, -cqx), qy = fmad(half6, Fy, -cqy), qz = fmad(half6, Fz, -cqz);
+  const T u1 = qx - cmx, v1 = qy + cmy;   // pairs 7: u1 + v1, 13: u1 - v1
+  const T u2 = qx + cmx, v2 = qz - cmz;   // pairs 9: u2 + v2, 15: u2 - v2
+  const T u3 = qy - cmy, v3 = qz + cmz;   // pairs 11: u3 + v3, 17: u3 - v3
+  // even part: G and H share u, with a = rho u - F and b = rho u + F
+  const T ax = fmad(T(-0.5), Fx, jx), ay = fmad(T(-0.5), Fy, jy), az = fmad(T(-0.5), Fz, jz);
+  const T bx = fmad(T(1.5), Fx, jx), by = fmad(T(1.5), Fy, jy), bz = fmad(T(1.5), Fz, jz);
+  const T KG = fmad(T(-1.5), fmad(ux, ax, fmad(uy, ay, uz * az)), drho);
+  const T KH = fmad(T(-1.5), fmad(ux, bx, fmad(uy, by, uz * bz)), drho);
+  const T hom = k.hom[0];
+  const T n0 = fmad(T(-1.0 / 3.0), KG, f[0]);
+  // n sums: S - 2 w (KG + 4.5 (c.u)(c.a)), w = 1/18 and 1/36
+  const T g9 = T(-1.0 / 9.0) * KG, g18 = T(-1.0 / 18.0) * KG;
+  const T px = T(-0.5) * ux, py = T(-0.5) * uy, pz = T(-0.5) * uz;
+  const T sx = fmad(px, ax, f[1] + g9), sy = fmad(py, ay, f[3] + g9), sz = fmad(pz, az, f[5] + g9);
+  const T rx = T(-0.25) * ux, ry = T(-0.25) * uy, rz = T(-0.25) * uz;
+  const T c7 = rx + ry, c13 = rx - ry, c9 = rx + rz, c15 = rx - rz, c11 = ry + rz, c17 = ry - rz;
+  const T s7 = fmad(c7, ax + ay, f[7] + g18), s13 = fmad(c13, ax - ay, f[13] + g18);
+  const T s9 = fmad(c9, ax + az, f[9] + g18), s15 = fmad(c15, ax - az, f[15] + g18);
+  const T s11 = fmad(c11, ay + az, f[11] + g18), s17 = fmad(c17, ay - az, f[17] + g18);
+  const T A = sx + sy + sz;
+  const T Dxy = s7 + s13, Dxz = s9 + s15, Dyz = s11 + s17, Dx = Dxy + Dxz;
+  const T D = Dx + Dyz;
+  const T m_e = fmad(T(-30), n0, fmad(T(-11), A, T(8) * D));
+  const T m_eps = fmad(T(12), n0, fmad(T(-4), A, D));
+  const T m_pxx = fmad(T(-4), sx, fmad(T(2), sy + sz, fmad(T(-2), Dyz, Dx)));
+  const T m_pww = fmad(T(2), sz - sy, Dxy - Dxz);
+  const T ce = k.mrt_g[0] * m_e, cs = k.mrt_g[1] * m_eps, cpx = k.mrt_g[5] * m_pxx, cpw = k.mrt_g[6] * m_pww;
+  f[0] = fmad(T(30), ce, fmad(T(-12), cs, fmad(T(2) * hom, n0, third * KH)));
+  // E of a pair = H_e + (1 - om) n_e - (projections)
+  const T h18 = T(1.0 / 18.0) * KH, h36 = T(1.0 / 36.0) * KH;
+  const T a0 = fmad(T(11), ce, fmad(T(4), cs, h18));
+  const T t = fmad(T(-2), cpx, a0);
+  const T Ex = fmad(px, T(-0.5) * bx, fmad(hom, sx, fmad(T(4), cpx, a0)));
+  const T Ey = fmad(py, T(-0.5) * by, fmad(hom, sy, fmad(T(2), cpw, t)));
+  const T Ez = fmad(pz, T(-0.5) * bz, fmad(hom, sz, fmad(T(-2), cpw, t)));
+  f[1] = Ex + Ox;
+  f[2] = Ex - Ox;
+  f[3] = Ey + Oy;
+  f[4] = Ey - Oy;
+  f[5] = Ez + Oz;
+  f[6] = Ez - Oz;
+  const T d0 = fmad(T(-8), ce, h36 - cs);
+  const T dxy = d0 - (cpx + cpw), dxz = d0 - (cpx - cpw), dyz = fmad(T(2), cpx, d0);
+  const T qbx = T(-0.5) * bx, qby = T(-0.5) * by, qbz = T(-0.5) * bz;
+  auto pair = [&](int i, T base, T s, T cu, T cb, T uv) {
+    const T E = fmad(cu, cb, fmad(hom, s, base)), O = fmad(half, f[i + 1], uv);
+    f[i] = E + O;
+    f[i + 1] = E - O;
+  };
+  pair(7, dxy, s7, c7, qbx + qby, u1 + v1);
+  pair(13, dxy, s13, c13, qbx - qby, u1 - v1);
+  pair(9, dxz, s9, c9, qbx + qbz, u2 + v2);
+  pair(15, dxz, s15, c15, qbx - qbz, u2 - v2);
+  pair(11, dyz, s11, c11, qby + qbz, u3 + v3);
+  pair(17, dyz, s17, c17, qby - qbz, u3 - v3);
 }
 
 // Everything after the gather for one fluid node: wet-node closure and its bookkeeping,
-// deposition, moments, forces, velocity, flow and scalar collision, in-place scatter.
-template <class L, class S, int NC, int NS, int COLL, int parity, bool BND, bool CACHE = false, int CS = 1,
-          bool VOFF = false>
-__device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typename Store<S>::T>& k, int n,
-                                                uint32_t m, long long sn,
+// deposition, moments, forces, velocity, flow and scalar collision, in-place scatter.  entry: the
+// node's fluid-list entry; c: its cells; o: its odd cells (parity 1).
+template <class L, class S, int NC, int NS, int COLL, int parity, bool BND, int CS>
+__device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typename Store<S>::T>& k, uint32_t entry, int n,
+                                                uint32_t m, long long c, const OddCells<L, S, NC, NS, CS, BND>& o,
                                                 typename Store<S>::T (&f)[NC][L::Q],
                                                 typename Store<S>::T (&h)[NS > 0 ? NS : 1][L::QC],
                                                 typename Store<S>::T& wallx, typename Store<S>::T& heatx,
-                                                typename Store<S>::T& prodx, const uint32_t* cache = nullptr) {
+                                                typename Store<S>::T& prodx) {
   using T = typename Store<S>::T;
+  using R = Rec<L, S, NC, NS>;
+  using SC = typename R::SC;
   constexpr int Q = L::Q, QC = L::QC;
-  const Nbr nb = nbr_of(a, n);
+  const Nbr nb = nbr_entry(a, n, entry);
   // ---- wet-node closure of scalar 0 and reaction bookkeeping (Eq. wetnode9, reactO2)
   if (NS > 0) {
     // the consumed totals are reductions (no value returned): the threshold test runs in
@@ -812,30 +959,28 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
     T rl[QC];
 #pragma unroll
     for (int j = 0; j < QC; ++j) rl[j] = T(0);
+    const auto solid_of = [&](int j) { return LBM_CHK(a.err, nb.at(-L::cx(j), -L::cy(j), -L::cz(j)), a.N); };
     if (BND && NS > 1 && a.conjugate) {
       // conduction in the solid: the rate constant of the link's last exchange
       close_conjugate<L, T>(h[0], h[NS > 1 ? 1 : 0], m, k, a, nb,
                             reinterpret_cast<const T*>(a.gs[parity]), [&](int j, T r, T exch) {
-        const int src = LBM_CHK(a.err, nb.at(-L::cx(j), -L::cy(j), -L::cz(j)), a.N);
-        atomicAdd(a.acc + src, widen(r));
+        atomicAdd(a.acc + solid_of(j), widen(r));
         wallx += exch;
         rl[j] = r;
       });
     } else if (BND && NS > 1 && a.arrhenius) {
       // temperature-dependent rate and reaction heat (the full kernel variant only)
       close_thermal<L, T>(h[0], h[NS > 1 ? 1 : 0], m, k, a.n_it, [&](int j, T r, T exch, T heat) {
-        const int src = LBM_CHK(a.err, nb.at(-L::cx(j), -L::cy(j), -L::cz(j)), a.N);
-        atomicAdd(a.acc + src, widen(r));
+        atomicAdd(a.acc + solid_of(j), widen(r));
         wallx += exch;
         heatx += heat;
         rl[j] = r;
       });
-    } else {
-      close_scalar<L, T>(h[0], m, k, [&](int j, T Cb, T exch) {
-        const int src = LBM_CHK(a.err, nb.at(-L::cx(j), -L::cy(j), -L::cz(j)), a.N);
-        atomicAdd(a.acc + src, widen(k.kr * Cb));
+    } else if (MaskBits<L>::reactive(m) != 0u) {
+      close_rate<L, T>(h[0], m, k, [&](int j, T r, T exch) {
+        atomicAdd(a.acc + solid_of(j), widen(r));
         wallx += exch;
-        rl[j] = k.kr * Cb;
+        rl[j] = r;
       });
     }
     if (NS > 1 && a.product) close_product<L, T>(h[NS - 1], m, k, rl, prodx);
@@ -862,17 +1007,20 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
       }
     }
   }
-  // ---- moments (Eq. 1.7, 1.8): rho = rref + sum of deviations
+  // ---- moments (Eq. 1.7, 1.8): rho = rref + sum of deviations, from pair sums and differences
   T drho[NC], rho[NC], jx[NC], jy[NC], jz[NC];
 #pragma unroll
   for (int s = 0; s < NC; ++s) {
-    T r = T(0), ax = T(0), ay = T(0), az = T(0);
+    to_pairs<L, T>(f[s]);
+    T r = f[s][0], ax = T(0), ay = T(0), az = T(0);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
+    for (int i = 1; i < Q; ++i) {
+      if (i > L::opp(i)) continue;
+      const T d = f[s][L::opp(i)];
       r += f[s][i];
-      if (L::cx(i)) ax += T(L::cx(i)) * f[s][i];
-      if (L::cy(i)) ay += T(L::cy(i)) * f[s][i];
-      if (L::cz(i)) az += T(L::cz(i)) * f[s][i];
+      if (L::cx(i)) ax += T(L::cx(i)) * d;
+      if (L::cy(i)) ay += T(L::cy(i)) * d;
+      if (L::cz(i)) az += T(L::cz(i)) * d;
     }
     drho[s] = r;
     rho[s] = k.rref[s] + r;
@@ -957,52 +1105,16 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
       const T ex = nxs * iden + k.tau[s] * Fx[s] * ir;
       const T ey = nys * iden + k.tau[s] * Fy[s] * ir;
       const T ez = nzs * iden + k.tau[s] * Fz[s] * ir;
-#pragma unroll
-      for (int i = 0; i < Q; ++i)
-        f[s][i] -= k.om[s] * (f[s][i] - feq_dev<L, T>(i, rho[s], drho[s], ex, ey, ez));
+      bgk_pairs<L, T>(f[s], k.om[s], k.hom[s], drho[s], rho[s], ex, ey, ez, T(0), T(0), T(0));
     }
+  } else if (COLL == 1) {
+    if constexpr (Q == 19) mrt_pairs_d3q19<T>(f[0], k, drho[0], jx[0], jy[0], jz[0], ux, uy, uz, Fx[0], Fy[0], Fz[0]);
+    else mrt_pairs_rows<L, T>(f[0], k, drho[0], jx[0], jy[0], jz[0], ux, uy, uz, Fx[0], Fy[0], Fz[0]);
   } else {
-    // Eq. 1.16 with Guo forcing (Eq. 1.21): f* = f + F_i - omega (f - f_eq + F_i / 2), for BGK;
-    // MRT adds the projections of n = f - f_eq + F_i / 2 on the non-hydrodynamic groups with
-    // rate (s_g - 1/tau).  Opposite directions are handled as pairs: the equilibrium and the
-    // Guo term split into even and odd parts, even MRT rows see n_i + n_opp(i), odd rows see
-    // n_i - n_opp(i).
-    const T uu = ux * ux + uy * uy + uz * uz;
 #pragma unroll
     for (int s = 0; s < NC; ++s) {
-      const T om = k.om[s];
-      const T uF = ux * Fx[s] + uy * Fy[s] + uz * Fz[s];
-      T sp[Q], dp[Q];   // pair sums / differences of n (MRT only), index of the first member
-      {
-        // rest population
-        const T w0 = T(L::w(0));
-        const T fe = w0 * (drho[s] - rho[s] * T(1.5) * uu);
-        const T Fi = w0 * (T(-3) * uF);
-        const T nq = f[s][0] - fe + T(0.5) * Fi;
-        if (COLL == 1) sp[0] = nq;
-        f[s][0] = f[s][0] + Fi - om * nq;
-      }
-#pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        if (i > L::opp(i)) continue;
-        const int o = L::opp(i);
-        const T w = T(L::w(i));
-        const T cu = T(L::cx(i)) * ux + T(L::cy(i)) * uy + T(L::cz(i)) * uz;
-        const T cF = T(L::cx(i)) * Fx[s] + T(L::cy(i)) * Fy[s] + T(L::cz(i)) * Fz[s];
-        const T fe_e = w * (drho[s] + rho[s] * (T(4.5) * cu * cu - T(1.5) * uu));
-        const T fe_o = w * (T(3) * rho[s] * cu);
-        const T Fi_e = w * (T(9) * cu * cF - T(3) * uF);
-        const T Fi_o = w * (T(3) * cF);
-        const T nq_i = f[s][i] - (fe_e + fe_o) + T(0.5) * (Fi_e + Fi_o);
-        const T nq_o = f[s][o] - (fe_e - fe_o) + T(0.5) * (Fi_e - Fi_o);
-        if (COLL == 1) {
-          sp[i] = nq_i + nq_o;
-          dp[i] = nq_i - nq_o;
-        }
-        f[s][i] = f[s][i] + (Fi_e + Fi_o) - om * nq_i;
-        f[s][o] = f[s][o] + (Fi_e - Fi_o) - om * nq_o;
-      }
-      if (COLL == 1) mrt_correct<L>(f[s], sp, dp, k.mrt_g);
+      const T b = T(1) - T(0.5) * k.om[s];
+      bgk_pairs<L, T>(f[s], k.om[s], k.hom[s], drho[s], rho[s], ux, uy, uz, b * Fx[s], b * Fy[s], b * Fz[s]);
     }
   }
   // ---- scalar collision (Eq. therpop_species, therpopeq_species), u = physical velocity
@@ -1041,75 +1153,49 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
   }
 #pragma unroll
   for (int s = 0; s < NC; ++s) {
+    Store<S>::st(R::f(a, c, s, 0), f[s][0]);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      S* p;
+    for (int i = 1; i < Q; ++i) {
       T v = f[s][i];
       bool keep = true;
-      if (VOFF && i != 0) {
-        const long long off = (long long)(int)cache[(i - 1) * CS];
-        const long long base_k = (long long)i * a.pitch;   // the plane's start in the array
-        p = reinterpret_cast<S*>(a.fplane[s][i]) + (LBM_CHK(a.err, off + base_k, (long long)L::Q * a.pitch) - base_k);
-      } else if (parity == 0 || i == 0 || flow_wall<L>(m, i)) {
-        p = reinterpret_cast<S*>(a.fplane[s][L::opp(i)]) + LBM_CHK(a.err, sn, a.pitch);
-        if (BND) {
-          if (L::cx(i) < 0 && xin && flow_wall<L>(m, i))
-            v += T(6.0 * L::w(i)) * rho[s] * uin;
-          else if (L::cx(i) > 0 && xout)
-            keep = false;   // leaves through the outlet; the cell is written below with opp(i)
-          else if (L::cy(i) > 0 && top && flow_wall<L>(m, i))
-            v -= T(L::w(i)) * rho[s] * (T(L::cx(i)) * k.uw6[0] + T(L::cz(i)) * k.uw6[2] + k.uw6[1]);
-        }
-      } else {
-        if (CACHE)
-          p = reinterpret_cast<S*>(a.fplane[s][i]) + cache[(i - 1) * CS];
-        else
-          p = reinterpret_cast<S*>(a.fplane[s][i]) +
-              LBM_CHK(a.err, (long long)__ldg(a.slot + LBM_CHK(a.err, nb.at(L::cx(i), L::cy(i), L::cz(i)), a.N)), a.pitch);
+      if (BND && (parity == 0 || flow_wall<L>(m, i))) {
+        if (L::cx(i) < 0 && xin && flow_wall<L>(m, i))
+          v += T(6.0 * L::w(i)) * rho[s] * uin;
+        else if (L::cx(i) > 0 && xout)
+          keep = false;   // leaves through the outlet; the cell is written below with opp(i)
+        else if (L::cy(i) > 0 && top && flow_wall<L>(m, i))
+          v -= T(L::w(i)) * rho[s] * (T(L::cx(i)) * k.uw6[0] + T(L::cz(i)) * k.uw6[2] + k.uw6[1]);
       }
-      if (keep) Store<S>::st(p, v);
+      if (keep) Store<S>::st(parity ? o.flow(s, i) : R::f(a, c, s, L::opp(i)), v);
       // zero-gradient outlet: the population entering through x = nx - 1 with direction i
       // repeats the node's own post-collision f_i, in the cell where link opp(i) reflects
-      if (BND && L::cx(i) < 0 && xout)
-        Store<S>::st(reinterpret_cast<S*>(a.fplane[s][i]) + LBM_CHK(a.err, sn, a.pitch), f[s][i]);
+      if (BND && L::cx(i) < 0 && xout) Store<S>::st(R::f(a, c, s, i), f[s][i]);
     }
   }
   // ---- scatter scalars: bounce-back at walls, inlet ghost / zero-gradient outlet at open faces
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
+    Store<SC>::st(R::h(a, c, s, 0), h[s][0]);
 #pragma unroll
-    for (int j = 0; j < QC; ++j) {
-      using SC = typename ScalarOf<S>::type;
-      const uint32_t code = j == 0 ? 0u : MaskBits<L>::code(m, j);
+    for (int j = 1; j < QC; ++j) {
       T v = h[s][j];
-      SC* p;
-      if (code == 3u) {
-        // open face: the population arriving from outside replaces the one leaving
+      if (L::cx(j) != 0 && MaskBits<L>::code(m, j) == 3u) {   // only the x faces are open
+        // open face: the population arriving from outside replaces the one leaving, in the own
+        // cell (row opp(j))
         const int jb = L::opp(j);
+        const long long row = LBM_CHK(a.err, s * (a.ny * a.nz) + int(fast_div(unsigned(n), a.div_x)), 3ll * a.ny * a.nz);
         T b;
-        const T sh = k.wca * k.cref[s];
         if (L::cx(j) < 0) {
-          const T cu = T(L::cx(jb)) * ux + T(L::cy(jb)) * uy + T(L::cz(jb)) * uz;
-          b = k.wca * k.C_in[s] * (T(1) + cu * k.ics2c) - sh;
-          a.inflow_row[LBM_CHK(a.err, s * (a.ny * a.nz) + int(fast_div(unsigned(n), a.div_x)), 3ll * a.ny * a.nz)] +=
-              widen(b) - widen(v);
+          const T cu = T(L::cx(jb)) * ux;
+          b = k.wca * k.C_in[s] * (T(1) + cu * k.ics2c) - k.wca * k.cref[s];
+          a.inflow_row[row] += widen(b) - widen(v);
         } else {
           b = h[s][jb];
-          a.outflow_row[LBM_CHK(a.err, s * (a.ny * a.nz) + int(fast_div(unsigned(n), a.div_x)), 3ll * a.ny * a.nz)] +=
-              widen(v) - widen(b);
+          a.outflow_row[row] += widen(v) - widen(b);
         }
         v = b;
-        p = reinterpret_cast<SC*>(a.hplane[s][jb]) + LBM_CHK(a.err, sn, a.pitch);
-      } else if (parity == 0 || j == 0 || code != 0u) {
-        p = reinterpret_cast<SC*>(a.hplane[s][L::opp(j)]) + LBM_CHK(a.err, sn, a.pitch);
-      } else {
-        if (CACHE)
-          p = reinterpret_cast<SC*>(a.hplane[s][j]) + cache[(j - 1) * CS];
-        else
-          p = reinterpret_cast<SC*>(a.hplane[s][j]) +
-              LBM_CHK(a.err, (long long)__ldg(a.slot + LBM_CHK(a.err, nb.at(L::cx(j), L::cy(j), L::cz(j)), a.N)), a.pitch);
       }
-      Store<SC>::st(p, v);
+      Store<SC>::st(parity ? o.scal(s, j) : R::h(a, c, s, L::opp(j)), v);
     }
   }
 }
@@ -1122,82 +1208,66 @@ template <class L, class S, int NC, int NS, int COLL, int parity, bool BND>
 __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) == 4 ? (parity ? LBM_STEP_MIN_BLOCKS_ODD : LBM_STEP_MIN_BLOCKS) : 2)) k_step(const Args a, const Coef<typename Store<S>::T> k) {
   using T = typename Store<S>::T;
   constexpr int Q = L::Q, QC = L::QC, NSD = NS > 0 ? NS : 1;
+  using R = Rec<L, S, NC, NS>;
+  using O = OddCells<L, S, NC, NS, LBM_STEP_CACHE_STRIDE, BND>;
   T wallx = T(0), heatx = T(0), prodx = T(0);
   const unsigned int count = a.fluid_count[0];
   const unsigned int base = a.fluid_count[1];   // entries below it have slot == entry
   const unsigned int stride = gridDim.x * blockDim.x;
   unsigned int e = blockIdx.x * blockDim.x + threadIdx.x;
-  // Odd parity with two cache buffers: the neighbour slots of the next entry are copied
-  // asynchronously into one while the current entry works from the other.
-  constexpr bool kPrefetch = LBM_ODD_SLOT_CACHE && LBM_ODD_SLOT_PREFETCH && parity == 1;
-#if LBM_ODD_SLOT_CACHE && LBM_ODD_SLOT_PREFETCH
-  if (kPrefetch) {
-    __shared__ uint32_t slot_buf[kPrefetch ? 2 * (L::Q - 1) * LBM_STEP_CACHE_STRIDE : 1];
+  const auto cell = [&](unsigned int en, int n) { return R::cell(en < base ? (long long)en : (long long)__ldg(a.slot + n)); };
+  // the list entry is fetched two iterations and the link mask one iteration ahead
+  uint32_t w_cur = e < count ? a.fluid_list[e] : 0u;
+  uint32_t w_nx = e + stride < count ? a.fluid_list[e + stride] : 0u;
+  uint32_t m_cur = e < count ? a.mask[list_node(a, w_cur)] : 0u;
+  if constexpr (parity == 1) {
+    // two cache buffers: the neighbours of the next entry are copied asynchronously into one while
+    // the current entry works from the other
+    __shared__ uint32_t slot_buf[2 * (L::Q - 1) * LBM_STEP_CACHE_STRIDE];
     uint32_t* cb = slot_buf + threadIdx.x;
     uint32_t* cn = slot_buf + (L::Q - 1) * LBM_STEP_CACHE_STRIDE + threadIdx.x;
-    int n_cur = e < count ? int(LBM_CHK(a.err, a.fluid_list[e], a.N)) : 0;
-    int n_nx = e + stride < count ? int(LBM_CHK(a.err, a.fluid_list[e + stride], a.N)) : 0;
-    uint32_t m_cur = e < count ? a.mask[n_cur] : 0u;
-    if (e < count) prefetch_slots<L, LBM_STEP_CACHE_STRIDE>(a, n_cur, cb);
+    const uint32_t* map = BND ? a.slot : a.off;
+    if (e < count) prefetch_nbrs<L, LBM_STEP_CACHE_STRIDE>(a, map, w_cur, cb);
     cp_async_commit();
     for (; e < count; e += stride) {
-      const int n = n_cur;
-      const uint32_t m = m_cur;
+      const uint32_t w = w_cur, m = m_cur;
       if (e + stride < count) {
-        n_cur = n_nx;
-        m_cur = a.mask[n_cur];
-        prefetch_slots<L, LBM_STEP_CACHE_STRIDE>(a, n_cur, cn);
+        w_cur = w_nx;
+        m_cur = a.mask[list_node(a, w_cur)];
+        prefetch_nbrs<L, LBM_STEP_CACHE_STRIDE>(a, map, w_cur, cn);
       }
-      if (e + 2 * stride < count) n_nx = int(LBM_CHK(a.err, a.fluid_list[e + 2 * stride], a.N));
+      if (e + 2 * stride < count) w_nx = a.fluid_list[e + 2 * stride];
       cp_async_commit();
-      cp_async_wait<1>();   // this entry's slots have arrived
+      cp_async_wait<1>();   // this entry's neighbours have arrived
       if (m & 1u) {
         T f[NC][Q], h[NSD][QC];
-        const long long sn = e < base ? (long long)e : (long long)__ldg(a.slot + n);
+        const int n = list_node(a, w);
+        const long long c = cell(e, n);
         // the plain variant addresses every flow link through its cache entry (wall_offsets);
         // the full variant keeps the per-link tests its boundary rules need
-        if (!BND) wall_offsets<L, LBM_STEP_CACHE_STRIDE>(a, sn, m, cb);
-        gather_entry_odd_cached<L, S, NC, NS, LBM_STEP_CACHE_STRIDE, true, !BND>(a, sn, n, m, cb, f, h);
-        collide_scatter<L, S, NC, NS, COLL, parity, BND, true, LBM_STEP_CACHE_STRIDE, !BND>(a, k, n, m, sn, f, h, wallx,
-                                                                                          heatx, prodx, cb);
+        if (!BND) wall_offsets<L, R, LBM_STEP_CACHE_STRIDE>(uint32_t(c) + uint32_t(kOffBias * R::FROW), m, cb);
+        const O o{a, c, m, cb};
+        gather_odd<L, S, NC, NS, LBM_STEP_CACHE_STRIDE, BND>(o, f, h);
+        collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, k, w, n, m, c, o, f, h, wallx, heatx, prodx);
       }
       uint32_t* t = cb;
       cb = cn;
       cn = t;
     }
     cp_async_wait<0>();
-  } else
-#endif
-  {
-#if LBM_ODD_SLOT_CACHE
-  __shared__ uint32_t slot_cache[(parity && !kPrefetch) ? (L::Q - 1) * LBM_STEP_CACHE_STRIDE : 1];
-  uint32_t* cache = slot_cache + threadIdx.x;
-#endif
-  // the list entry is fetched two iterations and the link mask one iteration ahead
-  int n_next = e < count ? int(LBM_CHK(a.err, a.fluid_list[e], a.N)) : 0;
-  int n_next2 = e + stride < count ? int(LBM_CHK(a.err, a.fluid_list[e + stride], a.N)) : 0;
-  uint32_t m_next = e < count ? a.mask[n_next] : 0u;
-  for (; e < count; e += stride) {
-    const int n = n_next;
-    const uint32_t m = m_next;
-    n_next = n_next2;
-    if (e + stride < count) m_next = a.mask[n_next];
-    if (e + 2 * stride < count) n_next2 = int(LBM_CHK(a.err, a.fluid_list[e + 2 * stride], a.N));
-    if (!(m & 1u)) continue;   // a node removed by deposition since the last list rebuild
-    T f[NC][Q], h[NSD][QC];
-#if LBM_ODD_SLOT_CACHE
-    if (parity) {
-      const long long sn = e < base ? (long long)e : (long long)__ldg(a.slot + n);
-      gather_entry_odd_cached<L, S, NC, NS, LBM_STEP_CACHE_STRIDE>(a, sn, n, m, cache, f, h);
-      collide_scatter<L, S, NC, NS, COLL, parity, BND, true, LBM_STEP_CACHE_STRIDE>(a, k, n, m, sn, f, h, wallx, heatx,
-                                                                                    prodx, cache);
-      continue;
+  } else {
+    for (; e < count; e += stride) {
+      const uint32_t w = w_cur, m = m_cur;
+      w_cur = w_nx;
+      if (e + stride < count) m_cur = a.mask[list_node(a, w_cur)];
+      if (e + 2 * stride < count) w_nx = a.fluid_list[e + 2 * stride];
+      if (!(m & 1u)) continue;   // a node removed by deposition since the last list rebuild
+      T f[NC][Q], h[NSD][QC];
+      const int n = list_node(a, w);
+      const long long c = cell(e, n);
+      gather_even<L, S, NC, NS>(a, c, f, h);
+      collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, k, w, n, m, c, O{a, c, m, nullptr}, f, h, wallx, heatx, prodx);
     }
-#endif
-    gather_entry<L, S, NC, NS, parity>(a, e, base, n, m, f, h);
-    const long long sn = e < base ? (long long)e : (long long)__ldg(a.slot + n);
-    collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, k, n, m, sn, f, h, wallx, heatx, prodx);
-  }
   }
   // ---- wall-exchange monitor: one reduction per warp that saw a reactive link
   if (NS > 0) {
@@ -1256,10 +1326,10 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   static_assert(sizeof(Args) % 4 == 0 && sizeof(Coef<T>) % 4 == 0, "word copies");
   __shared__ Args sa;
   __shared__ Coef<T> sk;
-#if LBM_ODD_SLOT_CACHE
-  extern __shared__ uint32_t slot_smem[];   // blockDim.x * Q words at odd parity (launcher)
+  using R = Rec<L, S, NC, NS>;
+  using O = OddCells<L, S, NC, NS, 1, BND>;
+  extern __shared__ uint32_t slot_smem[];   // 2 * blockDim.x * Q words at odd parity (launcher)
   uint32_t* cache = slot_smem + threadIdx.x * L::Q;
-#endif
   // blocks take chunks of LBM_TILE_CHUNK consecutive tiles in turn: the work list holds each
   // member's tiles together, so a chunk mostly stays within one member and its arguments are
   // staged again only when the chunk crosses into another; taking chunks in turn keeps a mix of
@@ -1267,15 +1337,12 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   auto next_tile = [&](unsigned int t) {
     return t + ((t % LBM_TILE_CHUNK == LBM_TILE_CHUNK - 1) ? (gridDim.x - 1) * LBM_TILE_CHUNK + 1 : 1);
   };
-#if LBM_ODD_SLOT_CACHE
-  // odd parity: two slot buffers, the next tile's neighbour slots are copied in (cp.async)
+  // odd parity: two neighbour buffers, the next tile's are copied in (cp.async)
   // while this tile computes, as in k_step; the next tile's list entry and link mask are loaded
   // one tile ahead at both parities whenever it belongs to the member already staged
   uint32_t* cn = slot_smem + (blockDim.x + threadIdx.x) * L::Q;
-#endif
   bool have_next = false;
-  int n_pf = 0;
-  uint32_t m_pf = 0u;
+  uint32_t w_pf = 0u, m_pf = 0u;
   unsigned int staged = 0xffffffffu;
   for (unsigned int t = blockIdx.x * LBM_TILE_CHUNK; t < ntiles; t = next_tile(t)) {
     const Tile tile = tiles[t];
@@ -1292,24 +1359,20 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
       have_next = false;
     }
     const Args& a = sa;
+    const uint32_t* map = BND ? a.slot : a.off;
     T wallx = T(0), heatx = T(0), prodx = T(0);
     const unsigned int e = tile.first + threadIdx.x;
     const unsigned int count = a.fluid_count[0];
-    int n = 0;
-    uint32_t m = 0u;
+    uint32_t w = 0u, m = 0u;
     if (have_next) {
-      n = n_pf;
+      w = w_pf;
       m = m_pf;
     } else if (e < count) {
-      n = int(LBM_CHK(a.err, a.fluid_list[e], a.N));
-      m = a.mask[n];
-#if LBM_ODD_SLOT_CACHE
-      if (parity) prefetch_slots<L, 1>(a, n, cache);
-#endif
+      w = a.fluid_list[e];
+      m = a.mask[list_node(a, w)];
+      if (parity) prefetch_nbrs<L, 1>(a, map, w, cache);
     }
-#if LBM_ODD_SLOT_CACHE
     if (parity) cp_async_commit();
-#endif
     // the next tile of this block, if it belongs to the staged member
     have_next = false;
     const unsigned int tn = next_tile(t);
@@ -1317,49 +1380,40 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
       const Tile tile2 = tiles[tn];
       if (tile2.member == staged) {
         const unsigned int e2 = tile2.first + threadIdx.x;
-        n_pf = 0;
+        w_pf = 0u;
         m_pf = 0u;
         if (e2 < count) {
-          n_pf = int(LBM_CHK(a.err, a.fluid_list[e2], a.N));
-          m_pf = a.mask[n_pf];
-#if LBM_ODD_SLOT_CACHE
-          if (parity) prefetch_slots<L, 1>(a, n_pf, cn);
-#endif
+          w_pf = a.fluid_list[e2];
+          m_pf = a.mask[list_node(a, w_pf)];
+          if (parity) prefetch_nbrs<L, 1>(a, map, w_pf, cn);
         }
         have_next = true;
       }
     }
-#if LBM_ODD_SLOT_CACHE
     if (parity) {
       cp_async_commit();
-      cp_async_wait<1>();   // this tile's slots have arrived
+      cp_async_wait<1>();   // this tile's neighbours have arrived
     }
-#endif
     if (e < count && (m & 1u)) {
       const unsigned int base = a.fluid_count[1];
       T f[NC][Q], h[NSD][QC];
-      const long long sn = e < base ? (long long)e : (long long)__ldg(a.slot + n);
-#if LBM_ODD_SLOT_CACHE
+      const int n = list_node(a, w);
+      const long long c = R::cell(e < base ? (long long)e : (long long)__ldg(a.slot + n));
+      const O o{a, c, m, cache};
       if (parity) {
         // the plain variant addresses every flow link through its cache entry (wall_offsets)
-        if (!BND) wall_offsets<L, 1>(a, sn, m, cache);
-        gather_entry_odd_cached<L, S, NC, NS, 1, true, !BND>(a, sn, n, m, cache, f, h);
-        collide_scatter<L, S, NC, NS, COLL, parity, BND, true, 1, !BND>(a, sk, n, m, sn, f, h, wallx, heatx, prodx,
-                                                                         cache);
-      } else
-#endif
-      {
-        gather_entry<L, S, NC, NS, parity>(a, e, base, n, m, f, h);
-        collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, sk, n, m, sn, f, h, wallx, heatx, prodx);
+        if (!BND) wall_offsets<L, R, 1>(uint32_t(c) + uint32_t(kOffBias * R::FROW), m, cache);
+        gather_odd<L, S, NC, NS, 1, BND>(o, f, h);
+      } else {
+        gather_even<L, S, NC, NS>(a, c, f, h);
       }
+      collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, sk, w, n, m, c, o, f, h, wallx, heatx, prodx);
     }
-#if LBM_ODD_SLOT_CACHE
     if (parity) {
       uint32_t* tmp = cache;
       cache = cn;
       cn = tmp;
     }
-#endif
     if (NS > 0) {
       const unsigned int any = __ballot_sync(0xffffffffu, wallx != T(0));
       if (any) {
@@ -1387,45 +1441,41 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
       }
     }
   }
-#if LBM_ODD_SLOT_CACHE
   if (parity) cp_async_wait<0>();
-#endif
 }
 
 // ================================================================ psi
 
-template <class L, class S, int NC, int parity>
+template <class L, class S, int NC, int NS, int parity>
 __global__ void __launch_bounds__(256) k_psi(const Args a, const Coef<typename Store<S>::T> k) {
   // Walks the fluid list in slot order, as k_step does: at parity 0 every population of the
   // node sits in its own cell (coalesced); at parity 1 population i sits in cell (n - c_i, opp i),
   // whose slot is looked up once for all components.  Sums in population order 0 .. Q-1 from
   // rho_ref, the order the gather of the step uses.
   using T = typename Store<S>::T;
+  using R = Rec<L, S, NC, NS>;
   const unsigned int count = a.fluid_count[0];
   const unsigned int base = a.fluid_count[1];   // entries below it have slot == entry
   const unsigned int stride = gridDim.x * blockDim.x;
   for (unsigned int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += stride) {
-    const int n = int(LBM_CHK(a.err, a.fluid_list[e], a.N));
+    const uint32_t w = a.fluid_list[e];
+    const int n = list_node(a, w);
     const uint32_t m = a.mask[n];
     if (!(m & 1u)) continue;   // a node removed by deposition since the last list rebuild
-    const long long sn = e < base ? (long long)e : (long long)__ldg(a.slot + n);
-    long long cell[L::Q];   // slot of the cell holding population i
-    const Nbr nb = parity ? nbr_of(a, n) : Nbr{};
+    const long long c = R::cell(e < base ? (long long)e : (long long)__ldg(a.slot + n));
+    long long cell[L::Q];   // offset of the row holding population i of component 0
+    const Nbr nb = parity ? nbr_entry(a, n, w) : Nbr{};
 #pragma unroll
     for (int i = 0; i < L::Q; ++i)
       cell[i] = (parity == 0 || i == 0 || flow_wall<L>(m, L::opp(i)))
-                    ? sn
-                    : (long long)__ldg(a.slot + LBM_CHK(a.err, nb.at(-L::cx(i), -L::cy(i), -L::cz(i)), a.N));
+                    ? c + R::frow(0, i)
+                    : cell_of<R>(a, nb.at(-L::cx(i), -L::cy(i), -L::cz(i))) + R::frow(0, L::opp(i));
 #pragma unroll
     for (int s = 0; s < NC; ++s) {
       T r = k.rref[s];
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i) {
-        // the own cell in plane i, a neighbour's in plane opp(i)
-        const bool own = parity == 0 || i == 0 || flow_wall<L>(m, L::opp(i));
-        const S* p = reinterpret_cast<const S*>(own ? a.fplane[s][i] : a.fplane[s][L::opp(i)]);
-        r += Store<S>::ld(p + LBM_CHK(a.err, cell[i], a.pitch));
-      }
+      for (int i = 0; i < L::Q; ++i)
+        r += Store<S>::ld(reinterpret_cast<const S*>(a.pop + LBM_CHK(a.err, cell[i] + s * L::Q * R::FROW, a.pop_bytes)));
       T p;
       if (a.psi_identity) p = r;
       else p = k.rho0 * (T(1) - exp(-r / k.rho0));   // Eq. 1.11
@@ -1476,17 +1526,18 @@ __global__ void __launch_bounds__(256) k_monitor(const Args a, const Coef<typena
   unsigned int nfluid = 0, nonfin = 0;
   const unsigned int count = a.fluid_count[0], base = a.fluid_count[1];
   for (unsigned int e = tid; e < count; e += nthr) {
-    const int n = int(a.fluid_list[e]);
+    const uint32_t w = a.fluid_list[e];
+    const int n = list_node(a, w);
     const uint32_t m = a.mask[n];
     if (!(m & 1u)) continue;
     ++nfluid;
-    const Nbr nb = parity ? nbr_of(a, n) : Nbr{};
-    const long long sn = e < base ? (long long)e : (long long)a.slot[n];
+    const Nbr nb = parity ? nbr_entry(a, n, w) : Nbr{};
+    const long long cell = Rec<L, S, NC, NS>::cell(e < base ? (long long)e : (long long)a.slot[n]);
     bool bad = false;
 #pragma unroll
     for (int s = 0; s < NC; ++s) {
       T f[Q];
-      gather_flow_pl<L, S>(a.fplane[s], sn, a.slot, m, nb, parity, f, a.err, a.N, a.pitch);
+      gather_flow<L, S, NC, NS>(a, s, cell, m, nb, parity, f);
       T r = T(0);
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
@@ -1501,7 +1552,7 @@ __global__ void __launch_bounds__(256) k_monitor(const Args a, const Coef<typena
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
       T h[QC];
-      gather_scal_pl<L, typename ScalarOf<S>::type>(a.hplane[s], sn, a.slot, m, nb, parity, h, a.err, a.N, a.pitch);
+      gather_scal<L, S, NC, NS>(a, s, cell, m, nb, parity, h);
       T c = T(0);
 #pragma unroll
       for (int j = 0; j < QC; ++j) c += h[j];
@@ -1561,17 +1612,16 @@ __global__ void __launch_bounds__(256) k_monitor(const Args a, const Coef<typena
 // rho^sigma, physical velocity (Eq. 1.19) and closed scalars of fluid node n; psi arrays must be
 // current when Shan-Chen forces are on.
 template <class L, class S, int NC, int NS>
-__device__ __forceinline__ void node_macros(const Args& a, const Coef<typename Store<S>::T>& k, int n,
-                                            uint32_t m, long long sn, int parity, typename Store<S>::T* rho_out,
+__device__ __forceinline__ void node_macros(const Args& a, const Coef<typename Store<S>::T>& k, int n, const Nbr& nb,
+                                            uint32_t m, long long cell, int parity, typename Store<S>::T* rho_out,
                                             typename Store<S>::T* u_out, typename Store<S>::T* C_out) {
   using T = typename Store<S>::T;
   constexpr int Q = L::Q, QC = L::QC;
-  const Nbr nb = nbr_of(a, n);
   T rho[NC], jx[NC], jy[NC], jz[NC], Fx[NC], Fy[NC], Fz[NC];
 #pragma unroll
   for (int s = 0; s < NC; ++s) {
     T f[Q];
-    gather_flow_pl<L, S>(a.fplane[s], sn, a.slot, m, nb, parity, f, a.err, a.N, a.pitch);
+    gather_flow<L, S, NC, NS>(a, s, cell, m, nb, parity, f);
     T r = T(0), ax = T(0), ay = T(0), az = T(0);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -1630,7 +1680,7 @@ __device__ __forceinline__ void node_macros(const Args& a, const Coef<typename S
   T hh[NS > 0 ? NS : 1][QC];
 #pragma unroll
   for (int s = 0; s < NS; ++s)
-    gather_scal_pl<L, typename ScalarOf<S>::type>(a.hplane[s], sn, a.slot, m, nb, parity, hh[s], a.err, a.N, a.pitch);
+    gather_scal<L, S, NC, NS>(a, s, cell, m, nb, parity, hh[s]);
   T rl[QC], gain = T(0);
 #pragma unroll
   for (int j = 0; j < QC; ++j) rl[j] = T(0);
@@ -1662,7 +1712,7 @@ __global__ void __launch_bounds__(256) k_moments(const Args a, const Coef<typena
   const uint32_t m = a.mask[n];
   T rho[NC], u[3], C[NS > 0 ? NS : 1];
   if (m & 1u) {
-    node_macros<L, S, NC, NS>(a, k, int(n), m, (long long)a.slot[n], parity, rho, u, C);
+    node_macros<L, S, NC, NS>(a, k, int(n), nbr_of(a, int(n)), m, Rec<L, S, NC, NS>::cell(a.slot[n]), parity, rho, u, C);
   } else {
     for (int s = 0; s < NC; ++s) rho[s] = T(0);
     u[0] = u[1] = u[2] = T(0);
@@ -1693,12 +1743,13 @@ __global__ void __launch_bounds__(256) k_resid(const Args a, const Coef<typename
   T du = T(0), uu = T(0), dc = T(0), cc = T(0);
   const unsigned int count = a.fluid_count[0], base = a.fluid_count[1];
   for (unsigned int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) {
-    const int n = int(a.fluid_list[e]);
+    const uint32_t w = a.fluid_list[e];
+    const int n = list_node(a, w);
     const uint32_t m = a.mask[n];
     if (!(m & 1u)) continue;
     const long long sn = e < base ? (long long)e : (long long)a.slot[n];
     T rho[NC], u[3], C[NS > 0 ? NS : 1];
-    node_macros<L, S, NC, NS>(a, k, n, m, sn, parity, rho, u, C);
+    node_macros<L, S, NC, NS>(a, k, n, nbr_entry(a, n, w), m, Rec<L, S, NC, NS>::cell(sn), parity, rho, u, C);
     for (int c = 0; c < 3; ++c) {
       const T d = u[c] - snap[c * P + sn];
       du += d * d;
@@ -1726,21 +1777,20 @@ __global__ void __launch_bounds__(256) k_init(const Args a, const Coef<typename 
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (n >= a.N) return;
   const bool fluid = a.flags[n] == FL_FLUID;
-  const long long sn = a.slot[n];
+  using R = Rec<L, S, NC, NS>;
+  const long long c = R::cell(a.slot[n]);
   const T ux = T(a.d_u[n]), uy = T(a.d_u[a.N + n]), uz = (L::D == 3) ? T(a.d_u[2 * a.N + n]) : T(0);
   for (int s = 0; s < NC; ++s) {
-    S* fs = reinterpret_cast<S*>(a.f[s]);
     const T r = T(a.d_rho[s * a.N + n]);
     const T dr = T(a.d_rho[s * a.N + n] - double(k.rref[s]));
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
       const T v = fluid ? feq_dev<L, T>(i, r, dr, ux, uy, uz) : T(0);
-      Store<S>::st(fs + (long long)i * a.pitch + sn, v);
+      Store<S>::st(R::f(a, c, s, i), v);
     }
   }
   for (int s = 0; s < NS; ++s) {
-    using SC = typename ScalarOf<S>::type;
-    SC* hs = reinterpret_cast<SC*>(a.h[s]);
+    using SC = typename R::SC;
     const T C = T(a.d_C[s * a.N + n]);
     const T dC = T(a.d_C[s * a.N + n] - double(k.cref[s]));
 #pragma unroll
@@ -1748,7 +1798,7 @@ __global__ void __launch_bounds__(256) k_init(const Args a, const Coef<typename 
       const T cu = T(L::cx(j)) * ux + T(L::cy(j)) * uy + T(L::cz(j)) * uz;
       const T wj = scal_w<T>(j, k);
       const T v = fluid ? wj * (dC + C * cu * k.ics2c) : T(0);
-      Store<SC>::st(hs + (long long)j * a.pitch + sn, v);
+      Store<SC>::st(R::h(a, c, s, j), v);
     }
   }
 }
@@ -1769,11 +1819,11 @@ __global__ void __launch_bounds__(256) k_pops_io(const Args a, const Coef<typena
   const uint32_t m = a.mask[n];
   const bool fluid = (m & 1u) != 0u;
   const Nbr nb = make_nbr(a, x, y, z);
-  const long long N = a.N, P = a.pitch;
-  const long long sn = a.slot[n];
+  using R = Rec<L, S, NC, NS>;
+  const long long N = a.N;
+  const long long c = R::cell(a.slot[n]);
   if (fio) {
     for (int s = 0; s < NC; ++s) {
-      S* fs = reinterpret_cast<S*>(a.f[s]);
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) {
         double* io = fio + ((long long)s * L::Q + i) * N + n;
@@ -1783,9 +1833,9 @@ __global__ void __launch_bounds__(256) k_pops_io(const Args a, const Coef<typena
         }
         S* p;
         if (parity == 0 || i == 0 || flow_wall<L>(m, L::opp(i)))
-          p = fs + (long long)i * P + sn;
+          p = R::f(a, c, s, i);
         else
-          p = fs + (long long)L::opp(i) * P + a.slot[nb.at(-L::cx(i), -L::cy(i), -L::cz(i))];
+          p = R::f(a, cell_of<R>(a, nb.at(-L::cx(i), -L::cy(i), -L::cz(i))), s, L::opp(i));
         const double sh = L::w(i) * double(k.rref[s]);
         if (dir == 0) *io = double(Store<S>::ldv(p)) + sh;
         else Store<S>::st(p, T(*io - sh));
@@ -1793,9 +1843,8 @@ __global__ void __launch_bounds__(256) k_pops_io(const Args a, const Coef<typena
     }
   }
   if (hio) {
-    using SC = typename ScalarOf<S>::type;
+    using SC = typename R::SC;
     for (int s = 0; s < NS; ++s) {
-      SC* hs = reinterpret_cast<SC*>(a.h[s]);
 #pragma unroll
       for (int j = 0; j < L::QC; ++j) {
         double* io = hio + ((long long)s * L::QC + j) * N + n;
@@ -1805,9 +1854,9 @@ __global__ void __launch_bounds__(256) k_pops_io(const Args a, const Coef<typena
         }
         SC* p;
         if (parity == 0 || j == 0 || MaskBits<L>::code(m, L::opp(j)) != 0u)
-          p = hs + (long long)j * P + sn;
+          p = R::h(a, c, s, j);
         else
-          p = hs + (long long)L::opp(j) * P + a.slot[nb.at(-L::cx(j), -L::cy(j), -L::cz(j))];
+          p = R::h(a, cell_of<R>(a, nb.at(-L::cx(j), -L::cy(j), -L::cz(j))), s, L::opp(j));
         const double sh = double(scal_w<T>(j, k)) * double(k.cref[s]);
         if (dir == 0) *io = double(Store<SC>::ldv(p)) + sh;
         else Store<SC>::st(p, T(*io - sh));
@@ -2004,9 +2053,10 @@ __device__ __forceinline__ unsigned int block_prefix(unsigned int b, unsigned in
 }
 
 // PRED 0 also assigns the new storage slots: fluid nodes take their list position, solid nodes
-// follow the fluid total in brick order (slot_new).
+// follow the fluid total in brick order (slot_new), and the byte offsets that go with them (off;
+// rec bytes per tile, elem per flow element).
 template <class L, int PRED>
-__global__ void __launch_bounds__(1024) k_list_write(const Args a, uint32_t* list) {
+__global__ void __launch_bounds__(1024) k_list_write(const Args a, uint32_t* list, const uint32_t rec, const uint32_t elem) {
   __shared__ unsigned int wsum[32];
   const long long t = blockIdx.x * 1024ll + threadIdx.x;
   long long n;
@@ -2014,10 +2064,15 @@ __global__ void __launch_bounds__(1024) k_list_write(const Args a, uint32_t* lis
   const unsigned int pos = block_prefix(__ballot_sync(0xffffffffu, f), a.block_counts[blockIdx.x], wsum);
   if (PRED == 0) {
     const unsigned int vpos = block_prefix(__ballot_sync(0xffffffffu, n >= 0), a.block_counts_v[blockIdx.x], wsum);
-    if (n >= 0) a.slot_new[n] = f ? pos : a.fluid_count[0] + (vpos - pos);
+    if (n >= 0) {
+      const unsigned int sl = f ? pos : a.fluid_count[0] + (vpos - pos);
+      a.slot_new[n] = sl;
+      if (a.off_ok) a.off[n] = (sl >> 5) * rec + (sl & 31u) * elem + uint32_t(kOffBias * 32) * elem;
+    }
   }
   if (f) {
-    list[pos] = (uint32_t)n;
+    list[pos] = PRED == 0 ? list_entry<L>(a, int(n), int(n % a.nx), int((n / a.nx) % a.ny), int(n / ((long long)a.nx * a.ny)))
+                          : (uint32_t)n;
     if (PRED == 1) a.listed[n] = 1;
   }
 }
@@ -2083,14 +2138,14 @@ template <class L, class S, int NC, int NS>
 __global__ void __launch_bounds__(1024) k_flip(const Args a, const Coef<typename Store<S>::T> k,
                                                const int parity_next) {
   using T = typename Store<S>::T;
-  using SC = typename ScalarOf<S>::type;   // scalar lattices' storage
+  using R = Rec<L, S, NC, NS>;
+  using SC = typename R::SC;   // scalar lattices' storage
   constexpr int Q = L::Q, QC = L::QC;
   const unsigned int cnt_raw = *a.flip_count;
   const unsigned int cnt = cnt_raw < a.flip_cap ? cnt_raw : a.flip_cap;
   if (cnt == 0) return;
   const int percf[3] = {a.per[0], a.per[1], a.per[2]};
   const int percs[3] = {a.open_x ? 0 : a.per[0], a.per[1], a.per[2]};
-  const long long P = a.pitch;
   const bool dissolve = a.geo_mode == GEO_DISSOLVE;
   // flip monitors: injected mass [0, 2), injected scalars [2, 5), removed mass [5, 7), removed
   // scalars [7, 10), solid temperature taken from the solid lattice [10]
@@ -2126,16 +2181,17 @@ __global__ void __launch_bounds__(1024) k_flip(const Args a, const Coef<typename
         coords_of(a, q, &qx, &qy, &qz);
         const Nbr nq = make_nbr(a, qx, qy, qz);
         const uint32_t mq = a.mask[q];
+        const long long cq = R::cell(a.slot[q]);
         for (int c = 0; c < NC; ++c) {
           T f[Q];
-          gather_flow<L, S>(reinterpret_cast<const S*>(a.f[c]), P, a.slot[q], a.slot, mq, nq, parity_next, f);
+          gather_flow<L, S, NC, NS>(a, c, cq, mq, nq, parity_next, f);
           double r = double(k.rref[c]);
           for (int j = 0; j < Q; ++j) r += double(f[j]);
           sr[c] += r;
         }
         T hh[NS > 0 ? NS : 1][QC];
         for (int c = 0; c < NS; ++c)
-          gather_scal<L, SC>(reinterpret_cast<const SC*>(a.h[c]), P, a.slot[q], a.slot, mq, nq, parity_next, hh[c]);
+          gather_scal<L, S, NC, NS>(a, c, cq, mq, nq, parity_next, hh[c]);
         T rl[QC], gain = T(0);
         for (int j = 0; j < QC; ++j) rl[j] = T(0);
         if (NS > 1 && a.conjugate)
@@ -2163,16 +2219,17 @@ __global__ void __launch_bounds__(1024) k_flip(const Args a, const Coef<typename
     } else {
       const Nbr ns = make_nbr(a, x, y, z);
       const uint32_t ms = a.mask[s];
+      const long long cs = R::cell(a.slot[s]);
       for (int c = 0; c < NC; ++c) {
         T f[Q];
-        gather_flow<L, S>(reinterpret_cast<const S*>(a.f[c]), P, a.slot[s], a.slot, ms, ns, parity_next, f);
+        gather_flow<L, S, NC, NS>(a, c, cs, ms, ns, parity_next, f);
         double r = double(k.rref[c]);
         for (int j = 0; j < Q; ++j) r += double(f[j]);
         atomicAdd(&sred[5 + c], r);
       }
       for (int c = 0; c < NS; ++c) {
         T h[QC];
-        gather_scal<L, SC>(reinterpret_cast<const SC*>(a.h[c]), P, a.slot[s], a.slot, ms, ns, parity_next, h);
+        gather_scal<L, S, NC, NS>(a, c, cs, ms, ns, parity_next, h);
         double C = double(k.cref[c]);
         for (int j = 0; j < QC; ++j) C += double(h[j]);
         atomicAdd(&sred[7 + c], C);
@@ -2184,37 +2241,35 @@ __global__ void __launch_bounds__(1024) k_flip(const Args a, const Coef<typename
   for (unsigned int e = threadIdx.x; e < cnt; e += blockDim.x) {
     if (a.flip_list[e] == 0xffffffffu) continue;
     const long long s = a.flip_list[e];
-    const long long ss = a.slot[s];   // storage slot of the flipping node
+    const long long ss = R::cell(a.slot[s]);   // cells of the flipping node
     int x, y, z;
     coords_of(a, s, &x, &y, &z);
     int ax;
     if (dissolve) {
       const double* sc4 = a.flip_scratch + 5ll * e;
       for (int c = 0; c < NC; ++c) {
-        S* fs = reinterpret_cast<S*>(a.f[c]);
         const double r = sc4[c];
         atomicAdd(&sred[c], r);
         for (int j = 0; j < Q; ++j) {
           const T tv = T(L::w(j) * (r - double(k.rref[c])));   // f_eq(rho_bar, u = 0) - w rref
           if (parity_next == 0 || j == 0) {
-            Store<S>::st(fs + (long long)j * P + ss, tv);
+            Store<S>::st(R::f(a, ss, c, j), tv);
             continue;
           }
           const long long src = nbr_checked(a, x, y, z, -L::cx(j), -L::cy(j), -L::cz(j), percf, &ax);
           const uint8_t fl = src < 0 ? FL_SOLID : a.flags[src];
           if (fl == FL_FLUID) {
-            S* from = fs + (long long)L::opp(j) * P + a.slot[src];
-            *(fs + (long long)j * P + ss) = *from;     // neighbour's bounced value moves
+            S* from = R::f(a, R::cell(a.slot[src]), c, L::opp(j));
+            *(R::f(a, ss, c, j)) = *from;     // neighbour's bounced value moves
             Store<S>::st(from, tv);
           } else if (fl == FL_FLIPPING) {
-            Store<S>::st(fs + (long long)L::opp(j) * P + a.slot[src], tv);
+            Store<S>::st(R::f(a, R::cell(a.slot[src]), c, L::opp(j)), tv);
           } else {
-            Store<S>::st(fs + (long long)j * P + ss, tv);
+            Store<S>::st(R::f(a, ss, c, j), tv);
           }
         }
       }
       for (int c = 0; c < NS; ++c) {
-        SC* hs = reinterpret_cast<SC*>(a.h[c]);
         double C = sc4[2 + c];
         if (c == 1 && a.conjugate) {
           // with conduction in the solid the new fluid node keeps its own temperature: its solid
@@ -2232,19 +2287,19 @@ __global__ void __launch_bounds__(1024) k_flip(const Args a, const Coef<typename
           const double wj = double(scal_w<T>(j, k));
           const T tv = T(wj * (C - double(k.cref[c])));       // h_eq(C_bar, u = 0) - w cref
           if (parity_next == 0 || j == 0) {
-            Store<SC>::st(hs + (long long)j * P + ss, tv);
+            Store<SC>::st(R::h(a, ss, c, j), tv);
             continue;
           }
           const long long src = nbr_checked(a, x, y, z, -L::cx(j), -L::cy(j), -L::cz(j), percs, &ax);
           const uint8_t fl = src < 0 ? FL_SOLID : a.flags[src];
           if (fl == FL_FLUID) {
-            SC* from = hs + (long long)L::opp(j) * P + a.slot[src];
-            *(hs + (long long)j * P + ss) = *from;
+            SC* from = R::h(a, R::cell(a.slot[src]), c, L::opp(j));
+            *(R::h(a, ss, c, j)) = *from;
             Store<SC>::st(from, tv);
           } else if (fl == FL_FLIPPING) {
-            Store<SC>::st(hs + (long long)L::opp(j) * P + a.slot[src], tv);
+            Store<SC>::st(R::h(a, R::cell(a.slot[src]), c, L::opp(j)), tv);
           } else {
-            Store<SC>::st(hs + (long long)j * P + ss, tv);
+            Store<SC>::st(R::h(a, ss, c, j), tv);
           }
         }
       }
@@ -2252,19 +2307,17 @@ __global__ void __launch_bounds__(1024) k_flip(const Args a, const Coef<typename
       // deposition in the swapped layout: a remaining fluid neighbour y = s + c_d now reads its
       // population from the new wall at (y, d); give it what s streamed toward it, (s, opp d)
       for (int c = 0; c < NC; ++c) {
-        S* fs = reinterpret_cast<S*>(a.f[c]);
         for (int d = 1; d < Q; ++d) {
           const long long yn = nbr_checked(a, x, y, z, L::cx(d), L::cy(d), L::cz(d), percf, &ax);
           if (yn < 0 || a.flags[yn] != FL_FLUID) continue;
-          *(fs + (long long)d * P + a.slot[yn]) = *(fs + (long long)L::opp(d) * P + ss);
+          *(R::f(a, R::cell(a.slot[yn]), c, d)) = *(R::f(a, ss, c, L::opp(d)));
         }
       }
       for (int c = 0; c < NS; ++c) {
-        SC* hs = reinterpret_cast<SC*>(a.h[c]);
         for (int d = 1; d < QC; ++d) {
           const long long yn = nbr_checked(a, x, y, z, L::cx(d), L::cy(d), L::cz(d), percs, &ax);
           if (yn < 0 || a.flags[yn] != FL_FLUID) continue;
-          *(hs + (long long)d * P + a.slot[yn]) = *(hs + (long long)L::opp(d) * P + ss);
+          *(R::h(a, R::cell(a.slot[yn]), c, d)) = *(R::h(a, ss, c, L::opp(d)));
         }
       }
     }
@@ -2277,7 +2330,9 @@ __global__ void __launch_bounds__(1024) k_flip(const Args a, const Coef<typename
     leave_flipping(a.flags, a.flip_list[e], dissolve ? FL_FLUID : FL_SOLID);
     if (dissolve) {
       const unsigned int pos = atomicAdd(a.fluid_count, 1u);
-      if (pos < a.N) a.fluid_list[pos] = a.flip_list[e];
+      int x, y, z;
+      coords_of(a, a.flip_list[e], &x, &y, &z);
+      if (pos < a.N) a.fluid_list[pos] = list_entry<L>(a, int(a.flip_list[e]), x, y, z);
       else atomicOr(a.err, ERR_CAPACITY);
     }
   }
@@ -2365,11 +2420,12 @@ __global__ void __launch_bounds__(256) k_solid(const Args a, const Coef<typename
 // gather reads it); T_b and C_b come from n_it + 1 fixed-point updates starting at the value
 // without reaction, and k is kept for the next step's species closure.  Monitors: heat gained by
 // the fluid side (bank HEAT), by the solid side (HEAT_S), reaction heat (HEAT_SRC).
-template <class L, class S>
+template <class L, class S, int NC, int NS>
 __global__ void __launch_bounds__(256) k_exchange(const Args a, const Coef<typename Store<S>::T> k,
                                                   const int parity_next) {
   using T = typename Store<S>::T;
-  using SC = typename ScalarOf<S>::type;
+  using R = Rec<L, S, NC, NS>;
+  using SC = typename R::SC;
   constexpr int QC = L::QC;
   T* g = reinterpret_cast<T*>(a.gs[parity_next]);
   T* kb = reinterpret_cast<T*>(a.kb);
@@ -2380,7 +2436,7 @@ __global__ void __launch_bounds__(256) k_exchange(const Args a, const Coef<typen
   T heat = T(0), heat_s = T(0), src_q = T(0);
   const unsigned int count = a.fluid_count[0], base = a.fluid_count[1];
   for (unsigned int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) {
-    const int n = int(LBM_CHK(a.err, a.fluid_list[e], a.N));
+    const int n = list_node(a, a.fluid_list[e]);
     const uint32_t m = a.mask[n];
     if (!(m & 1u)) continue;
     bool any = false;
@@ -2390,7 +2446,7 @@ __global__ void __launch_bounds__(256) k_exchange(const Args a, const Coef<typen
       any |= (c == 1u || c == 2u);
     }
     if (!any) continue;
-    const long long sn = e < base ? (long long)e : (long long)a.slot[n];
+    const long long cell = R::cell(e < base ? (long long)e : (long long)a.slot[n]);
     int x, y, z, ax;
     coords_of(a, n, &x, &y, &z);
     const Nbr nb = make_nbr(a, x, y, z);
@@ -2401,7 +2457,7 @@ __global__ void __launch_bounds__(256) k_exchange(const Args a, const Coef<typen
       const long long s = nbr_checked(a, x, y, z, L::cx(j), L::cy(j), L::cz(j), perc, &ax);
       if (s < 0) continue;   // a closed face: plain bounce-back
       const int i = L::opp(j);
-      SC* hp = reinterpret_cast<SC*>(a.hplane[1][i]) + LBM_CHK(a.err, sn, a.pitch);
+      SC* hp = R::h(a, cell, 1, i);
       T* gp = g + (long long)j * a.N + s;
       const T ho = Store<SC>::ld(hp) + sh1;
       const T go = *gp;
@@ -2411,11 +2467,9 @@ __global__ void __launch_bounds__(256) k_exchange(const Args a, const Coef<typen
         // the species population moving toward the wall, where the next step gathers it
         const SC* bp;
         if (parity_next == 0 || MaskBits<L>::code(m, i) != 0u)
-          bp = reinterpret_cast<const SC*>(a.hplane[0][j]) + LBM_CHK(a.err, sn, a.pitch);
+          bp = R::h(a, cell, 0, j);
         else
-          bp = reinterpret_cast<const SC*>(a.hplane[0][i]) +
-               LBM_CHK(a.err, (long long)__ldg(a.slot + LBM_CHK(a.err, nb.at(-L::cx(j), -L::cy(j), -L::cz(j)), a.N)),
-                       a.pitch);
+          bp = R::h(a, cell_of<R>(a, nb.at(-L::cx(j), -L::cy(j), -L::cz(j))), 0, i);
         const T hb = Store<SC>::ld(bp) + sh0;
         T kt = T(0);
         for (int it = 0; it <= a.n_it; ++it) {

@@ -126,6 +126,11 @@ struct MaskBits {
   __host__ __device__ static constexpr uint32_t code(uint32_t m, int j) {
     return (m >> (SC_BASE + 2 * (j - 1))) & 3u;
   }
+  // nonzero if any scalar link is reactive (code 2): bit 2 (j - 1) for direction j
+  __host__ __device__ static constexpr uint32_t reactive(uint32_t m) {
+    const uint32_t c = m >> SC_BASE;
+    return (c >> 1) & ~c & (L::QC == 7 ? 0x555u : 0x55u);
+  }
 };
 
 }  // namespace lbm

@@ -30,6 +30,7 @@ struct KernelSet {
   void (*coefs)(const Args* a, int n, void* out);
   cudaError_t (*step_tiles)(const Args* d_args, const void* d_coefs, const Tile* d_tiles, unsigned int ntiles,
                             int n_comp, int n_scal, int coll, int parity, int bnd, int threads, cudaStream_t);
+  long long (*rec_bytes)(const Args&);   // bytes per tile of 32 slots of all populations
   int psi_bytes;   // bytes per psi element (compute type)
   int coef_bytes;
 };
@@ -69,6 +70,7 @@ Coef<T> make_coef(const Args& a, bool shifted) {
     k.G_ads[s] = T(a.G_ads[s]);
     for (int t = 0; t < 2; ++t) k.G[s][t] = T(a.G[s][t]);
     k.rref[s] = shifted ? T(a.rho_ref[s]) : T(0);
+    k.hom[s] = T(0.5 * (1.0 - 1.0 / a.tau[s]));
   }
   for (int s = 0; s < 3; ++s) {
     k.omc[s] = T(1.0 / a.tau_c[s]);
@@ -90,6 +92,14 @@ Coef<T> make_coef(const Args& a, bool shifted) {
   k.ics2c = T(double(L::QC - 1) / (2.0 * (1.0 - a.J0)));
   k.icb = T(1.0 / (2.0 * (1.0 - a.J0) / double(L::QC - 1) + a.k_react * a.tau_c[0] / (a.tau_c[0] - 0.5)));
   k.kr = T(a.k_react);
+  {
+    const double wa = (1.0 - a.J0) / double(L::QC - 1);
+    const double icb = 1.0 / (2.0 * wa + a.k_react * a.tau_c[0] / (a.tau_c[0] - 0.5));
+    k.cl1 = T(4.0 * wa * icb - 1.0);
+    k.cl2 = T(2.0 * a.k_react * icb);
+  }
+  k.oq = T(a.s_grp[2] / 8.0);
+  k.omm = T(a.s_grp[4] / 8.0);
   k.DP = T(a.DP);
   k.keep = T(1.0 - a.DP);
   for (int c = 0; c < 3; ++c) k.uw6[c] = T(6.0 * a.u_wall[c]);
@@ -113,7 +123,7 @@ struct Launchers {
   // dynamic shared memory of the tile kernel's odd-step neighbour-slot caches: two buffers of Q
   // words per thread (the current tile's and the next tile's)
   static size_t slot_smem_bytes(int parity, int threads) {
-    if (!parity || !LBM_ODD_SLOT_CACHE) return 0;
+    if (!parity) return 0;
     return 2 * (size_t)threads * L::Q * sizeof(uint32_t);
   }
 
@@ -136,10 +146,10 @@ struct Launchers {
   }
   // BND: a moving plate, a velocity inlet or the temperature-dependent reaction needs the full
   // variant of the step kernel, and so does a domain too large for the plain variant's 32-bit
-  // wall offsets
+  // byte offsets (4 GB of populations, 41 M nodes of D3Q19 + D3Q7 in FP32)
   template <int NC, int NS, int COLL>
   static cudaError_t step_t(const Args& a, int parity, cudaStream_t st) {
-    if (a.moving_wall || a.flow_open_x || a.arrhenius || !a.voff_ok)
+    if (a.moving_wall || a.flow_open_x || a.arrhenius || !a.off_ok)
       return parity ? step_p<NC, NS, COLL, 1, true>(a, st) : step_p<NC, NS, COLL, 0, true>(a, st);
     return parity ? step_p<NC, NS, COLL, 1, false>(a, st) : step_p<NC, NS, COLL, 0, false>(a, st);
   }
@@ -168,24 +178,35 @@ struct Launchers {
   }
 
   // psi pass: resident waves of 256-thread blocks over the fluid list (grid-stride)
-  template <int NC, int PAR>
+  template <int NC, int NS, int PAR>
   static cudaError_t psi_p(const Args& a, cudaStream_t st) {
     static int cached_blocks = 0;
     if (!cached_blocks) {
       int dev = 0, sms = 0, occ = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_psi<L, S, NC, PAR>, 256, 0);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_psi<L, S, NC, NS, PAR>, 256, 0);
       cached_blocks = (occ > 0 ? occ : 1) * (sms > 0 ? sms : 1);
     }
     const long long need = (a.N + 255) / 256;
     const unsigned int blocks = (unsigned int)(need < cached_blocks ? need : cached_blocks);
-    k_psi<L, S, NC, PAR><<<blocks > 0 ? blocks : 1, 256, 0, st>>>(a, coef(a));
+    k_psi<L, S, NC, NS, PAR><<<blocks > 0 ? blocks : 1, 256, 0, st>>>(a, coef(a));
     return cudaGetLastError();
   }
   static cudaError_t psi(const Args& a, int parity, cudaStream_t st) {
-    if (a.n_comp == 1) return parity ? psi_p<1, 1>(a, st) : psi_p<1, 0>(a, st);
-    return parity ? psi_p<2, 1>(a, st) : psi_p<2, 0>(a, st);
+    cudaError_t e = cudaSuccess;
+    by_nc_ns(a, [&](auto nc, auto ns) {
+      constexpr int NC = decltype(nc)::value, NS = decltype(ns)::value;
+      e = parity ? psi_p<NC, NS, 1>(a, st) : psi_p<NC, NS, 0>(a, st);
+    });
+    return e;
+  }
+
+  // bytes per tile of 32 slots (before the context's buffers exist, from the lattice counts alone)
+  static long long rec_bytes(const Args& a) {
+    long long r = 0;
+    by_nc_ns(a, [&](auto nc, auto ns) { r = Rec<L, S, decltype(nc)::value, decltype(ns)::value>::BYTES; });
+    return r;
   }
 
   template <class F>
@@ -264,7 +285,11 @@ struct Launchers {
     return cudaGetLastError();
   }
   static cudaError_t exchange(const Args& a, int parity_next, cudaStream_t st) {
-    k_exchange<L, S><<<box_blocks(a), 256, 0, st>>>(a, coef(a), parity_next);
+    // conduction in the solid needs the species and the temperature: two or three scalar lattices
+    by_nc_ns(a, [&](auto nc, auto ns) {
+      if constexpr (decltype(ns)::value >= 2)
+        k_exchange<L, S, decltype(nc)::value, decltype(ns)::value><<<box_blocks(a), 256, 0, st>>>(a, coef(a), parity_next);
+    });
     return cudaGetLastError();
   }
   static cudaError_t solid_init(const Args& a, cudaStream_t st) {
@@ -287,12 +312,12 @@ struct Launchers {
       k_list_count<L, 0><<<bchunks, 1024, 0, st>>>(a);
       k_list_scan<<<1, 1024, 0, st>>>(a.block_counts, bchunks, a.fluid_count);
       k_list_scan<<<1, 1024, 0, st>>>(a.block_counts_v, bchunks, a.fluid_count + 2);
-      k_list_write<L, 0><<<bchunks, 1024, 0, st>>>(a, a.fluid_list);
+      k_list_write<L, 0><<<bchunks, 1024, 0, st>>>(a, a.fluid_list, (uint32_t)rec_bytes(a), (uint32_t)sizeof(S));
     }
     if (which & 2) {
       k_list_count<L, 1><<<chunks, 1024, 0, st>>>(a);
       k_list_scan<<<1, 1024, 0, st>>>(a.block_counts, chunks, a.iface_count);
-      k_list_write<L, 1><<<chunks, 1024, 0, st>>>(a, a.iface_list);
+      k_list_write<L, 1><<<chunks, 1024, 0, st>>>(a, a.iface_list, 0u, 0u);
     }
     return cudaGetLastError();
   }
@@ -351,6 +376,7 @@ struct Launchers {
     k.step_tiles = &step_tiles;
     k.coef_bytes = (int)sizeof(Coef<T>);
     k.step = &step;
+    k.rec_bytes = &rec_bytes;
     k.psi = &psi;
     k.moments = &moments;
     k.monitor = &monitor;
@@ -386,8 +412,14 @@ const KernelSet& kernels_d3_bf16s32();
 cudaError_t launch_reduce(const double* partials, long long nblocks, int K, double* out, int* err,
                           int nonfin_slot, cudaStream_t st);
 cudaError_t launch_detect(const Args& a, cudaStream_t st);
-cudaError_t launch_permute(const void* src, void* dst, int elem, long long pitch, int planes,
-                           const uint8_t* flags, long long N, const uint32_t* from, const uint32_t* to,
+// Placement of one lattice's rows (elem bytes per element) in a population buffer: tiles of 32 slots
+// (tile bytes apart, row bytes first within one) or planes (tile = 0: row r at first + r * pitch).
+struct Place {
+  unsigned char* p;
+  long long tile, first, pitch;
+  const uint32_t* map;   // slot of each node; NULL: node order
+};
+cudaError_t launch_permute(const Place& src, const Place& dst, int elem, int rows, const uint8_t* flags, long long N,
                            cudaStream_t st);
 cudaError_t launch_iota(uint32_t* v, long long N, cudaStream_t st);
 

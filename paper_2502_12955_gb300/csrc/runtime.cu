@@ -43,8 +43,8 @@ struct lbm_ctx {
   std::string err;
   std::vector<void*> allocs;
   double* mon_host = nullptr;      // pinned [NMON + 12]: monitors, then the 11 flip monitors
-  void* f_alt[2] = {nullptr, nullptr};   // second population buffers: targets of re-slotting
-  void* h_alt[3] = {nullptr, nullptr, nullptr};
+  unsigned char* pop_alt = nullptr;   // second population buffer: target of re-slotting, staging of checkpoints
+  long long rec = 0;               // bytes of one tile of 32 slots
   int nlat = 0;                    // scalar lattices: the given scalars, then the product if any
   // CUDA graphs of one even + odd step pair, keyed by which of the two steps end with a
   // geometry update; rebuilt whenever the kernel arguments change (re-slotting)
@@ -216,7 +216,6 @@ void fill_args(lbm_ctx* c) {
   Args& a = c->a;
   const lbm_params& p = c->p;
   a.pitch = c->pitch;
-  a.voff_ok = 3ll * c->pitch < (1ll << 31) ? 1 : 0;
   a.N = c->N;
   a.nx = c->nx; a.ny = c->ny; a.nz = c->nz;
   a.n_comp = p.n_comp;
@@ -291,25 +290,28 @@ constexpr long long kListRebuild = 1024;   // steps between sorted rebuilds of t
 #define LBM_STEP_GRAPHS 1
 #endif
 
-void set_planes(lbm_ctx* c) {
-  for (int s = 0; s < c->p.n_comp; ++s)
-    for (int i = 0; i < c->Qf; ++i)
-      c->a.fplane[s][i] = static_cast<char*>(c->a.f[s]) + (size_t)i * c->pitch * c->elem;
-  for (int s = 0; s < c->nlat; ++s)
-    for (int j = 0; j < c->Qc; ++j)
-      c->a.hplane[s][j] = static_cast<char*>(c->a.h[s]) + (size_t)j * c->pitch * c->elem_h;
+// Rows of flow component s (s < n_comp) or scalar lattice s - n_comp: element size, row count and
+// placement in the tiled buffer p, or as planes in node order (checkpoints: the lattices one
+// after the other) in p.
+Place lattice_place(const lbm_ctx* c, int s, unsigned char* p, bool tiled, const uint32_t* map, int* elem, int* rows) {
+  const int nc = c->p.n_comp;
+  const bool flow = s < nc;
+  *elem = (int)(flow ? c->elem : c->elem_h);
+  *rows = flow ? c->Qf : c->Qc;
+  const long long before = (long long)std::min(s, nc) * c->Qf * c->elem + (long long)std::max(0, s - nc) * c->Qc * c->elem_h;
+  if (tiled) return Place{p, c->rec, before * 32, 32ll * *elem, map};
+  return Place{p, 0, before * c->pitch, c->pitch * *elem, map};
 }
 
-// Copies the populations of every fluid node between two population buffers.  A NULL map
-// means node order; otherwise the map gives the slot of each node.
-lbm_status move_pops(lbm_ctx* c, void* const* src_f, void* const* dst_f, void* const* src_h,
-                     void* const* dst_h, const uint32_t* from, const uint32_t* to) {
-  for (int s = 0; s < c->p.n_comp; ++s)
-    LAUNCH(launch_permute(src_f[s], dst_f[s], (int)c->elem, c->pitch, c->Qf, c->a.flags, c->N, from, to,
-                          c->stream));
-  for (int s = 0; s < c->nlat; ++s)
-    LAUNCH(launch_permute(src_h[s], dst_h[s], (int)c->elem_h, c->pitch, c->Qc, c->a.flags, c->N, from, to,
-                          c->stream));
+// Copies the populations of every fluid node between two population buffers (see lattice_place).
+lbm_status move_pops(lbm_ctx* c, unsigned char* src, bool src_tiled, const uint32_t* from, unsigned char* dst, bool dst_tiled,
+                     const uint32_t* to) {
+  for (int s = 0; s < c->p.n_comp + c->nlat; ++s) {
+    int elem, rows;
+    const Place ps = lattice_place(c, s, src, src_tiled, from, &elem, &rows);
+    const Place pd = lattice_place(c, s, dst, dst_tiled, to, &elem, &rows);
+    LAUNCH(launch_permute(ps, pd, elem, rows, c->a.flags, c->N, c->stream));
+  }
   return LBM_OK;
 }
 
@@ -331,13 +333,9 @@ lbm_status relist(lbm_ctx* c, bool carry) {
   CK(cudaMemsetAsync(c->a.listed, 0, (c->N + 3) / 4 * 4, c->stream));
   LAUNCH(c->ks->lists(c->a, 3, c->stream));
   if (carry) {
-    lbm_status st = move_pops(c, c->a.f, c->f_alt, c->a.h, c->h_alt, c->a.slot, c->a.slot_new);
+    lbm_status st = move_pops(c, c->a.pop, true, c->a.slot, c->pop_alt, true, c->a.slot_new);
     if (st != LBM_OK) return st;
-    for (int s = 0; s < 2; ++s) {
-      std::swap(c->a.f[s], c->f_alt[s]);
-      std::swap(c->a.h[s], c->h_alt[s]);
-    }
-    set_planes(c);
+    std::swap(c->a.pop, c->pop_alt);
   }
   std::swap(c->a.slot, c->a.slot_new);
   return LBM_OK;
@@ -443,36 +441,29 @@ __global__ void __launch_bounds__(256) k_detect(const Args a) {
   }
 }
 
-// Population copy of every fluid node between buffers of one lattice: dst[i][to(n)] =
-// src[i][from(n)], where a NULL map is node order.
+// Copy of one lattice's populations of every fluid node from one placement to another.
 template <class E>
-__global__ void __launch_bounds__(256) k_permute(const E* __restrict__ src, E* __restrict__ dst, long long pitch,
-                                                 int planes, const uint8_t* __restrict__ flags, long long N,
-                                                 const uint32_t* __restrict__ from, const uint32_t* __restrict__ to) {
+__global__ void __launch_bounds__(256) k_permute(const Place src, const Place dst, int rows,
+                                                 const uint8_t* __restrict__ flags, long long N) {
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (n >= N || flags[n] != FL_FLUID) return;
-  const long long s = from ? (long long)from[n] : n;
-  const long long d = to ? (long long)to[n] : n;
-  for (int i = 0; i < planes; ++i) dst[i * pitch + d] = src[i * pitch + s];
+  const auto cell = [&](const Place& p) {
+    const long long s = p.map ? (long long)p.map[n] : n;
+    return p.p + p.first + (p.tile ? (s >> 5) * p.tile + (s & 31) * (long long)sizeof(E) : s * (long long)sizeof(E));
+  };
+  const unsigned char* from = cell(src);
+  unsigned char* to = cell(dst);
+  for (int i = 0; i < rows; ++i)
+    *reinterpret_cast<E*>(to + i * dst.pitch) = *reinterpret_cast<const E*>(from + i * src.pitch);
 }
 
-cudaError_t launch_permute(const void* src, void* dst, int elem, long long pitch, int planes,
-                           const uint8_t* flags, long long N, const uint32_t* from, const uint32_t* to,
+cudaError_t launch_permute(const Place& src, const Place& dst, int elem, int rows, const uint8_t* flags, long long N,
                            cudaStream_t st) {
   const unsigned int nb = (unsigned int)((N + 255) / 256);
   switch (elem) {
-    case 2:
-      k_permute<uint16_t><<<nb, 256, 0, st>>>(static_cast<const uint16_t*>(src), static_cast<uint16_t*>(dst),
-                                              pitch, planes, flags, N, from, to);
-      break;
-    case 4:
-      k_permute<uint32_t><<<nb, 256, 0, st>>>(static_cast<const uint32_t*>(src), static_cast<uint32_t*>(dst),
-                                              pitch, planes, flags, N, from, to);
-      break;
-    default:
-      k_permute<unsigned long long><<<nb, 256, 0, st>>>(static_cast<const unsigned long long*>(src),
-                                                        static_cast<unsigned long long*>(dst), pitch, planes,
-                                                        flags, N, from, to);
+    case 2: k_permute<uint16_t><<<nb, 256, 0, st>>>(src, dst, rows, flags, N); break;
+    case 4: k_permute<uint32_t><<<nb, 256, 0, st>>>(src, dst, rows, flags, N); break;
+    default: k_permute<unsigned long long><<<nb, 256, 0, st>>>(src, dst, rows, flags, N);
   }
   return cudaGetLastError();
 }
@@ -574,12 +565,13 @@ lbm_status lbm_create(lbm_lattice lattice, int32_t nx, int32_t ny, int32_t nz, c
     if (st != LBM_OK) return bail(st);                      \
     ptr = reinterpret_cast<decltype(ptr)>(v);               \
   } while (0)
-  for (int s = 0; s < params->n_comp; ++s) DA(a.f[s], P * c->Qf * c->elem);
-  for (int s = 0; s < c->nlat; ++s) DA(a.h[s], P * c->Qc * c->elem_h);
-  for (int s = 0; s < params->n_comp; ++s) DA(c->f_alt[s], P * c->Qf * c->elem);
-  for (int s = 0; s < c->nlat; ++s) DA(c->h_alt[s], P * c->Qc * c->elem_h);
-  set_planes(c);
+  c->rec = c->ks->rec_bytes(a);
+  a.pop_bytes = P / 32 * c->rec;
+  a.off_ok = a.pop_bytes + 64 * kOffBias * (long long)c->elem < (1ll << 32) ? 1 : 0;
+  DA(a.pop, a.pop_bytes);
+  DA(c->pop_alt, a.pop_bytes);
   DA(a.slot, N * 4);
+  if (a.off_ok) DA(a.off, N * 4);
   DA(a.slot_new, N * 4);
   if (a.sc_on)
     for (int s = 0; s < params->n_comp; ++s) DA(a.psi[s], P * c->ks->psi_bytes);
@@ -640,8 +632,7 @@ lbm_status lbm_create(lbm_lattice lattice, int32_t nx, int32_t ny, int32_t nz, c
   if (e == cudaSuccess) e = cudaMemsetAsync(a.inflow_row, 0, 3 * rows * 8, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(a.outflow_row, 0, 3 * rows * 8, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(a.mon_out, 0, (NMON + 8) * 8, c->stream);
-  for (int s = 0; s < params->n_comp && e == cudaSuccess; ++s) e = cudaMemsetAsync(a.f[s], 0, P * c->Qf * c->elem, c->stream);
-  for (int s = 0; s < c->nlat && e == cudaSuccess; ++s) e = cudaMemsetAsync(a.h[s], 0, P * c->Qc * c->elem_h, c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(a.pop, 0, a.pop_bytes, c->stream);
   if (e == cudaSuccess) e = launch_iota(a.slot, N, c->stream);   // node order until a geometry is set
   if (e == cudaSuccess) {
     // inlet profile u_x(y) = 6 U s (1 - s), s = (y + 1/2) / ny (zero without a velocity inlet)
@@ -1061,8 +1052,8 @@ size_t solid_state_bytes(const lbm_ctx* c) {
   return (2 * c->Qc + (c->Qc - 1)) * N * e + 2 * WALLX_SLOTS * 8 + 8;
 }
 size_t state_bytes(const lbm_ctx* c) {
-  const size_t N = (size_t)c->N, P = (size_t)c->pitch, rows = (size_t)c->ny * c->nz;
-  return sizeof(StateHeader) + (c->p.n_comp * c->Qf * c->elem + c->nlat * c->Qc * c->elem_h) * P +
+  const size_t N = (size_t)c->N, rows = (size_t)c->ny * c->nz;
+  return sizeof(StateHeader) + (size_t)c->a.pop_bytes +
          (N + 3) / 4 * 4 + N * 8 + 3 * WALLX_SLOTS * 8 + 6 * rows * 8 + 10 * 8 + solid_state_bytes(c);
 }
 }  // namespace
@@ -1083,20 +1074,13 @@ lbm_status lbm_get_state(lbm_ctx* c, void* host, size_t* nbytes) {
   hd.step = c->step;
   std::memcpy(o, &hd, sizeof hd);
   o += sizeof hd;
-  const size_t P = (size_t)c->pitch, N = (size_t)c->N, rows = (size_t)c->ny * c->nz;
-  // populations in node order (solid nodes 0), staged in the second population buffers
-  for (int s = 0; s < c->p.n_comp; ++s) CK(cudaMemsetAsync(c->f_alt[s], 0, c->Qf * P * c->elem, c->stream));
-  for (int s = 0; s < c->nlat; ++s) CK(cudaMemsetAsync(c->h_alt[s], 0, c->Qc * P * c->elem_h, c->stream));
-  lbm_status st = move_pops(c, c->a.f, c->f_alt, c->a.h, c->h_alt, c->a.slot, nullptr);
+  const size_t N = (size_t)c->N, rows = (size_t)c->ny * c->nz;
+  // populations as planes in node order (solid nodes 0), staged in the second population buffer
+  CK(cudaMemsetAsync(c->pop_alt, 0, c->a.pop_bytes, c->stream));
+  lbm_status st = move_pops(c, c->a.pop, true, c->a.slot, c->pop_alt, false, nullptr);
   if (st != LBM_OK) return st;
-  for (int s = 0; s < c->p.n_comp; ++s) {
-    CK(cudaMemcpyAsync(o, c->f_alt[s], c->Qf * P * c->elem, cudaMemcpyDeviceToHost, c->stream));
-    o += c->Qf * P * c->elem;
-  }
-  for (int s = 0; s < c->nlat; ++s) {
-    CK(cudaMemcpyAsync(o, c->h_alt[s], c->Qc * P * c->elem_h, cudaMemcpyDeviceToHost, c->stream));
-    o += c->Qc * P * c->elem_h;
-  }
+  CK(cudaMemcpyAsync(o, c->pop_alt, c->a.pop_bytes, cudaMemcpyDeviceToHost, c->stream));
+  o += c->a.pop_bytes;
   CK(cudaMemcpyAsync(o, c->a.flags, (N + 3) / 4 * 4, cudaMemcpyDeviceToHost, c->stream)); o += (N + 3) / 4 * 4;
   CK(cudaMemcpyAsync(o, c->a.acc, N * 8, cudaMemcpyDeviceToHost, c->stream)); o += N * 8;
   CK(cudaMemcpyAsync(o, c->a.wallx_slot, 3 * WALLX_SLOTS * 8, cudaMemcpyDeviceToHost, c->stream)); o += 3 * WALLX_SLOTS * 8;
@@ -1129,17 +1113,11 @@ lbm_status lbm_set_state(lbm_ctx* c, const void* host, size_t nbytes) {
       hd.n_comp != c->p.n_comp || hd.n_scal != c->nlat || hd.nx != c->nx || hd.ny != c->ny || hd.nz != c->nz)
     return fail(c, LBM_ERR_INVALID_ARG, "checkpoint does not match this context");
   o += sizeof hd;
-  const size_t P = (size_t)c->pitch, N = (size_t)c->N, rows = (size_t)c->ny * c->nz;
-  // node-order populations go to the second buffers; they move to their slots once the slot
+  const size_t N = (size_t)c->N, rows = (size_t)c->ny * c->nz;
+  // node-order populations go to the second buffer; they move to their slots once the slot
   // map of the restored geometry exists
-  for (int s = 0; s < c->p.n_comp; ++s) {
-    CK(cudaMemcpyAsync(c->f_alt[s], o, c->Qf * P * c->elem, cudaMemcpyHostToDevice, c->stream));
-    o += c->Qf * P * c->elem;
-  }
-  for (int s = 0; s < c->nlat; ++s) {
-    CK(cudaMemcpyAsync(c->h_alt[s], o, c->Qc * P * c->elem_h, cudaMemcpyHostToDevice, c->stream));
-    o += c->Qc * P * c->elem_h;
-  }
+  CK(cudaMemcpyAsync(c->pop_alt, o, c->a.pop_bytes, cudaMemcpyHostToDevice, c->stream));
+  o += c->a.pop_bytes;
   CK(cudaMemcpyAsync(c->a.flags, o, (N + 3) / 4 * 4, cudaMemcpyHostToDevice, c->stream)); o += (N + 3) / 4 * 4;
   CK(cudaMemcpyAsync(c->a.acc, o, N * 8, cudaMemcpyHostToDevice, c->stream)); o += N * 8;
   CK(cudaMemcpyAsync(c->a.wallx_slot, o, 3 * WALLX_SLOTS * 8, cudaMemcpyHostToDevice, c->stream)); o += 3 * WALLX_SLOTS * 8;
@@ -1160,7 +1138,7 @@ lbm_status lbm_set_state(lbm_ctx* c, const void* host, size_t nbytes) {
   CK(cudaMemsetAsync(c->a.err, 0, 16, c->stream));
   lbm_status st = rebuild_geometry(c, false);
   if (st != LBM_OK) return st;
-  st = move_pops(c, c->f_alt, c->a.f, c->h_alt, c->a.h, nullptr, c->a.slot);
+  st = move_pops(c, c->pop_alt, false, nullptr, c->a.pop, true, c->a.slot);
   if (st != LBM_OK) return st;
   CK(cudaStreamSynchronize(c->stream));
   c->step = hd.step;
@@ -1320,7 +1298,7 @@ lbm_status ens_launch(lbm_ensemble* e, int parity, cudaStream_t st) {
   int bnd = 0;   // the boundary-rule kernel variant when any member has a moving plate or an inlet
   // (or a domain too large for the plain variant's 32-bit wall offsets)
   for (size_t k = 0; k < e->m.size(); ++k)
-    bnd |= e->m[k]->a.moving_wall | e->m[k]->a.flow_open_x | e->m[k]->a.arrhenius | !e->m[k]->a.voff_ok;
+    bnd |= e->m[k]->a.moving_wall | e->m[k]->a.flow_open_x | e->m[k]->a.arrhenius | !e->m[k]->a.off_ok;
   const cudaError_t r = e->ks->step_tiles(e->d_args, e->d_coefs, e->d_tiles, e->ntiles, p.n_comp, p.n_scal,
                                           p.collision, parity, bnd, e->threads, st);
   e->launches += 1;
