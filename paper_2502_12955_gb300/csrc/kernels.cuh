@@ -2128,22 +2128,32 @@ __device__ __forceinline__ void coords_of(const Args& a, long long n, int* x, in
   *z = int(n / ((long long)a.nx * a.ny));
 }
 
-// One block processes the whole flip list in phases separated by __syncthreads:
+// The flip list in phases separated by barriers of one cluster of kFlipBlocks blocks, a warp per entry with
+// its lanes over the neighbours or directions (a warp keeps its entries through all phases):
 //   0 claim entries (validate, mark FLIPPING, drop duplicates)
 //   1 dissolution: neighbour means (flags before the flip);  deposition: removed sums
 //   2 write populations of the new fluid nodes / hand populations to remaining neighbours
 //   3 final flags;  4 link masks of every node around a flipped one;  5 clear the list
 // parity_next is the layout parity of the state the flips act on (steps completed & 1).
+// What bounds it is the chain of dependent loads of an entry: flag, slot and mask of 18 neighbours, their
+// populations, then the 18 flags around each of them.
+constexpr int kFlipBlocks = 8, kFlipThreads = 512;
+__device__ __forceinline__ void cluster_barrier() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
 template <class L, class S, int NC, int NS>
-__global__ void __launch_bounds__(1024) k_flip(const Args a, const Coef<typename Store<S>::T> k,
-                                               const int parity_next) {
+__global__ void __cluster_dims__(kFlipBlocks, 1, 1) __launch_bounds__(kFlipThreads)
+    k_flip(const Args a, const Coef<typename Store<S>::T> k, const int parity_next) {
   using T = typename Store<S>::T;
   using R = Rec<L, S, NC, NS>;
   using SC = typename R::SC;   // scalar lattices' storage
   constexpr int Q = L::Q, QC = L::QC;
   const unsigned int cnt_raw = *a.flip_count;
   const unsigned int cnt = cnt_raw < a.flip_cap ? cnt_raw : a.flip_cap;
-  if (cnt == 0) return;
+  if (cnt == 0) return;   // the same in every block: nothing writes the count before the last barrier
+  const int lane = threadIdx.x & 31;
+  const unsigned int first = (blockIdx.x * kFlipThreads + threadIdx.x) >> 5, step = kFlipBlocks * kFlipThreads / 32;
   const int percf[3] = {a.per[0], a.per[1], a.per[2]};
   const int percs[3] = {a.open_x ? 0 : a.per[0], a.per[1], a.per[2]};
   const bool dissolve = a.geo_mode == GEO_DISSOLVE;
@@ -2152,121 +2162,152 @@ __global__ void __launch_bounds__(1024) k_flip(const Args a, const Coef<typename
   __shared__ double sred[11];
   if (threadIdx.x < 11) sred[threadIdx.x] = 0.0;
   // ---- phase 0: claim
-  for (unsigned int e = threadIdx.x; e < cnt; e += blockDim.x) {
+  for (unsigned int e = first; e < cnt; e += step) {
     const long long s = a.flip_list[e];
-    bool ok;
-    if (dissolve)
-      ok = a.flags[s] == FL_REACTIVE && consumed(a, a.acc[s]) &&
-           cas_flag(a.flags, s, FL_REACTIVE, FL_FLIPPING, a.err);
-    else
-      ok = a.flags[s] == FL_FLUID && a.acc[s] > 1.0 && cas_flag(a.flags, s, FL_FLUID, FL_FLIPPING, a.err);
-    if (!ok) a.flip_list[e] = 0xffffffffu;
+    bool ok = false;
+    if (lane == 0) {
+      if (dissolve)
+        ok = a.flags[s] == FL_REACTIVE && consumed(a, a.acc[s]) &&
+             cas_flag(a.flags, s, FL_REACTIVE, FL_FLIPPING, a.err);
+      else
+        ok = a.flags[s] == FL_FLUID && a.acc[s] > 1.0 && cas_flag(a.flags, s, FL_FLUID, FL_FLIPPING, a.err);
+      if (!ok) a.flip_list[e] = 0xffffffffu;
+    }
+    __syncwarp();
   }
   __syncthreads();
+  cluster_barrier();
   // ---- phase 1
-  for (unsigned int e = threadIdx.x; e < cnt; e += blockDim.x) {
+  for (unsigned int e = first; e < cnt; e += step) {
     if (a.flip_list[e] == 0xffffffffu) continue;
     const long long s = a.flip_list[e];
     int x, y, z;
     coords_of(a, s, &x, &y, &z);
     if (dissolve) {
-      double sr[2] = {0.0, 0.0}, sc[3] = {0.0, 0.0, 0.0};
-      int count = 0;
+      // lane i - 1: neighbour i
+      double sr[NC] = {}, sc[NS > 0 ? NS : 1] = {};
+      bool fluid = false;
       int ax;
-      for (int i = 1; i < Q; ++i) {
+      const int i = lane + 1;
+      if (i < Q) {
         const long long q = nbr_checked(a, x, y, z, L::cx(i), L::cy(i), L::cz(i), percf, &ax);
-        if (q < 0 || a.flags[q] != FL_FLUID) continue;
-        ++count;
-        int qx, qy, qz;
-        coords_of(a, q, &qx, &qy, &qz);
-        const Nbr nq = make_nbr(a, qx, qy, qz);
-        const uint32_t mq = a.mask[q];
-        const long long cq = R::cell(a.slot[q]);
-        for (int c = 0; c < NC; ++c) {
-          T f[Q];
-          gather_flow<L, S, NC, NS>(a, c, cq, mq, nq, parity_next, f);
-          double r = double(k.rref[c]);
-          for (int j = 0; j < Q; ++j) r += double(f[j]);
-          sr[c] += r;
-        }
-        T hh[NS > 0 ? NS : 1][QC];
-        for (int c = 0; c < NS; ++c)
-          gather_scal<L, S, NC, NS>(a, c, cq, mq, nq, parity_next, hh[c]);
-        T rl[QC], gain = T(0);
-        for (int j = 0; j < QC; ++j) rl[j] = T(0);
-        if (NS > 1 && a.conjugate)
-          close_conjugate<L, T>(hh[0], hh[NS > 1 ? 1 : 0], mq, k, a, nq,
-                                reinterpret_cast<const T*>(a.gs[parity_next]), [&](int j, T r, T) { rl[j] = r; });
-        else if (NS > 1 && a.arrhenius)
-          close_thermal<L, T>(hh[0], hh[NS > 1 ? 1 : 0], mq, k, a.n_it, [&](int j, T r, T, T) { rl[j] = r; });
-        else if (NS > 0)
-          close_scalar<L, T>(hh[0], mq, k, [&](int j, T Cb, T) { rl[j] = k.kr * Cb; });
-        if (NS > 1 && a.product) close_product<L, T>(hh[NS - 1], mq, k, rl, gain);
-        for (int c = 0; c < NS; ++c) {
-          double C = double(k.cref[c]);
-          for (int j = 0; j < QC; ++j) C += double(hh[c][j]);
-          sc[c] += C;
+        fluid = q >= 0 && a.flags[q] == FL_FLUID;
+        if (fluid) {
+          const Nbr nq = nbr_of(a, int(q));
+          const uint32_t mq = a.mask[q];
+          const long long cq = R::cell(a.slot[q]);
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            T f[Q];
+            gather_flow<L, S, NC, NS>(a, c, cq, mq, nq, parity_next, f);
+            double r = double(k.rref[c]);
+#pragma unroll
+            for (int j = 0; j < Q; ++j) r += double(f[j]);
+            sr[c] = r;
+          }
+          T hh[NS > 0 ? NS : 1][QC];
+#pragma unroll
+          for (int c = 0; c < NS; ++c) gather_scal<L, S, NC, NS>(a, c, cq, mq, nq, parity_next, hh[c]);
+          T rl[QC], gain = T(0);
+#pragma unroll
+          for (int j = 0; j < QC; ++j) rl[j] = T(0);
+          if (NS > 1 && a.conjugate)
+            close_conjugate<L, T>(hh[0], hh[NS > 1 ? 1 : 0], mq, k, a, nq,
+                                  reinterpret_cast<const T*>(a.gs[parity_next]), [&](int j, T r, T) { rl[j] = r; });
+          else if (NS > 1 && a.arrhenius)
+            close_thermal<L, T>(hh[0], hh[NS > 1 ? 1 : 0], mq, k, a.n_it, [&](int j, T r, T, T) { rl[j] = r; });
+          else if (NS > 0)
+            close_scalar<L, T>(hh[0], mq, k, [&](int j, T Cb, T) { rl[j] = k.kr * Cb; });
+          if (NS > 1 && a.product) close_product<L, T>(hh[NS - 1], mq, k, rl, gain);
+#pragma unroll
+          for (int c = 0; c < NS; ++c) {
+            double C = double(k.cref[c]);
+#pragma unroll
+            for (int j = 0; j < QC; ++j) C += double(hh[c][j]);
+            sc[c] = C;
+          }
         }
       }
-      double* sc4 = a.flip_scratch + 5ll * e;
-      if (count == 0) {
-        leave_flipping(a.flags, s, FL_REACTIVE);   // nothing to average: stays solid
-        a.flip_list[e] = 0xffffffffu;
+      const int count = __popc(__ballot_sync(0xffffffffu, fluid));
+      if (count == 0) {   // nothing to average: stays solid
+        if (lane == 0) {
+          leave_flipping(a.flags, s, FL_REACTIVE);
+          a.flip_list[e] = 0xffffffffu;
+        }
+        __syncwarp();
         continue;
       }
-      for (int c = 0; c < 2; ++c) sc4[c] = sr[c] / count;
-      for (int c = 0; c < 3; ++c) sc4[2 + c] = sc[c] / count;
-    } else {
-      const Nbr ns = make_nbr(a, x, y, z);
+      double* sc4 = a.flip_scratch + 5ll * e;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const double r = warp_sum(sr[c]);
+        if (lane == 0) sc4[c] = r / count;
+      }
+#pragma unroll
+      for (int c = 0; c < NS; ++c) {
+        const double r = warp_sum(sc[c]);
+        if (lane == 0) sc4[2 + c] = r / count;
+      }
+      __syncwarp();
+    } else if (lane == 0) {
+      const Nbr ns = nbr_of(a, int(s));
       const uint32_t ms = a.mask[s];
       const long long cs = R::cell(a.slot[s]);
+#pragma unroll
       for (int c = 0; c < NC; ++c) {
         T f[Q];
         gather_flow<L, S, NC, NS>(a, c, cs, ms, ns, parity_next, f);
         double r = double(k.rref[c]);
+#pragma unroll
         for (int j = 0; j < Q; ++j) r += double(f[j]);
         atomicAdd(&sred[5 + c], r);
       }
+#pragma unroll
       for (int c = 0; c < NS; ++c) {
         T h[QC];
         gather_scal<L, S, NC, NS>(a, c, cs, ms, ns, parity_next, h);
         double C = double(k.cref[c]);
+#pragma unroll
         for (int j = 0; j < QC; ++j) C += double(h[j]);
         atomicAdd(&sred[7 + c], C);
       }
     }
   }
-  __syncthreads();
-  // ---- phase 2
-  for (unsigned int e = threadIdx.x; e < cnt; e += blockDim.x) {
+  cluster_barrier();
+  // ---- phase 2: lane j moves or sets the population of direction j
+  for (unsigned int e = first; e < cnt; e += step) {
     if (a.flip_list[e] == 0xffffffffu) continue;
     const long long s = a.flip_list[e];
     const long long ss = R::cell(a.slot[s]);   // cells of the flipping node
-    int x, y, z;
+    int x, y, z, ax;
     coords_of(a, s, &x, &y, &z);
-    int ax;
+    const int j = lane;
+    // where direction j of the node comes from: a node (flow and scalar periodicity) or a face
+    long long srcf = -1, srcs = -1;
+    if (j < Q) {
+      const int d = dissolve ? -1 : 1;
+      srcf = nbr_checked(a, x, y, z, d * L::cx(j), d * L::cy(j), d * L::cz(j), percf, &ax);
+      if (j < QC) srcs = nbr_checked(a, x, y, z, d * L::cx(j), d * L::cy(j), d * L::cz(j), percs, &ax);
+    }
+    const uint8_t flf = srcf < 0 ? FL_SOLID : a.flags[srcf], fls = srcs < 0 ? FL_SOLID : a.flags[srcs];
+    const int o = j < Q ? L::opp(j) : 0;
     if (dissolve) {
       const double* sc4 = a.flip_scratch + 5ll * e;
       for (int c = 0; c < NC; ++c) {
         const double r = sc4[c];
-        atomicAdd(&sred[c], r);
-        for (int j = 0; j < Q; ++j) {
-          const T tv = T(L::w(j) * (r - double(k.rref[c])));   // f_eq(rho_bar, u = 0) - w rref
-          if (parity_next == 0 || j == 0) {
-            Store<S>::st(R::f(a, ss, c, j), tv);
-            continue;
-          }
-          const long long src = nbr_checked(a, x, y, z, -L::cx(j), -L::cy(j), -L::cz(j), percf, &ax);
-          const uint8_t fl = src < 0 ? FL_SOLID : a.flags[src];
-          if (fl == FL_FLUID) {
-            S* from = R::f(a, R::cell(a.slot[src]), c, L::opp(j));
-            *(R::f(a, ss, c, j)) = *from;     // neighbour's bounced value moves
-            Store<S>::st(from, tv);
-          } else if (fl == FL_FLIPPING) {
-            Store<S>::st(R::f(a, R::cell(a.slot[src]), c, L::opp(j)), tv);
-          } else {
-            Store<S>::st(R::f(a, ss, c, j), tv);
-          }
+        if (lane == 0) atomicAdd(&sred[c], r);
+        if (j >= Q) continue;
+        const T tv = T(L::w(j) * (r - double(k.rref[c])));   // f_eq(rho_bar, u = 0) - w rref
+        if (parity_next == 0 || j == 0) {
+          Store<S>::st(R::f(a, ss, c, j), tv);
+        } else if (flf == FL_FLUID) {
+          S* from = R::f(a, R::cell(a.slot[srcf]), c, o);
+          *R::f(a, ss, c, j) = *from;     // neighbour's bounced value moves
+          Store<S>::st(from, tv);
+        } else if (flf == FL_FLIPPING) {
+          Store<S>::st(R::f(a, R::cell(a.slot[srcf]), c, o), tv);
+        } else {
+          Store<S>::st(R::f(a, ss, c, j), tv);
         }
       }
       for (int c = 0; c < NS; ++c) {
@@ -2275,58 +2316,45 @@ __global__ void __launch_bounds__(1024) k_flip(const Args a, const Coef<typename
           // with conduction in the solid the new fluid node keeps its own temperature: its solid
           // populations leave the solid lattice
           T* g = reinterpret_cast<T*>(a.gs[parity_next]);
-          C = 0.0;
-          for (int q = 0; q < QC; ++q) {
-            C += double(g[(long long)q * a.N + s]);
-            g[(long long)q * a.N + s] = T(0);
+          double own = 0.0;
+          if (j < QC) {
+            own = double(g[(long long)j * a.N + s]);
+            g[(long long)j * a.N + s] = T(0);
           }
-          atomicAdd(&sred[10], C);
+          C = warp_sum(own);
+          if (lane == 0) atomicAdd(&sred[10], C);
         }
-        atomicAdd(&sred[2 + c], C);
-        for (int j = 0; j < QC; ++j) {
-          const double wj = double(scal_w<T>(j, k));
-          const T tv = T(wj * (C - double(k.cref[c])));       // h_eq(C_bar, u = 0) - w cref
-          if (parity_next == 0 || j == 0) {
-            Store<SC>::st(R::h(a, ss, c, j), tv);
-            continue;
-          }
-          const long long src = nbr_checked(a, x, y, z, -L::cx(j), -L::cy(j), -L::cz(j), percs, &ax);
-          const uint8_t fl = src < 0 ? FL_SOLID : a.flags[src];
-          if (fl == FL_FLUID) {
-            SC* from = R::h(a, R::cell(a.slot[src]), c, L::opp(j));
-            *(R::h(a, ss, c, j)) = *from;
-            Store<SC>::st(from, tv);
-          } else if (fl == FL_FLIPPING) {
-            Store<SC>::st(R::h(a, R::cell(a.slot[src]), c, L::opp(j)), tv);
-          } else {
-            Store<SC>::st(R::h(a, ss, c, j), tv);
-          }
+        if (lane == 0) atomicAdd(&sred[2 + c], C);
+        if (j >= QC) continue;
+        const double wj = double(scal_w<T>(j, k));
+        const T tv = T(wj * (C - double(k.cref[c])));       // h_eq(C_bar, u = 0) - w cref
+        if (parity_next == 0 || j == 0) {
+          Store<SC>::st(R::h(a, ss, c, j), tv);
+        } else if (fls == FL_FLUID) {
+          SC* from = R::h(a, R::cell(a.slot[srcs]), c, o);
+          *R::h(a, ss, c, j) = *from;
+          Store<SC>::st(from, tv);
+        } else if (fls == FL_FLIPPING) {
+          Store<SC>::st(R::h(a, R::cell(a.slot[srcs]), c, o), tv);
+        } else {
+          Store<SC>::st(R::h(a, ss, c, j), tv);
         }
       }
-    } else if (parity_next == 1) {
+    } else if (parity_next == 1 && j > 0) {
       // deposition in the swapped layout: a remaining fluid neighbour y = s + c_d now reads its
       // population from the new wall at (y, d); give it what s streamed toward it, (s, opp d)
-      for (int c = 0; c < NC; ++c) {
-        for (int d = 1; d < Q; ++d) {
-          const long long yn = nbr_checked(a, x, y, z, L::cx(d), L::cy(d), L::cz(d), percf, &ax);
-          if (yn < 0 || a.flags[yn] != FL_FLUID) continue;
-          *(R::f(a, R::cell(a.slot[yn]), c, d)) = *(R::f(a, ss, c, L::opp(d)));
-        }
-      }
-      for (int c = 0; c < NS; ++c) {
-        for (int d = 1; d < QC; ++d) {
-          const long long yn = nbr_checked(a, x, y, z, L::cx(d), L::cy(d), L::cz(d), percs, &ax);
-          if (yn < 0 || a.flags[yn] != FL_FLUID) continue;
-          *(R::h(a, R::cell(a.slot[yn]), c, d)) = *(R::h(a, ss, c, L::opp(d)));
-        }
-      }
+      if (j < Q && srcf >= 0 && flf == FL_FLUID)
+        for (int c = 0; c < NC; ++c) *R::f(a, R::cell(a.slot[srcf]), c, j) = *R::f(a, ss, c, o);
+      if (j < QC && srcs >= 0 && fls == FL_FLUID)
+        for (int c = 0; c < NS; ++c) *R::h(a, R::cell(a.slot[srcs]), c, j) = *R::h(a, ss, c, o);
     }
+    __syncwarp();
   }
-  __syncthreads();
+  cluster_barrier();
   // ---- phase 3: final flags; new fluid nodes join the fluid list (removed ones are skipped by
   // their mask until the next rebuild)
-  for (unsigned int e = threadIdx.x; e < cnt; e += blockDim.x) {
-    if (a.flip_list[e] == 0xffffffffu) continue;
+  for (unsigned int e = first; e < cnt; e += step) {
+    if (a.flip_list[e] == 0xffffffffu || lane != 0) continue;
     leave_flipping(a.flags, a.flip_list[e], dissolve ? FL_FLUID : FL_SOLID);
     if (dissolve) {
       const unsigned int pos = atomicAdd(a.fluid_count, 1u);
@@ -2336,32 +2364,32 @@ __global__ void __launch_bounds__(1024) k_flip(const Args a, const Coef<typename
       else atomicOr(a.err, ERR_CAPACITY);
     }
   }
-  __syncthreads();
-  // ---- phase 4: masks around every flipped node
-  for (unsigned int e = threadIdx.x; e < cnt; e += blockDim.x) {
+  __syncwarp();
+  cluster_barrier();
+  // ---- phase 4: masks around every flipped node, lane i: neighbour i (lane 0: the node itself)
+  for (unsigned int e = first; e < cnt; e += step) {
     if (a.flip_list[e] == 0xffffffffu) continue;
     const long long s = a.flip_list[e];
     int x, y, z, ax;
     coords_of(a, s, &x, &y, &z);
-    a.mask[s] = compute_mask<L>(a, x, y, z);
-    for (int i = 1; i < Q; ++i) {
-      const long long q = nbr_checked(a, x, y, z, L::cx(i), L::cy(i), L::cz(i), percf, &ax);
-      if (q < 0) continue;
-      int qx, qy, qz;
-      coords_of(a, q, &qx, &qy, &qz);
-      a.mask[q] = compute_mask<L>(a, qx, qy, qz);
-    }
-    if (dissolve) {
-      // reactive solids that now touch the new fluid node join the interface list
-      for (int j = 1; j < QC; ++j) {
-        const long long q = nbr_checked(a, x, y, z, L::cx(j), L::cy(j), L::cz(j), percs, &ax);
-        if (q >= 0 && a.flags[q] == FL_REACTIVE && cas_flag(a.listed, q, 0, 1, a.err)) push_iface(a, q);
+    if (lane < Q) {
+      const long long q = lane == 0 ? s : nbr_checked(a, x, y, z, L::cx(lane), L::cy(lane), L::cz(lane), percf, &ax);
+      if (q >= 0) {
+        int qx, qy, qz;
+        coords_of(a, q, &qx, &qy, &qz);
+        a.mask[q] = compute_mask<L>(a, qx, qy, qz);
       }
     }
+    if (dissolve && lane > 0 && lane < QC) {
+      // reactive solids that now touch the new fluid node join the interface list
+      const long long q = nbr_checked(a, x, y, z, L::cx(lane), L::cy(lane), L::cz(lane), percs, &ax);
+      if (q >= 0 && a.flags[q] == FL_REACTIVE && cas_flag(a.listed, q, 0, 1, a.err)) push_iface(a, q);
+    }
+    __syncwarp();
   }
   __syncthreads();
   if (threadIdx.x < 11 && sred[threadIdx.x] != 0.0) atomicAdd(a.flip_mon + threadIdx.x, sred[threadIdx.x]);
-  if (threadIdx.x == 0) *a.flip_count = 0u;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.flip_count = 0u;
 }
 
 // ================================================================ conduction in the solid

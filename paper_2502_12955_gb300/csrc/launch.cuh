@@ -269,7 +269,7 @@ struct Launchers {
 
   static cudaError_t flip(const Args& a, int parity_next, cudaStream_t st) {
     by_nc_ns(a, [&](auto nc, auto ns) {
-      k_flip<L, S, decltype(nc)::value, decltype(ns)::value><<<1, 1024, 0, st>>>(a, coef(a), parity_next);
+      k_flip<L, S, decltype(nc)::value, decltype(ns)::value><<<kFlipBlocks, kFlipThreads, 0, st>>>(a, coef(a), parity_next);
     });
     return cudaGetLastError();
   }
