@@ -60,6 +60,12 @@ lbm_status lbm_nn_transpose(const void* x, void* y, int64_t R, int32_t Cc, void*
 lbm_status lbm_nn_reduce_splits(const float* part, float* out, int64_t n, int32_t splits, int64_t stride, void* stream);
 /* dx = dy where y > 0, else 0 (gradient through y = relu(x)); n BF16 elements. */
 lbm_status lbm_nn_relu_grad(const void* y, const void* dy, void* dx, int64_t n, void* stream);
+/* Gradient through y = relu(conv + b) with the bias gradient: dx = dy where y > 0, else 0; db[c] = sum_v
+   dx[v][c] (FP32, overwritten).  With dskip, dy is the gradient of the 2x average pooling of y (coarse
+   sizes D/2, H/2, W/2) and dskip the one of its skip connection: the layer's gradient is
+   BF16(BF16(dy / 8) + dskip).  C % 8 == 0, C <= 2048, 16-byte aligned arrays of D*H*W voxels. */
+lbm_status lbm_nn_relu_grad_bias(const void* y, const void* dy, const void* dskip, void* dx, float* db, int32_t D, int32_t H,
+                                 int32_t W, int32_t C, void* stream);
 /* 2x average pooling of in [D*H*W][C] into out [D/2*H/2*W/2][C] (D, H, W even), or with
    backward = 1 its gradient: in = dL/dout (coarse), out = dL/din (fine, D*H*W). */
 lbm_status lbm_nn_pool2(const void* in, void* out, int32_t D, int32_t H, int32_t W, int32_t C, int32_t backward,
@@ -95,6 +101,28 @@ lbm_status lbm_nn_pack_weights(const float* w, void* wk, void* wt, int32_t Co, i
                                void* stream);
 /* dwcol [27 Ci][Co] (k = tap Ci + c, FP32) -> dw [Co][Ci][27]. */
 lbm_status lbm_nn_unpack_wgrad(const float* dwcol, float* dw, int32_t Co, int32_t Ci, void* stream);
+/* 3^3 convolution without im2col rows (tcgen05, implicit GEMM): y [D*H*W][N] = conv(x) + bias (bias may be
+   NULL), then max(., 0) with relu.  x is xa [.][Ca], on the coarse grid (D/2, H/2, W/2) and upsampled 2x if up,
+   followed along the channels by xb [D*H*W][Cb] (Cb == 0: none).  Ca and Cb multiples of 16, or one input of at
+   most 8 channels.  N % 16 == 0, N <= 256.  Columns [0, n0) go to y0 [.][n0], the rest to y1 [.][N - n0] (n0 == N:
+   y1 unused).  wp: the weights from lbm_nn_conv3_pack (wp for the convolution with N = Co; wtp with dL/dy as x and
+   N = Ci for its input gradient).  Arrays 16-byte aligned (the narrow input excepted).  The same sums
+   in the same order as lbm_nn_im2col + lbm_nn_gemm_tn. */
+lbm_status lbm_nn_conv3(const void* xa, int32_t Ca, int32_t up, const void* xb, int32_t Cb, int32_t D, int32_t H, int32_t W,
+                        const void* wp, int32_t N, const float* bias, int32_t relu, void* y0, int32_t n0, void* y1,
+                        void* stream);
+/* Weight gradient of that convolution: dw [Co][Ca+Cb][27] (FP32) from dy [D*H*W][Co] (Co % 16 == 0), with
+   lbm_nn_conv3_wgrad_scratch floats of device scratch. */
+lbm_status lbm_nn_conv3_wgrad(const void* xa, int32_t Ca, int32_t up, const void* xb, int32_t Cb, int32_t D, int32_t H,
+                              int32_t W, const void* dy, int32_t Co, float* scratch, float* dw, void* stream);
+int64_t lbm_nn_conv3_wgrad_scratch(int32_t D, int32_t H, int32_t W, int32_t C, int32_t Co);
+/* Weights w [Co][Ci][27] (FP32) in the operand order of lbm_nn_conv3: wp (lbm_nn_conv3_packed(Co, Ci) BF16 elements)
+   and, if wtp is not NULL, the flipped transpose for the input gradient (lbm_nn_conv3_packed(Ci, Co)). */
+lbm_status lbm_nn_conv3_pack(const float* w, void* wp, void* wtp, int32_t Co, int32_t Ci, void* stream);
+int64_t lbm_nn_conv3_packed(int32_t Co, int32_t Ci);
+/* 1 if lbm_nn_conv3 and lbm_nn_conv3_wgrad take a layer of these channels, its input gradient included
+   (shared and tensor memory hold its operands), else 0. */
+int32_t lbm_nn_conv3_fits(int32_t Ca, int32_t up, int32_t Cb, int32_t Co);
 /* y = a + b, n BF16 elements. */
 lbm_status lbm_nn_add(const void* a, const void* b, void* y, int64_t n, void* stream);
 /* y = BF16(x), n elements. */

@@ -29,91 +29,13 @@
 #include <cstring>
 
 #include "../../include/lbm_nn.h"
+#include "tc.cuh"
 
 namespace lbmnn {
-
-using bf16 = __nv_bfloat16;
 
 constexpr int BM = 128;         // output rows per CTA (TMEM lanes)
 constexpr int BK = 64;          // K per stage: 64 BF16 = one 128-byte swizzle row
 constexpr int STAGES = 4;
-constexpr unsigned kWaitLimit = 1u << 22;   // polls of an mbarrier before a wait gives up
-
-// ------------------------------------------------------------------ PTX helpers
-
-__device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* b, unsigned n) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(saddr(b)), "r"(n) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(saddr(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity) {
-  for (unsigned it = 0; it < kWaitLimit; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(saddr(b)), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-// 2D tiled TMA load of box {x .. x + 63, y .. y + rows - 1} into shared memory, counted on bar
-__device__ __forceinline__ void tma_load_2d(const CUtensorMap* map, void* dst, uint64_t* bar, int x, int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n" ::"r"(
-          saddr(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(saddr(bar))
-      : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-
-// Shared-memory matrix descriptor of a K-major tile written by TMA with the 128-byte swizzle:
-// rows of 128 bytes, 8-row groups 1024 bytes apart (stride byte offset); the leading byte offset
-// is not used by this layout.  Bits: start address >> 4 [0, 14), leading offset >> 4 [16, 30),
-// stride offset >> 4 [32, 46), descriptor version 1 [46, 48), layout 2 = 128-byte swizzle [61, 64).
-__device__ __forceinline__ uint64_t desc_sw128(const void* p) {
-  uint64_t d = (uint64_t)((saddr(p) >> 4) & 0x3FFFu);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-// Instruction descriptor of kind::f16: FP32 accumulator [4, 6) = 1, A and B BF16 [7, 10) = 1,
-// [10, 13) = 1, both K-major (bits 15, 16 clear), N >> 3 at [17, 23), M >> 4 at [24, 29).
-__host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-// arrive on bar once every tcgen05 operation this thread issued before has completed
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(saddr(bar))
-               : "memory");
-}
-// 16 consecutive FP32 columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
-      "[%16];\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 // ------------------------------------------------------------------ GEMM
 
@@ -364,6 +286,90 @@ __global__ void k_relu_grad(const bf16* __restrict__ y, const bf16* __restrict__
     dx[i] = __bfloat162float(y[i]) > 0.f ? dy[i] : __float2bfloat16_rn(0.f);
 }
 
+// 8 BF16 values as one 16-byte word
+union Vec8 {
+  uint4 u;
+  bf16 v[8];
+};
+__device__ __forceinline__ Vec8 ld8(const bf16* p) {
+  Vec8 r;
+  r.u = *reinterpret_cast<const uint4*>(p);
+  return r;
+}
+
+// Gradient through y = relu(conv + b), together with the bias gradient: dx = dy where y > 0, else 0, and
+// db[c] += sum_v dx[v][c].  With POOL, dy is itself the gradient of the layer's 2x average pooling plus the one of
+// its skip connection: dy = BF16(BF16(dpool / 8) + dskip), rounded like the separate passes it replaces.
+// One thread per 8 channels; a block's threads keep their channels from voxel to voxel (256 is a multiple of
+// C / 8 threads per voxel, or the rest of the block idles), so the bias sums stay in registers and the block adds
+// each of them once.
+template <bool POOL>
+__global__ void __launch_bounds__(256) k_relu_grad_bias(const bf16* __restrict__ y, const bf16* __restrict__ dy,
+                                                        const bf16* __restrict__ dskip, bf16* __restrict__ dx,
+                                                        float* __restrict__ db, long long V, int C, int H, int W) {
+  __shared__ float red[256][9];
+  const int c8n = C / 8, rows = 256 / c8n;   // voxels per block and pass
+  const int c8 = threadIdx.x % c8n, r = threadIdx.x / c8n;
+  float s[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) s[i] = 0.f;
+  if (r < rows)
+    for (long long v = (long long)blockIdx.x * rows + r; v < V; v += (long long)gridDim.x * rows) {
+      const long long at = v * C + c8 * 8;
+      const Vec8 a = ld8(y + at);
+      Vec8 d;
+      if (POOL) {
+        const int xx = (int)(v % W), yy = (int)((v / W) % H), zz = (int)(v / ((long long)W * H));
+        const Vec8 p = ld8(dy + (((long long)(zz / 2) * (H / 2) + yy / 2) * (W / 2) + xx / 2) * C + c8 * 8);
+        const Vec8 k = ld8(dskip + at);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          d.v[i] = __float2bfloat16_rn(__bfloat162float(__float2bfloat16_rn(__bfloat162float(p.v[i]) * 0.125f)) +
+                                       __bfloat162float(k.v[i]));
+      } else {
+        d = ld8(dy + at);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (!(__bfloat162float(a.v[i]) > 0.f)) d.v[i] = __float2bfloat16_rn(0.f);
+        s[i] += __bfloat162float(d.v[i]);
+      }
+      *reinterpret_cast<uint4*>(dx + at) = d.u;
+    }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) red[threadIdx.x][i] = s[i];
+  __syncthreads();
+  for (int c = threadIdx.x; c < C; c += 256) {
+    float t = 0.f;
+    for (int k = 0; k < rows; ++k) t += red[k * c8n + c / 8][c % 8];
+    atomicAdd(&db[c], t);
+  }
+}
+
+// The pooling and upsampling passes for C % 8 == 0: one thread per 8 channels, the same sums in the same order.
+__global__ void __launch_bounds__(256) k_pool2_vec(const bf16* __restrict__ in, bf16* __restrict__ out, int D, int H, int W,
+                                                   int C, float scale) {
+  // out[coarse] = scale * sum over its 2x2x2 block of in (D, H, W: the fine sizes)
+  const int d = D / 2, h = H / 2, w = W / 2, c8n = C / 8;
+  const long long total = (long long)d * h * w * c8n;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    const int c8 = (int)(i % c8n);
+    const int v = (int)(i / c8n);
+    const int xx = v % w, yy = (v / w) % h, zz = v / (w * h);
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const Vec8 p = ld8(in + (((long long)(2 * zz + (a >> 2)) * H + 2 * yy + ((a >> 1) & 1)) * W + 2 * xx + (a & 1)) * C + c8 * 8);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s[k] += __bfloat162float(p.v[k]);
+    }
+    Vec8 o;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) o.v[k] = __float2bfloat16_rn(s[k] * scale);
+    *reinterpret_cast<uint4*>(out + (long long)v * C + c8 * 8) = o.u;
+  }
+}
+
 // 2x average pooling (forward: x fine -> y coarse) and its gradient (dy coarse -> dx fine)
 __global__ void k_pool2(const bf16* __restrict__ in, bf16* __restrict__ out, int D, int H, int W, int C, int backward) {
   const int d = D / 2, h = H / 2, w = W / 2;
@@ -458,13 +464,35 @@ __global__ void k_head_fwd(const bf16* __restrict__ h, const float* __restrict__
     }
 }
 
+// The same for the network's head (16 channels, 4 outputs): a voxel's row is two 16-byte words, its result one.
+__global__ void __launch_bounds__(256) k_head_fwd_16x4(const bf16* __restrict__ h, const float* __restrict__ w,
+                                                       const float* __restrict__ b, float* __restrict__ y, long long V) {
+  float wr[64], br[4];
+#pragma unroll
+  for (int i = 0; i < 64; ++i) wr[i] = __ldg(w + i);
+#pragma unroll
+  for (int o = 0; o < 4; ++o) br[o] = __ldg(b + o);
+  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
+    const Vec8 p[2] = {ld8(h + v * 16), ld8(h + v * 16 + 8)};
+    float s[4];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      s[o] = br[o];
+#pragma unroll
+      for (int c = 0; c < 16; ++c) s[o] = fmaf(wr[o * 16 + c], __bfloat162float(p[c >> 3].v[c & 7]), s[o]);
+    }
+    *reinterpret_cast<float4*>(y + v * 4) = make_float4(s[0], s[1], s[2], s[3]);
+  }
+}
+
 // Head gradients: dh[v][c] = sum_o w[o][c] dy[v][o] (BF16); dw[o][c] = sum_v dy[v][o] h[v][c] and
-// db[o] = sum_v dy[v][o] (FP32: per-thread sums, then one warp reduction and one atomic per warp and
+// db[o] = sum_v dy[v][o] (FP32: per-thread sums, a block reduction and one atomic per block and
 // entry; dw, db zeroed first).  C and Co are the head's fixed sizes.
 template <int C, int Co>
 __global__ void __launch_bounds__(256) k_head_bwd(const bf16* __restrict__ h, const float* __restrict__ w,
                                                   const float* __restrict__ dy, bf16* __restrict__ dh,
                                                   float* __restrict__ dw, float* __restrict__ db, long long V) {
+  __shared__ float red[8][Co * (C + 1)];
   float acc[Co * (C + 1)];
 #pragma unroll
   for (int i = 0; i < Co * (C + 1); ++i) acc[i] = 0.f;
@@ -492,17 +520,23 @@ __global__ void __launch_bounds__(256) k_head_bwd(const bf16* __restrict__ h, co
   for (int i = 0; i < Co * (C + 1); ++i) {
     float s = acc[i];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) {
-      const int o = i / (C + 1), c = i % (C + 1);
-      atomicAdd(c < C ? &dw[o * C + c] : &db[o], s);
-    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][i] = s;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < Co * (C + 1); i += 256) {
+    float s = 0.f;
+    for (int k = 0; k < 8; ++k) s += red[k][i];
+    const int o = i / (C + 1), c = i % (C + 1);
+    atomicAdd(c < C ? &dw[o * C + c] : &db[o], s);
   }
 }
 
 // Masked mean squared error over fluid voxels: loss += sum (y - t)^2 / (n_fluid Co) and
 // dy = 2 (y - t) / (n_fluid Co) on fluid voxels, 0 elsewhere (loss zeroed first)
-__global__ void k_mse(const float* __restrict__ y, const float* __restrict__ t, const uint8_t* __restrict__ fluid,
-                      float* __restrict__ dy, double* __restrict__ loss, long long V, int Co, double inv_n) {
+__global__ void __launch_bounds__(256) k_mse(const float* __restrict__ y, const float* __restrict__ t,
+                                             const uint8_t* __restrict__ fluid, float* __restrict__ dy,
+                                             double* __restrict__ loss, long long V, int Co, double inv_n) {
+  __shared__ double red[8];
   double s = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V * Co; i += (long long)gridDim.x * blockDim.x) {
     const long long v = i / Co;
@@ -511,7 +545,12 @@ __global__ void k_mse(const float* __restrict__ y, const float* __restrict__ t, 
     dy[i] = (float)(2.0 * d * inv_n);
   }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, s * inv_n);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) s += red[k];
+    atomicAdd(loss, s * inv_n);
+  }
 }
 
 // Adam (Kingma and Ba 2015) on FP32 master weights
@@ -617,6 +656,12 @@ cudaError_t launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, int M, int
   dim3 grid(N / BN, M / BM, splits);
   k_gemm_tn<BN><<<grid, 128, SM::bytes, st>>>(ta, tb, K, kbs, o, err_word());
   return cudaGetLastError();
+}
+
+// 16-byte vector access: channels in groups of 8 and aligned pointers
+bool vec8_ok(int C, const void* a, const void* b, const void* c = nullptr, const void* d = nullptr) {
+  return C % 8 == 0 && ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b) | reinterpret_cast<uintptr_t>(c) |
+                         reinterpret_cast<uintptr_t>(d)) & 15u) == 0;
 }
 
 unsigned grid_for(long long n) {
@@ -735,10 +780,34 @@ lbm_status lbm_nn_relu_grad(const void* y, const void* dy, void* dx, int64_t n, 
   return LBM_OK;
 }
 
+lbm_status lbm_nn_relu_grad_bias(const void* y, const void* dy, const void* dskip, void* dx, float* db, int32_t D, int32_t H,
+                                 int32_t W, int32_t C, void* stream) {
+  if (!y || !dy || !dx || !db || D <= 0 || H <= 0 || W <= 0 || C <= 0 || C > 2048 || !vec8_ok(C, y, dy, dskip, dx))
+    return LBM_ERR_INVALID_ARG;
+  if (dskip && ((D | H | W) & 1)) return LBM_ERR_INVALID_ARG;
+  const long long V = (long long)D * H * W;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  NN_CK(cudaMemsetAsync(db, 0, sizeof(float) * C, st));
+  const int rows = 256 / (C / 8);
+  long long g = (V + 8ll * rows - 1) / (8ll * rows);   // at least 8 voxels per thread
+  if (g > 152 * 6) g = 152 * 6;
+  auto* kern = dskip ? k_relu_grad_bias<true> : k_relu_grad_bias<false>;
+  kern<<<(unsigned)(g < 1 ? 1 : g), 256, 0, st>>>(static_cast<const bf16*>(y), static_cast<const bf16*>(dy),
+                                                 static_cast<const bf16*>(dskip), static_cast<bf16*>(dx), db, V, C, H, W);
+  NN_CK(cudaGetLastError());
+  return LBM_OK;
+}
+
 lbm_status lbm_nn_pool2(const void* in, void* out, int32_t D, int32_t H, int32_t W, int32_t C, int32_t backward,
                         void* stream) {
   if (!in || !out || D < 2 || H < 2 || W < 2 || (D | H | W) & 1 || C <= 0) return LBM_ERR_INVALID_ARG;
   const long long n = (long long)D * H * W * C;
+  if (!backward && vec8_ok(C, in, out) && (long long)D * H * W < (1ll << 31)) {
+    k_pool2_vec<<<grid_for(n / 64), 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<const bf16*>(in),
+                                                                                static_cast<bf16*>(out), D, H, W, C, 0.125f);
+    NN_CK(cudaGetLastError());
+    return LBM_OK;
+  }
   k_pool2<<<grid_for(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<const bf16*>(in),
                                                                       static_cast<bf16*>(out), D, H, W, C, backward);
   NN_CK(cudaGetLastError());
@@ -749,6 +818,12 @@ lbm_status lbm_nn_up2(const void* in, void* out, int32_t D, int32_t H, int32_t W
                       void* stream) {
   if (!in || !out || D <= 0 || H <= 0 || W <= 0 || C <= 0) return LBM_ERR_INVALID_ARG;
   const long long n = 8LL * D * H * W * C;
+  if (backward && vec8_ok(C, in, out) && 8LL * D * H * W < (1ll << 31)) {
+    k_pool2_vec<<<grid_for(n / 64), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+        static_cast<const bf16*>(in), static_cast<bf16*>(out), 2 * D, 2 * H, 2 * W, C, 1.f);
+    NN_CK(cudaGetLastError());
+    return LBM_OK;
+  }
   k_up2<<<grid_for(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<const bf16*>(in), static_cast<bf16*>(out),
                                                                     D, H, W, C, backward);
   NN_CK(cudaGetLastError());
@@ -779,6 +854,11 @@ lbm_status lbm_nn_colsum(const void* x, float* out, int64_t V, int32_t C, void* 
 lbm_status lbm_nn_head_fwd(const void* h, const float* w, const float* b, float* y, int64_t V, int32_t C, int32_t Co,
                            void* stream) {
   if (!h || !w || !b || !y || V <= 0 || C <= 0 || Co <= 0) return LBM_ERR_INVALID_ARG;
+  if (C == 16 && Co == 4 && vec8_ok(16, h, y)) {
+    k_head_fwd_16x4<<<grid_for(V), 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<const bf16*>(h), w, b, y, V);
+    NN_CK(cudaGetLastError());
+    return LBM_OK;
+  }
   k_head_fwd<<<grid_for(V), 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<const bf16*>(h), w, b, y, V, C, Co);
   NN_CK(cudaGetLastError());
   return LBM_OK;
@@ -803,7 +883,9 @@ lbm_status lbm_nn_mse(const float* y, const float* t, const uint8_t* fluid, floa
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   NN_CK(cudaMemsetAsync(loss, 0, sizeof(double), st));
   const double inv_n = 1.0 / ((double)(n_fluid > 0 ? n_fluid : 1) * Co);
-  k_mse<<<grid_for(V * Co), 256, 0, st>>>(y, t, fluid, dy, loss, V, Co, inv_n);
+  unsigned g = grid_for(V * Co);
+  if (g > 152 * 6) g = 152 * 6;   // one FP64 atomic per block
+  k_mse<<<g, 256, 0, st>>>(y, t, fluid, dy, loss, V, Co, inv_n);
   NN_CK(cudaGetLastError());
   return LBM_OK;
 }

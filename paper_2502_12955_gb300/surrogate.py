@@ -8,8 +8,8 @@ arbiter of the network's error.
 
 Binding: the `lbm_nn_*` functions below carry the C ABI's names (include/lbm_nn.h) and only
 marshal torch tensors into device pointers; every operation runs in liblbm.so's sm_103a kernels
-(the 3^3 convolutions as im2col + tcgen05 GEMMs, BF16 storage, FP32 accumulation).  PyTorch is
-used for device memory and the stream only.
+(the 3^3 convolutions as implicit GEMMs on the tcgen05 tensor cores, BF16 storage, FP32 accumulation).
+PyTorch is used for device memory and the stream only.
 
 Network (the same plan as the FP64 reference of the test suite): encoder levels of two 3^3
 convolutions (ReLU) and 2x average pooling, a bottleneck of two 3^3 convolutions, decoder levels
@@ -66,6 +66,10 @@ def nn_lib():
         "lbm_nn_unpack_wgrad": [vp, vp, i32, i32, vp],
         "lbm_nn_add": [vp, vp, vp, i64, vp],
         "lbm_nn_cast_bf16": [vp, vp, i64, vp],
+        "lbm_nn_relu_grad_bias": [vp, vp, vp, vp, vp, i32, i32, i32, i32, vp],
+        "lbm_nn_conv3": [vp, i32, i32, vp, i32, i32, i32, i32, vp, i32, vp, i32, vp, i32, vp, vp],
+        "lbm_nn_conv3_wgrad": [vp, i32, i32, vp, i32, i32, i32, i32, vp, i32, vp, vp, vp],
+        "lbm_nn_conv3_pack": [vp, vp, vp, i32, i32, vp],
     }
     for name, args in sig.items():
         fn = getattr(lib, name)
@@ -73,6 +77,12 @@ def nn_lib():
         fn.restype = C.c_int
     lib.lbm_nn_gemm_splits.argtypes = [i32, i32]
     lib.lbm_nn_gemm_splits.restype = i32
+    lib.lbm_nn_conv3_packed.argtypes = [i32, i32]
+    lib.lbm_nn_conv3_packed.restype = i64
+    lib.lbm_nn_conv3_fits.argtypes = [i32, i32, i32, i32]
+    lib.lbm_nn_conv3_fits.restype = i32
+    lib.lbm_nn_conv3_wgrad_scratch.argtypes = [i32, i32, i32, i32, i32]
+    lib.lbm_nn_conv3_wgrad_scratch.restype = i64
     _NN = lib
     return lib
 
@@ -177,6 +187,37 @@ def lbm_nn_cast_bf16(x, y, n):
     _call("lbm_nn_cast_bf16", _p(x), _p(y), n)
 
 
+def lbm_nn_relu_grad_bias(y, dy, dskip, dx, db, shape, Cc):
+    _call("lbm_nn_relu_grad_bias", _p(y), _p(dy), _p(dskip), _p(dx), _p(db), *shape, Cc)
+
+
+def lbm_nn_conv3(src, shape, wp, N, y0, n0, y1=None, bias=None, relu=0):
+    """src: (xa, Ca, up, xb, Cb), the input's parts (xb None with Cb 0)."""
+    xa, ca, up, xb, cb = src
+    _call("lbm_nn_conv3", _p(xa), ca, up, _p(xb), cb, *shape, _p(wp), N, _p(bias), relu, _p(y0), n0, _p(y1))
+
+
+def lbm_nn_conv3_wgrad(src, shape, dy, Co, scratch, dw):
+    xa, ca, up, xb, cb = src
+    _call("lbm_nn_conv3_wgrad", _p(xa), ca, up, _p(xb), cb, *shape, _p(dy), Co, _p(scratch), _p(dw))
+
+
+def lbm_nn_conv3_wgrad_scratch(shape, Cc, Co):
+    return int(nn_lib().lbm_nn_conv3_wgrad_scratch(*shape, Cc, Co))
+
+
+def lbm_nn_conv3_pack(w, wp, wtp, Co, Ci):
+    _call("lbm_nn_conv3_pack", _p(w), _p(wp), _p(wtp), Co, Ci)
+
+
+def lbm_nn_conv3_packed(Co, Ci):
+    return int(nn_lib().lbm_nn_conv3_packed(Co, Ci))
+
+
+def lbm_nn_conv3_fits(Ca, up, Cb, Co):
+    return bool(nn_lib().lbm_nn_conv3_fits(Ca, up, Cb, Co))
+
+
 # ------------------------------------------------------------------ network
 
 def kpad(k):
@@ -259,180 +300,185 @@ class WarmStartNet:
         return {k: v.detach().cpu().numpy().copy() for k, v in self.g.items()}
 
     def _pack(self):
-        """BF16 GEMM copies of the 3^3 kernels: wk [Co][Kp] and the flipped transpose wt [Ci][Kpt]."""
+        """BF16 operands of the 3^3 kernels: wp for the convolution, wt (flipped, transposed) for its
+        input gradient; layers that lbm_nn_conv3 does not take get the im2col GEMM's."""
         torch = self.torch
-        if not hasattr(self, "wk"):
-            self.wk, self.wt = {}, {}
+        if not hasattr(self, "wp"):
+            bf = dict(dtype=torch.bfloat16, device=self.dev)
+            self.wp, self.wt, self.rows = {}, {}, {}
             for name, kind, ci, co in self.plan:
-                if kind == "conv3":
-                    self.wk[name] = torch.empty((co, kpad(27 * ci)), dtype=torch.bfloat16, device=self.dev)
-                    self.wt[name] = torch.empty((ci, kpad(27 * co)), dtype=torch.bfloat16, device=self.dev)
+                if kind != "conv3":
+                    continue
+                cb = self.width[int(name[3])] if name.startswith("dec") else 0
+                self.rows[name] = not lbm_nn_conv3_fits(ci - cb, cb > 0, cb, co)
+                if self.rows[name]:
+                    self.wp[name] = torch.empty((co, kpad(27 * ci)), **bf)
+                    self.wt[name] = torch.empty((ci, kpad(27 * co)), **bf)
+                else:
+                    self.wp[name] = torch.empty(lbm_nn_conv3_packed(co, ci), **bf)
+                    self.wt[name] = torch.empty(lbm_nn_conv3_packed(ci, co), **bf) if ci % 16 == 0 else None
         for name, kind, ci, co in self.plan:
-            if kind == "conv3":
-                lbm_nn_pack_weights(self.p[name + ".w"], self.wk[name], self.wt[name], co, ci, kpad(27 * ci),
-                                    kpad(27 * co))
-
-    # -------------------------------------------------------------- buffers
-
-    def _scratch_for(self, shape):
-        """BF16 im2col scratch and FP32 split-K partials sized for an input of this shape."""
-        D, H, W = shape
-        need, part = 0, 0
-        for l, (name, kind, ci, co) in enumerate(self.plan):
             if kind != "conv3":
                 continue
-            V = self._level_volume(name, shape)
-            need = max(need, V * kpad(27 * ci), V * kpad(27 * co))
-            part = max(part, kpad(27 * ci) * co * 64)
-        if self._scratch is None or self._scratch[0] < need or self._scratch[2] < part:
-            torch = self.torch
-            self._scratch = (need, torch.empty(need, dtype=torch.bfloat16, device=self.dev), part,
-                             torch.empty(part, dtype=torch.float32, device=self.dev))
-        return self._scratch[1], self._scratch[3]
-
-    def _level_volume(self, name, shape):
-        D, H, W = shape
-        if name.startswith("enc"):
-            lv = int(name[3])
-        elif name.startswith("dec"):
-            lv = int(name[3])
-        else:
-            lv = self.L
-        return (D >> lv) * (H >> lv) * (W >> lv)
+            if self.rows[name]:
+                lbm_nn_pack_weights(self.p[name + ".w"], self.wp[name], self.wt[name], co, ci, kpad(27 * ci), kpad(27 * co))
+            else:
+                lbm_nn_conv3_pack(self.p[name + ".w"], self.wp[name], self.wt[name], co, ci)
 
     # -------------------------------------------------------------- layers
+    # An input is (xa, Ca, up, xb, Cb): one tensor, or the decoder's pair of a coarse tensor, upsampled as it is
+    # read, and the encoder's output of the level.
 
-    def _conv3(self, name, x, shape, ci, co):
-        torch = self.torch
-        D, H, W = shape
-        V = D * H * W
-        kp = kpad(27 * ci)
-        col, _ = self._scratch_for(self._in_shape)
-        lbm_nn_im2col(x, col, D, H, W, ci, kp, 0)
-        y = torch.empty((V, co), dtype=torch.bfloat16, device=self.dev)
-        lbm_nn_gemm_tn(col, self.wk[name], y, co, V, co, kp, 1, OUT_BF16_RELU, self.p[name + ".b"])
+    def _empty(self, rows, cols, dtype=None):
+        return self.torch.empty((rows, cols), dtype=dtype or self.torch.bfloat16, device=self.dev)
+
+    def _scratch_for(self, n):
+        if self._scratch is None or self._scratch.numel() < n:
+            self._scratch = self.torch.empty(n, dtype=self.torch.float32, device=self.dev)
+        return self._scratch
+
+    def _conv3(self, name, src, shape, co):
+        V = shape[0] * shape[1] * shape[2]
+        if V % 128:
+            raise _lbm.LbmError(-1, f"{name}: the number of voxels must be a multiple of 128")
+        y = self._empty(V, co)
+        if self.rows[name]:
+            x, ci = self._joined(src, shape)
+            kp = kpad(27 * ci)
+            col = self._empty(V, kp)
+            lbm_nn_im2col(x, col, *shape, ci, kp, 0)
+            lbm_nn_gemm_tn(col, self.wp[name], y, co, V, co, kp, 1, OUT_BF16_RELU, self.p[name + ".b"])
+        else:
+            lbm_nn_conv3(src, shape, self.wp[name], co, y, co, bias=self.p[name + ".b"], relu=1)
         return y
 
-    def _conv3_backward(self, name, xin, yout, dy, shape, ci, co, need_dx=True):
-        torch = self.torch
+    def _conv3_backward(self, name, src, yout, dy, dskip, shape, co, need_dx=True):
+        """Gradients of a layer's weights and bias from dy (with dskip: dy is the gradient of the pooled
+        output and dskip the skip connection's); returns those of the parts of its input."""
+        V = shape[0] * shape[1] * shape[2]
+        _, ca, _, _, cb = src
+        dpre = self._empty(V, co)
+        lbm_nn_relu_grad_bias(yout, dy, dskip, dpre, self.g[name + ".b"], shape, co)
+        if self.rows[name]:
+            return self._rows_backward(name, src, dpre, shape, co, need_dx)
+        lbm_nn_conv3_wgrad(src, shape, dpre, co, self._scratch_for(lbm_nn_conv3_wgrad_scratch(shape, ca + cb, co)),
+                           self.g[name + ".w"])
+        if not need_dx:
+            return None, None
+        # input gradient: a convolution of dpre with the flipped, transposed kernel
+        da, db = self._empty(V, ca), self._empty(V, cb) if cb else None
+        lbm_nn_conv3((dpre, co, 0, None, 0), shape, self.wt[name], ca + cb, da, ca, db)
+        return da, db
+
+    # Layers outside lbm_nn_conv3's range (an input of 9 or more channels that is no multiple of 16, very wide
+    # layers): im2col rows and plain GEMMs.
+
+    def _joined(self, src, shape):
+        xa, ca, up, xb, cb = src
+        if not cb:
+            return xa, ca
+        D, H, W = shape
+        fine = self._empty(D * H * W, ca)
+        lbm_nn_up2(xa, fine, D // 2, H // 2, W // 2, ca, 0)
+        cat = self._empty(D * H * W, ca + cb)
+        lbm_nn_concat(fine, ca, xb, cb, cat, D * H * W, 0)
+        return cat, ca + cb
+
+    def _rows_backward(self, name, src, dpre, shape, co, need_dx):
         D, H, W = shape
         V = D * H * W
+        _, ca, _, _, cb = src
+        x, ci = self._joined(src, shape)
         kp, kpt = kpad(27 * ci), kpad(27 * co)
-        col, part = self._scratch_for(self._in_shape)
-        dpre = torch.empty_like(dy)
-        lbm_nn_relu_grad(yout, dy, dpre, V * co)
-        lbm_nn_colsum(dpre, self.g[name + ".b"], V, co)
         # weight gradient: dW[k][o] = sum_v colT[k][v] dpreT[o][v], split over v; colT is built
         # from a channel-major copy of the input when the rows allow 8-voxel vectors
+        col = self._empty(kp, V)
         if W % 8 == 0:
-            xT = torch.empty((ci, V), dtype=torch.bfloat16, device=self.dev)
-            lbm_nn_transpose(xin, xT, V, ci)
+            xT = self._empty(ci, V)
+            lbm_nn_transpose(x, xT, V, ci)
             lbm_nn_im2col_cv(xT, col, D, H, W, ci, kp)
         else:
-            lbm_nn_im2col(xin, col, D, H, W, ci, kp, 1)
-        dpreT = torch.empty((co, V), dtype=torch.bfloat16, device=self.dev)
+            lbm_nn_im2col(x, col, D, H, W, ci, kp, 1)
+        dpreT = self._empty(co, V)
         lbm_nn_transpose(dpre, dpreT, V, co)
         tiles = (kp // 128) * max(1, co // 128)
-        want = max(1, min(64, (4 * 152) // max(1, tiles), V // 64))
-        splits = lbm_nn_gemm_splits(V, want)
+        splits = lbm_nn_gemm_splits(V, max(1, min(64, (4 * 152) // max(1, tiles), V // 64)))
+        part = self._scratch_for(splits * kp * co)
         lbm_nn_gemm_tn(col, dpreT, part, co, kp, co, V, splits, OUT_F32, None)
-        dwcol = torch.empty((kp, co), dtype=torch.float32, device=self.dev)
+        dwcol = self._empty(kp, co, self.torch.float32)
         lbm_nn_reduce_splits(part, dwcol, kp * co, splits, kp * co)
         lbm_nn_unpack_wgrad(dwcol, self.g[name + ".w"], co, ci)
         if not need_dx:
-            return None
-        # input gradient: a convolution of dpre with the flipped, transposed kernel
+            return None, None
+        col = self._empty(V, kpt)
         lbm_nn_im2col(dpre, col, D, H, W, co, kpt, 0)
-        dx = torch.empty((V, ci), dtype=torch.bfloat16, device=self.dev)
+        dx = self._empty(V, ci)
         lbm_nn_gemm_tn(col, self.wt[name], dx, ci, V, ci, kpt, 1, OUT_BF16, None)
-        return dx
+        if not cb:
+            return dx, None
+        da, db = self._empty(V, ca), self._empty(V, cb)
+        lbm_nn_concat(da, ca, db, cb, dx, V, 1)
+        return da, db
 
     # -------------------------------------------------------------- passes
 
     def forward(self, x, shape):
         """x: BF16 [V][c_in] channel-last; returns FP32 [V][c_out] and keeps the activations."""
-        torch = self.torch
-        self._in_shape = tuple(shape)
-        acts = {"in": (x, tuple(shape), self.c_in)}
+        # per layer: its input, its output and the sizes
+        acts = {}
         h, shp, c = x, tuple(shape), self.c_in
         skips = []
         for l, wd in enumerate(self.width[:-1]):
             for s in "ab":
-                n = f"enc{l}{s}"
-                h = self._conv3(n, h, shp, c, wd)
+                n, src = f"enc{l}{s}", (h, c, 0, None, 0)
+                h = self._conv3(n, src, shp, wd)
                 c = wd
-                acts[n] = (h, shp, c)
+                acts[n] = (src, h, shp)
             skips.append((h, shp, c))
             D, H, W = shp
-            nxt = (D // 2, H // 2, W // 2)
-            pooled = torch.empty((nxt[0] * nxt[1] * nxt[2], c), dtype=torch.bfloat16, device=self.dev)
+            shp = (D // 2, H // 2, W // 2)
+            pooled = self._empty(shp[0] * shp[1] * shp[2], c)
             lbm_nn_pool2(h, pooled, D, H, W, c, 0)
-            h, shp = pooled, nxt
-            acts[f"pool{l}"] = (h, shp, c)
+            h = pooled
         for n in ("mid_a", "mid_b"):
-            h = self._conv3(n, h, shp, c, self.width[-1])
+            src = (h, c, 0, None, 0)
+            h = self._conv3(n, src, shp, self.width[-1])
             c = self.width[-1]
-            acts[n] = (h, shp, c)
+            acts[n] = (src, h, shp)
         for l in reversed(range(self.L)):
-            sk, sshp, sc = skips[l]
-            D, H, W = shp
-            up = torch.empty((8 * D * H * W, c), dtype=torch.bfloat16, device=self.dev)
-            lbm_nn_up2(h, up, D, H, W, c, 0)
-            V = sshp[0] * sshp[1] * sshp[2]
-            cat = torch.empty((V, c + sc), dtype=torch.bfloat16, device=self.dev)
-            lbm_nn_concat(up, c, sk, sc, cat, V, 0)
-            acts[f"cat{l}"] = (cat, sshp, c + sc)
-            n = f"dec{l}"
-            h = self._conv3(n, cat, sshp, c + sc, self.width[l])
-            shp, c = sshp, self.width[l]
-            acts[n] = (h, shp, c)
+            sk, shp, sc = skips[l]
+            n, src = f"dec{l}", (h, c, 1, sk, sc)
+            h = self._conv3(n, src, shp, self.width[l])
+            c = self.width[l]
+            acts[n] = (src, h, shp)
         V = shp[0] * shp[1] * shp[2]
-        y = torch.empty((V, self.c_out), dtype=torch.float32, device=self.dev)
+        y = self._empty(V, self.c_out, self.torch.float32)
         lbm_nn_head_fwd(h, self.p["head.w"], self.p["head.b"], y, V, c, self.c_out)
         self._acts = acts
         return y
 
     def backward(self, dy):
         """dy: FP32 [V][c_out] = dL/dy of the last forward; fills the gradients."""
-        torch = self.torch
         acts = self._acts
-        h, shp, c = acts["dec0"]
-        V = shp[0] * shp[1] * shp[2]
-        dh = torch.empty((V, c), dtype=torch.bfloat16, device=self.dev)
+        _, h, shp = acts["dec0"]
+        V, c = h.shape
+        dh = self._empty(V, c)
         lbm_nn_head_bwd(h, self.p["head.w"], dy, dh, self.g["head.w"], self.g["head.b"], V, c, self.c_out)
         dskip = {}
         for l in range(self.L):
-            n = f"dec{l}"
-            cat, cshp, cc = acts[f"cat{l}"]
-            y, _, co = acts[n]
-            dcat = self._conv3_backward(n, cat, y, dh, cshp, cc, co)
-            sc = self.width[l]
-            cu = cc - sc
-            Vf = cshp[0] * cshp[1] * cshp[2]
-            du = torch.empty((Vf, cu), dtype=torch.bfloat16, device=self.dev)
-            ds = torch.empty((Vf, sc), dtype=torch.bfloat16, device=self.dev)
-            lbm_nn_concat(du, cu, ds, sc, dcat, Vf, 1)
-            dskip[l] = ds
-            D, H, W = cshp
-            dh = torch.empty((Vf // 8, cu), dtype=torch.bfloat16, device=self.dev)
-            lbm_nn_up2(du, dh, D // 2, H // 2, W // 2, cu, 1)
-        for n, prev in (("mid_b", "mid_a"), ("mid_a", f"pool{self.L - 1}")):
-            xin, xshp, ci = acts[prev]
-            y, _, co = acts[n]
-            dh = self._conv3_backward(n, xin, y, dh, xshp, ci, co)
+            src, y, (D, H, W) = acts[f"dec{l}"]
+            du, dskip[l] = self._conv3_backward(f"dec{l}", src, y, dh, None, (D, H, W), self.width[l])
+            dh = self._empty(D * H * W // 8, src[1])
+            lbm_nn_up2(du, dh, D // 2, H // 2, W // 2, src[1], 1)
+        for n in ("mid_b", "mid_a"):
+            src, y, shp = acts[n]
+            dh, _ = self._conv3_backward(n, src, y, dh, None, shp, self.width[-1])
         for l in reversed(range(self.L)):
-            sk, sshp, sc = acts[f"enc{l}b"]
-            D, H, W = sshp
-            Vf = D * H * W
-            up = torch.empty((Vf, sc), dtype=torch.bfloat16, device=self.dev)
-            lbm_nn_pool2(dh, up, D, H, W, sc, 1)
-            dh = torch.empty_like(up)
-            lbm_nn_add(up, dskip[l], dh, Vf * sc)
-            for s, prev in (("b", f"enc{l}a"), ("a", f"pool{l - 1}" if l > 0 else "in")):
-                n = f"enc{l}{s}"
-                xin, xshp, ci = acts[prev]
-                y, _, co = acts[n]
-                dh = self._conv3_backward(n, xin, y, dh, xshp, ci, co, need_dx=not (l == 0 and s == "a"))
+            # the pooling's gradient and the skip connection's meet in the layer's ReLU gradient
+            src, y, shp = acts[f"enc{l}b"]
+            dh, _ = self._conv3_backward(f"enc{l}b", src, y, dh, dskip[l], shp, self.width[l])
+            src, y, shp = acts[f"enc{l}a"]
+            dh, _ = self._conv3_backward(f"enc{l}a", src, y, dh, None, shp, self.width[l], need_dx=l > 0)
 
     def loss_and_grad(self, y, t, fluid, n_fluid):
         torch = self.torch
