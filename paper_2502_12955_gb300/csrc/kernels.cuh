@@ -1,7 +1,7 @@
 // kernels.cuh -- sm_103a kernels of the reactive multi-component LBM step.
 //
-// Storage: tiles of 32 slots (see Rec).  A tile holds one row of 32 elements per population of
-// every lattice, the flow components first, so all populations of a warp's 32 slots are one
+// Storage: tiles of kTile slots (see Rec).  A tile holds one row of kTile elements per population of
+// every lattice, the flow components first, so all populations of a warp's 32 slots lie in one
 // contiguous record.  Node n = x + nx*(y + ny*z) sits at slot[n]; the slot map puts the fluid nodes
 // first, in list order, so a warp's lanes touch consecutive elements of every row and no cache
 // line carries solid-node bytes.  The cells named (n, i) below are row i at slot[n].
@@ -122,7 +122,7 @@ __host__ __device__ __forceinline__ unsigned int fast_div(unsigned int n, FastDi
 
 // Everything a kernel needs, in double; kernels convert to their compute type.
 struct Args {
-  unsigned char* pop;        // every population, in tiles of 32 slots (see Rec): the flow components,
+  unsigned char* pop;        // every population, in tiles of kTile slots (see Rec): the flow components,
                              // the given scalars, then the reaction product (if any)
   long long pop_bytes;
   void* psi[2];              // compute-type psi per component (Shan-Chen only)
@@ -313,27 +313,33 @@ __device__ __forceinline__ Nbr nbr_entry(const Args& a, int n, uint32_t entry) {
 
 // ------------------------------------------------------------- population tiles
 
-// Record of one tile of 32 slots: NC * Q rows of 32 flow elements, then NS * QC rows of 32 scalar
+// Record of one tile of kTile slots: NC * Q rows of kTile flow elements, then NS * QC rows of kTile scalar
 // elements.  One record is a contiguous stretch (3.3 KB for D3Q19 + D3Q7 in FP32), so an even step
 // reads and writes each of a warp's rows from one base address with constant offsets and within
 // a few DRAM pages, where planes of the whole domain put every population in a page of its own.
+// kTile is 64 for 16-bit flow elements and 32 otherwise: a row is then at least one 128-byte line.  An unaligned run
+// of 32 neighbour cells (odd steps) in rows of 32 16-bit elements always crosses into another line, in rows of
+// 64 half of the time: 232 x 203 x 181 with FP16 flow and FP32 scalars, odd step 200 us with 32, 188 us with 64.
+// FP32 rows of 64 are no faster (256^3, both parities together 638 us each way).
+__host__ __device__ constexpr int tile_slots(int elem) { return elem == 2 ? 64 : 32; }
 template <class L, class S, int NC, int NS>
 struct Rec {
   using SC = typename ScalarOf<S>::type;
-  static constexpr int FROW = 32 * (int)sizeof(S), HROW = 32 * (int)sizeof(SC);
+  static constexpr int kTile = tile_slots((int)sizeof(S));
+  static constexpr int FROW = kTile * (int)sizeof(S), HROW = kTile * (int)sizeof(SC);
   static constexpr int H0 = NC * L::Q * FROW;
   static constexpr int BYTES = H0 + NS * L::QC * HROW;
   static constexpr bool kSameElem = sizeof(S) == sizeof(SC);
   __host__ __device__ static constexpr int frow(int s, int i) { return (s * L::Q + i) * FROW; }
   __host__ __device__ static constexpr int hrow(int s, int j) { return H0 + (s * L::QC + j) * HROW; }
   // byte offset of the first flow cell of a slot, and of its first scalar cell less H0
-  __device__ __forceinline__ static long long cell(long long sn) {
-    return (sn >> 5) * BYTES + (sn & 31) * (long long)sizeof(S);
+  __device__ __forceinline__ static long long cell(unsigned long long sn) {
+    return (long long)((sn / kTile) * BYTES + (sn % kTile) * sizeof(S));
   }
   template <class O>
   __device__ __forceinline__ static O scell(O c) {
     if (kSameElem) return c;
-    return c + ((c / O(sizeof(S))) & O(31)) * O(sizeof(SC) - sizeof(S));
+    return c + ((c / O(sizeof(S))) % O(kTile)) * O(sizeof(SC) - sizeof(S));
   }
   __device__ __forceinline__ static S* f(const Args& a, long long c, int s, int i) {
     return reinterpret_cast<S*>(a.pop + LBM_CHK(a.err, c + frow(s, i), a.pop_bytes));
@@ -2067,7 +2073,10 @@ __global__ void __launch_bounds__(1024) k_list_write(const Args a, uint32_t* lis
     if (n >= 0) {
       const unsigned int sl = f ? pos : a.fluid_count[0] + (vpos - pos);
       a.slot_new[n] = sl;
-      if (a.off_ok) a.off[n] = (sl >> 5) * rec + (sl & 31u) * elem + uint32_t(kOffBias * 32) * elem;
+      if (a.off_ok) {
+        const uint32_t tile = (uint32_t)tile_slots((int)elem);
+        a.off[n] = (sl / tile) * rec + (sl % tile + kOffBias * tile) * elem;
+      }
     }
   }
   if (f) {

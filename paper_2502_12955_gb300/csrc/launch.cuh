@@ -30,7 +30,7 @@ struct KernelSet {
   void (*coefs)(const Args* a, int n, void* out);
   cudaError_t (*step_tiles)(const Args* d_args, const void* d_coefs, const Tile* d_tiles, unsigned int ntiles,
                             int n_comp, int n_scal, int coll, int parity, int bnd, int threads, cudaStream_t);
-  long long (*rec_bytes)(const Args&);   // bytes per tile of 32 slots of all populations
+  long long (*rec_bytes)(const Args&);   // bytes per tile of kTile slots of all populations
   int psi_bytes;   // bytes per psi element (compute type)
   int coef_bytes;
 };
@@ -202,7 +202,7 @@ struct Launchers {
     return e;
   }
 
-  // bytes per tile of 32 slots (before the context's buffers exist, from the lattice counts alone)
+  // bytes per tile of kTile slots (before the context's buffers exist, from the lattice counts alone)
   static long long rec_bytes(const Args& a) {
     long long r = 0;
     by_nc_ns(a, [&](auto nc, auto ns) { r = Rec<L, S, decltype(nc)::value, decltype(ns)::value>::BYTES; });
@@ -412,11 +412,12 @@ const KernelSet& kernels_d3_bf16s32();
 cudaError_t launch_reduce(const double* partials, long long nblocks, int K, double* out, int* err,
                           int nonfin_slot, cudaStream_t st);
 cudaError_t launch_detect(const Args& a, cudaStream_t st);
-// Placement of one lattice's rows (elem bytes per element) in a population buffer: tiles of 32 slots
+// Placement of one lattice's rows (elem bytes per element) in a population buffer: tiles of slots
 // (tile bytes apart, row bytes first within one) or planes (tile = 0: row r at first + r * pitch).
 struct Place {
   unsigned char* p;
   long long tile, first, pitch;
+  int slots;             // slots per tile
   const uint32_t* map;   // slot of each node; NULL: node order
 };
 cudaError_t launch_permute(const Place& src, const Place& dst, int elem, int rows, const uint8_t* flags, long long N,

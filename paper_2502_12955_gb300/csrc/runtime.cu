@@ -44,7 +44,7 @@ struct lbm_ctx {
   std::vector<void*> allocs;
   double* mon_host = nullptr;      // pinned [NMON + 12]: monitors, then the 11 flip monitors
   unsigned char* pop_alt = nullptr;   // second population buffer: target of re-slotting, staging of checkpoints
-  long long rec = 0;               // bytes of one tile of 32 slots
+  long long rec = 0;               // bytes of one tile of kTile slots
   int nlat = 0;                    // scalar lattices: the given scalars, then the product if any
   // CUDA graphs of one even + odd step pair, keyed by which of the two steps end with a
   // geometry update; rebuilt whenever the kernel arguments change (re-slotting)
@@ -299,8 +299,9 @@ Place lattice_place(const lbm_ctx* c, int s, unsigned char* p, bool tiled, const
   *elem = (int)(flow ? c->elem : c->elem_h);
   *rows = flow ? c->Qf : c->Qc;
   const long long before = (long long)std::min(s, nc) * c->Qf * c->elem + (long long)std::max(0, s - nc) * c->Qc * c->elem_h;
-  if (tiled) return Place{p, c->rec, before * 32, 32ll * *elem, map};
-  return Place{p, 0, before * c->pitch, c->pitch * *elem, map};
+  const int tile = tile_slots((int)c->elem);
+  if (tiled) return Place{p, c->rec, before * tile, (long long)tile * *elem, tile, map};
+  return Place{p, 0, before * c->pitch, c->pitch * *elem, tile, map};
 }
 
 // Copies the populations of every fluid node between two population buffers (see lattice_place).
@@ -449,7 +450,7 @@ __global__ void __launch_bounds__(256) k_permute(const Place src, const Place ds
   if (n >= N || flags[n] != FL_FLUID) return;
   const auto cell = [&](const Place& p) {
     const long long s = p.map ? (long long)p.map[n] : n;
-    return p.p + p.first + (p.tile ? (s >> 5) * p.tile + (s & 31) * (long long)sizeof(E) : s * (long long)sizeof(E));
+    return p.p + p.first + (p.tile ? (s / p.slots) * p.tile + (s % p.slots) * (long long)sizeof(E) : s * (long long)sizeof(E));
   };
   const unsigned char* from = cell(src);
   unsigned char* to = cell(dst);
@@ -566,8 +567,9 @@ lbm_status lbm_create(lbm_lattice lattice, int32_t nx, int32_t ny, int32_t nz, c
     ptr = reinterpret_cast<decltype(ptr)>(v);               \
   } while (0)
   c->rec = c->ks->rec_bytes(a);
-  a.pop_bytes = P / 32 * c->rec;
-  a.off_ok = a.pop_bytes + 64 * kOffBias * (long long)c->elem < (1ll << 32) ? 1 : 0;
+  const int tile = tile_slots((int)c->elem);
+  a.pop_bytes = (N + tile - 1) / tile * c->rec;
+  a.off_ok = a.pop_bytes + tile * kOffBias * (long long)c->elem < (1ll << 32) ? 1 : 0;
   DA(a.pop, a.pop_bytes);
   DA(c->pop_alt, a.pop_bytes);
   DA(a.slot, N * 4);
@@ -1044,6 +1046,10 @@ struct StateHeader {
   int32_t version, lattice, precision, n_comp, n_scal, nx, ny, nz;
   int64_t step;
 };
+// bytes of the populations in a checkpoint: planes of pitch slots
+size_t plane_bytes(const lbm_ctx* c) {
+  return (size_t)(c->p.n_comp * c->Qf * c->elem + c->nlat * c->Qc * c->elem_h) * (size_t)c->pitch;
+}
 // bytes of the solid thermal lattice's state (conduction in the solid): both node-indexed copies,
 // the exchange's rate constants, the two heat banks and the removed-solid monitor
 size_t solid_state_bytes(const lbm_ctx* c) {
@@ -1053,7 +1059,7 @@ size_t solid_state_bytes(const lbm_ctx* c) {
 }
 size_t state_bytes(const lbm_ctx* c) {
   const size_t N = (size_t)c->N, rows = (size_t)c->ny * c->nz;
-  return sizeof(StateHeader) + (size_t)c->a.pop_bytes +
+  return sizeof(StateHeader) + plane_bytes(c) +
          (N + 3) / 4 * 4 + N * 8 + 3 * WALLX_SLOTS * 8 + 6 * rows * 8 + 10 * 8 + solid_state_bytes(c);
 }
 }  // namespace
@@ -1079,8 +1085,8 @@ lbm_status lbm_get_state(lbm_ctx* c, void* host, size_t* nbytes) {
   CK(cudaMemsetAsync(c->pop_alt, 0, c->a.pop_bytes, c->stream));
   lbm_status st = move_pops(c, c->a.pop, true, c->a.slot, c->pop_alt, false, nullptr);
   if (st != LBM_OK) return st;
-  CK(cudaMemcpyAsync(o, c->pop_alt, c->a.pop_bytes, cudaMemcpyDeviceToHost, c->stream));
-  o += c->a.pop_bytes;
+  CK(cudaMemcpyAsync(o, c->pop_alt, plane_bytes(c), cudaMemcpyDeviceToHost, c->stream));
+  o += plane_bytes(c);
   CK(cudaMemcpyAsync(o, c->a.flags, (N + 3) / 4 * 4, cudaMemcpyDeviceToHost, c->stream)); o += (N + 3) / 4 * 4;
   CK(cudaMemcpyAsync(o, c->a.acc, N * 8, cudaMemcpyDeviceToHost, c->stream)); o += N * 8;
   CK(cudaMemcpyAsync(o, c->a.wallx_slot, 3 * WALLX_SLOTS * 8, cudaMemcpyDeviceToHost, c->stream)); o += 3 * WALLX_SLOTS * 8;
@@ -1116,8 +1122,8 @@ lbm_status lbm_set_state(lbm_ctx* c, const void* host, size_t nbytes) {
   const size_t N = (size_t)c->N, rows = (size_t)c->ny * c->nz;
   // node-order populations go to the second buffer; they move to their slots once the slot
   // map of the restored geometry exists
-  CK(cudaMemcpyAsync(c->pop_alt, o, c->a.pop_bytes, cudaMemcpyHostToDevice, c->stream));
-  o += c->a.pop_bytes;
+  CK(cudaMemcpyAsync(c->pop_alt, o, plane_bytes(c), cudaMemcpyHostToDevice, c->stream));
+  o += plane_bytes(c);
   CK(cudaMemcpyAsync(c->a.flags, o, (N + 3) / 4 * 4, cudaMemcpyHostToDevice, c->stream)); o += (N + 3) / 4 * 4;
   CK(cudaMemcpyAsync(c->a.acc, o, N * 8, cudaMemcpyHostToDevice, c->stream)); o += N * 8;
   CK(cudaMemcpyAsync(c->a.wallx_slot, o, 3 * WALLX_SLOTS * 8, cudaMemcpyHostToDevice, c->stream)); o += 3 * WALLX_SLOTS * 8;
