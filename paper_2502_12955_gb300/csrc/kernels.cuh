@@ -595,6 +595,14 @@ __device__ __forceinline__ double widen(float v) {
                                           ((unsigned long long)(b & 0x7fffffu) << 29)));
 }
 
+// Programmatic dependent launch: the kernels of a time step are launched so that each may start while its
+// predecessor still runs.  A kernel lets its successor start at once, reads what no step changes (without
+// geometry updates: lists, masks, maps), and waits for the completion of its predecessor before it touches
+// anything else.  Every thread waits, so completion still runs in launch order.  On a small domain this hides the launch
+// and the first dependent loads, which are most of a 4 us kernel.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 template <class T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
@@ -1217,6 +1225,8 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   using R = Rec<L, S, NC, NS>;
   using O = OddCells<L, S, NC, NS, LBM_STEP_CACHE_STRIDE, BND>;
   T wallx = T(0), heatx = T(0), prodx = T(0);
+  pdl_trigger();
+  if (a.geo_mode != GEO_NONE) pdl_wait();
   const unsigned int count = a.fluid_count[0];
   const unsigned int base = a.fluid_count[1];   // entries below it have slot == entry
   const unsigned int stride = gridDim.x * blockDim.x;
@@ -1235,6 +1245,7 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
     const uint32_t* map = BND ? a.slot : a.off;
     if (e < count) prefetch_nbrs<L, LBM_STEP_CACHE_STRIDE>(a, map, w_cur, cb);
     cp_async_commit();
+    if (a.geo_mode == GEO_NONE) pdl_wait();
     for (; e < count; e += stride) {
       const uint32_t w = w_cur, m = m_cur;
       if (e + stride < count) {
@@ -1262,6 +1273,7 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
     }
     cp_async_wait<0>();
   } else {
+    if (a.geo_mode == GEO_NONE) pdl_wait();
     for (; e < count; e += stride) {
       const uint32_t w = w_cur, m = m_cur;
       w_cur = w_nx;
@@ -1326,7 +1338,7 @@ struct Tile {
 template <class L, class S, int NC, int NS, int COLL, int parity, bool BND>
 __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) == 4 ? (parity ? LBM_TILES_MIN_BLOCKS_ODD : LBM_STEP_MIN_BLOCKS) : 2)) k_step_tiles(
     const Args* __restrict__ args, const Coef<typename Store<S>::T>* __restrict__ coefs,
-    const Tile* __restrict__ tiles, unsigned int ntiles) {
+    const Tile* __restrict__ tiles, unsigned int ntiles, unsigned int chunk) {
   using T = typename Store<S>::T;
   constexpr int Q = L::Q, QC = L::QC, NSD = NS > 0 ? NS : 1;
   static_assert(sizeof(Args) % 4 == 0 && sizeof(Coef<T>) % 4 == 0, "word copies");
@@ -1336,21 +1348,22 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   using O = OddCells<L, S, NC, NS, 1, BND>;
   extern __shared__ uint32_t slot_smem[];   // 2 * blockDim.x * Q words at odd parity (launcher)
   uint32_t* cache = slot_smem + threadIdx.x * L::Q;
-  // blocks take chunks of LBM_TILE_CHUNK consecutive tiles in turn: the work list holds each
-  // member's tiles together, so a chunk mostly stays within one member and its arguments are
-  // staged again only when the chunk crosses into another; taking chunks in turn keeps a mix of
-  // 2D and 3D members on every block
+  // blocks take chunks of consecutive tiles in turn (at most LBM_TILE_CHUNK, fewer where that would leave
+  // blocks idle): the work list holds each member's tiles together, so a chunk mostly stays within
+  // one member and its arguments are staged again only when the chunk crosses into another; taking
+  // chunks in turn keeps a mix of uneven members on every block
   auto next_tile = [&](unsigned int t) {
-    return t + ((t % LBM_TILE_CHUNK == LBM_TILE_CHUNK - 1) ? (gridDim.x - 1) * LBM_TILE_CHUNK + 1 : 1);
+    return t + ((t % chunk == chunk - 1) ? (gridDim.x - 1) * chunk + 1 : 1);
   };
   // odd parity: two neighbour buffers, the next tile's are copied in (cp.async)
   // while this tile computes, as in k_step; the next tile's list entry and link mask are loaded
   // one tile ahead at both parities whenever it belongs to the member already staged
   uint32_t* cn = slot_smem + (blockDim.x + threadIdx.x) * L::Q;
-  bool have_next = false;
+  bool have_next = false, waited = false;
   uint32_t w_pf = 0u, m_pf = 0u;
   unsigned int staged = 0xffffffffu;
-  for (unsigned int t = blockIdx.x * LBM_TILE_CHUNK; t < ntiles; t = next_tile(t)) {
+  pdl_trigger();
+  for (unsigned int t = blockIdx.x * chunk; t < ntiles; t = next_tile(t)) {
     const Tile tile = tiles[t];
     if (tile.member != staged) {   // block-uniform
       __syncthreads();   // the previous member's tiles are done with sa / sk
@@ -1400,6 +1413,8 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
       cp_async_commit();
       cp_async_wait<1>();   // this tile's neighbours have arrived
     }
+    if (!waited) pdl_wait();   // ensembles keep their geometry: everything read so far is static
+    waited = true;
     if (e < count && (m & 1u)) {
       const unsigned int base = a.fluid_count[1];
       T f[NC][Q], h[NSD][QC];
@@ -1448,6 +1463,7 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
     }
   }
   if (parity) cp_async_wait<0>();
+  if (!waited) pdl_wait();
 }
 
 // ================================================================ psi
@@ -1460,22 +1476,33 @@ __global__ void __launch_bounds__(256) k_psi(const Args a, const Coef<typename S
   // rho_ref, the order the gather of the step uses.
   using T = typename Store<S>::T;
   using R = Rec<L, S, NC, NS>;
+  pdl_trigger();
+  if (a.geo_mode != GEO_NONE) pdl_wait();
   const unsigned int count = a.fluid_count[0];
   const unsigned int base = a.fluid_count[1];   // entries below it have slot == entry
   const unsigned int stride = gridDim.x * blockDim.x;
-  for (unsigned int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += stride) {
-    const uint32_t w = a.fluid_list[e];
+  unsigned int e = blockIdx.x * blockDim.x + threadIdx.x;
+  uint32_t w = e < count ? a.fluid_list[e] : 0u;
+  uint32_t m = e < count ? a.mask[list_node(a, w)] : 0u;
+  bool waited = a.geo_mode != GEO_NONE;
+  for (; e < count; e += stride) {
     const int n = list_node(a, w);
-    const uint32_t m = a.mask[n];
-    if (!(m & 1u)) continue;   // a node removed by deposition since the last list rebuild
     const long long c = R::cell(e < base ? (long long)e : (long long)__ldg(a.slot + n));
     long long cell[L::Q];   // offset of the row holding population i of component 0
     const Nbr nb = parity ? nbr_entry(a, n, w) : Nbr{};
+    const uint32_t mn = m;
 #pragma unroll
     for (int i = 0; i < L::Q; ++i)
-      cell[i] = (parity == 0 || i == 0 || flow_wall<L>(m, L::opp(i)))
+      cell[i] = (parity == 0 || i == 0 || flow_wall<L>(mn, L::opp(i)))
                     ? c + R::frow(0, i)
                     : cell_of<R>(a, nb.at(-L::cx(i), -L::cy(i), -L::cz(i))) + R::frow(0, L::opp(i));
+    if (e + stride < count) {   // the next entry and its mask, one iteration ahead
+      w = a.fluid_list[e + stride];
+      m = a.mask[list_node(a, w)];
+    }
+    if (!waited) pdl_wait();
+    waited = true;
+    if (!(mn & 1u)) continue;   // a node removed by deposition since the last list rebuild
 #pragma unroll
     for (int s = 0; s < NC; ++s) {
       T r = k.rref[s];
@@ -1488,6 +1515,7 @@ __global__ void __launch_bounds__(256) k_psi(const Args a, const Coef<typename S
       reinterpret_cast<T*>(a.psi[s])[n] = p;
     }
   }
+  if (!waited) pdl_wait();
 }
 
 // ================================================================ monitors
@@ -2158,6 +2186,8 @@ __global__ void __cluster_dims__(kFlipBlocks, 1, 1) __launch_bounds__(kFlipThrea
   using R = Rec<L, S, NC, NS>;
   using SC = typename R::SC;   // scalar lattices' storage
   constexpr int Q = L::Q, QC = L::QC;
+  pdl_trigger();
+  pdl_wait();
   const unsigned int cnt_raw = *a.flip_count;
   const unsigned int cnt = cnt_raw < a.flip_cap ? cnt_raw : a.flip_cap;
   if (cnt == 0) return;   // the same in every block: nothing writes the count before the last barrier
@@ -2414,6 +2444,8 @@ __global__ void __launch_bounds__(256) k_solid(const Args a, const Coef<typename
                                                const int parity) {
   using T = typename Store<S>::T;
   constexpr int QC = L::QC;
+  pdl_trigger();
+  pdl_wait();
   const T* gin = reinterpret_cast<const T*>(a.gs[parity]);
   T* gout = reinterpret_cast<T*>(a.gs[parity ^ 1]);
   const int perc[3] = {a.open_x ? 0 : a.per[0], a.per[1], a.per[2]};
@@ -2464,6 +2496,8 @@ __global__ void __launch_bounds__(256) k_exchange(const Args a, const Coef<typen
   using R = Rec<L, S, NC, NS>;
   using SC = typename R::SC;
   constexpr int QC = L::QC;
+  pdl_trigger();
+  pdl_wait();
   T* g = reinterpret_cast<T*>(a.gs[parity_next]);
   T* kb = reinterpret_cast<T*>(a.kb);
   const int perc[3] = {a.open_x ? 0 : a.per[0], a.per[1], a.per[2]};

@@ -35,6 +35,25 @@ struct KernelSet {
   int coef_bytes;
 };
 
+// Launch of a kernel that may start before its predecessor in the stream has finished (see pdl_wait).  FP64 kernels
+// are launched in full order: they are bound by the FP64 units, and blocks placed while the predecessor still holds
+// some SMs share them unevenly (128 x 64 channel: 9.8 us per step in order, 12.3 us with early starts; FP32 200 x 80
+// droplet: 7.2 us in order, 6.6 us with).
+template <class... P, class... A>
+cudaError_t launch_pdl(bool early, void (*kernel)(P...), unsigned int grid, unsigned int block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 inline dim3 node_grid(const Args& a, dim3 blk) {
   return dim3((a.nx + blk.x - 1) / blk.x, (a.ny + blk.y - 1) / blk.y, a.nz);
 }
@@ -117,6 +136,7 @@ template <class L, class S>
 struct Launchers {
   using T = typename Store<S>::T;
   static constexpr bool kShifted = !std::is_same<S, double>::value;
+  static constexpr bool kEarly = sizeof(T) == 4;
   static Coef<T> coef(const Args& a) { return make_coef<L, T>(a, kShifted); }
 
   // one resident wave of blocks; the kernel walks the fluid list with a grid-stride loop
@@ -141,8 +161,7 @@ struct Launchers {
     }
     long long need = (a.N + threads - 1) / threads;
     const unsigned int blocks = (unsigned int)(need < cached_blocks ? need : cached_blocks);
-    k_step<L, S, NC, NS, COLL, PAR, BND><<<blocks > 0 ? blocks : 1, threads, 0, st>>>(a, coef(a));
-    return cudaGetLastError();
+    return launch_pdl(kEarly, k_step<L, S, NC, NS, COLL, PAR, BND>, blocks > 0 ? blocks : 1, threads, 0, st, a, coef(a));
   }
   // BND: a moving plate, a velocity inlet or the temperature-dependent reaction needs the full
   // variant of the step kernel, and so does a domain too large for the plain variant's 32-bit
@@ -177,21 +196,22 @@ struct Launchers {
     return a.n_comp == 1 ? step_s<1>(a, parity, coll, st) : step_s<2>(a, parity, coll, st);
   }
 
-  // psi pass: resident waves of 256-thread blocks over the fluid list (grid-stride)
+  // psi pass: resident waves of the step kernel's blocks over the fluid list (grid-stride)
   template <int NC, int NS, int PAR>
   static cudaError_t psi_p(const Args& a, cudaStream_t st) {
-    static int cached_blocks = 0;
-    if (!cached_blocks) {
+    const int threads = a.bx;
+    static int cached_threads = -1, cached_blocks = 0;
+    if (cached_threads != threads) {
       int dev = 0, sms = 0, occ = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_psi<L, S, NC, NS, PAR>, 256, 0);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_psi<L, S, NC, NS, PAR>, threads, 0);
       cached_blocks = (occ > 0 ? occ : 1) * (sms > 0 ? sms : 1);
+      cached_threads = threads;
     }
-    const long long need = (a.N + 255) / 256;
+    const long long need = (a.N + threads - 1) / threads;
     const unsigned int blocks = (unsigned int)(need < cached_blocks ? need : cached_blocks);
-    k_psi<L, S, NC, NS, PAR><<<blocks > 0 ? blocks : 1, 256, 0, st>>>(a, coef(a));
-    return cudaGetLastError();
+    return launch_pdl(kEarly, k_psi<L, S, NC, NS, PAR>, blocks > 0 ? blocks : 1, threads, 0, st, a, coef(a));
   }
   static cudaError_t psi(const Args& a, int parity, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
@@ -268,29 +288,31 @@ struct Launchers {
   }
 
   static cudaError_t flip(const Args& a, int parity_next, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
     by_nc_ns(a, [&](auto nc, auto ns) {
-      k_flip<L, S, decltype(nc)::value, decltype(ns)::value><<<kFlipBlocks, kFlipThreads, 0, st>>>(a, coef(a), parity_next);
+      e = launch_pdl(kEarly, k_flip<L, S, decltype(nc)::value, decltype(ns)::value>, kFlipBlocks, kFlipThreads, 0, st, a, coef(a), parity_next);
     });
-    return cudaGetLastError();
+    return e;
   }
 
   // grid-stride kernels over the box (k_solid) and the fluid list (k_exchange): two waves of
   // blocks, fewer on a small domain
   static unsigned int box_blocks(const Args& a) {
-    const long long need = (a.N + 255) / 256, cap = 2ll * wave_blocks();
+    const long long need = (a.N + a.bx - 1) / a.bx, cap = 2ll * wave_blocks() * 256 / a.bx;
     return (unsigned int)(need < cap ? (need > 0 ? need : 1) : cap);
   }
   static cudaError_t solid(const Args& a, int parity, cudaStream_t st) {
-    k_solid<L, S><<<box_blocks(a), 256, 0, st>>>(a, coef(a), parity);
-    return cudaGetLastError();
+    return launch_pdl(kEarly, k_solid<L, S>, box_blocks(a), a.bx, 0, st, a, coef(a), parity);
   }
   static cudaError_t exchange(const Args& a, int parity_next, cudaStream_t st) {
     // conduction in the solid needs the species and the temperature: two or three scalar lattices
+    cudaError_t e = cudaErrorInvalidValue;
     by_nc_ns(a, [&](auto nc, auto ns) {
       if constexpr (decltype(ns)::value >= 2)
-        k_exchange<L, S, decltype(nc)::value, decltype(ns)::value><<<box_blocks(a), 256, 0, st>>>(a, coef(a), parity_next);
+        e = launch_pdl(kEarly, k_exchange<L, S, decltype(nc)::value, decltype(ns)::value>, box_blocks(a), a.bx, 0, st, a, coef(a),
+                       parity_next);
     });
-    return cudaGetLastError();
+    return e;
   }
   static cudaError_t solid_init(const Args& a, cudaStream_t st) {
     const unsigned int nb = (unsigned int)((a.N + 255) / 256);
@@ -336,9 +358,11 @@ struct Launchers {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step_tiles<L, S, NC, NS, COLL, PAR, BND>, threads, smem);
     const unsigned int wave = (unsigned int)((occ > 0 ? occ : 1) * (sms > 0 ? sms : 1));
     const unsigned int blocks = ntiles < wave ? (ntiles > 0 ? ntiles : 1) : wave;
-    k_step_tiles<L, S, NC, NS, COLL, PAR, BND><<<blocks, threads, smem, st>>>(
-        d_args, static_cast<const Coef<T>*>(d_coefs), d_tiles, ntiles);
-    return cudaGetLastError();
+    // consecutive tiles per turn: whole chunks for every block first, LBM_TILE_CHUNK at most
+    unsigned int chunk = ntiles / blocks;
+    chunk = chunk < 1 ? 1 : (chunk > LBM_TILE_CHUNK ? LBM_TILE_CHUNK : chunk);
+    return launch_pdl(kEarly, k_step_tiles<L, S, NC, NS, COLL, PAR, BND>, blocks, threads, smem, st, d_args,
+                      static_cast<const Coef<T>*>(d_coefs), d_tiles, ntiles, chunk);
   }
   template <int NC, int NS, int COLL>
   static cudaError_t step_tiles_b(const Args* d, const void* k, const Tile* t, unsigned int nt, int parity, int bnd,
@@ -411,7 +435,7 @@ const KernelSet& kernels_d3_bf16s32();
 // Storage-independent kernels (runtime.cu)
 cudaError_t launch_reduce(const double* partials, long long nblocks, int K, double* out, int* err,
                           int nonfin_slot, cudaStream_t st);
-cudaError_t launch_detect(const Args& a, cudaStream_t st);
+cudaError_t launch_detect(const Args& a, bool early, cudaStream_t st);
 // Placement of one lattice's rows (elem bytes per element) in a population buffer: tiles of slots
 // (tile bytes apart, row bytes first within one) or planes (tile = 0: row r at first + r * pitch).
 struct Place {

@@ -47,11 +47,12 @@ struct lbm_ctx {
   long long rec = 0;               // bytes of one tile of kTile slots
   int nlat = 0;                    // scalar lattices: the given scalars, then the product if any
   // CUDA graphs of one even + odd step pair, keyed by which of the two steps end with a
-  // geometry update; rebuilt whenever the kernel arguments change (re-slotting)
+  // geometry update, and of kChain steps of one kind ([4]: none does, [5]: every one does); rebuilt
+  // whenever the kernel arguments change (re-slotting)
   cudaStream_t cap_stream = nullptr;
   long long gen = 0;               // bumped whenever the arguments or the fluid list change
-  cudaGraphExec_t pair_exec[4] = {nullptr, nullptr, nullptr, nullptr};
-  long long pair_launches[4] = {0, 0, 0, 0};
+  cudaGraphExec_t pair_exec[6] = {};
+  long long pair_launches[6] = {};
   bool graphs_ok = true;
 };
 
@@ -265,7 +266,13 @@ void fill_args(lbm_ctx* c) {
   a.deposit_conservative = p.deposit_conservative ? 1 : 0;
   a.V_m = p.V_m; a.m_s0 = p.m_s0; a.DP = p.DP;
   int bx = p.block_x;
-  if (bx == 0) bx = 256;   // the step kernel walks the fluid list: the block shape is not tied to nx
+  if (bx == 0) {
+    // the step kernel walks the fluid list: the block shape is not tied to nx.  256 threads, fewer on a domain
+    // whose blocks of that size would not reach every SM (152 on this GPU): 128 x 64 nodes in FP64 take
+    // 15.1 us per step as 32 blocks of 256 and 9.8 us as 128 blocks of 64 (16.0 us as 256 blocks of 32)
+    bx = 256;
+    while (bx > 64 && (c->N + bx - 1) / bx < 152) bx /= 2;
+  }
   a.bx = bx;
   a.by = 1;
   a.div_x = make_fast_div(c->nx);
@@ -434,6 +441,8 @@ cudaError_t launch_reduce(const double* partials, long long nblocks, int K, doub
 
 // Dissolution test (V_m acc >= m_s0) over the interface list.
 __global__ void __launch_bounds__(256) k_detect(const Args a) {
+  pdl_trigger();
+  pdl_wait();
   const unsigned int cnt = *a.iface_count;
   for (unsigned int e = blockIdx.x * blockDim.x + threadIdx.x; e < cnt; e += gridDim.x * blockDim.x) {
     const long long n = a.iface_list[e];
@@ -479,12 +488,11 @@ cudaError_t launch_iota(uint32_t* v, long long N, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_detect(const Args& a, cudaStream_t st) {
+cudaError_t launch_detect(const Args& a, bool early, cudaStream_t st) {
   long long nb = (a.N / 8 + 255) / 256;
   if (nb < 1) nb = 1;
   if (nb > 152 * 16) nb = 152 * 16;
-  k_detect<<<(unsigned int)nb, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(early, k_detect, (unsigned int)nb, 256, 0, st, a);
 }
 
 }  // namespace lbm
@@ -618,7 +626,7 @@ lbm_status lbm_create(lbm_lattice lattice, int32_t nx, int32_t ny, int32_t nz, c
   DA(a.d_C, std::max<long long>(1, c->nlat) * N * 8);
   DA(a.snap, 4 * P * c->ks->psi_bytes);
 #undef DA
-  e = cudaMallocHost(reinterpret_cast<void**>(&c->mon_host), (NMON + 12) * sizeof(double));
+  e = cudaMallocHost(reinterpret_cast<void**>(&c->mon_host), (NMON + 16) * sizeof(double));
   if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMallocHost"));
   // zero everything the kernels accumulate into
   e = cudaMemsetAsync(a.flags, 0, (N + 3) / 4 * 4, c->stream);
@@ -736,30 +744,34 @@ lbm_status enqueue_step(lbm_ctx* c, long long step, cudaStream_t st, bool timed)
     c->ev_used.push_back({e0, e1});
   }
   if (geo_after(c, step + 1)) {
-    if (c->p.geo_mode == LBM_GEO_DISSOLVE) LAUNCH(launch_detect(c->a, st));
+    if (c->p.geo_mode == LBM_GEO_DISSOLVE) LAUNCH(launch_detect(c->a, c->ks->psi_bytes == 4, st));
     LAUNCH(c->ks->flip(c->a, parity_of(step + 1), st));
   }
   return LBM_OK;
 }
 
-// Steps step+1 and step+2 complete neither a list rebuild nor a monitor evaluation.
-bool plain_pair(const lbm_ctx* c, long long step) {
-  for (long long d = step + 1; d <= step + 2; ++d) {
+// Steps step+1 .. step+n complete neither a list rebuild nor a monitor evaluation.
+bool plain_run(const lbm_ctx* c, long long step, int n) {
+  for (long long d = step + 1; d <= step + n; ++d) {
     if (c->p.geo_mode != LBM_GEO_NONE && (d % kListRebuild) == 0) return false;
     if (c->p.N_mon > 0 && (d % c->p.N_mon) == 0) return false;
   }
   return true;
 }
 
-// Captures an even + odd step pair into a graph (once per geometry-update pattern).
-lbm_status pair_graph(lbm_ctx* c, long long step, cudaGraphExec_t* out, long long* launches) {
-  const int key = (geo_after(c, step + 1) ? 1 : 0) | (geo_after(c, step + 2) ? 2 : 0);
+// Steps of the longer graph.  Between two graphs the GPU idles for about as long as a small domain's kernel runs.
+constexpr int kChain = 8;
+
+// Captures n steps (2, or kChain of one kind) from an even one into a graph, once per geometry-update pattern.
+lbm_status step_graph(lbm_ctx* c, long long step, int n, cudaGraphExec_t* out, long long* launches) {
+  const int key = n == kChain ? (geo_after(c, step + 1) ? 5 : 4)
+                              : (geo_after(c, step + 1) ? 1 : 0) | (geo_after(c, step + 2) ? 2 : 0);
   if (!c->pair_exec[key]) {
     if (!c->cap_stream) CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
     const long long l0 = c->launches;
     CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-    lbm_status st = enqueue_step(c, step, c->cap_stream, false);
-    if (st == LBM_OK) st = enqueue_step(c, step + 1, c->cap_stream, false);
+    lbm_status st = LBM_OK;
+    for (int k = 0; k < n && st == LBM_OK; ++k) st = enqueue_step(c, step + k, c->cap_stream, false);
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
     if (st != LBM_OK) {
@@ -789,16 +801,18 @@ lbm_status lbm_step(lbm_ctx* c, int64_t nsteps) {
   if (!c || nsteps < 0) return LBM_ERR_INVALID_ARG;
   if (!c->fields_set) return fail(c, LBM_ERR_STATE, "lbm_set_fields must precede lbm_step");
   for (int64_t k = 0; k < nsteps;) {
-    // two plain steps from an even step: one graph launch
+    // plain steps from an even step: one graph launch for kChain or for two of them
     if (LBM_STEP_GRAPHS && c->graphs_ok && !c->profile && (c->step & 1) == 0 && nsteps - k >= 2 &&
-        plain_pair(c, c->step)) {
+        plain_run(c, c->step, 2)) {
+      const bool one_kind = c->p.geo_mode == LBM_GEO_NONE || c->p.N_geo == 1;
+      const int n = one_kind && nsteps - k >= kChain && plain_run(c, c->step, kChain) ? kChain : 2;
       cudaGraphExec_t g = nullptr;
       long long nl = 0;
-      if (pair_graph(c, c->step, &g, &nl) == LBM_OK) {
+      if (step_graph(c, c->step, n, &g, &nl) == LBM_OK) {
         CK(cudaGraphLaunch(g, c->stream));
         c->launches += nl;
-        c->step += 2;
-        k += 2;
+        c->step += n;
+        k += n;
         continue;
       }
       c->graphs_ok = false;   // capture unavailable: launch the kernels one by one from now on
@@ -1403,7 +1417,7 @@ lbm_status lbm_ensemble_create(lbm_lattice lattice, int32_t n, const int32_t* di
   e->active.assign(n, 1);
   e->built_gen.assign(n, -1);
   e->ks = e->m[0]->ks;
-  e->threads = e->m[0]->a.bx;
+  e->threads = p0.block_x ? p0.block_x : 256;   // the work list spans all members
   *out = e;
   return LBM_OK;
 }
