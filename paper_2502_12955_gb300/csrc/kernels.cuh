@@ -1520,24 +1520,34 @@ __global__ void __launch_bounds__(256) k_psi(const Args a, const Coef<typename S
 
 // ================================================================ monitors
 
+// Sums of K values over a block of 256 threads into out[0 .. K), in a fixed order; only the values with their bit in
+// used (block-uniform) are added up, the others are 0 in every thread.  A warp takes every eighth value: 8 values per
+// lane from shared memory, then 5 shuffle stages, a third of the FP64 additions of reducing every value in every warp
+// (the FP64 unit is narrow: with 25 values per warp it was 56 % busy and most of the kernel's time).
 template <int K>
-__device__ __forceinline__ void block_reduce_store(double (&v)[K], double* out) {
-  __shared__ double sh[32][K];
-  const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  const int lane = tid & 31, wid = tid >> 5;
-  const int nw = (blockDim.x * blockDim.y + 31) >> 5;
+__device__ __forceinline__ void block_reduce_store(double (&v)[K], unsigned int used, double* out) {
+  constexpr int KB = K < 8 ? K : 8;   // values held at once
+  __shared__ double sh[KB][256];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 #pragma unroll
-  for (int q = 0; q < K; ++q) {
-    double s = warp_sum(v[q]);
-    if (lane == 0) sh[wid][q] = s;
-  }
-  __syncthreads();
-  if (wid == 0) {
+  for (int q0 = 0; q0 < K; q0 += KB) {
+    if ((used >> q0 & ((1u << KB) - 1u)) == 0u) {
+      if (tid < KB && q0 + tid < K) out[q0 + tid] = 0.0;
+      continue;
+    }
+    __syncthreads();
 #pragma unroll
-    for (int q = 0; q < K; ++q) {
-      double s = lane < nw ? sh[lane][q] : 0.0;
-      s = warp_sum(s);
-      if (lane == 0) out[q] = s;
+    for (int q = 0; q < KB; ++q)
+      if (q0 + q < K && (used >> (q0 + q) & 1u)) sh[q][tid] = v[q0 + q];
+    __syncthreads();
+    if (wid < KB && q0 + wid < K) {
+      double s = 0.0;
+      if (used >> (q0 + wid) & 1u) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s += sh[wid][lane + 32 * i];
+        s = warp_sum(s);
+      }
+      if (lane == 0) out[q0 + wid] = s;
     }
   }
 }
@@ -1605,11 +1615,12 @@ __global__ void __launch_bounds__(256) k_monitor(const Args a, const Coef<typena
   v[M_NONFIN] = double(nonfin);
   // bookkeeping over every node
   const bool dep = a.geo_mode == GEO_DEPOSIT;
-  double react = 0.0, depo = 0.0, nsolid = 0.0, tsolid = 0.0;
+  double react = 0.0, depo = 0.0, tsolid = 0.0;
+  unsigned int nsolid = 0;
   const T* gcur = a.conjugate ? reinterpret_cast<const T*>(a.gs[parity]) : nullptr;
   for (long long n = tid; n < a.N; n += nthr) {
     const uint8_t fl = a.flags[n];
-    nsolid += fl != FL_FLUID ? 1.0 : 0.0;
+    nsolid += fl != FL_FLUID ? 1u : 0u;
     const double acc = a.acc[n];
     if (acc != 0.0) {
       if (dep && fl != FL_REACTIVE) depo += acc; else react += acc;
@@ -1623,7 +1634,7 @@ __global__ void __launch_bounds__(256) k_monitor(const Args a, const Coef<typena
   }
   v[M_REACT] = react;
   v[M_DEPO] = depo;
-  v[M_NSOLID] = nsolid;
+  v[M_NSOLID] = double(nsolid);
   v[M_TSOLID] = tsolid;
   const int rows = a.ny * a.nz;
   for (int r = tid; r < rows; r += nthr)
@@ -1638,7 +1649,16 @@ __global__ void __launch_bounds__(256) k_monitor(const Args a, const Coef<typena
     v[M_HEAT_S] += a.wallx_slot[BANK_HEAT_S * WALLX_SLOTS + q];
     v[M_HEAT_SRC] += a.wallx_slot[BANK_HEAT_SRC * WALLX_SLOTS + q];
   }
-  block_reduce_store<NMON>(v, a.partials + (long long)blockIdx.x * NMON);
+  // what this kind of context can have in its sums
+  unsigned int used = 1u << M_MASS | (NC > 1 ? 1u << (M_MASS + 1) : 0u) | 7u << M_MOM | 1u << M_NFLUID | 1u << M_NSOLID | 1u << M_NONFIN;
+  if (NS > 0) used |= 1u << M_REACT | 1u << M_DEPO | 1u << M_WALLX;
+  for (int s = 0; s < NS; ++s) {
+    used |= 1u << mon_spec(s);
+    if (a.open_x) used |= 1u << mon_in(s) | 1u << mon_out(s);
+  }
+  if (NS > 1) used |= 1u << M_HEAT | 1u << M_PROD;
+  if (a.conjugate) used |= 1u << M_TSOLID | 1u << M_HEAT_S | 1u << M_HEAT_SRC;
+  block_reduce_store<NMON>(v, used, a.partials + (long long)blockIdx.x * NMON);
 }
 
 // ================================================================ node macroscopics
@@ -1798,7 +1818,7 @@ __global__ void __launch_bounds__(256) k_resid(const Args a, const Coef<typename
     }
   }
   double v[4] = {double(du), double(uu), double(dc), double(cc)};
-  block_reduce_store<4>(v, a.partials + (long long)blockIdx.x * 4);
+  block_reduce_store<4>(v, 15u, a.partials + (long long)blockIdx.x * 4);
 }
 
 // ================================================================ init / pop I/O

@@ -42,7 +42,7 @@ struct lbm_ctx {
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_used;
   std::string err;
   std::vector<void*> allocs;
-  double* mon_host = nullptr;      // pinned [NMON + 12]: monitors, then the 11 flip monitors
+  double* mon_host = nullptr;      // pinned [NMON + 16]: monitors, the last residual's 4 sums, the 11 flip monitors
   unsigned char* pop_alt = nullptr;   // second population buffer: target of re-slotting, staging of checkpoints
   long long rec = 0;               // bytes of one tile of kTile slots
   int nlat = 0;                    // scalar lattices: the given scalars, then the product if any
@@ -400,42 +400,35 @@ lbm_status check_err(lbm_ctx* c) {
 
 namespace lbm {
 
-// Fixed-order sum of the per-block partials (deterministic): each thread adds a fixed set of
-// blocks for all K values at once (K <= 32), then warp shuffles and one pass over the warps.
-__global__ void __launch_bounds__(256) k_reduce_partials(const double* __restrict__ partials,
-                                                         long long nblocks, int K,
-                                                         double* __restrict__ out, int* err,
-                                                         int nonfin_slot) {
-  __shared__ double sh[8][32];
+// Fixed-order sum of the per-block partials (deterministic): a warp per row of K values (K <= 32), 32 rows at a time,
+// then one pass over the warps.
+__global__ void __launch_bounds__(1024) k_reduce_partials(const double* __restrict__ partials,
+                                                          long long nblocks, int K,
+                                                          double* __restrict__ out, int* err,
+                                                          int nonfin_slot) {
+  __shared__ double sh[32][33];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  double acc[32];
-#pragma unroll
-  for (int k = 0; k < 32; ++k) acc[k] = 0.0;
-  for (long long b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < 32; ++k)
-      if (k < K) acc[k] += partials[b * K + k];
-#pragma unroll
-  for (int k = 0; k < 32; ++k) {
-    if (k >= K) break;
-    double v = acc[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[wid][k] = v;
+  double acc = 0.0;
+  if (lane < K) {
+#pragma unroll 4
+    for (long long b = wid; b < nblocks; b += 32) acc += partials[b * K + lane];
   }
+  sh[wid][lane] = acc;
   __syncthreads();
-  if (wid == 0 && lane < K) {
-    double v = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += sh[w][lane];
-    out[lane] = v;
-    if (nonfin_slot == lane && v > 0.0) atomicOr(err, ERR_NONFINITE);
+  // warp k: value k of every warp
+  if (wid < K) {
+    const double v = warp_sum(sh[lane][wid]);
+    if (lane == 0) {
+      out[wid] = v;
+      if (nonfin_slot == wid && v > 0.0) atomicOr(err, ERR_NONFINITE);
+    }
   }
 }
 
 cudaError_t launch_reduce(const double* partials, long long nblocks, int K, double* out, int* err,
                           int nonfin_slot, cudaStream_t st) {
   if (K > 32) return cudaErrorInvalidValue;
-  k_reduce_partials<<<1, 256, 0, st>>>(partials, nblocks, K, out, err, nonfin_slot);
+  k_reduce_partials<<<1, 1024, 0, st>>>(partials, nblocks, K, out, err, nonfin_slot);
   return cudaGetLastError();
 }
 
@@ -976,9 +969,11 @@ lbm_status lbm_get_monitors(lbm_ctx* c, lbm_monitors* out) {
   lbm_status st = run_monitor(c);
   if (st != LBM_OK) return st;
   double* hm = c->mon_host;
-  CK(cudaMemcpyAsync(hm, c->a.mon_out, NMON * 8, cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaMemcpyAsync(hm + NMON, c->a.flip_mon, 11 * 8, cudaMemcpyDeviceToHost, c->stream));
+  const double* r4 = hm + NMON;
+  CK(cudaMemcpyAsync(hm, c->a.mon_out, (NMON + 4) * 8, cudaMemcpyDeviceToHost, c->stream));
+  CK(cudaMemcpyAsync(hm + NMON + 4, c->a.flip_mon, 11 * 8, cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
+  const double* fm = hm + NMON + 4;
   std::memset(out, 0, sizeof(*out));
   out->step = double(c->step);
   out->mass[0] = hm[M_MASS]; out->mass[1] = hm[M_MASS + 1];
@@ -992,12 +987,12 @@ lbm_status lbm_get_monitors(lbm_ctx* c, lbm_monitors* out) {
     sp[s] = hm[mon_spec(s)];
     in[s] = hm[mon_in(s)];
     outf[s] = hm[mon_out(s)];
-    inj[s] = hm[NMON + 2 + s];
-    rem[s] = hm[NMON + 7 + s];
+    inj[s] = fm[2 + s];
+    rem[s] = fm[7 + s];
   }
   for (int s = 0; s < 2; ++s) {
-    out->injected_mass[s] = hm[NMON + s];
-    out->removed_mass[s] = hm[NMON + 5 + s];
+    out->injected_mass[s] = fm[s];
+    out->removed_mass[s] = fm[5 + s];
   }
   const int ns = c->p.n_scal;
   for (int s = 0; s < 2; ++s) {
@@ -1022,19 +1017,14 @@ lbm_status lbm_get_monitors(lbm_ctx* c, lbm_monitors* out) {
     out->t_solid = hm[M_TSOLID];
     out->heat_solid = hm[M_HEAT_S];
     out->heat_source = hm[M_HEAT_SRC];
-    out->solid_removed = hm[NMON + 10];
+    out->solid_removed = fm[10];
   }
   out->n_solid = hm[M_NSOLID];
   out->n_fluid = hm[M_NFLUID];
   out->nonfinite = hm[M_NONFIN];
   // latest residual evaluation (automatic every N_mon steps, or lbm_residual)
   out->residual = -1.0;
-  if (c->res_evals >= 2) {
-    double r4[4];
-    CK(cudaMemcpyAsync(r4, c->a.mon_out + NMON, 32, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    out->residual = residual_from(r4);
-  }
+  if (c->res_evals >= 2) out->residual = residual_from(r4);
   return LBM_OK;
 }
 
