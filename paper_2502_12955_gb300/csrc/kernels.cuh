@@ -464,7 +464,9 @@ __device__ __forceinline__ void close_thermal(T* h0, T* h1, uint32_t m, const Co
         const T kt = k.arrA * exp(-k.arrTa / Tb);
         const T Cb = T(2) * hb / (w2 + kt * k.fc);
         const T Q = k.hr * kt * Cb;
+        const T was = Tb;
         Tb = (T(2) * gb + Q * k.fT) / w2;
+        if (Tb == was) break;   // every further iteration would repeat this one
       }
       const T kt = k.arrA * exp(-k.arrTa / Tb);
       const T Cb = T(2) * hb / (w2 + kt * k.fc);
@@ -2507,7 +2509,8 @@ __global__ void __launch_bounds__(256) k_solid(const Args a, const Coef<typename
 // Qp = h_r k(T_b) C_b at a reactive link, where C_b = 2 hb / (2 w + k tau_c / (tau_c - 1/2)) closes
 // the species population hb = h_C,j that has just streamed into n (read as the next step's
 // gather reads it); T_b and C_b come from n_it + 1 fixed-point updates starting at the value
-// without reaction, and k is kept for the next step's species closure.  Monitors: heat gained by
+// without reaction, and k is kept for the next step's species closure.  The updates end early once T_b repeats: a
+// fixed point of the rounded arithmetic, so the result is that of all of them.  Monitors: heat gained by
 // the fluid side (bank HEAT), by the solid side (HEAT_S), reaction heat (HEAT_SRC).
 template <class L, class S, int NC, int NS>
 __global__ void __launch_bounds__(256) k_exchange(const Args a, const Coef<typename Store<S>::T> k,
@@ -2526,60 +2529,58 @@ __global__ void __launch_bounds__(256) k_exchange(const Args a, const Coef<typen
   const T den = w * (cf + T(1));
   T heat = T(0), heat_s = T(0), src_q = T(0);
   const unsigned int count = a.fluid_count[0], base = a.fluid_count[1];
-  for (unsigned int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) {
-    const int n = list_node(a, a.fluid_list[e]);
+  // one thread per link: the links of a node are independent, and the chain of a link (its iterations) is long
+  constexpr unsigned int LN = QC <= 5 ? 4 : 8;   // threads per node (two of eight idle in 3D)
+  const unsigned int j1 = threadIdx.x % LN;
+  const int j = int(j1) + 1;
+  for (unsigned int e = (blockIdx.x * blockDim.x + threadIdx.x) / LN; e < count; e += gridDim.x * blockDim.x / LN) {
+    if (j >= QC) continue;
+    const uint32_t wd = a.fluid_list[e];
+    const int n = list_node(a, wd);
     const uint32_t m = a.mask[n];
     if (!(m & 1u)) continue;
-    bool any = false;
-#pragma unroll
-    for (int j = 1; j < QC; ++j) {
-      const uint32_t c = MaskBits<L>::code(m, j);
-      any |= (c == 1u || c == 2u);
-    }
-    if (!any) continue;
-    const long long cell = R::cell(e < base ? (long long)e : (long long)a.slot[n]);
+    const uint32_t c = MaskBits<L>::code(m, j);
+    if (c != 1u && c != 2u) continue;
+    const int i = L::opp(j);
     int x, y, z, ax;
     coords_of(a, n, &x, &y, &z);
-    const Nbr nb = make_nbr(a, x, y, z);
-#pragma unroll
-    for (int j = 1; j < QC; ++j) {
-      const uint32_t c = MaskBits<L>::code(m, j);
-      if (c != 1u && c != 2u) continue;
-      const long long s = nbr_checked(a, x, y, z, L::cx(j), L::cy(j), L::cz(j), perc, &ax);
-      if (s < 0) continue;   // a closed face: plain bounce-back
-      const int i = L::opp(j);
-      SC* hp = R::h(a, cell, 1, i);
-      T* gp = g + (long long)j * a.N + s;
-      const T ho = Store<SC>::ld(hp) + sh1;
-      const T go = *gp;
-      T Tb = (cf * ho + go) / den;
-      T Qp = T(0);
-      if (c == 2u) {
-        // the species population moving toward the wall, where the next step gathers it
-        const SC* bp;
-        if (parity_next == 0 || MaskBits<L>::code(m, i) != 0u)
-          bp = R::h(a, cell, 0, j);
-        else
-          bp = R::h(a, cell_of<R>(a, nb.at(-L::cx(j), -L::cy(j), -L::cz(j))), 0, i);
-        const T hb = Store<SC>::ld(bp) + sh0;
-        T kt = T(0);
-        for (int it = 0; it <= a.n_it; ++it) {
-          kt = k.arrA * exp(-k.arrTa / Tb);
-          const T Cb = T(2) * hb / (T(2) * w + kt * k.fc);
-          Qp = k.hr * kt * Cb;
-          Tb = (cf * ho + go + T(0.5) * cf * Qp) / den;
-        }
-        kb[(long long)(i - 1) * a.N + n] = kt;
+    const long long s = nbr_checked(a, x, y, z, L::cx(j), L::cy(j), L::cz(j), perc, &ax);
+    if (s < 0) continue;   // a closed face: plain bounce-back
+    const long long cell = R::cell(e < base ? (long long)e : (long long)a.slot[n]);
+    SC* hp = R::h(a, cell, 1, i);
+    T* gp = g + (long long)j * a.N + s;
+    const T ho = Store<SC>::ld(hp) + sh1;
+    const T go = *gp;
+    T Tb = (cf * ho + go) / den;
+    T Qp = T(0);
+    if (c == 2u) {
+      // the species population moving toward the wall, where the next step gathers it
+      const SC* bp;
+      if (parity_next == 0 || MaskBits<L>::code(m, i) != 0u)
+        bp = R::h(a, cell, 0, j);
+      else
+        bp = R::h(a, cell_of<R>(a, nbr_entry(a, n, wd).at(-L::cx(j), -L::cy(j), -L::cz(j))), 0, i);
+      const T hb = Store<SC>::ld(bp) + sh0;
+      T kt = T(0);
+      for (int it = 0; it <= a.n_it; ++it) {
+        const T was = Tb;
+        kt = k.arrA * exp(-k.arrTa / Tb);
+        const T Cb = T(2) * hb / (T(2) * w + kt * k.fc);
+        Qp = k.hr * kt * Cb;
+        Tb = (cf * ho + go + T(0.5) * cf * Qp) / den;
+        if (Tb == was) break;   // every further iteration would repeat this one
       }
-      const T hn = T(2) * w * Tb - ho;
-      const T gn = T(2) * w * Tb - go;
-      Store<SC>::st(hp, hn - sh1);
-      *gp = gn;
-      heat += hn - ho;
-      heat_s += gn - go;
-      src_q += Qp;
+      kb[(long long)(i - 1) * a.N + n] = kt;
     }
+    const T hn = T(2) * w * Tb - ho;
+    const T gn = T(2) * w * Tb - go;
+    Store<SC>::st(hp, hn - sh1);
+    *gp = gn;
+    heat += hn - ho;
+    heat_s += gn - go;
+    src_q += Qp;
   }
+  __syncwarp();
   const int lane_slot = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) % WALLX_SLOTS;
   const T vals[3] = {heat, heat_s, src_q};
   const int banks[3] = {BANK_HEAT, BANK_HEAT_S, BANK_HEAT_SRC};

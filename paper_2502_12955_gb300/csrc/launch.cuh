@@ -305,8 +305,8 @@ struct Launchers {
 
   // grid-stride kernels over the box (k_solid) and the fluid list (k_exchange): two waves of
   // blocks, fewer on a small domain
-  static unsigned int box_blocks(const Args& a) {
-    const long long need = (a.N + a.bx - 1) / a.bx, cap = 2ll * wave_blocks() * 256 / a.bx;
+  static unsigned int box_blocks(const Args& a, int per_node = 1) {
+    const long long need = (a.N * per_node + a.bx - 1) / a.bx, cap = 2ll * wave_blocks() * 256 / a.bx;
     return (unsigned int)(need < cap ? (need > 0 ? need : 1) : cap);
   }
   static cudaError_t solid(const Args& a, int parity, cudaStream_t st) {
@@ -317,8 +317,8 @@ struct Launchers {
     cudaError_t e = cudaErrorInvalidValue;
     by_nc_ns(a, [&](auto nc, auto ns) {
       if constexpr (decltype(ns)::value >= 2)
-        e = launch_pdl(kEarly, k_exchange<L, S, decltype(nc)::value, decltype(ns)::value>, box_blocks(a), a.bx, 0, st, a, coef(a),
-                       parity_next);
+        e = launch_pdl(kEarly, k_exchange<L, S, decltype(nc)::value, decltype(ns)::value>, box_blocks(a, L::QC <= 5 ? 4 : 8), a.bx,
+                       0, st, a, coef(a), parity_next);
     });
     return e;
   }
