@@ -955,13 +955,13 @@ __device__ __forceinline__ void mrt_pairs_d3q19(T* f, const K& k, T drho, T jx, 
 // Everything after the gather for one fluid node: wet-node closure and its bookkeeping,
 // deposition, moments, forces, velocity, flow and scalar collision, in-place scatter.  entry: the
 // node's fluid-list entry; c: its cells; o: its odd cells (parity 1).
-template <class L, class S, int NC, int NS, int COLL, int parity, bool BND, int CS>
+template <class L, class S, int NC, int NS, int COLL, int parity, bool BND, int CS, class Pre>
 __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typename Store<S>::T>& k, uint32_t entry, int n,
                                                 uint32_t m, long long c, const OddCells<L, S, NC, NS, CS, BND>& o,
                                                 typename Store<S>::T (&f)[NC][L::Q],
                                                 typename Store<S>::T (&h)[NS > 0 ? NS : 1][L::QC],
                                                 typename Store<S>::T& wallx, typename Store<S>::T& heatx,
-                                                typename Store<S>::T& prodx) {
+                                                typename Store<S>::T& prodx, Pre pre) {
   using T = typename Store<S>::T;
   using R = Rec<L, S, NC, NS>;
   using SC = typename R::SC;
@@ -1167,6 +1167,14 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
       if (xin) uin = T(a.u_in_row[yy]);
     }
   }
+  // the cache entries move to registers, and the cache takes the next node's while this one is stored
+  uint32_t ent[parity ? Q - 1 : 1];
+  if (parity) {
+#pragma unroll
+    for (int i = 0; i < Q - 1; ++i) ent[i] = o.cache[i * CS];
+  }
+  pre();
+  const OddCells<L, S, NC, NS, 1, BND> to{a, c, m, ent};
 #pragma unroll
   for (int s = 0; s < NC; ++s) {
     Store<S>::st(R::f(a, c, s, 0), f[s][0]);
@@ -1182,7 +1190,7 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
         else if (L::cy(i) > 0 && top && flow_wall<L>(m, i))
           v -= T(L::w(i)) * rho[s] * (T(L::cx(i)) * k.uw6[0] + T(L::cz(i)) * k.uw6[2] + k.uw6[1]);
       }
-      if (keep) Store<S>::st(parity ? o.flow(s, i) : R::f(a, c, s, L::opp(i)), v);
+      if (keep) Store<S>::st(parity ? to.flow(s, i) : R::f(a, c, s, L::opp(i)), v);
       // zero-gradient outlet: the population entering through x = nx - 1 with direction i
       // repeats the node's own post-collision f_i, in the cell where link opp(i) reflects
       if (BND && L::cx(i) < 0 && xout) Store<S>::st(R::f(a, c, s, i), f[s][i]);
@@ -1211,7 +1219,7 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
         }
         v = b;
       }
-      Store<SC>::st(parity ? o.scal(s, j) : R::h(a, c, s, L::opp(j)), v);
+      Store<SC>::st(parity ? to.scal(s, j) : R::h(a, c, s, L::opp(j)), v);
     }
   }
 }
@@ -1239,25 +1247,26 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   uint32_t w_nx = e + stride < count ? a.fluid_list[e + stride] : 0u;
   uint32_t m_cur = e < count ? a.mask[list_node(a, w_cur)] : 0u;
   if constexpr (parity == 1) {
-    // two cache buffers: the neighbours of the next entry are copied asynchronously into one while
-    // the current entry works from the other
-    __shared__ uint32_t slot_buf[2 * (L::Q - 1) * LBM_STEP_CACHE_STRIDE];
+    // the neighbours of the next entry are copied in (asynchronously) while this entry is stored
+    __shared__ uint32_t slot_buf[(L::Q - 1) * LBM_STEP_CACHE_STRIDE];
     uint32_t* cb = slot_buf + threadIdx.x;
-    uint32_t* cn = slot_buf + (L::Q - 1) * LBM_STEP_CACHE_STRIDE + threadIdx.x;
     const uint32_t* map = BND ? a.slot : a.off;
     if (e < count) prefetch_nbrs<L, LBM_STEP_CACHE_STRIDE>(a, map, w_cur, cb);
     cp_async_commit();
     if (a.geo_mode == GEO_NONE) pdl_wait();
     for (; e < count; e += stride) {
       const uint32_t w = w_cur, m = m_cur;
-      if (e + stride < count) {
+      const bool more = e + stride < count;
+      if (more) {
         w_cur = w_nx;
         m_cur = a.mask[list_node(a, w_cur)];
-        prefetch_nbrs<L, LBM_STEP_CACHE_STRIDE>(a, map, w_cur, cn);
       }
       if (e + 2 * stride < count) w_nx = a.fluid_list[e + 2 * stride];
-      cp_async_commit();
-      cp_async_wait<1>();   // this entry's neighbours have arrived
+      cp_async_wait<0>();   // this entry's neighbours have arrived
+      const auto pre = [&]() {
+        if (more) prefetch_nbrs<L, LBM_STEP_CACHE_STRIDE>(a, map, w_cur, cb);
+        cp_async_commit();
+      };
       if (m & 1u) {
         T f[NC][Q], h[NSD][QC];
         const int n = list_node(a, w);
@@ -1267,11 +1276,10 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
         if (!BND) wall_offsets<L, R, LBM_STEP_CACHE_STRIDE>(uint32_t(c) + uint32_t(kOffBias * R::FROW), m, cb);
         const O o{a, c, m, cb};
         gather_odd<L, S, NC, NS, LBM_STEP_CACHE_STRIDE, BND>(o, f, h);
-        collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, k, w, n, m, c, o, f, h, wallx, heatx, prodx);
+        collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, k, w, n, m, c, o, f, h, wallx, heatx, prodx, pre);
+      } else {
+        pre();
       }
-      uint32_t* t = cb;
-      cb = cn;
-      cn = t;
     }
     cp_async_wait<0>();
   } else {
@@ -1286,7 +1294,7 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
       const int n = list_node(a, w);
       const long long c = cell(e, n);
       gather_even<L, S, NC, NS>(a, c, f, h);
-      collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, k, w, n, m, c, O{a, c, m, nullptr}, f, h, wallx, heatx, prodx);
+      collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, k, w, n, m, c, O{a, c, m, nullptr}, f, h, wallx, heatx, prodx, []() {});
     }
   }
   // ---- wall-exchange monitor: one reduction per warp that saw a reactive link
@@ -1348,7 +1356,7 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   __shared__ Coef<T> sk;
   using R = Rec<L, S, NC, NS>;
   using O = OddCells<L, S, NC, NS, 1, BND>;
-  extern __shared__ uint32_t slot_smem[];   // 2 * blockDim.x * Q words at odd parity (launcher)
+  extern __shared__ uint32_t slot_smem[];   // blockDim.x * Q words at odd parity (launcher)
   uint32_t* cache = slot_smem + threadIdx.x * L::Q;
   // blocks take chunks of consecutive tiles in turn (at most LBM_TILE_CHUNK, fewer where that would leave
   // blocks idle): the work list holds each member's tiles together, so a chunk mostly stays within
@@ -1357,10 +1365,9 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   auto next_tile = [&](unsigned int t) {
     return t + ((t % chunk == chunk - 1) ? (gridDim.x - 1) * chunk + 1 : 1);
   };
-  // odd parity: two neighbour buffers, the next tile's are copied in (cp.async)
-  // while this tile computes, as in k_step; the next tile's list entry and link mask are loaded
-  // one tile ahead at both parities whenever it belongs to the member already staged
-  uint32_t* cn = slot_smem + (blockDim.x + threadIdx.x) * L::Q;
+  // odd parity: the next tile's neighbours are copied in (cp.async) while this tile is stored, as in
+  // k_step; the next tile's list entry and link mask are loaded one tile ahead at both parities
+  // whenever it belongs to the member already staged
   bool have_next = false, waited = false;
   uint32_t w_pf = 0u, m_pf = 0u;
   unsigned int staged = 0xffffffffu;
@@ -1393,9 +1400,13 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
       m = a.mask[list_node(a, w)];
       if (parity) prefetch_nbrs<L, 1>(a, map, w, cache);
     }
-    if (parity) cp_async_commit();
+    if (parity) {
+      cp_async_commit();
+      cp_async_wait<0>();   // this tile's neighbours have arrived
+    }
     // the next tile of this block, if it belongs to the staged member
     have_next = false;
+    bool next_in = false;
     const unsigned int tn = next_tile(t);
     if (tn < ntiles) {
       const Tile tile2 = tiles[tn];
@@ -1406,15 +1417,14 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
         if (e2 < count) {
           w_pf = a.fluid_list[e2];
           m_pf = a.mask[list_node(a, w_pf)];
-          if (parity) prefetch_nbrs<L, 1>(a, map, w_pf, cn);
+          next_in = true;
         }
         have_next = true;
       }
     }
-    if (parity) {
-      cp_async_commit();
-      cp_async_wait<1>();   // this tile's neighbours have arrived
-    }
+    const auto pre = [&]() {
+      if (parity && next_in) prefetch_nbrs<L, 1>(a, map, w_pf, cache);
+    };
     if (!waited) pdl_wait();   // ensembles keep their geometry: everything read so far is static
     waited = true;
     if (e < count && (m & 1u)) {
@@ -1430,12 +1440,9 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
       } else {
         gather_even<L, S, NC, NS>(a, c, f, h);
       }
-      collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, sk, w, n, m, c, o, f, h, wallx, heatx, prodx);
-    }
-    if (parity) {
-      uint32_t* tmp = cache;
-      cache = cn;
-      cn = tmp;
+      collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, sk, w, n, m, c, o, f, h, wallx, heatx, prodx, pre);
+    } else {
+      pre();
     }
     if (NS > 0) {
       const unsigned int any = __ballot_sync(0xffffffffu, wallx != T(0));
