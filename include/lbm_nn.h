@@ -103,11 +103,11 @@ lbm_status lbm_nn_pack_weights(const float* w, void* wk, void* wt, int32_t Co, i
 lbm_status lbm_nn_unpack_wgrad(const float* dwcol, float* dw, int32_t Co, int32_t Ci, void* stream);
 /* 3^3 convolution without im2col rows (tcgen05, implicit GEMM): y [D*H*W][N] = conv(x) + bias (bias may be
    NULL), then max(., 0) with relu.  x is xa [.][Ca], on the coarse grid (D/2, H/2, W/2) and upsampled 2x if up,
-   followed along the channels by xb [D*H*W][Cb] (Cb == 0: none).  Ca and Cb multiples of 16, or one input of at
-   most 8 channels.  N % 16 == 0, N <= 256.  Columns [0, n0) go to y0 [.][n0], the rest to y1 [.][N - n0] (n0 == N:
+   followed along the channels by xb [D*H*W][Cb] (Cb == 0: none).  Ca and Cb multiples of 16, or one input of
+   Ca <= 8 channels in rows of 8 (lbm_nn_pad8).  N % 16 == 0, N <= 256.  Columns [0, n0) go to y0 [.][n0], the rest to y1 [.][N - n0] (n0 == N:
    y1 unused).  wp: the weights from lbm_nn_conv3_pack (wp for the convolution with N = Co; wtp with dL/dy as x and
-   N = Ci for its input gradient).  Arrays 16-byte aligned (the narrow input excepted).  The same sums
-   in the same order as lbm_nn_im2col + lbm_nn_gemm_tn. */
+   N = Ci for its input gradient).  Arrays 16-byte aligned.  The same sums in
+   the same order as lbm_nn_im2col + lbm_nn_gemm_tn. */
 lbm_status lbm_nn_conv3(const void* xa, int32_t Ca, int32_t up, const void* xb, int32_t Cb, int32_t D, int32_t H, int32_t W,
                         const void* wp, int32_t N, const float* bias, int32_t relu, void* y0, int32_t n0, void* y1,
                         void* stream);
@@ -116,6 +116,8 @@ lbm_status lbm_nn_conv3(const void* xa, int32_t Ca, int32_t up, const void* xb, 
 lbm_status lbm_nn_conv3_wgrad(const void* xa, int32_t Ca, int32_t up, const void* xb, int32_t Cb, int32_t D, int32_t H,
                               int32_t W, const void* dy, int32_t Co, float* scratch, float* dw, void* stream);
 int64_t lbm_nn_conv3_wgrad_scratch(int32_t D, int32_t H, int32_t W, int32_t C, int32_t Co);
+/* x8 [V][8] = x [V][C], C <= 8, zero padded. */
+lbm_status lbm_nn_pad8(const void* x, void* x8, int64_t V, int32_t C, void* stream);
 /* Weights w [Co][Ci][27] (FP32) in the operand order of lbm_nn_conv3: wp (lbm_nn_conv3_packed(Co, Ci) BF16 elements)
    and, if wtp is not NULL, the flipped transpose for the input gradient (lbm_nn_conv3_packed(Ci, Co)). */
 lbm_status lbm_nn_conv3_pack(const float* w, void* wp, void* wtp, int32_t Co, int32_t Ci, void* stream);

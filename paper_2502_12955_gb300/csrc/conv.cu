@@ -24,6 +24,7 @@
 // LBM_ERR_TIMEOUT) and the kernel still releases its TMEM before it returns.
 #include <algorithm>
 #include <initializer_list>
+#include <type_traits>
 
 #include "../../include/lbm_nn.h"
 #include "tc.cuh"
@@ -237,8 +238,14 @@ __global__ void __launch_bounds__(192, 4) k_conv3(const ConvSrc src, const bf16*
     }
   } else if (warp == 4) {
     if (lane == 0) {
+      // one thread issues 27 C / 16 MMAs per output, so the loop is kept to a few instructions each: descriptors
+      // differ in their start address only, in 16-byte units
       const uint32_t idesc = idesc_bf16(128, N);
-      int b = 0;   // weight stage counter
+      const uint64_t a_desc = desc_plain(saddr(sA), CHUNK, HX * ROW16), b_desc = desc_plain(saddr(sB), (uint32_t)N * 16, 128);
+      const uint32_t a_step = 2 * CHUNK / 16, b_step = 2 * (uint32_t)N, plane16 = plane_bytes / 16, stage16 = stage_bytes / 16;
+      const int n16 = (p.stages ? p.sc : C) / 16;
+      int st = 0;              // weight stage and the parity of its current fill
+      unsigned st_ph = 0;
       if (!p.stages && !mbar_wait(&fullB[0], 0)) ok = false;
       for (int t = 0; t < nz && ok; ++t) {
         const int ac = t % p.accs;
@@ -246,37 +253,42 @@ __global__ void __launch_bounds__(192, 4) k_conv3(const ConvSrc src, const bf16*
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)(ac * N);
         uint32_t acc = 0;
+        uint64_t bd = b_desc;
+#pragma unroll 1
         for (int dz = 0; dz < 3 && ok; ++dz) {
           const int q = p.seq ? 3 * t + dz : t + dz;
-          if (!mbar_wait(&fullA[q % P], (unsigned)(q / P) & 1u)) {
+          if ((p.seq || t == 0 || dz == 2) && !mbar_wait(&fullA[q % P], (unsigned)(q / P) & 1u)) {
             ok = false;
             break;
           }
-          const uint32_t pa = saddr(sA) + (uint32_t)(q % P) * plane_bytes;
-          for (int tap = 0; tap < 9 && ok; ++tap) {
-            const uint32_t ta = pa + (uint32_t)((tap / 3) * HX + tap % 3) * ROW16;
-            for (int ch = 0; ch < nch; ++ch) {
-              uint32_t wb;
-              int st = 0;
-              if (p.stages) {
-                st = b % p.stages;
-                if (!mbar_wait(&fullB[st], (unsigned)(b / p.stages) & 1u)) {
-                  ok = false;
-                  break;
+          uint64_t ad = a_desc + (uint64_t)((uint32_t)(q % P) * plane16);
+#pragma unroll 1
+          for (int dy = 0; dy < 3 && ok; ++dy, ad += HX) {
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+              uint64_t a = ad + dx;
+              if (!p.stages) {
+#pragma unroll 2
+                for (int kk = 0; kk < n16; ++kk, a += a_step, bd += b_step) {
+                  mma_bf16(d, a, bd, idesc, acc);
+                  acc = 1;
                 }
-                wb = saddr(sB) + (uint32_t)st * stage_bytes;
               } else {
-                wb = saddr(sB) + (uint32_t)(dz * 9 + tap) * tap_bytes;
+                for (int ch = 0; ch < nch && ok; ++ch) {
+                  if (!mbar_wait(&fullB[st], st_ph)) ok = false;
+                  bd = b_desc + (uint64_t)((uint32_t)st * stage16);
+#pragma unroll 2
+                  for (int kk = 0; kk < n16; ++kk, a += a_step, bd += b_step) {
+                    mma_bf16(d, a, bd, idesc, acc);
+                    acc = 1;
+                  }
+                  mma_commit(&emptyB[st]);
+                  if (++st == p.stages) {
+                    st = 0;
+                    st_ph ^= 1u;
+                  }
+                }
               }
-              const int n16 = (p.stages ? p.sc : C) / 16;
-              for (int kk = 0; kk < n16; ++kk) {
-                const uint32_t a = ta + (uint32_t)((p.stages ? ch * p.sc / 8 : 0) + 2 * kk) * CHUNK;
-                mma_bf16(d, desc_plain(a, CHUNK, HX * ROW16), desc_plain(wb + (uint32_t)kk * N * 32, (uint32_t)N * 16, 128),
-                         idesc, acc);
-                acc = 1;
-              }
-              if (p.stages) mma_commit(&emptyB[st]);
-              ++b;
             }
           }
           if (p.seq) mma_commit(&emptyA[q % P]);
@@ -313,86 +325,92 @@ __global__ void __launch_bounds__(192, 4) k_conv3(const ConvSrc src, const bf16*
   if (warp == 0) tmem_free(tmem, (uint32_t)p.cols);
 }
 
-// The first layer: C <= 8 channels, not a multiple of 16.  K runs over tap * C + c as in the im2col GEMM (in
-// 16s across taps), so the 128 x K16 operand is assembled row by row from the halo planes in shared memory.
-constexpr int kFirstMaxK16 = 14;   // ceil(27 * 8 / 16)
-__global__ void __launch_bounds__(128) k_conv3_first(const bf16* __restrict__ x, const bf16* __restrict__ wp, const ConvOut out,
-                                                     int C, int N, int nz, int D, int H, int W, int cols, int* err) {
+// The first layer: C <= 8 channels in rows of 8 (lbm_nn_pad8).  K runs over tap * C + c as in the im2col GEMM (in 16s
+// across taps), so a row of the operand is put together from the 27 neighbours' 16-byte rows in registers: chunk q
+// holds the values k = 8 q .. 8 q + 7, all positions known at compile time.
+template <int C>
+struct FirstRow {
+  static constexpr int K16 = (27 * C + 15) / 16, CHUNKS = 2 * K16, USED = (27 * C + 7) / 8;
+  uint4 t[27];
+  __device__ __forceinline__ void load(const bf16* __restrict__ x8, long long v, int x, int y, int z, int D, int H, int W, bool in) {
+#pragma unroll
+    for (int i = 0; i < 27; ++i) {
+      const int dz = i / 9 - 1, dy = (i / 3) % 3 - 1, dx = i % 3 - 1;
+      const bool ok = in && (unsigned)(x + dx) < (unsigned)W && (unsigned)(y + dy) < (unsigned)H && (unsigned)(z + dz) < (unsigned)D;
+      t[i] = ok ? __ldg(reinterpret_cast<const uint4*>(x8 + (v + (long long)(dz * H + dy) * W + dx) * 8)) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+  __device__ __forceinline__ uint32_t half_at(int k) const {   // 16-bit value k
+    if (k >= 27 * C) return 0u;
+    const int tap = k / C, c = k % C;
+    const uint32_t w = c / 2 == 0 ? t[tap].x : (c / 2 == 1 ? t[tap].y : (c / 2 == 2 ? t[tap].z : t[tap].w));
+    return c % 2 ? w >> 16 : w & 0xffffu;
+  }
+  __device__ __forceinline__ uint4 chunk(int q) const {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = half_at(8 * q + 2 * i) | half_at(8 * q + 2 * i + 1) << 16;
+    return make_uint4(w[0], w[1], w[2], w[3]);
+  }
+};
+
+// x [V][C] -> x8 [V][8], zero padded
+__global__ void __launch_bounds__(256) k_pad8(const bf16* __restrict__ x, bf16* __restrict__ x8, long long V, int C) {
+  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
+    __align__(16) bf16 w[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) w[c] = c < C ? x[v * C + c] : __float2bfloat16_rn(0.f);
+    *reinterpret_cast<uint4*>(x8 + v * 8) = *reinterpret_cast<const uint4*>(w);
+  }
+}
+
+// Tiles of 128 consecutive voxels, one thread per voxel; the CTAs of an SM hide one another's phases.
+template <int C>
+__global__ void __launch_bounds__(128, 3) k_conv3_first(const bf16* __restrict__ x8, const bf16* __restrict__ wp, const ConvOut out,
+                                                        int N, int D, int H, int W, int cols, int* err) {
+  using F = FirstRow<C>;
   extern __shared__ unsigned char raw[];
   unsigned char* base = raw + ((128u - (saddr(raw) & 127u)) & 127u);
-  const int k16 = (27 * C + 15) / 16;
-  unsigned char* sA = base;                                        // [2 k16][128 rows][16 bytes]
-  unsigned char* sB = sA + (size_t)k16 * 4096;                     // [k16][2][N][16 bytes]
-  bf16* halo = reinterpret_cast<bf16*>(sB + (size_t)k16 * N * 32);  // ring of 3 planes [PV][C]
+  unsigned char* sA = base;                                        // [CHUNKS][128 rows][16 bytes]
+  unsigned char* sB = sA + F::CHUNKS * 2048;                       // [K16][2][N][16 bytes]
   __shared__ uint64_t full, done;
   __shared__ uint32_t slot;
   const int warp = threadIdx.x >> 5;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * nz;
+  const long long V = (long long)D * H * W;
   if (threadIdx.x == 0) {
     mbar_init(&full, 1);
     mbar_init(&done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    mbar_expect_tx(&full, (unsigned)(k16 * N * 32));
-    bulk_load(sB, wp, (unsigned)(k16 * N * 32), &full);
+    mbar_expect_tx(&full, (unsigned)(F::K16 * N * 32));
+    bulk_load(sB, wp, (unsigned)(F::K16 * N * 32), &full);
   }
   if (warp == 0) tmem_alloc(&slot, (uint32_t)cols);
-  auto load_plane = [&](int z) {
-    bf16* dst = halo + (size_t)((z + 3) % 3) * PV * C;
-    for (int i = threadIdx.x; i < PV * C; i += 128) {
-      const int v = i / C, c = i - v * C;
-      const int xx = x0 - 1 + v % HX, yy = y0 - 1 + v / HX;
-      bf16 val = __float2bfloat16_rn(0.f);
-      if (xx >= 0 && xx < W && yy >= 0 && yy < H && z >= 0 && z < D) val = x[((long long)(z * H + yy) * W + xx) * C + c];
-      dst[i] = val;
-    }
-  };
-  load_plane(z0 - 1);
-  load_plane(z0);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = slot;
   bool ok = warp_wait(&full, 0);
-  const int m = threadIdx.x, mx = m % TX, my = m / TX;
-  for (int t = 0; t < nz && z0 + t < D; ++t) {
-    const int z = z0 + t;
-    load_plane(z + 1);
-    __syncthreads();
-    // this thread's row of the operand
+  unsigned ph = 0;
+  for (long long v0 = (long long)blockIdx.x * 128; v0 < V; v0 += (long long)gridDim.x * 128, ph ^= 1u) {
+    const long long v = v0 + threadIdx.x;
     {
-      int tap = 0, c = 0;
-      const bf16* row = nullptr;
-      auto tap_row = [&]() {
-        const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-        row = halo + ((size_t)((z + dz - 1 + 3) % 3) * PV + (my + dy) * HX + mx + dx) * C;
-      };
-      tap_row();
-      for (int k8 = 0; k8 < 2 * k16; ++k8) {
-        __align__(16) bf16 w[8];
+      F row;
+      const int r = (int)(v / W);
+      row.load(x8, v, (int)(v - (long long)r * W), r % H, r / H, D, H, W, v < V);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          w[i] = tap < 27 ? row[c] : __float2bfloat16_rn(0.f);
-          if (++c == C) {
-            c = 0;
-            if (++tap < 27) tap_row();
-          }
-        }
-        *reinterpret_cast<uint4*>(sA + (size_t)k8 * 2048 + m * 16) = *reinterpret_cast<const uint4*>(w);
-      }
+      for (int q = 0; q < F::CHUNKS; ++q) *reinterpret_cast<uint4*>(sA + q * 2048 + threadIdx.x * 16) = row.chunk(q);
     }
     fence_async();
     __syncthreads();
     if (threadIdx.x == 0 && ok) {
       const uint32_t idesc = idesc_bf16(128, N);
-      for (int kk = 0; kk < k16; ++kk)
-        mma_bf16(tmem, desc_plain(saddr(sA) + (uint32_t)kk * 4096, 2048, 128),
-                 desc_plain(saddr(sB) + (uint32_t)kk * N * 32, (uint32_t)N * 16, 128), idesc, kk > 0 ? 1u : 0u);
+      const uint64_t ad = desc_plain(saddr(sA), 2048, 128), bd = desc_plain(saddr(sB), (uint32_t)N * 16, 128);
+      for (int kk = 0; kk < F::K16; ++kk) mma_bf16(tmem, ad + kk * 256, bd + (uint64_t)(kk * 2 * N), idesc, kk > 0 ? 1u : 0u);
       mma_commit(&done);
     }
-    if (ok && !warp_wait(&done, (unsigned)t & 1u)) ok = false;
+    if (ok && !warp_wait(&done, ph)) ok = false;
     tc_fence_after();
-    store_row(tmem + ((uint32_t)(warp * 32) << 16), out, N, ((long long)z * H + y0 + my) * W + x0 + mx,
-              ok && x0 + mx < W && y0 + my < H);
+    store_row(tmem + ((uint32_t)(warp * 32) << 16), out, N, v, ok && v < V);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -415,41 +433,49 @@ struct WgradPlan {
   int C, Co;
   int tiles, tj, jobs;       // 128-row tiles of k, tiles per CTA, CTAs along k
   int nkb, kbs, splits;      // 64-voxel blocks, blocks per split, splits
-  int nb, cols;              // dy buffers, TMEM columns
+  int ws, nb, cols;          // im2col tiles in the ring, dy buffers, TMEM columns
   unsigned smem;
 };
-constexpr int WSTAGES = 4;                 // ring of 16 KB im2col tiles
+constexpr int WSTAGES = 6;                 // ring of 16 KB im2col tiles, fewer (more than WLAG) for wide layers
+constexpr int WLAG = 3;                    // tiles whose copies are in flight behind the one being issued
 constexpr int WBLOCK = 64 * 16;            // bytes of an 8-row chunk of 64 voxels
 
 __device__ __forceinline__ void cp16_ca(void* dst, const void* src, bool in) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n" ::"r"(saddr(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
 }
 
-__global__ void __launch_bounds__(160, 4) k_wgrad(const ConvSrc src, const bf16* __restrict__ dy, float* __restrict__ part,
+template <int FIRST>   // 0: channels in 16s; else the narrow input of FIRST channels in rows of 8
+__global__ void __launch_bounds__(288, FIRST ? 1 : 2) k_wgrad(const ConvSrc src, const bf16* __restrict__ dy, float* __restrict__ part,
                                                const WgradPlan p, int D, int H, int W, int* err) {
   extern __shared__ unsigned char raw[];
   unsigned char* base = raw + ((128u - (saddr(raw) & 127u)) & 127u);
   __shared__ uint64_t full[WSTAGES], empty[WSTAGES], done;
   __shared__ uint32_t slot;
   unsigned char* sA = base;
-  unsigned char* sB = base + WSTAGES * 16 * WBLOCK;
+  unsigned char* sB = base + (size_t)p.ws * 16 * WBLOCK;
   const uint32_t bbytes = (uint32_t)(p.Co / 8) * WBLOCK;
-  int* table = reinterpret_cast<int*>(sB + (size_t)p.nb * bbytes);   // [16 tj] tap | c << 8, or -1 past 27 C
+  // per pair of 8-row chunks (16 channels of a tap): tap, part of the input (0 a, 1 a on the coarse grid, 2 b, -1 past
+  // 27 C), element offset from the voxel's own row (channel alone on the coarse grid)
+  int4* table = reinterpret_cast<int4*>(sB + (size_t)p.nb * bbytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int C = p.C, Co = p.Co;
+  const int C = p.C, Co = p.Co, ws = p.ws;
   const int t0 = blockIdx.y * p.tj, nt = min(p.tj, p.tiles - t0);
   const int kb0 = blockIdx.x * p.kbs, kb1 = min(p.nkb, kb0 + p.kbs);
   if (threadIdx.x == 0) {
     for (int i = 0; i < WSTAGES; ++i) {
-      mbar_init(&full[i], 128);
+      mbar_init(&full[i], 256);
       mbar_init(&empty[i], 1);
     }
     mbar_init(&done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  for (int i = threadIdx.x; i < 16 * nt; i += 160) {
-    const int k = (t0 * 16 + i) * 8;
-    table[i] = k < 27 * C ? (k / C) | (k % C) << 8 : -1;
+  for (int i = threadIdx.x; i < 8 * nt; i += 288) {
+    const int k = (t0 * 8 + i) * 16, tap = k / C, c = k % C;
+    const int shift = ((tap / 9 - 1) * H + (tap / 3) % 3 - 1) * W + tap % 3 - 1;
+    table[i] = k >= 27 * C ? make_int4(0, -1, 0, 0)
+               : c >= src.ca ? make_int4(tap, 2, shift * src.cb + c - src.ca, 0)
+               : src.up ? make_int4(tap, 1, c, 0)
+                        : make_int4(tap, 0, shift * src.ca + c, 0);
   }
   if (warp == 0) tmem_alloc(&slot, (uint32_t)p.cols);
   tc_fence_before();
@@ -459,73 +485,91 @@ __global__ void __launch_bounds__(160, 4) k_wgrad(const ConvSrc src, const bf16*
   bool ok = true;
   const int total = (kb1 - kb0) * nt;
 
-  if (warp < 4) {
-    const int vox = threadIdx.x & 63, half = threadIdx.x >> 6;
-    const bool vec = C % 8 == 0;
-    int v = kb0 * 64 + vox;
-    int x = v % W, y = (v / W) % H, z = v / (W * H);
+  if (warp < 8) {
     int a = 0;
-    for (int kb = kb0; kb < kb1 && ok; ++kb) {
-      // taps whose voxel is inside: bits tap = (dz + 1) 9 + (dy + 1) 3 + dx + 1
-      const uint32_t mx = (x > 0 ? 1u : 0u) | 2u | (x < W - 1 ? 4u : 0u);
-      const uint32_t my = (y > 0 ? mx : 0u) | mx << 3 | (y < H - 1 ? mx << 6 : 0u);
-      const uint32_t mz = (z > 0 ? my : 0u) | my << 9 | (z < D - 1 ? my << 18 : 0u);
-      for (int ti = 0; ti < nt && ok; ++ti, ++a) {
-        const int s = a % WSTAGES;
-        if (a >= WSTAGES && !warp_wait(&empty[s], (unsigned)(a / WSTAGES - 1) & 1u)) ok = false;
-        if (ti == 0) {   // the block's dy, for all of its tiles
-          unsigned char* d = sB + (size_t)((kb - kb0) % p.nb) * bbytes + vox * 16;
-          for (int o8 = half; o8 < Co / 8; o8 += 2) cp16_ca(d + o8 * WBLOCK, dy + (long long)v * Co + o8 * 8, true);
-        }
-        unsigned char* d = sA + (size_t)s * 16 * WBLOCK + vox * 16;
-#pragma unroll 4
-        for (int j = half; j < 16; j += 2) {
-          const int e = table[ti * 16 + j];
-          const int tap = e & 255, c = e >> 8;
-          if (vec) {
-            const bool in = e >= 0 && ((mz >> tap) & 1u);
-            const int dz = tap / 9 - 1, dy3 = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
+    auto publish_behind = [&]() {
+      cp_commit();
+      asm volatile("cp.async.wait_group %0;\n" ::"n"(WLAG) : "memory");
+      if (a >= WLAG) {
+        fence_async();
+        mbar_arrive(&full[(a - WLAG) % ws]);
+      }
+    };
+    if constexpr (FIRST > 0) {
+      // a warp pair per 64-voxel block, four blocks at a time: every thread puts one voxel's row together, then the
+      // blocks' tiles are written in order
+      using F = FirstRow<FIRST>;
+      const int vox = threadIdx.x & 63, grp = threadIdx.x >> 6;
+      for (int kb = kb0; kb < kb1 && ok; kb += 4) {
+        const bool mine = kb + grp < kb1;
+        const int v = (kb + grp) * 64 + vox;
+        const int r = v / W;
+        F row;
+        row.load(src.a, v, v - r * W, r % H, r / H, D, H, W, mine);
+        for (int g = 0; g < 4 && kb + g < kb1 && ok; ++g)
+          for (int ti = 0; ti < nt && ok; ++ti, ++a) {
+            const int s = a % ws;
+            if (a >= ws && !warp_wait(&empty[s], (unsigned)(a / ws - 1) & 1u)) ok = false;
+            if (g == grp) {
+              unsigned char* d = sA + (size_t)s * 16 * WBLOCK + vox * 16;
+              if (ti == 0)
+                for (int o8 = 0; o8 < Co / 8; ++o8)
+                  cp16_ca(sB + (size_t)((kb + g - kb0) % p.nb) * bbytes + vox * 16 + o8 * WBLOCK, dy + (long long)v * Co + o8 * 8, true);
+#pragma unroll
+              for (int q = 0; q < F::USED; ++q)
+                if (q / 16 == t0 + ti) *reinterpret_cast<uint4*>(d + (q % 16) * WBLOCK) = row.chunk(q);
+            }
+            publish_behind();
+          }
+      }
+    } else {
+      // two lanes per voxel take the two chunks of a pair, so that they read 32 contiguous bytes
+      const int sub = threadIdx.x & 1, vox = (threadIdx.x >> 1) & 63, half = threadIdx.x >> 7;
+      int v = kb0 * 64 + vox;
+      int x = v % W, y = (v / W) % H, z = v / (W * H);
+      for (int kb = kb0; kb < kb1 && ok; ++kb) {
+        // taps whose voxel is inside: bits tap = (dz + 1) 9 + (dy + 1) 3 + dx + 1
+        const uint32_t mx = (x > 0 ? 1u : 0u) | 2u | (x < W - 1 ? 4u : 0u);
+        const uint32_t my = (y > 0 ? mx : 0u) | mx << 3 | (y < H - 1 ? mx << 6 : 0u);
+        const uint32_t mz = (z > 0 ? my : 0u) | my << 9 | (z < D - 1 ? my << 18 : 0u);
+        const bf16* pa = src.a + (src.up ? 0 : (long long)v * src.ca) + sub * 8;
+        const bf16* pb = src.b + (long long)v * src.cb + sub * 8;
+        for (int ti = 0; ti < nt && ok; ++ti, ++a) {
+          const int s = a % ws;
+          if (a >= ws && !warp_wait(&empty[s], (unsigned)(a / ws - 1) & 1u)) ok = false;
+          if (ti == 0) {   // the block's dy, for all of its tiles
+            unsigned char* d = sB + (size_t)((kb - kb0) % p.nb) * bbytes + vox * 16;
+            for (int o8 = 2 * half + sub; o8 < Co / 8; o8 += 4) cp16_ca(d + o8 * WBLOCK, dy + (long long)v * Co + o8 * 8, true);
+          }
+          unsigned char* d = sA + (size_t)s * 16 * WBLOCK + (8 * half + sub) * WBLOCK + vox * 16;
+#pragma unroll
+          for (int jj = 0; jj < 4; ++jj, d += 2 * WBLOCK) {
+            const int4 e = table[ti * 8 + half * 4 + jj];
+            const bool in = e.y >= 0 && ((mz >> e.x) & 1u);
             const bf16* q = src.a;
             if (in) {
-              if (c >= src.ca) q = src.b + ((long long)v + (dz * H + dy3) * W + dx) * src.cb + (c - src.ca);
-              else if (src.up) q = src_at(src, c, x + dx, y + dy3, z + dz, H, W);
-              else q = src.a + ((long long)v + (dz * H + dy3) * W + dx) * src.ca + c;
+              if (e.y == 0) q = pa + e.z;
+              else if (e.y == 2) q = pb + e.z;
+              else
+                q = pa + ((long long)(((z + e.x / 9 - 1) >> 1) * (H >> 1) + ((y + (e.x / 3) % 3 - 1) >> 1)) * (W >> 1) +
+                          ((x + e.x % 3 - 1) >> 1)) * src.ca + e.z;
             }
-            cp16_ca(d + j * WBLOCK, q, in);
-          } else {
-            // a narrow input: the chunk's 8 values come from one or more taps
-            __align__(16) bf16 w[8];
-            int t = tap, cc = c;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const bool in = e >= 0 && t < 27 && ((mz >> t) & 1u);
-              w[i] = in ? src.a[((long long)v + ((t / 9 - 1) * H + (t / 3) % 3 - 1) * W + t % 3 - 1) * C + cc] : __float2bfloat16_rn(0.f);
-              if (++cc == C) {
-                cc = 0;
-                ++t;
-              }
-            }
-            *reinterpret_cast<uint4*>(d + j * WBLOCK) = *reinterpret_cast<const uint4*>(w);
+            cp16_ca(d, q, in);
           }
+          publish_behind();
         }
-        cp_commit();
-        // publish two tiles behind, so that two are in flight
-        asm volatile("cp.async.wait_group 2;\n" ::: "memory");
-        if (a >= 2) {
-          fence_async();
-          mbar_arrive(&full[(a - 2) % WSTAGES]);
-        }
+        v += 64;
+        for (x += 64; x >= W; x -= W)
+          if (++y == H) {
+            y = 0;
+            ++z;
+          }
       }
-      v += 64;
-      for (x += 64; x >= W; x -= W)
-        if (++y == H) {
-          y = 0;
-          ++z;
-        }
     }
     cp_wait_all();
     fence_async();
-    for (int i = max(0, a - 2); i < a; ++i) mbar_arrive(&full[i % WSTAGES]);
+    for (int i = max(0, a - WLAG); i < a; ++i) mbar_arrive(&full[i % ws]);
+    if (warp >= 4) goto tail;
     if (!warp_wait(&done, 0)) ok = false;
     tc_fence_after();
     float* dst = part + (size_t)blockIdx.x * 27 * C * Co;
@@ -545,8 +589,8 @@ __global__ void __launch_bounds__(160, 4) k_wgrad(const ConvSrc src, const bf16*
     // both operands MN-major (bits 15, 16)
     const uint32_t idesc = idesc_bf16(128, Co) | (1u << 15) | (1u << 16);
     for (int a = 0; a < total && ok; ++a) {
-      const int s = a % WSTAGES, kb = a / nt, ti = a - kb * nt;
-      if (!mbar_wait(&full[s], (unsigned)(a / WSTAGES) & 1u)) {
+      const int s = a % ws, kb = a / nt, ti = a - kb * nt;
+      if (!mbar_wait(&full[s], (unsigned)(a / ws) & 1u)) {
         ok = false;
         break;
       }
@@ -559,6 +603,7 @@ __global__ void __launch_bounds__(160, 4) k_wgrad(const ConvSrc src, const bf16*
     }
     mma_commit(&done);
   }
+tail:
   if (!ok) atomicOr(err, 1);
   __syncwarp();
   tc_fence_before();
@@ -641,7 +686,7 @@ static bool conv_plan(ConvPlan* p, int C, int N, int D, int H, int W) {
       if (p->smem > limit) continue;
       const int tiles = ((W + TX - 1) / TX) * ((H + TY - 1) / TY);
       int per_sm = (int)(kSmemOne / p->smem);
-      if (per_sm > 8) per_sm = 8;
+      if (per_sm > 4) per_sm = 4;   // registers
       // accumulators of the CTAs of an SM share 512 TMEM columns
       while (per_sm > 1 && per_sm * pow2_cols(2 * N) > 512) --per_sm;
       const int slots = sm_count() * per_sm;
@@ -671,17 +716,20 @@ static bool wgrad_plan(WgradPlan* p, int C, int Co, int D, int H, int W) {
   p->splits = (p->nkb + p->kbs - 1) / p->kbs;
   // tiles per CTA: all that fit into half of TMEM, fewer where that leaves SMs without a CTA
   p->tj = std::max(1, std::min(p->tiles, 256 / Co));
-  while (p->tj > 1 && p->splits * ((p->tiles + p->tj - 1) / p->tj) < 2 * sm_count()) --p->tj;
+  while (C % 16 == 0 && p->tj > 1 && p->splits * ((p->tiles + p->tj - 1) / p->tj) < 2 * sm_count()) --p->tj;
   p->jobs = (p->tiles + p->tj - 1) / p->tj;
   p->tj = (p->tiles + p->jobs - 1) / p->jobs;
-  p->cols = pow2_cols(p->tj * Co);
-  // before a tile is written, the one WSTAGES back has been multiplied; the dy buffer of a block is written with the
+  // before a tile is written, the one ws back has been multiplied; the dy buffer of a block is written with the
   // block's first tile, so the last tile of the buffer's previous block has to lie that far back: (nb - 1) tiles + 1 >=
-  // WSTAGES for the CTA with the fewest tiles per block
+  // ws for the CTA with the fewest tiles per block
   const int fewest = p->tiles - (p->jobs - 1) * p->tj;
-  p->nb = (WSTAGES - 1 + fewest - 1) / fewest + 1;
-  p->smem = WSTAGES * 16u * WBLOCK + (unsigned)p->nb * (Co / 8) * WBLOCK + 16u * p->tj * 4 + 128;
-  return p->smem <= kSmemOne && p->jobs <= 65535;
+  p->cols = pow2_cols(p->tj * Co);
+  for (p->ws = WSTAGES; p->ws > WLAG; --p->ws) {
+    p->nb = (p->ws - 1 + fewest - 1) / fewest + 1;
+    p->smem = p->ws * 16u * WBLOCK + (unsigned)p->nb * (Co / 8) * WBLOCK + 8u * p->tj * 16 + 128;
+    if (p->smem <= kSmemOne) break;
+  }
+  return p->ws > WLAG && p->jobs <= 65535;
 }
 
 template <class K>
@@ -697,6 +745,22 @@ using namespace lbmnn;
   do {                                           \
     if ((x) != cudaSuccess) return LBM_ERR_CUDA; \
   } while (0)
+
+// calls f with the narrow input's channel count as a constant
+template <class F>
+static bool by_narrow(int C, F&& f) {
+  switch (C) {
+    case 1: f(std::integral_constant<int, 1>()); return true;
+    case 2: f(std::integral_constant<int, 2>()); return true;
+    case 3: f(std::integral_constant<int, 3>()); return true;
+    case 4: f(std::integral_constant<int, 4>()); return true;
+    case 5: f(std::integral_constant<int, 5>()); return true;
+    case 6: f(std::integral_constant<int, 6>()); return true;
+    case 7: f(std::integral_constant<int, 7>()); return true;
+    case 8: f(std::integral_constant<int, 8>()); return true;
+  }
+  return false;
+}
 
 static bool conv_args_ok(const void* xa, int Ca, int up, const void* xb, int Cb, int D, int H, int W) {
   if (!xa || Ca <= 0 || Cb < 0 || (Cb > 0 && !xb) || D <= 0 || H <= 0 || W <= 0) return false;
@@ -727,6 +791,13 @@ int32_t lbm_nn_conv3_fits(int32_t Ca, int32_t up, int32_t Cb, int32_t Co) {
   return wgrad_plan(&w, C, Co, 8, 8, 8) ? 1 : 0;
 }
 
+lbm_status lbm_nn_pad8(const void* x, void* x8, int64_t V, int32_t C, void* stream) {
+  if (!x || !x8 || V <= 0 || C <= 0 || C > 8 || !aligned16({x8})) return LBM_ERR_INVALID_ARG;
+  k_pad8<<<grid_for(V), 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<const bf16*>(x), static_cast<bf16*>(x8), V, C);
+  NN_CK(cudaGetLastError());
+  return LBM_OK;
+}
+
 lbm_status lbm_nn_conv3_pack(const float* w, void* wp, void* wtp, int32_t Co, int32_t Ci, void* stream) {
   if (!w || !wp || Co <= 0 || Ci <= 0 || Co > 4096 || Ci > 4096) return LBM_ERR_INVALID_ARG;
   const long long n = lbm_nn_conv3_packed(Co, Ci) + (wtp ? lbm_nn_conv3_packed(Ci, Co) : 0);
@@ -741,7 +812,7 @@ lbm_status lbm_nn_conv3(const void* xa, int32_t Ca, int32_t up, const void* xb, 
                         const void* wp, int32_t N, const float* bias, int32_t relu, void* y0, int32_t n0, void* y1,
                         void* stream) {
   if (!conv_args_ok(xa, Ca, up, xb, Cb, D, H, W) || !wp || !y0 || N <= 0 || N % 16 || N > 256 || n0 <= 0 || n0 > N ||
-      n0 % 16 || (n0 < N && !y1) || !aligned16({Ca % 16 ? nullptr : xa, xb, wp, bias, y0, y1}))
+      n0 % 16 || (n0 < N && !y1) || !aligned16({xa, xb, wp, bias, y0, y1}))
     return LBM_ERR_INVALID_ARG;
   int* err = err_word();
   if (!err) return LBM_ERR_CUDA;
@@ -750,13 +821,19 @@ lbm_status lbm_nn_conv3(const void* xa, int32_t Ca, int32_t up, const void* xb, 
   const int tx = (W + TX - 1) / TX, ty = (H + TY - 1) / TY;
   if (Ca % 16) {
     const int k16 = (27 * Ca + 15) / 16;
-    const unsigned smem = (unsigned)k16 * 4096 + (unsigned)k16 * N * 32 + 3u * PV * Ca * 2 + 128;
-    NN_CK(allow_smem(k_conv3_first, smem));
-    const int slots = sm_count() * 4;
-    const int zs = std::max(1, std::min(D, slots / (tx * ty)));
-    const int nz = (D + zs - 1) / zs;
-    k_conv3_first<<<dim3(tx, ty, (D + nz - 1) / nz), 128, smem, st>>>(static_cast<const bf16*>(xa), static_cast<const bf16*>(wp),
-                                                                     out, Ca, N, nz, D, H, W, pow2_cols(N), err);
+    const unsigned smem = (unsigned)k16 * (4096 + N * 32) + 128;
+    if (smem > kSmemOne) return LBM_ERR_INVALID_ARG;
+    cudaError_t e = cudaSuccess;
+    by_narrow(Ca, [&](auto c) {
+      constexpr int C = decltype(c)::value;
+      e = allow_smem(k_conv3_first<C>, smem);
+      if (e != cudaSuccess) return;
+      const long long need = ((long long)D * H * W + 127) / 128;
+      const unsigned grid = (unsigned)std::min<long long>(need, sm_count() * std::max(1u, std::min(3u, kSmemOne / smem)));
+      k_conv3_first<C><<<grid, 128, smem, st>>>(static_cast<const bf16*>(xa), static_cast<const bf16*>(wp), out, N, D, H, W,
+                                               pow2_cols(N), err);
+    });
+    NN_CK(e);
   } else {
     ConvPlan p;
     if (!conv_plan(&p, Ca + Cb, N, D, H, W)) return LBM_ERR_INVALID_ARG;
@@ -777,17 +854,24 @@ int64_t lbm_nn_conv3_wgrad_scratch(int32_t D, int32_t H, int32_t W, int32_t C, i
 lbm_status lbm_nn_conv3_wgrad(const void* xa, int32_t Ca, int32_t up, const void* xb, int32_t Cb, int32_t D, int32_t H,
                               int32_t W, const void* dy, int32_t Co, float* scratch, float* dw, void* stream) {
   if (!conv_args_ok(xa, Ca, up, xb, Cb, D, H, W) || !dy || Co <= 0 || Co % 16 || !scratch || !dw ||
-      !aligned16({Ca % 16 ? nullptr : xa, xb, dy, scratch}))
+      !aligned16({xa, xb, dy, scratch}))
     return LBM_ERR_INVALID_ARG;
   WgradPlan p;
   if (!wgrad_plan(&p, Ca + Cb, Co, D, H, W)) return LBM_ERR_INVALID_ARG;
   int* err = err_word();
   if (!err) return LBM_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  NN_CK(allow_smem(k_wgrad, p.smem));
   const ConvSrc src{static_cast<const bf16*>(xa), static_cast<const bf16*>(xb), Ca, Cb, up ? 1 : 0};
-  k_wgrad<<<dim3(p.splits, p.jobs), 160, p.smem, st>>>(src, static_cast<const bf16*>(dy), scratch, p, D, H, W, err);
-  NN_CK(cudaGetLastError());
+  auto launch = [&](auto* kern) {
+    cudaError_t e = allow_smem(kern, p.smem);
+    if (e != cudaSuccess) return e;
+    kern<<<dim3(p.splits, p.jobs), 288, p.smem, st>>>(src, static_cast<const bf16*>(dy), scratch, p, D, H, W, err);
+    return cudaGetLastError();
+  };
+  cudaError_t e = cudaSuccess;
+  if (Ca % 16) by_narrow(Ca, [&](auto c) { e = launch(k_wgrad<decltype(c)::value>); });
+  else e = launch(k_wgrad<0>);
+  NN_CK(e);
   k_wgrad_sum<<<grid_for(27ll * (Ca + Cb) * Co), 256, 0, st>>>(scratch, dw, p.splits, Ca + Cb, Co);
   NN_CK(cudaGetLastError());
   return LBM_OK;

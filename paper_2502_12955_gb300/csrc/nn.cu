@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(256) k_head_fwd_16x4(const bf16* __restrict__ 
 // Head gradients: dh[v][c] = sum_o w[o][c] dy[v][o] (BF16); dw[o][c] = sum_v dy[v][o] h[v][c] and
 // db[o] = sum_v dy[v][o] (FP32: per-thread sums, a block reduction and one atomic per block and
 // entry; dw, db zeroed first).  C and Co are the head's fixed sizes.
-template <int C, int Co>
+template <int C, int Co, bool VEC>
 __global__ void __launch_bounds__(256) k_head_bwd(const bf16* __restrict__ h, const float* __restrict__ w,
                                                   const float* __restrict__ dy, bf16* __restrict__ dh,
                                                   float* __restrict__ dw, float* __restrict__ db, long long V) {
@@ -498,16 +498,40 @@ __global__ void __launch_bounds__(256) k_head_bwd(const bf16* __restrict__ h, co
   for (int i = 0; i < Co * (C + 1); ++i) acc[i] = 0.f;
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
     float g[Co], hv[C];
+    if (VEC) {
+      static_assert(Co == 4 && C % 8 == 0, "vector rows");
+      const float4 q = *reinterpret_cast<const float4*>(dy + v * Co);
+      g[0] = q.x; g[1] = q.y; g[2] = q.z; g[3] = q.w;
 #pragma unroll
-    for (int o = 0; o < Co; ++o) g[o] = dy[v * Co + o];
+      for (int c8 = 0; c8 < C / 8; ++c8) {
+        const Vec8 r = ld8(h + v * C + c8 * 8);
 #pragma unroll
-    for (int c = 0; c < C; ++c) hv[c] = __bfloat162float(h[v * C + c]);
+        for (int i = 0; i < 8; ++i) hv[c8 * 8 + i] = __bfloat162float(r.v[i]);
+      }
+    } else {
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      float s = 0.f;
+      for (int o = 0; o < Co; ++o) g[o] = dy[v * Co + o];
 #pragma unroll
-      for (int o = 0; o < Co; ++o) s = fmaf(w[o * C + c], g[o], s);
-      if (dh) dh[v * C + c] = __float2bfloat16_rn(s);
+      for (int c = 0; c < C; ++c) hv[c] = __bfloat162float(h[v * C + c]);
+    }
+    if (dh) {
+#pragma unroll
+      for (int c8 = 0; c8 < C / 8; ++c8) {
+        Vec8 r;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          float s = 0.f;
+#pragma unroll
+          for (int o = 0; o < Co; ++o) s = fmaf(__ldg(w + o * C + c8 * 8 + i), g[o], s);
+          r.v[i] = __float2bfloat16_rn(s);
+        }
+        if (VEC) {
+          *reinterpret_cast<uint4*>(dh + v * C + c8 * 8) = r.u;
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) dh[v * C + c8 * 8 + i] = r.v[i];
+        }
+      }
     }
 #pragma unroll
     for (int o = 0; o < Co; ++o) {
@@ -538,11 +562,13 @@ __global__ void __launch_bounds__(256) k_mse(const float* __restrict__ y, const 
                                              double* __restrict__ loss, long long V, int Co, double inv_n) {
   __shared__ double red[8];
   double s = 0.0;
+  const double inv2 = 2.0 * inv_n;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V * Co; i += (long long)gridDim.x * blockDim.x) {
     const long long v = i / Co;
     const float d = fluid[v] ? y[i] - t[i] : 0.f;
-    s += (double)d * d;
-    dy[i] = (float)(2.0 * d * inv_n);
+    const double dd = d;
+    s = fma(dd, dd, s);                // dd dd is exact, so this rounds as the separate product and sum
+    dy[i] = (float)(dd * inv2);        // inv2 = 2 inv_n exactly
   }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -872,7 +898,8 @@ lbm_status lbm_nn_head_bwd(const void* h, const float* w, const float* dy, void*
   NN_CK(cudaMemsetAsync(db, 0, sizeof(float) * Co, st));
   unsigned g = grid_for(V);
   if (g > 152 * 4) g = 152 * 4;
-  k_head_bwd<16, 4><<<g, 256, 0, st>>>(static_cast<const bf16*>(h), w, dy, static_cast<bf16*>(dh), dw, db, V);
+  auto* kern = vec8_ok(16, h, dy, dh) ? k_head_bwd<16, 4, true> : k_head_bwd<16, 4, false>;
+  kern<<<g, 256, 0, st>>>(static_cast<const bf16*>(h), w, dy, static_cast<bf16*>(dh), dw, db, V);
   NN_CK(cudaGetLastError());
   return LBM_OK;
 }

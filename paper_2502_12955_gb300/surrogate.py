@@ -70,6 +70,7 @@ def nn_lib():
         "lbm_nn_conv3": [vp, i32, i32, vp, i32, i32, i32, i32, vp, i32, vp, i32, vp, i32, vp, vp],
         "lbm_nn_conv3_wgrad": [vp, i32, i32, vp, i32, i32, i32, i32, vp, i32, vp, vp, vp],
         "lbm_nn_conv3_pack": [vp, vp, vp, i32, i32, vp],
+        "lbm_nn_pad8": [vp, vp, i64, i32, vp],
     }
     for name, args in sig.items():
         fn = getattr(lib, name)
@@ -204,6 +205,10 @@ def lbm_nn_conv3_wgrad(src, shape, dy, Co, scratch, dw):
 
 def lbm_nn_conv3_wgrad_scratch(shape, Cc, Co):
     return int(nn_lib().lbm_nn_conv3_wgrad_scratch(*shape, Cc, Co))
+
+
+def lbm_nn_pad8(x, x8, V, Cc):
+    _call("lbm_nn_pad8", _p(x), _p(x8), V, Cc)
 
 
 def lbm_nn_conv3_pack(w, wp, wtp, Co, Ci):
@@ -427,6 +432,9 @@ class WarmStartNet:
         # per layer: its input, its output and the sizes
         acts = {}
         h, shp, c = x, tuple(shape), self.c_in
+        if not self.rows["enc0a"] and c <= 8:   # the narrow input, in rows of 8 channels
+            h = self._empty(shp[0] * shp[1] * shp[2], 8)
+            lbm_nn_pad8(x, h, h.shape[0], c)
         skips = []
         for l, wd in enumerate(self.width[:-1]):
             for s in "ab":

@@ -20,6 +20,12 @@ def _rand(shape, seed, dtype=torch.bfloat16):
     return torch.randn(shape, generator=g).to(dtype).cuda()
 
 
+def _padded(x):
+    x8 = torch.empty((x.shape[0], 8), dtype=torch.bfloat16, device="cuda")
+    sg.lbm_nn_pad8(x, x8, x.shape[0], x.shape[1])
+    return x8
+
+
 # shapes (D, H, W): a partial tile along x and y, several z ranges per column, one plane, whole tiles
 SHAPES = [(6, 16, 12), (16, 8, 8), (1, 16, 40), (40, 32, 16), (2, 20, 48)]
 LAYERS = [(5, 0, 0, 16), (4, 0, 0, 48), (16, 0, 0, 16), (32, 0, 0, 32), (48, 0, 0, 64), (64, 0, 0, 224), (160, 0, 0, 160),
@@ -51,6 +57,8 @@ def test_conv3_repeats_the_im2col_gemm(shape, ca, up, cb, co):
     sg.lbm_nn_im2col(x, col, D, H, W, C, kp, 0)
     want = torch.empty((V, co), dtype=torch.bfloat16, device="cuda")
     sg.lbm_nn_gemm_tn(col, wk, want, co, V, co, kp, 1, sg.OUT_BF16_RELU, bias)
+    if ca <= 8:
+        xa = _padded(xa)
     # implicit, with the columns split over two outputs where there are several 16s
     wp = torch.empty(sg.lbm_nn_conv3_packed(co, C), dtype=torch.bfloat16, device="cuda")
     sg.lbm_nn_conv3_pack(w, wp, None, co, C)
@@ -88,6 +96,8 @@ def test_conv3_wgrad_repeats_the_split_gemm(shape, ca, up, cb, co):
     sg.lbm_nn_reduce_splits(part, rows, kp * co, splits, kp * co)
     want = torch.empty((co, C, 27), dtype=torch.float32, device="cuda")
     sg.lbm_nn_unpack_wgrad(rows, want, co, C)
+    if ca <= 8:
+        xa = _padded(xa)
     scratch = torch.empty(sg.lbm_nn_conv3_wgrad_scratch(shape, C, co), dtype=torch.float32, device="cuda")
     dw = torch.full((co, C, 27), float("nan"), dtype=torch.float32, device="cuda")
     sg.lbm_nn_conv3_wgrad((xa, ca, up, xb, cb), shape, dy, co, scratch, dw)
