@@ -270,7 +270,9 @@ void fill_args(lbm_ctx* c) {
     // the step kernel walks the fluid list: the block shape is not tied to nx.  256 threads, fewer on a domain
     // whose blocks of that size would not reach every SM (152 on this GPU): 128 x 64 nodes in FP64 take
     // 15.1 us per step as 32 blocks of 256 and 9.8 us as 128 blocks of 64 (16.0 us as 256 blocks of 32)
-    bx = 256;
+    // FP64 arithmetic: 64 threads at every size.  Those kernels are bound by the FP64 units, and small blocks
+    // share them out more evenly in the last wave (64^3 dissolution: 103.3 us per step with 256, 87.5 us with 64).
+    bx = p.precision == LBM_FP64 ? 64 : 256;
     while (bx > 64 && (c->N + bx - 1) / bx < 152) bx /= 2;
   }
   a.bx = bx;
