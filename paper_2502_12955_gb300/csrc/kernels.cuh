@@ -1239,8 +1239,18 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   if (a.geo_mode != GEO_NONE) pdl_wait();
   const unsigned int count = a.fluid_count[0];
   const unsigned int base = a.fluid_count[1];   // entries below it have slot == entry
-  const unsigned int stride = gridDim.x * blockDim.x;
+  // Block rounds over the list, forwards or backwards.  Each kernel that reads the populations starts where its
+  // predecessor ended, so that the populations L2 still holds are read there: odd steps go backwards, and
+  // after a psi pass (always forwards) so does every step.
+  const bool back = parity == 1 || a.sc_on;
+  unsigned int stride = gridDim.x * blockDim.x;
   unsigned int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (back) {
+    // whole blocks from the list's end; below its start e and e + stride wrap past count
+    e = ((count + blockDim.x - 1) / blockDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
+    stride = 0u - stride;
+    if (e >= count) e += stride;   // the last block's threads past the end
+  }
   const auto cell = [&](unsigned int en, int n) { return R::cell(en < base ? (long long)en : (long long)__ldg(a.slot + n)); };
   // the list entry is fetched two iterations and the link mask one iteration ahead
   uint32_t w_cur = e < count ? a.fluid_list[e] : 0u;
@@ -1371,9 +1381,11 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   bool have_next = false, waited = false;
   uint32_t w_pf = 0u, m_pf = 0u;
   unsigned int staged = 0xffffffffu;
+  // odd steps take the tiles backwards, from those whose populations L2 still holds (see k_step)
+  const auto tile_at = [&](unsigned int t) { return tiles[parity ? ntiles - 1 - t : t]; };
   pdl_trigger();
   for (unsigned int t = blockIdx.x * chunk; t < ntiles; t = next_tile(t)) {
-    const Tile tile = tiles[t];
+    const Tile tile = tile_at(t);
     if (tile.member != staged) {   // block-uniform
       __syncthreads();   // the previous member's tiles are done with sa / sk
       const uint32_t* src = reinterpret_cast<const uint32_t*>(args + tile.member);
@@ -1409,7 +1421,7 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
     bool next_in = false;
     const unsigned int tn = next_tile(t);
     if (tn < ntiles) {
-      const Tile tile2 = tiles[tn];
+      const Tile tile2 = tile_at(tn);
       if (tile2.member == staged) {
         const unsigned int e2 = tile2.first + threadIdx.x;
         w_pf = 0u;
