@@ -1492,13 +1492,19 @@ lbm_status lbm_ensemble_run_to_steady(lbm_ensemble* e, double r_tol, int64_t max
     if (st != LBM_OK) return st;
     done += chunk;
     if ((ens_step_of(e) % Nm) != 0) continue;
-    // per-member exit: a member whose residual reached the tolerance stops stepping
+    // per-member exit: a member whose residual reached the tolerance stops stepping.  The step that ended the
+    // interval has evaluated it: four sums per member, read together behind one wait
     for (size_t k = 0; k < e->m.size(); ++k) {
+      lbm_ctx* c = e->m[k];
       if (!e->active[k]) continue;
-      lbm_monitors mon;
-      st = lbm_get_monitors(e->m[k], &mon);
-      if (st != LBM_OK) return efail(e, st, "member %zu: %s", k, e->m[k]->err.c_str());
-      if (mon.residual >= 0.0 && mon.residual <= r_tol) {
+      ECK(cudaMemcpyAsync(c->mon_host + NMON, c->a.mon_out + NMON, 32, cudaMemcpyDeviceToHost, c->stream));
+    }
+    for (size_t k = 0; k < e->m.size(); ++k) {
+      lbm_ctx* c = e->m[k];
+      if (!e->active[k]) continue;
+      ECK(cudaStreamSynchronize(c->stream));
+      const double r = c->res_evals >= 2 ? residual_from(c->mon_host + NMON) : -1.0;
+      if (r >= 0.0 && r <= r_tol) {
         e->active[k] = 0;
         e->dirty = true;
       }
