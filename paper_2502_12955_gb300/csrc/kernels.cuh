@@ -1577,12 +1577,12 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[K], unsigned int 
 // (deviations from the reference, so the sums stay accurate), bookkeeping sums over all nodes
 // in FP64, per-block partials in FP64 (summed in fixed order by k_reduce_partials).
 template <class L, class S, int NC, int NS>
-__global__ void __launch_bounds__(256) k_monitor(const Args a, const Coef<typename Store<S>::T> k,
-                                                 const int parity) {
+__device__ __forceinline__ void monitor_block(const Args& a, const Coef<typename Store<S>::T>& k, const int parity,
+                                              const unsigned int block, const unsigned int blocks) {
   using T = typename Store<S>::T;
   constexpr int Q = L::Q, QC = L::QC;
-  const unsigned int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned int nthr = gridDim.x * blockDim.x;
+  const unsigned int tid = block * blockDim.x + threadIdx.x;
+  const unsigned int nthr = blocks * blockDim.x;
   T dm[NC > 0 ? NC : 1], mom[3] = {T(0), T(0), T(0)}, dsp[NS > 0 ? NS : 1];
 #pragma unroll
   for (int s = 0; s < NC; ++s) dm[s] = T(0);
@@ -1679,7 +1679,12 @@ __global__ void __launch_bounds__(256) k_monitor(const Args a, const Coef<typena
   }
   if (NS > 1) used |= 1u << M_HEAT | 1u << M_PROD;
   if (a.conjugate) used |= 1u << M_TSOLID | 1u << M_HEAT_S | 1u << M_HEAT_SRC;
-  block_reduce_store<NMON>(v, used, a.partials + (long long)blockIdx.x * NMON);
+  block_reduce_store<NMON>(v, used, a.partials + (long long)block * NMON);
+}
+
+template <class L, class S, int NC, int NS>
+__global__ void __launch_bounds__(256) k_monitor(const Args a, const Coef<typename Store<S>::T> k, const int parity) {
+  monitor_block<L, S, NC, NS>(a, k, parity, blockIdx.x, gridDim.x);
 }
 
 // ================================================================ node macroscopics
@@ -1810,14 +1815,14 @@ __global__ void __launch_bounds__(256) k_moments(const Args a, const Coef<typena
 // at the nodes' storage slots, which are replaced: sum (u - u_s)^2, sum u^2, sum (C - C_s)^2,
 // sum C^2.  (A re-slotting invalidates the snapshots; the runtime then skips one evaluation.)
 template <class L, class S, int NC, int NS>
-__global__ void __launch_bounds__(256) k_resid(const Args a, const Coef<typename Store<S>::T> k,
-                                               const int parity) {
+__device__ __forceinline__ void resid_block(const Args& a, const Coef<typename Store<S>::T>& k, const int parity,
+                                            const unsigned int block, const unsigned int blocks) {
   using T = typename Store<S>::T;
   T* snap = reinterpret_cast<T*>(a.snap);
   const long long P = a.pitch;
   T du = T(0), uu = T(0), dc = T(0), cc = T(0);
   const unsigned int count = a.fluid_count[0], base = a.fluid_count[1];
-  for (unsigned int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) {
+  for (unsigned int e = block * blockDim.x + threadIdx.x; e < count; e += blocks * blockDim.x) {
     const uint32_t w = a.fluid_list[e];
     const int n = list_node(a, w);
     const uint32_t m = a.mask[n];
@@ -1839,7 +1844,36 @@ __global__ void __launch_bounds__(256) k_resid(const Args a, const Coef<typename
     }
   }
   double v[4] = {double(du), double(uu), double(dc), double(cc)};
-  block_reduce_store<4>(v, 15u, a.partials + (long long)blockIdx.x * 4);
+  block_reduce_store<4>(v, 15u, a.partials + (long long)block * 4);
+}
+
+template <class L, class S, int NC, int NS>
+__global__ void __launch_bounds__(256) k_resid(const Args a, const Coef<typename Store<S>::T> k, const int parity) {
+  resid_block<L, S, NC, NS>(a, k, parity, blockIdx.x, gridDim.x);
+}
+
+// One block of an evaluation of every member of an ensemble: `block` of `blocks` of its member.
+struct EvalBlock {
+  unsigned int member, block, blocks;
+};
+
+// Monitors or residual partials of all members in one launch, each block as k_monitor's or k_resid's of its
+// member.  Launched member by member they are bound by latency: 15 us for the monitors of any small member.
+template <class L, class S, int NC, int NS>
+__global__ void __launch_bounds__(256) k_eval_members(const Args* __restrict__ args,
+                                                      const Coef<typename Store<S>::T>* __restrict__ coefs,
+                                                      const EvalBlock* __restrict__ list, const int resid,
+                                                      const int parity) {
+  __shared__ Args sa;
+  __shared__ Coef<typename Store<S>::T> sk;
+  const EvalBlock b = list[blockIdx.x];
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(args + b.member);
+  for (unsigned int i = threadIdx.x; i < sizeof(Args) / 4; i += blockDim.x) reinterpret_cast<uint32_t*>(&sa)[i] = src[i];
+  const uint32_t* ksrc = reinterpret_cast<const uint32_t*>(coefs + b.member);
+  for (unsigned int i = threadIdx.x; i < sizeof(sk) / 4; i += blockDim.x) reinterpret_cast<uint32_t*>(&sk)[i] = ksrc[i];
+  __syncthreads();
+  if (resid) resid_block<L, S, NC, NS>(sa, sk, parity, b.block, b.blocks);
+  else monitor_block<L, S, NC, NS>(sa, sk, parity, b.block, b.blocks);
 }
 
 // ================================================================ init / pop I/O

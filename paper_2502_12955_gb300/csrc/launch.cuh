@@ -30,6 +30,8 @@ struct KernelSet {
   void (*coefs)(const Args* a, int n, void* out);
   cudaError_t (*step_tiles)(const Args* d_args, const void* d_coefs, const Tile* d_tiles, unsigned int ntiles,
                             int n_comp, int n_scal, int coll, int parity, int bnd, int threads, cudaStream_t);
+  cudaError_t (*eval_members)(const Args* d_args, const void* d_coefs, const EvalBlock* d_list, unsigned int blocks,
+                              const Args& kind, int resid, int parity, cudaStream_t);
   long long (*rec_bytes)(const Args&);   // bytes per tile of kTile slots of all populations
   int psi_bytes;   // bytes per psi element (compute type)
   int coef_bytes;
@@ -277,6 +279,16 @@ struct Launchers {
     return cudaGetLastError();
   }
 
+  // kind: any member's arguments (the lattice counts)
+  static cudaError_t eval_members(const Args* d_args, const void* d_coefs, const EvalBlock* d_list, unsigned int blocks,
+                                  const Args& kind, int resid, int parity, cudaStream_t st) {
+    by_nc_ns(kind, [&](auto nc, auto ns) {
+      k_eval_members<L, S, decltype(nc)::value, decltype(ns)::value>
+          <<<blocks, 256, 0, st>>>(d_args, static_cast<const Coef<T>*>(d_coefs), d_list, resid, parity);
+    });
+    return cudaGetLastError();
+  }
+
   static cudaError_t init(const Args& a, cudaStream_t st) {
     const unsigned int nb = (unsigned int)((a.N + 255) / 256);
     by_nc_ns(a, [&](auto nc, auto ns) {
@@ -405,6 +417,7 @@ struct Launchers {
     KernelSet k;
     k.coefs = &coefs;
     k.step_tiles = &step_tiles;
+    k.eval_members = &eval_members;
     k.coef_bytes = (int)sizeof(Coef<T>);
     k.step = &step;
     k.rec_bytes = &rec_bytes;

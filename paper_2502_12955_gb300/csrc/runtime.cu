@@ -404,10 +404,8 @@ namespace lbm {
 
 // Fixed-order sum of the per-block partials (deterministic): a warp per row of K values (K <= 32), 32 rows at a time,
 // then one pass over the warps.
-__global__ void __launch_bounds__(1024) k_reduce_partials(const double* __restrict__ partials,
-                                                          long long nblocks, int K,
-                                                          double* __restrict__ out, int* err,
-                                                          int nonfin_slot) {
+__device__ __forceinline__ void reduce_partials(const double* __restrict__ partials, long long nblocks, int K,
+                                                double* __restrict__ out, int* err, int nonfin_slot) {
   __shared__ double sh[32][33];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double acc = 0.0;
@@ -427,6 +425,21 @@ __global__ void __launch_bounds__(1024) k_reduce_partials(const double* __restri
   }
 }
 
+__global__ void __launch_bounds__(1024) k_reduce_partials(const double* __restrict__ partials,
+                                                          long long nblocks, int K,
+                                                          double* __restrict__ out, int* err,
+                                                          int nonfin_slot) {
+  reduce_partials(partials, nblocks, K, out, err, nonfin_slot);
+}
+
+// The same for every member of an ensemble, a block each.
+__global__ void __launch_bounds__(1024) k_reduce_members(const Args* __restrict__ args, const EvalBlock* __restrict__ heads,
+                                                         const int resid) {
+  const EvalBlock b = heads[blockIdx.x];
+  const Args& a = args[b.member];
+  reduce_partials(a.partials, b.blocks, resid ? 4 : NMON, a.mon_out + (resid ? NMON : 0), a.err, resid ? -1 : M_NONFIN);
+}
+
 cudaError_t launch_reduce(const double* partials, long long nblocks, int K, double* out, int* err,
                           int nonfin_slot, cudaStream_t st) {
   if (K > 32) return cudaErrorInvalidValue;
@@ -434,7 +447,9 @@ cudaError_t launch_reduce(const double* partials, long long nblocks, int K, doub
   return cudaGetLastError();
 }
 
-// Dissolution test (V_m acc >= m_s0) over the interface list.
+// Dissolution test (V_m acc >= m_s0) over the interface list.  Bound by DRAM sectors: 8 bytes of each 64 that a
+// listed node's total brings in (256^3 packing: 1.49 M nodes in 18 us, the same with four nodes per thread in flight
+// and with the list walked from the end the step left in L2).
 __global__ void __launch_bounds__(256) k_detect(const Args a) {
   pdl_trigger();
   pdl_wait();
@@ -1224,6 +1239,9 @@ struct lbm_ensemble {
   Tile* d_tiles = nullptr;
   size_t tile_cap = 0;
   unsigned int ntiles = 0;
+  EvalBlock* d_eval = nullptr;   // blocks of an evaluation of the active members, then one head entry per member
+  size_t eval_cap = 0;
+  unsigned int neval = 0, nheads = 0;
   bool dirty = true;
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t pair = nullptr;
@@ -1281,6 +1299,16 @@ lbm_status ens_prepare(lbm_ensemble* e) {
     if (!e->active[k]) continue;
     for (unsigned int f = 0; f < counts[k]; f += (unsigned int)e->threads) tiles.push_back(Tile{(unsigned int)k, f});
   }
+  std::vector<EvalBlock> eval, heads;
+  for (int k = 0; k < n; ++k) {
+    if (!e->active[k]) continue;
+    const unsigned int blocks = reduce_blocks(args[k]);
+    for (unsigned int b = 0; b < blocks; ++b) eval.push_back(EvalBlock{(unsigned int)k, b, blocks});
+    heads.push_back(EvalBlock{(unsigned int)k, 0u, blocks});
+  }
+  e->neval = (unsigned int)eval.size();
+  e->nheads = (unsigned int)heads.size();
+  eval.insert(eval.end(), heads.begin(), heads.end());
   std::vector<char> coefs((size_t)n * e->ks->coef_bytes);
   e->ks->coefs(args.data(), n, coefs.data());
   if (!e->d_args) {
@@ -1293,6 +1321,15 @@ lbm_status ens_prepare(lbm_ensemble* e) {
     ECK(cudaMalloc(&e->d_tiles, std::max<size_t>(1, tiles.size()) * sizeof(Tile)));
     e->tile_cap = tiles.size();
   }
+  if (eval.size() > e->eval_cap) {
+    if (e->d_eval) cudaFree(e->d_eval);
+    e->d_eval = nullptr;
+    e->eval_cap = 0;
+    ECK(cudaMalloc(&e->d_eval, eval.size() * sizeof(EvalBlock)));
+    e->eval_cap = eval.size();
+  }
+  if (!eval.empty())
+    ECK(cudaMemcpyAsync(e->d_eval, eval.data(), eval.size() * sizeof(EvalBlock), cudaMemcpyHostToDevice, e->stream));
   ECK(cudaMemcpyAsync(e->d_args, args.data(), n * sizeof(Args), cudaMemcpyHostToDevice, e->stream));
   ECK(cudaMemcpyAsync(e->d_coefs, coefs.data(), coefs.size(), cudaMemcpyHostToDevice, e->stream));
   if (!tiles.empty())
@@ -1318,19 +1355,50 @@ lbm_status ens_launch(lbm_ensemble* e, int parity, cudaStream_t st) {
   return LBM_OK;
 }
 
+long long ens_step_of(const lbm_ensemble* e) {
+  for (size_t k = 0; k < e->m.size(); ++k)
+    if (e->active[k]) return e->m[k]->step;
+  return 0;
+}
+
+// The monitors and the residual of every active member in four launches on the members' common stream.
+lbm_status ens_evaluate(lbm_ensemble* e, int parity) {
+  const Args& kind = e->m[0]->a;
+  for (int resid = 0; resid < 2; ++resid) {
+    ECK(e->ks->eval_members(e->d_args, e->d_coefs, e->d_eval, e->neval, kind, resid, parity, e->stream));
+    k_reduce_members<<<e->nheads, 1024, 0, e->stream>>>(e->d_args, e->d_eval + e->neval, resid);
+    ECK(cudaGetLastError());
+    e->launches += 2;
+  }
+  return LBM_OK;
+}
+
 // after a step: the members' counters, and their monitors when due
 lbm_status ens_after_step(lbm_ensemble* e) {
+  const auto due = [](const lbm_ctx* c) { return c->p.N_mon > 0 && (c->step % c->p.N_mon) == 0; };
+  size_t n_due = 0, n_active = 0;
   for (size_t k = 0; k < e->m.size(); ++k) {
     if (!e->active[k]) continue;
+    e->m[k]->step += 1;
+    n_active += 1;
+    n_due += due(e->m[k]) ? 1 : 0;
+  }
+  if (n_due == 0) return LBM_OK;
+  const bool together = n_due == n_active;   // members with other intervals are evaluated one by one
+  if (together) {
+    lbm_status st = ens_evaluate(e, parity_of(ens_step_of(e)));
+    if (st != LBM_OK) return st;
+  }
+  for (size_t k = 0; k < e->m.size(); ++k) {
     lbm_ctx* c = e->m[k];
-    c->step += 1;
-    if (c->p.N_mon > 0 && (c->step % c->p.N_mon) == 0) {
+    if (!e->active[k] || !due(c)) continue;
+    if (!together) {
       lbm_status st = run_monitor(c);
       if (st == LBM_OK) st = run_residual(c);
       if (st != LBM_OK) return efail(e, st, "member %zu: %s", k, c->err.c_str());
-      c->have_snap = true;
-      c->res_evals += 1;
     }
+    c->have_snap = true;
+    c->res_evals += 1;
   }
   return LBM_OK;
 }
@@ -1342,12 +1410,6 @@ bool ens_plain_pair(const lbm_ensemble* e, long long step) {
     if (Nm > 0 && ((step + 1) % Nm == 0 || (step + 2) % Nm == 0)) return false;
   }
   return true;
-}
-
-long long ens_step_of(const lbm_ensemble* e) {
-  for (size_t k = 0; k < e->m.size(); ++k)
-    if (e->active[k]) return e->m[k]->step;
-  return 0;
 }
 
 }  // namespace
