@@ -624,6 +624,9 @@ __device__ __forceinline__ T warp_sum(T v) {
 #ifndef LBM_STEP_MIN_BLOCKS_ODD
 #define LBM_STEP_MIN_BLOCKS_ODD 3   // k_step's odd parity: the slot prefetch hides the lookups, registers pay
 #endif
+#ifndef LBM_TILES_MIN_BLOCKS_2D
+#define LBM_TILES_MIN_BLOCKS_2D 4   // k_step_tiles in 2D (64 registers; 3 / 4 / 5 blocks: 22.6 / 18.5 / 20.6 us, spills at 5)
+#endif
 #ifndef LBM_TILES_MIN_BLOCKS_ODD
 #define LBM_TILES_MIN_BLOCKS_ODD 3  // k_step_tiles: odd parity, slots prefetched a tile ahead (as k_step)
 #endif
@@ -1356,7 +1359,7 @@ struct Tile {
 // arguments and constants in shared memory, and for each tile it updates entries first ..
 // first + blockDim - 1 exactly as k_step updates them.
 template <class L, class S, int NC, int NS, int COLL, int parity, bool BND>
-__global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) == 4 ? (parity ? LBM_TILES_MIN_BLOCKS_ODD : LBM_STEP_MIN_BLOCKS) : 2)) k_step_tiles(
+__global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) == 4 ? (L::D == 2 ? LBM_TILES_MIN_BLOCKS_2D : (parity ? LBM_TILES_MIN_BLOCKS_ODD : LBM_STEP_MIN_BLOCKS)) : 2)) k_step_tiles(
     const Args* __restrict__ args, const Coef<typename Store<S>::T>* __restrict__ coefs,
     const Tile* __restrict__ tiles, unsigned int ntiles, unsigned int chunk) {
   using T = typename Store<S>::T;

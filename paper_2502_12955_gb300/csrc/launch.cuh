@@ -377,8 +377,10 @@ struct Launchers {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step_tiles<L, S, NC, NS, COLL, PAR, BND>, threads, smem);
     const unsigned int wave = (unsigned int)((occ > 0 ? occ : 1) * (sms > 0 ? sms : 1));
     const unsigned int blocks = ntiles < wave ? (ntiles > 0 ? ntiles : 1) : wave;
-    // consecutive tiles per turn: whole chunks for every block first, LBM_TILE_CHUNK at most
-    unsigned int chunk = ntiles / blocks;
+    // consecutive tiles per turn: about eight turns for every block, LBM_TILE_CHUNK tiles at most.  Fewer turns
+    // leave the last one uneven: six 3D members (27 tiles per block) take 222 us per step in chunks of 8 and 212 us in
+    // chunks of 2, twelve 2D members (7 tiles per block) 18.5 us in chunks of 8 and 16.5 us in chunks of 1
+    unsigned int chunk = ntiles / (8 * blocks);
     chunk = chunk < 1 ? 1 : (chunk > LBM_TILE_CHUNK ? LBM_TILE_CHUNK : chunk);
     return launch_pdl(kEarly, k_step_tiles<L, S, NC, NS, COLL, PAR, BND>, blocks, threads, smem, st, d_args,
                       static_cast<const Coef<T>*>(d_coefs), d_tiles, ntiles, chunk);
