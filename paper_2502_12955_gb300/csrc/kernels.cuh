@@ -187,6 +187,7 @@ struct Args {
   // conduction in the solid (with arrhenius): the solid thermal lattice in two compute-type
   // buffers [QC][N] by node (full values); step t reads gs[t & 1] and writes gs[(t + 1) & 1]
   int conjugate;
+  unsigned int solid_blocks;   // blocks at the end of a step launch that advance the solid lattice
   double tau_s, c_fs;
   void* gs[2];
   void* kb;                  // compute-type [QC - 1][N]: k(T_b) of the link arriving in
@@ -1227,6 +1228,9 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
   }
 }
 
+template <class L, class S>
+__device__ __forceinline__ void solid_nodes(const Args& a, const Coef<typename Store<S>::T>& k, int parity, unsigned int block, unsigned int blocks);
+
 // One fused time step for every fluid node: gather (A-A parity), wet-node closure and its
 // bookkeeping, deposition, moments, forces, velocity, flow collision (BGK / MRT, Guo or
 // velocity shift), scalar collision, in-place scatter with bounce-back / inlet / outlet.
@@ -1239,6 +1243,17 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   using O = OddCells<L, S, NC, NS, LBM_STEP_CACHE_STRIDE, BND>;
   T wallx = T(0), heatx = T(0), prodx = T(0);
   pdl_trigger();
+  unsigned int blocks = gridDim.x;
+  if constexpr (BND && NS > 1) {
+    // conduction in the solid: the last blocks advance the solid lattice, of which the fluid's step reads the old state
+    // only.  A launch of its own adds its latency to every step (420 x 80: 4.8 us beside a step of 8).
+    blocks -= a.solid_blocks;
+    if (blockIdx.x >= blocks) {
+      pdl_wait();
+      solid_nodes<L, S>(a, k, parity, blockIdx.x - blocks, a.solid_blocks);
+      return;
+    }
+  }
   if (a.geo_mode != GEO_NONE) pdl_wait();
   const unsigned int count = a.fluid_count[0];
   const unsigned int base = a.fluid_count[1];   // entries below it have slot == entry
@@ -1246,7 +1261,7 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   // predecessor ended, so that the populations L2 still holds are read there: odd steps go backwards, and
   // after a psi pass (always forwards) so does every step.
   const bool back = parity == 1 || a.sc_on;
-  unsigned int stride = gridDim.x * blockDim.x;
+  unsigned int stride = blocks * blockDim.x;
   unsigned int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (back) {
     // whole blocks from the list's end; below its start e and e + stride wrap past count
@@ -2518,18 +2533,15 @@ __global__ void __cluster_dims__(kFlipBlocks, 1, 1) __launch_bounds__(kFlipThrea
 // the node as the arriving population of the opposite direction: at a closed face that is the
 // reflection, at a fluid neighbour it is the solid side of the link that k_exchange replaces.
 template <class L, class S>
-__global__ void __launch_bounds__(256) k_solid(const Args a, const Coef<typename Store<S>::T> k,
-                                               const int parity) {
+__device__ __forceinline__ void solid_nodes(const Args& a, const Coef<typename Store<S>::T>& k, const int parity, const unsigned int block,
+                            const unsigned int blocks) {
   using T = typename Store<S>::T;
   constexpr int QC = L::QC;
-  pdl_trigger();
-  pdl_wait();
   const T* gin = reinterpret_cast<const T*>(a.gs[parity]);
   T* gout = reinterpret_cast<T*>(a.gs[parity ^ 1]);
   const int perc[3] = {a.open_x ? 0 : a.per[0], a.per[1], a.per[2]};
   const long long N = a.N;
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
-       n += (long long)gridDim.x * blockDim.x) {
+  for (long long n = block * (long long)blockDim.x + threadIdx.x; n < N; n += (long long)blocks * blockDim.x) {
     if (a.flags[n] == FL_FLUID) continue;
     T g[QC];
     T Ts = T(0);
@@ -2558,7 +2570,7 @@ __global__ void __launch_bounds__(256) k_solid(const Args a, const Coef<typename
 // reacRate), after the fluid step and the solid lattice's streaming.  For fluid node n and a
 // direction j toward a solid node s = n + c_j (arriving direction i = opp(j)): the fluid
 // population ho = h*_T,j that left n toward s (kept at n by the bounce-back of the step, in plane
-// i) and the solid population go = g*_s,i that left s toward n (kept at s in plane j by k_solid)
+// i) and the solid population go = g*_s,i that left s toward n (kept at s in plane j by solid_nodes)
 // meet at one interface temperature T_b.  Each side receives 2 w T_b minus what it sent, and the
 // link's energy in units of the fluid's rho c_p grows by the reaction heat Qp:
 //     T_b = (c_fs ho + go + c_fs Qp / 2) / (w (c_fs + 1)).

@@ -22,7 +22,6 @@ struct KernelSet {
   cudaError_t (*resid)(const Args&, int parity, cudaStream_t, long long* nblocks);
   // conduction in the solid: the solid lattice's step, the link exchange after the fluid step
   // (parity of the next step), and the solid's initial state from the staged fields
-  cudaError_t (*solid)(const Args&, int parity, cudaStream_t);
   cudaError_t (*exchange)(const Args&, int parity_next, cudaStream_t);
   cudaError_t (*solid_init)(const Args&, cudaStream_t);
   // ensembles: compute-type constants of n members into host memory (coef_bytes each), and one
@@ -169,8 +168,11 @@ struct Launchers {
       cached_threads = threads;
     }
     long long need = (a.N + threads - 1) / threads;
-    const unsigned int blocks = (unsigned int)(need < cached_blocks ? need : cached_blocks);
-    return launch_pdl(kEarly, k_step<L, S, NC, NS, COLL, PAR, BND>, blocks > 0 ? blocks : 1, threads, 0, st, a, coef(a));
+    unsigned int blocks = (unsigned int)(need < cached_blocks ? need : cached_blocks);
+    if (blocks == 0) blocks = 1;
+    Args b = a;
+    if (BND && NS > 1 && a.conjugate) blocks += b.solid_blocks = box_blocks(a);   // behind the step's own blocks
+    return launch_pdl(kEarly, k_step<L, S, NC, NS, COLL, PAR, BND>, blocks, threads, 0, st, b, coef(a));
   }
   // BND: a moving plate, a velocity inlet or the temperature-dependent reaction needs the full
   // variant of the step kernel, and so does a domain too large for the plain variant's 32-bit
@@ -314,14 +316,11 @@ struct Launchers {
     return e;
   }
 
-  // grid-stride kernels over the box (k_solid) and the fluid list (k_exchange): two waves of
+  // grid-stride kernels over the box (solid_nodes) and the fluid list (k_exchange): two waves of
   // blocks, fewer on a small domain
   static unsigned int box_blocks(const Args& a, int per_node = 1) {
     const long long need = (a.N * per_node + a.bx - 1) / a.bx, cap = 2ll * wave_blocks() * 256 / a.bx;
     return (unsigned int)(need < cap ? (need > 0 ? need : 1) : cap);
-  }
-  static cudaError_t solid(const Args& a, int parity, cudaStream_t st) {
-    return launch_pdl(kEarly, k_solid<L, S>, box_blocks(a), a.bx, 0, st, a, coef(a), parity);
   }
   static cudaError_t exchange(const Args& a, int parity_next, cudaStream_t st) {
     // conduction in the solid needs the species and the temperature: two or three scalar lattices
@@ -432,7 +431,6 @@ struct Launchers {
     k.masks = &masks;
     k.lists = &lists;
     k.resid = &resid;
-    k.solid = &solid;
     k.exchange = &exchange;
     k.solid_init = &solid_init;
     k.psi_bytes = (int)sizeof(typename Store<S>::T);

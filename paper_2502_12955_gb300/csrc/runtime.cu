@@ -745,8 +745,7 @@ lbm_status enqueue_step(lbm_ctx* c, long long step, cudaStream_t st, bool timed)
   if (c->a.sc_on) LAUNCH(c->ks->psi(c->a, par, st));
   LAUNCH(c->ks->step(c->a, par, c->p.collision, st));
   if (c->p.conjugate) {
-    // conduction in the solid: the solid lattice's step, then the exchange across its links
-    LAUNCH(c->ks->solid(c->a, par, st));
+    // conduction in the solid: the step has advanced the solid lattice too; the exchange across its links
     LAUNCH(c->ks->exchange(c->a, par ^ 1, st));
   }
   if (timed) {
