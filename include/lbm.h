@@ -102,7 +102,8 @@ typedef struct lbm_params {
   double rho_ref[2];          /* storage shift references for 16-bit modes (flow) */
   double C_ref[2];            /* storage shift references for 16-bit modes (scalars) */
   void* stream;               /* cudaStream_t for all work of this context */
-  int32_t block_x;            /* threads per block of the step kernel: 0 (automatic: 256) or a
+  int32_t block_x;            /* threads per block of the step kernel: 0 (automatic: 64 in FP64, else 256, and
+                                 128 or 64 on domains whose blocks would not reach every SM) or a
                                  multiple of 32 up to 256 */
   int32_t device;             /* CUDA device ordinal */
   int32_t l2_fetch_bytes;     /* L2 fetch granularity hint for this process's context
@@ -199,8 +200,8 @@ lbm_status lbm_params_default(lbm_params* p);
 
 /* Allocate a context for an nx x ny x nz domain (Sec. 2.1.4 lattices).  Validates every
    parameter (tau > 0.5, n_comp, n_scal, J0, MRT only with one component and Guo forcing,
-   nz == 1 for 2D, nx >= 2 with ade_open_x).  Device memory: populations in SoA planes
-   pop[q][n], one in-place copy per lattice, plus flags, link masks and FP64 bookkeeping.
+   nz == 1 for 2D, nx >= 2 with ade_open_x).  Device memory: two buffers of populations in tiles of 32 or 64
+   nodes (one holds the live in-place copy), flags, link masks and FP64 bookkeeping.
    *out is NULL on error; lbm_last_error(NULL) then holds the reason. */
 lbm_status lbm_create(lbm_lattice lattice, int32_t nx, int32_t ny, int32_t nz,
                       const lbm_params* params, lbm_ctx** out);

@@ -12,7 +12,8 @@
  *  - Pointers are DEVICE pointers owned by the caller; nothing is allocated except one 4-byte
  *    error word per process (lbm_nn_gemm_tn's bounded waits) on first use.
  *  - Activations are channel-last BF16, x[v][c], voxel v = x + W (y + H z).
- *  - A 3^3 convolution ("same", zero outside) uses im2col rows col[v][k], k = tap C + c,
+ *  - A 3^3 convolution ("same", zero outside) runs without rows (lbm_nn_conv3, lbm_nn_conv3_wgrad) or
+ *    over im2col rows col[v][k]; both sum over k = tap C + c,
  *    tap = (dz+1) 9 + (dy+1) 3 + (dx+1), zero for k >= 27 C up to the padded width Kp.
  *  - Work is enqueued on `stream` (a cudaStream_t; NULL = legacy default); no call synchronises
  *    except lbm_nn_status.  Invalid sizes or pointers return LBM_ERR_INVALID_ARG before anything

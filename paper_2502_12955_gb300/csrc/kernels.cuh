@@ -615,10 +615,6 @@ __device__ __forceinline__ T warp_sum(T v) {
 
 // ================================================================ step
 
-// One fused time step for every fluid node: gather (A-A parity), wet-node closure and its
-// bookkeeping, deposition, moments, forces, velocity, flow collision (BGK / MRT, Guo or
-// velocity shift), scalar collision, in-place scatter with bounce-back / inlet / outlet.
-// Registers hold deviations from w_i * ref throughout.
 #ifndef LBM_STEP_MIN_BLOCKS
 #define LBM_STEP_MIN_BLOCKS 3   // resident 256-thread blocks per SM, one component in FP32 math (80 registers)
 #endif
@@ -1235,6 +1231,13 @@ __device__ __forceinline__ void solid_nodes(const Args& a, const Coef<typename S
 // bookkeeping, deposition, moments, forces, velocity, flow collision (BGK / MRT, Guo or
 // velocity shift), scalar collision, in-place scatter with bounce-back / inlet / outlet.
 // Registers hold deviations from w_i * ref throughout.
+//
+// What bounds it (256^3 packing, D3Q19 MRT + D3Q7, 6.7 M fluid nodes): the even step in FP32 DRAM traffic, 1.1 times
+// the 208 bytes per node (273 us with planes over the domain and a collision per population, 248 us now); the odd step
+// the latency of its scattered neighbour cells (390 -> 362 us); with 16-bit storage instruction issue (232 x 203 x
+// 181, FP16 flow and FP32 scalars: 140 / 190 -> 117 / 180 us); FP64 the FP64 units (64^3: 163 -> 88 us per
+// step).  128^3 FP32, where half of the 0.17 GB of populations fit into L2: 49 -> 39 us per step, of which the walk
+// back and forth gives 5.
 template <class L, class S, int NC, int NS, int COLL, int parity, bool BND>
 __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) == 4 ? (parity ? LBM_STEP_MIN_BLOCKS_ODD : LBM_STEP_MIN_BLOCKS) : 2)) k_step(const Args a, const Coef<typename Store<S>::T> k) {
   using T = typename Store<S>::T;
@@ -1512,7 +1515,8 @@ __global__ void __launch_bounds__(256) k_psi(const Args a, const Coef<typename S
   // Walks the fluid list in slot order, as k_step does: at parity 0 every population of the
   // node sits in its own cell (coalesced); at parity 1 population i sits in cell (n - c_i, opp i),
   // whose slot is looked up once for all components.  Sums in population order 0 .. Q-1 from
-  // rho_ref, the order the gather of the step uses.
+  // rho_ref, the order the gather of the step uses.  Bound by DRAM (parity 0: 128^3 with two components, 0.32 GB in
+  // 57 us) and by the scattered cells (parity 1: 70 us; 62 and 94 us with planes over the domain).
   using T = typename Store<S>::T;
   using R = Rec<L, S, NC, NS>;
   pdl_trigger();
@@ -1593,7 +1597,8 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[K], unsigned int 
 
 // Monitors, one wave of blocks: population sums over the fluid list in the compute type
 // (deviations from the reference, so the sums stay accurate), bookkeeping sums over all nodes
-// in FP64, per-block partials in FP64 (summed in fixed order by k_reduce_partials).
+// in FP64, per-block partials in FP64 (summed in fixed order by k_reduce_partials).  Bound by latency on small
+// domains (15 us at any size up to 512 x 512, 38 to 44 us when every warp reduced every value), else by DRAM.
 template <class L, class S, int NC, int NS>
 __device__ __forceinline__ void monitor_block(const Args& a, const Coef<typename Store<S>::T>& k, const int parity,
                                               const unsigned int block, const unsigned int blocks) {
@@ -2266,7 +2271,9 @@ __device__ __forceinline__ void coords_of(const Args& a, long long n, int* x, in
 //   3 final flags;  4 link masks of every node around a flipped one;  5 clear the list
 // parity_next is the layout parity of the state the flips act on (steps completed & 1).
 // What bounds it is the chain of dependent loads of an entry: flag, slot and mask of 18 neighbours, their
-// populations, then the 18 flags around each of them.
+// populations, then the 18 flags around each of them.  One block with a thread per entry took longer than the step
+// once a few hundred nodes flipped together (64^3 FP64 dissolution: 2.4 ms for ten steps, 1.3 ms with the cluster
+// and all); an update without flips takes 2 us.
 constexpr int kFlipBlocks = 8, kFlipThreads = 512;
 __device__ __forceinline__ void cluster_barrier() {
   __syncwarp();
