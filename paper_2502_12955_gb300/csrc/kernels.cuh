@@ -35,34 +35,32 @@ namespace lbm {
 
 // ------------------------------------------------------------------ storage
 
+// Populations are loaded with ordinary loads.  The read-only path (__ldg) wants data that does not change while the
+// kernel lives, and a step kernel lives from before its predecessor, which writes them, has ended (see pdl_wait).
 template <class S>
 struct Store;
 template <>
 struct Store<double> {
   using T = double;
-  __device__ static T ld(const double* p) { return __ldg(p); }
-  __device__ static T ldv(const double* p) { return *p; }
+  __device__ static T ld(const double* p) { return *p; }
   __device__ static void st(double* p, T v) { *p = v; }
 };
 template <>
 struct Store<float> {
   using T = float;
-  __device__ static T ld(const float* p) { return __ldg(p); }
-  __device__ static T ldv(const float* p) { return *p; }
+  __device__ static T ld(const float* p) { return *p; }
   __device__ static void st(float* p, T v) { *p = v; }
 };
 template <>
 struct Store<__half> {
   using T = float;
-  __device__ static T ld(const __half* p) { return __half2float(__ldg(p)); }
-  __device__ static T ldv(const __half* p) { return __half2float(*p); }
+  __device__ static T ld(const __half* p) { return __half2float(*p); }
   __device__ static void st(__half* p, T v) { *p = __float2half_rn(v); }
 };
 template <>
 struct Store<__nv_bfloat16> {
   using T = float;
-  __device__ static T ld(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
-  __device__ static T ldv(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+  __device__ static T ld(const __nv_bfloat16* p) { return __bfloat162float(*p); }
   __device__ static void st(__nv_bfloat16* p, T v) { *p = __float2bfloat16_rn(v); }
 };
 
@@ -78,15 +76,13 @@ struct bf16_s32 {
 template <>
 struct Store<half_s32> {
   using T = float;
-  __device__ static T ld(const half_s32* p) { return __half2float(__ldg(&p->v)); }
-  __device__ static T ldv(const half_s32* p) { return __half2float(p->v); }
+  __device__ static T ld(const half_s32* p) { return __half2float(p->v); }
   __device__ static void st(half_s32* p, T v) { p->v = __float2half_rn(v); }
 };
 template <>
 struct Store<bf16_s32> {
   using T = float;
-  __device__ static T ld(const bf16_s32* p) { return __bfloat162float(__ldg(&p->v)); }
-  __device__ static T ldv(const bf16_s32* p) { return __bfloat162float(p->v); }
+  __device__ static T ld(const bf16_s32* p) { return __bfloat162float(p->v); }
   __device__ static void st(bf16_s32* p, T v) { p->v = __float2bfloat16_rn(v); }
 };
 template <class S>
@@ -609,7 +605,10 @@ __device__ __forceinline__ double widen(float v) {
 // Programmatic dependent launch: the kernels of a time step are launched so that each may start while its
 // predecessor still runs.  A kernel lets its successor start at once, reads what no step changes (without
 // geometry updates: lists, masks, maps), and waits for the completion of its predecessor before it touches
-// anything else.  Every thread waits, so completion still runs in launch order.  On a small domain this hides the launch
+// anything else.  Every thread waits, so completion still runs in launch order.  What a step changes (populations, psi,
+// totals, the solid lattice) is read after the wait and with ordinary loads: the wait makes the predecessor's writes
+// visible to those, while the read-only path (__ldg) may only be used for data that is constant from this kernel's
+// start to its end, which includes the end of its predecessor: slots, lists, masks.  On a small domain this hides the launch
 // and the first dependent loads, which are most of a 4 us kernel.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
@@ -1977,7 +1976,7 @@ __global__ void __launch_bounds__(256) k_pops_io(const Args a, const Coef<typena
         else
           p = R::f(a, cell_of<R>(a, nb.at(-L::cx(i), -L::cy(i), -L::cz(i))), s, L::opp(i));
         const double sh = L::w(i) * double(k.rref[s]);
-        if (dir == 0) *io = double(Store<S>::ldv(p)) + sh;
+        if (dir == 0) *io = double(Store<S>::ld(p)) + sh;
         else Store<S>::st(p, T(*io - sh));
       }
     }
@@ -1998,7 +1997,7 @@ __global__ void __launch_bounds__(256) k_pops_io(const Args a, const Coef<typena
         else
           p = R::h(a, cell_of<R>(a, nb.at(-L::cx(j), -L::cy(j), -L::cz(j))), s, L::opp(j));
         const double sh = double(scal_w<T>(j, k)) * double(k.cref[s]);
-        if (dir == 0) *io = double(Store<SC>::ldv(p)) + sh;
+        if (dir == 0) *io = double(Store<SC>::ld(p)) + sh;
         else Store<SC>::st(p, T(*io - sh));
       }
     }
