@@ -98,8 +98,8 @@ Coef<T> make_coef(const Args& a, bool shifted) {
     k.G_ads[s] = T(a.G_ads[s]);
     for (int t = 0; t < 2; ++t) k.G[s][t] = T(a.G[s][t]);
     k.rref[s] = shifted ? T(a.rho_ref[s]) : T(0);
-    k.hom[s] = T(0.5 * (1.0 - 1.0 / a.tau[s]));
   }
+  k.hom = T(0.5 * (1.0 - 1.0 / a.tau[0]));
   for (int s = 0; s < 3; ++s) {
     k.omc[s] = T(1.0 / a.tau_c[s]);
     k.C_in[s] = T(a.C_in[s]);
