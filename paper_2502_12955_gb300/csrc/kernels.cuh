@@ -822,38 +822,37 @@ __device__ __forceinline__ T cdot(int i, T x, T y, T z) {
   return r;
 }
 
-// BGK of one component on pairs (Eq. 1.16, 1.21), f* = f + om (f_eq - f) + (1 - om/2) F.  With b = (1 - om/2) F the
-// odd part of the equilibrium and the force is 3 w c.o, o = om rho u + b, and their even part, the density's share
-// om w drho aside, w (4.5 (c.u)(c.e) - 1.5 u.e), e = o + b.  Velocity-shift forcing (Eq. 1.17, 1.18) is the same
-// with b = 0 and its own u.
-// Mass and momentum: om multiplies differences (w drho - f, w rho (c.u) - f) that carry neither up to rounding.  With
-// f* = (1 - om) f + om f_eq, one operation less per sum and difference, the two rounded factors add up to 1 for some
-// relaxation times only, and else every step changes mass and momentum by the same factor, up to 6e-8 in FP32 (32 x 32
-// box, 2000 steps, tau 0.9: 1.3e-4 of the mass deviation, 2.2e-5 this way); om drho rounded ahead of the weights
-// costs FP64 a drift of 1.2e-17 per step in the same way.  The factor 3 is applied to the vector and not folded into
-// the weights: 1/18, 1/36 and 1/9 round to FP32 within 7e-9, 1/6, 1/12 and 1/3 only within 3e-8, which would change
-// the momentum by that factor every step.
+// BGK of one component on pairs (Eq. 1.16, 1.21), f* = f + om (f_eq - f) + (1 - om/2) F, from its drho, velocity u,
+// momentum m = rho u and b = (1 - om/2) F.  The odd part of the equilibrium is 3 w c.m and of the force 3 w c.b, the
+// even part of both, the density's share w drho aside, w (4.5 (c.u)(c.e) - 1.5 u.e), e = om m + 2 b.  Velocity-shift
+// forcing (Eq. 1.17, 1.18) is the same with b = 0 and its own u.
+// Mass and momentum: om multiplies the differences w drho - f and 3 w c.m - f, whose products are not rounded, and
+// each pair takes an increment that is zero at equilibrium.  So no factor that is rounded once, the same way at every
+// node, acts on mass or momentum: (1 - om) f + om f_eq, two operations less per pair, has two factors that add up to 1
+// for some relaxation times only and else changes both by up to 6e-8 of themselves per step in FP32 (32 x 32 box, 2000
+// steps, tau 0.9: 1.3e-4 of the mass deviation, 2e-5 this way), and rounded products that drift once a flow is
+// uniform (momentum 5e-5, 2e-5 this way).  What is left is the weights' own rounding: 1/18, 1/36 and 1/9 round to
+// FP32 within 7e-9 (1/6, 1/12 and 1/3 only within 3e-8, which is why the factor 3 goes to the vector).
 template <class L, class T>
-__device__ __forceinline__ void bgk_pairs(T* f, T om, T drho, T rho, T ux, T uy, T uz, T bx, T by, T bz) {
-  const T wa = T(L::w(1)), wd = T(L::w(L::Q - 1));
-  const T ro = om * rho, omh = T(0.5) * om;
-  const T ox = fmad(ro, ux, bx), oy = fmad(ro, uy, by), oz = fmad(ro, uz, bz);
-  const T ex = ox + bx, ey = oy + by, ez = oz + bz;
+__device__ __forceinline__ void bgk_pairs(T* f, T om, T drho, T ux, T uy, T uz, T mx, T my, T mz, T bx, T by, T bz) {
+  const T wa = T(L::w(1)), wd = T(L::w(L::Q - 1)), omh = T(0.5) * om;
+  const T ex = fmad(om, mx, T(2) * bx), ey = fmad(om, my, T(2) * by), ez = fmad(om, mz, T(2) * bz);
   const T K = T(-1.5) * fmad(ux, ex, fmad(uy, ey, uz * ez));
-  f[0] = fmad(om, fmad(T(L::w(0)), drho, -f[0]), fmad(T(L::w(0)), K, f[0]));
-  const T Ra = wa * drho, Rd = wd * drho, Ka = wa * K, Kd = wd * K;
+  f[0] += fmad(om, fmad(T(L::w(0)), drho, -f[0]), T(L::w(0)) * K);
+  const T Ka = wa * K, Kd = wd * K;
   const T a45 = T(4.5 * L::w(1)), d45 = T(4.5 * L::w(L::Q - 1));
-  const T o3x = T(3) * ox, o3y = T(3) * oy, o3z = T(3) * oz;
+  const T m3x = T(3) * mx, m3y = T(3) * my, m3z = T(3) * mz, b3x = T(3) * bx, b3y = T(3) * by, b3z = T(3) * bz;
 #pragma unroll
   for (int i = 1; i < L::Q; ++i) {
     const int o = L::opp(i);
     if (i > o) continue;
     const bool axis = L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i) + L::cz(i) * L::cz(i) == 1;
+    const T w2 = T(2) * (axis ? wa : wd);
     const T cu = axis ? cdot<L>(i, a45 * ux, a45 * uy, a45 * uz) : cdot<L>(i, d45 * ux, d45 * uy, d45 * uz);
     const T Ee = fmad(cu, cdot<L>(i, ex, ey, ez), axis ? Ka : Kd);
-    const T Eo = axis ? cdot<L>(i, wa * o3x, wa * o3y, wa * o3z) : cdot<L>(i, wd * o3x, wd * o3y, wd * o3z);
-    const T E = fmad(om, fmad(T(-0.5), f[i], axis ? Ra : Rd), fmad(T(0.5), f[i], Ee));
-    const T O = fmad(T(0.5), f[o], fmad(-omh, f[o], Eo));
+    const T Oe = axis ? cdot<L>(i, wa * b3x, wa * b3y, wa * b3z) : cdot<L>(i, wd * b3x, wd * b3y, wd * b3z);
+    const T E = fmad(T(0.5), f[i], fmad(omh, fmad(w2, drho, -f[i]), Ee));
+    const T O = fmad(T(0.5), f[o], fmad(omh, fmad(w2, cdot<L>(i, m3x, m3y, m3z), -f[o]), Oe));
     f[i] = E + O;
     f[o] = E - O;
   }
@@ -1134,7 +1133,10 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
       const T ex = nxs * iden + k.tau[s] * Fx[s] * ir;
       const T ey = nys * iden + k.tau[s] * Fy[s] * ir;
       const T ez = nzs * iden + k.tau[s] * Fz[s] * ir;
-      bgk_pairs<L, T>(f[s], k.om[s], drho[s], rho[s], ex, ey, ez, T(0), T(0), T(0));
+      // rho u: of a single component its own momentum and the shift
+      const T tx = NC == 1 ? fmad(k.tau[s], Fx[s], jx[s]) : rho[s] * ex, ty = NC == 1 ? fmad(k.tau[s], Fy[s], jy[s]) : rho[s] * ey,
+              tz = NC == 1 ? fmad(k.tau[s], Fz[s], jz[s]) : rho[s] * ez;
+      bgk_pairs<L, T>(f[s], k.om[s], drho[s], ex, ey, ez, tx, ty, tz, T(0), T(0), T(0));
     }
   } else if (COLL == 1) {
     if constexpr (Q == 19) mrt_pairs_d3q19<T>(f[0], k, drho[0], jx[0], jy[0], jz[0], ux, uy, uz, Fx[0], Fy[0], Fz[0]);
@@ -1143,7 +1145,9 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
 #pragma unroll
     for (int s = 0; s < NC; ++s) {
       const T b = T(1) - T(0.5) * k.om[s];
-      bgk_pairs<L, T>(f[s], k.om[s], drho[s], rho[s], ux, uy, uz, b * Fx[s], b * Fy[s], b * Fz[s]);
+      // rho u: of a single component mx, which carries no rounding of the velocity's division
+      const T tx = NC == 1 ? mx : rho[s] * ux, ty = NC == 1 ? my : rho[s] * uy, tz = NC == 1 ? mz : rho[s] * uz;
+      bgk_pairs<L, T>(f[s], k.om[s], drho[s], ux, uy, uz, tx, ty, tz, b * Fx[s], b * Fy[s], b * Fz[s]);
     }
   }
   // ---- scalar collision (Eq. therpop_species, therpopeq_species), u = physical velocity
