@@ -1635,6 +1635,7 @@ void lbm_ensemble_destroy(lbm_ensemble* e) {
   if (e->d_args) cudaFree(e->d_args);
   if (e->d_coefs) cudaFree(e->d_coefs);
   if (e->d_tiles) cudaFree(e->d_tiles);
+  if (e->d_eval) cudaFree(e->d_eval);
   delete e;
 }
 
