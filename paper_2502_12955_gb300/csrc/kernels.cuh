@@ -28,6 +28,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cstdint>
+#include <type_traits>
 
 #include "lattice.cuh"
 
@@ -133,9 +134,10 @@ struct Args {
   // slot e) and the solid nodes to F .. N-1; nodes that become fluid later keep their slot.
   uint32_t* slot;
   uint32_t* slot_new;         // rebuild scratch
-  // Byte offset of every node's first cell in pop, plus kOffBias rows (see wall_offsets); kept
-  // beside slot when pop fits in 32 bits (off_ok), for the plain step kernels
+  // Byte offset of every node's first cell in pop, plus kOffBias rows (see wall_offsets), for the odd step of the plain
+  // kernels: in 32 bits while they hold it (off_ok), else in 64
   uint32_t* off;
+  unsigned long long* off64;
   unsigned int* block_counts; // ordered-compaction scratch [chunks + 1]
   unsigned int* block_counts_v;   // the same for the in-domain positions of the fluid-list order
   double* wallx_slot;        // [NBANKS][WALLX_SLOTS] wall-exchange accumulators
@@ -176,7 +178,7 @@ struct Args {
   int moving_wall;           // the top plate moves (closed y axis)
   int flow_open_x;           // flow velocity inlet at x = 0, zero-gradient outlet at x = nx - 1
   double* u_in_row;          // [ny] inlet velocity u_x(y)
-  int off_ok;                // pop fits in 32-bit byte offsets: the plain step kernels apply
+  int off_ok;                // 32-bit byte offsets reach all of pop
   int arrhenius;             // scalar 1 is the temperature: rate k(T_b), reaction heat into T
   int n_it;                  // fixed-point iterations of the C_b - T_b coupling per link
   double arr_A, arr_Ta, heat_release;
@@ -322,7 +324,7 @@ __host__ __device__ constexpr int tile_slots(int elem) { return elem == 2 ? 64 :
 template <class L, class S, int NC, int NS>
 struct Rec {
   using SC = typename ScalarOf<S>::type;
-  static constexpr int kTile = tile_slots((int)sizeof(S));
+  static constexpr int kTile = tile_slots((int)sizeof(S)), kElem = (int)sizeof(S);
   static constexpr int FROW = kTile * (int)sizeof(S), HROW = kTile * (int)sizeof(SC);
   static constexpr int H0 = NC * L::Q * FROW;
   static constexpr int BYTES = H0 + NS * L::QC * HROW;
@@ -330,8 +332,9 @@ struct Rec {
   __host__ __device__ static constexpr int frow(int s, int i) { return (s * L::Q + i) * FROW; }
   __host__ __device__ static constexpr int hrow(int s, int j) { return H0 + (s * L::QC + j) * HROW; }
   // byte offset of the first flow cell of a slot, and of its first scalar cell less H0
-  __device__ __forceinline__ static long long cell(unsigned long long sn) {
-    return (long long)((sn / kTile) * BYTES + (sn % kTile) * sizeof(S));
+  __device__ __forceinline__ static long long cell(long long sn) {
+    const uint32_t n = uint32_t(sn);   // slots are below 2^31
+    return (long long)(n / kTile) * (BYTES - FROW) + (long long)n * (int)sizeof(S);
   }
   template <class O>
   __device__ __forceinline__ static O scell(O c) {
@@ -639,7 +642,7 @@ __device__ __forceinline__ T warp_sum(T v) {
 // (n + c_i, i): every neighbour it needs on the way in, it needs again on the way out, and the
 // scalar lattices' axis links use the flow lattice's neighbours.  One shared-memory entry per
 // direction k (entry k - 1, for the neighbour n + c_k) serves all of them.  The entries are copied
-// in asynchronously (cp.async) while the previous node of the thread computes: the byte offset of the
+// in asynchronously (cp.async) while the previous node of the thread computes: the offset of the
 // neighbour's cells (Args::off) for the plain kernels, its slot for the full ones.
 //
 // k_step keeps the cache as rows of LBM_STEP_CACHE_STRIDE threads per direction (consecutive
@@ -647,11 +650,12 @@ __device__ __forceinline__ T warp_sum(T v) {
 // tile kernel gives each thread Q consecutive words of dynamic shared memory instead, sized
 // to its block (Q - 1 used; the odd stride puts the threads of a warp on distinct banks).
 #define LBM_STEP_CACHE_STRIDE 256
-// Asynchronous copies (cp.async, sm_80 and later) of one 4-byte word from global to shared
+// Asynchronous copies (cp.async, sm_80 and later) of one 4- or 8-byte word from global to shared
 // memory; a thread waits for its own groups with cp_async_wait.
-__device__ __forceinline__ void cp_async4(uint32_t* smem, const uint32_t* gmem) {
+template <class E>
+__device__ __forceinline__ void cp_async_word(E* smem, const E* gmem) {
   const unsigned int s = (unsigned int)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(s), "l"(gmem), "n"((int)sizeof(E)) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -659,59 +663,92 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 
 // Start copying the map's values of all Q - 1 neighbours n + c_i of a list entry's node into the
 // cache.  Links into walls copy a value that is never read (the periodic image is a valid node).
-template <class L, int CS>
-__device__ __forceinline__ void prefetch_nbrs(const Args& a, const uint32_t* map, uint32_t entry, uint32_t* cache) {
+template <class L, int CS, class E>
+__device__ __forceinline__ void prefetch_nbrs(const Args& a, const E* map, uint32_t entry, E* cache) {
   const int n = list_node(a, entry);
   const Nbr nb = nbr_entry(a, n, entry);
 #pragma unroll
   for (int i = 1; i < L::Q; ++i)
-    cp_async4(cache + (i - 1) * CS, map + LBM_CHK(a.err, nb.at(L::cx(i), L::cy(i), L::cz(i)), a.N));
+    cp_async_word(cache + (i - 1) * CS, map + LBM_CHK(a.err, nb.at(L::cx(i), L::cy(i), L::cz(i)), a.N));
 }
 
-// Byte offsets in the cache are biased by kOffBias rows.  Flow links into walls read and write the
+// Offsets in the cache are biased by kOffBias rows.  Flow links into walls read and write the
 // node's own cell: (n, i) for the population arriving in direction i, which sits in row i while
 // a fluid link's cell sits in row opp(i).  Writing into a wall link's cache entry the own offset moved
 // by opp(k) - k rows (at most two rows down, so the biased offset stays positive) lets every flow
 // access take row + entry without testing the link.
+// The entries are 32-bit byte offsets up to 4 GB of populations (41 M nodes of D3Q19 + D3Q7 in FP32) and 64-bit ones
+// beyond (kWide), which cost registers and shared memory: 384^3 FP32, 22.6 M fluid nodes, 1053 us per step, 1050 us
+// with 32-bit offsets in flow elements (whose multiply slows the 16-bit ensemble's odd step, 253 -> 266 us) and 1286
+// us with slots and tests per link; 448^3 FP16 1439 us and 1704 us; 576^3 FP32 3726 us.
 constexpr int kOffBias = 4;
-template <class L, class R, int CS>
-__device__ __forceinline__ void wall_offsets(uint32_t own, uint32_t m, uint32_t* cache) {
+
+// Variants of the step: plain; full with the boundary rules of a moving plate, a velocity inlet or the
+// temperature-dependent reaction; plain with wide offsets (odd steps).  A cache entry is an offset, in the
+// full variant a slot.
+enum : int { kPlain = 0, kFull = 1, kWide = 2 };
+template <int VAR>
+struct Entries {
+  using type = uint32_t;
+  __device__ __forceinline__ static const uint32_t* map(const Args& a) { return VAR == kPlain ? a.off : a.slot; }
+};
+template <>
+struct Entries<kWide> {
+  using type = unsigned long long;
+  __device__ __forceinline__ static const unsigned long long* map(const Args& a) { return a.off64; }
+};
+
+template <class L, class R, int CS, class E>
+__device__ __forceinline__ void wall_offsets(long long slot, uint32_t m, E* cache) {
+  const uint32_t n = uint32_t(slot);
+  const E own = E(n / R::kTile) * E(R::BYTES - R::FROW) + E(n) * E(R::kElem) + E(kOffBias * R::FROW);
 #pragma unroll
   for (int k = 1; k < L::Q; ++k)
-    if (flow_wall<L>(m, k)) cache[(k - 1) * CS] = own + uint32_t((L::opp(k) - k) * R::FROW);
+    if (flow_wall<L>(m, k)) cache[(k - 1) * CS] = own + E((L::opp(k) - k) * R::FROW);
 }
 
 // The cells an odd step reads and writes through cache entry k: flow row (s, k) and scalar row (s, k)
 // of the neighbour n + c_k, or of the own node behind a wall (rows opp(k)).
-template <class L, class S, int NC, int NS, int CS, bool BND>
+template <class L, class S, int NC, int NS, int CS, int VAR>
 struct OddCells {
   using R = Rec<L, S, NC, NS>;
   using SC = typename R::SC;
+  using E = typename Entries<VAR>::type;
   static constexpr long long kBias = (long long)kOffBias * R::FROW;
   const Args& a;
   long long c;      // the node's own cells
   uint32_t m;
-  const uint32_t* cache;
+  const E* cache;
+  // row at byte `row` of the cells at an entry's offset, and the cells of the slot that an entry names
+  __device__ __forceinline__ unsigned char* at(E e, long long row) const {
+    return a.pop + LBM_CHK(a.err, (long long)e + (row - kBias), a.pop_bytes);
+  }
+  __device__ __forceinline__ long long cell(E e) const { return R::cell((long long)LBM_CHK(a.err, e, a.pitch)); }
   __device__ __forceinline__ S* flow(int s, int k) const {
-    if (!BND) return reinterpret_cast<S*>(a.pop + LBM_CHK(a.err, (long long)cache[(k - 1) * CS] + (R::frow(s, k) - kBias), a.pop_bytes));
+    const E e = cache[(k - 1) * CS];
+    if (VAR != kFull) return reinterpret_cast<S*>(at(e, R::frow(s, k)));
     if (flow_wall<L>(m, k)) return R::f(a, c, s, L::opp(k));
-    return R::f(a, R::cell((long long)LBM_CHK(a.err, cache[(k - 1) * CS], a.pitch)), s, k);
+    return R::f(a, cell(e), s, k);
   }
   // A scalar link to a fluid neighbour is a fluid flow link and a wall or reactive link a flow wall,
   // so the entry serves both; only an open face (x links) may be a fluid link of a periodic flow.
   __device__ __forceinline__ SC* scal(int s, int k) const {
-    if (!BND && R::kSameElem) {
+    const E e = cache[(k - 1) * CS];
+    if (VAR != kFull && R::kSameElem) {
       if (L::cx(k) != 0 && MaskBits<L>::code(m, k) == 3u) return R::h(a, c, s, L::opp(k));
-      return reinterpret_cast<SC*>(a.pop + LBM_CHK(a.err, (long long)cache[(k - 1) * CS] + (R::hrow(s, k) - kBias), a.pop_bytes));
+      return reinterpret_cast<SC*>(at(e, R::hrow(s, k)));
     }
     if (MaskBits<L>::code(m, k) != 0u) return R::h(a, c, s, L::opp(k));
-    if (!BND) return R::h(a, (long long)cache[(k - 1) * CS] - kBias, s, k);
-    return R::h(a, R::cell((long long)LBM_CHK(a.err, cache[(k - 1) * CS], a.pitch)), s, k);
+    if (VAR != kFull) {
+      const uint32_t lane = uint32_t(e) / R::kElem % R::kTile;
+      return reinterpret_cast<SC*>(at(e, R::hrow(s, k) + lane * (uint32_t)(sizeof(SC) - sizeof(S))));
+    }
+    return R::h(a, cell(e), s, k);
   }
 };
 
-template <class L, class S, int NC, int NS, int CS, bool BND>
-__device__ __forceinline__ void gather_odd(const OddCells<L, S, NC, NS, CS, BND>& o, typename Store<S>::T (&f)[NC][L::Q],
+template <class L, class S, int NC, int NS, int CS, int VAR>
+__device__ __forceinline__ void gather_odd(const OddCells<L, S, NC, NS, CS, VAR>& o, typename Store<S>::T (&f)[NC][L::Q],
                                            typename Store<S>::T (&h)[NS > 0 ? NS : 1][L::QC]) {
   using R = Rec<L, S, NC, NS>;
 #pragma unroll
@@ -967,9 +1004,9 @@ __device__ __forceinline__ void mrt_pairs_d3q19(T* f, const K& k, T drho, T jx, 
 // Everything after the gather for one fluid node: wet-node closure and its bookkeeping,
 // deposition, moments, forces, velocity, flow and scalar collision, in-place scatter.  entry: the
 // node's fluid-list entry; c: its cells; o: its odd cells (parity 1).
-template <class L, class S, int NC, int NS, int COLL, int parity, bool BND, int CS, class Pre>
+template <class L, class S, int NC, int NS, int COLL, int parity, int VAR, int CS, class Pre>
 __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typename Store<S>::T>& k, uint32_t entry, int n,
-                                                uint32_t m, long long c, const OddCells<L, S, NC, NS, CS, BND>& o,
+                                                uint32_t m, long long c, const OddCells<L, S, NC, NS, CS, VAR>& o,
                                                 typename Store<S>::T (&f)[NC][L::Q],
                                                 typename Store<S>::T (&h)[NS > 0 ? NS : 1][L::QC],
                                                 typename Store<S>::T& wallx, typename Store<S>::T& heatx,
@@ -978,6 +1015,7 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
   using R = Rec<L, S, NC, NS>;
   using SC = typename R::SC;
   constexpr int Q = L::Q, QC = L::QC;
+  constexpr bool BND = VAR == kFull;
   const Nbr nb = nbr_entry(a, n, entry);
   // ---- wet-node closure of scalar 0 and reaction bookkeeping (Eq. wetnode9, reactO2)
   if (NS > 0) {
@@ -1185,13 +1223,13 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
     }
   }
   // the cache entries move to registers, and the cache takes the next node's while this one is stored
-  uint32_t ent[parity ? Q - 1 : 1];
+  typename Entries<VAR>::type ent[parity ? Q - 1 : 1];
   if (parity) {
 #pragma unroll
     for (int i = 0; i < Q - 1; ++i) ent[i] = o.cache[i * CS];
   }
   pre();
-  const OddCells<L, S, NC, NS, 1, BND> to{a, c, m, ent};
+  const OddCells<L, S, NC, NS, 1, VAR> to{a, c, m, ent};
 #pragma unroll
   for (int s = 0; s < NC; ++s) {
     Store<S>::st(R::f(a, c, s, 0), f[s][0]);
@@ -1244,6 +1282,11 @@ __device__ __forceinline__ void collide_scatter(const Args& a, const Coef<typena
 template <class L, class S>
 __device__ __forceinline__ void solid_nodes(const Args& a, const Coef<typename Store<S>::T>& k, int parity, unsigned int block, unsigned int blocks);
 
+// Blocks per SM of the odd step with 64-bit offsets: two leave the registers it needs (576^3 FP32 3726 us, 3929 us with
+// three and spills), but mixed storage with its two address forms does better with three (3546 us, 3617 us with two).
+template <class S>
+constexpr int wide_min_blocks() { return std::is_same<S, typename ScalarOf<S>::type>::value ? 2 : 3; }
+
 // One fused time step for every fluid node: gather (A-A parity), wet-node closure and its
 // bookkeeping, deposition, moments, forces, velocity, flow collision (BGK / MRT, Guo or
 // velocity shift), scalar collision, in-place scatter with bounce-back / inlet / outlet.
@@ -1255,12 +1298,13 @@ __device__ __forceinline__ void solid_nodes(const Args& a, const Coef<typename S
 // 181, FP16 flow and FP32 scalars: 140 / 190 -> 117 / 180 us); FP64 the FP64 units (64^3: 163 -> 88 us per
 // step).  128^3 FP32, where half of the 0.17 GB of populations fit into L2: 49 -> 39 us per step, of which the walk
 // back and forth gives 5.
-template <class L, class S, int NC, int NS, int COLL, int parity, bool BND>
-__global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) == 4 ? (parity ? LBM_STEP_MIN_BLOCKS_ODD : LBM_STEP_MIN_BLOCKS) : 2)) k_step(const Args a, const Coef<typename Store<S>::T> k) {
+template <class L, class S, int NC, int NS, int COLL, int parity, int VAR>
+__global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) == 4 ? (VAR == kWide ? wide_min_blocks<S>() : parity ? LBM_STEP_MIN_BLOCKS_ODD : LBM_STEP_MIN_BLOCKS) : 2)) k_step(const Args a, const Coef<typename Store<S>::T> k) {
   using T = typename Store<S>::T;
   constexpr int Q = L::Q, QC = L::QC, NSD = NS > 0 ? NS : 1;
+  constexpr bool BND = VAR == kFull;
   using R = Rec<L, S, NC, NS>;
-  using O = OddCells<L, S, NC, NS, LBM_STEP_CACHE_STRIDE, BND>;
+  using O = OddCells<L, S, NC, NS, LBM_STEP_CACHE_STRIDE, VAR>;
   T wallx = T(0), heatx = T(0), prodx = T(0);
   pdl_trigger();
   unsigned int blocks = gridDim.x;
@@ -1289,16 +1333,17 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
     stride = 0u - stride;
     if (e >= count) e += stride;   // the last block's threads past the end
   }
-  const auto cell = [&](unsigned int en, int n) { return R::cell(en < base ? (long long)en : (long long)__ldg(a.slot + n)); };
+  const auto slot = [&](unsigned int en, int n) { return en < base ? (long long)en : (long long)__ldg(a.slot + n); };
   // the list entry is fetched two iterations and the link mask one iteration ahead
   uint32_t w_cur = e < count ? a.fluid_list[e] : 0u;
   uint32_t w_nx = e + stride < count ? a.fluid_list[e + stride] : 0u;
   uint32_t m_cur = e < count ? a.mask[list_node(a, w_cur)] : 0u;
   if constexpr (parity == 1) {
     // the neighbours of the next entry are copied in (asynchronously) while this entry is stored
-    __shared__ uint32_t slot_buf[(L::Q - 1) * LBM_STEP_CACHE_STRIDE];
-    uint32_t* cb = slot_buf + threadIdx.x;
-    const uint32_t* map = BND ? a.slot : a.off;
+    using E = typename Entries<VAR>::type;
+    __shared__ E slot_buf[(L::Q - 1) * LBM_STEP_CACHE_STRIDE];
+    E* cb = slot_buf + threadIdx.x;
+    const E* map = Entries<VAR>::map(a);
     if (e < count) prefetch_nbrs<L, LBM_STEP_CACHE_STRIDE>(a, map, w_cur, cb);
     cp_async_commit();
     if (a.geo_mode == GEO_NONE) pdl_wait();
@@ -1318,13 +1363,13 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
       if (m & 1u) {
         T f[NC][Q], h[NSD][QC];
         const int n = list_node(a, w);
-        const long long c = cell(e, n);
+        const long long sn = slot(e, n), c = R::cell(sn);
         // the plain variant addresses every flow link through its cache entry (wall_offsets);
         // the full variant keeps the per-link tests its boundary rules need
-        if (!BND) wall_offsets<L, R, LBM_STEP_CACHE_STRIDE>(uint32_t(c) + uint32_t(kOffBias * R::FROW), m, cb);
+        if (VAR != kFull) wall_offsets<L, R, LBM_STEP_CACHE_STRIDE>(sn, m, cb);
         const O o{a, c, m, cb};
-        gather_odd<L, S, NC, NS, LBM_STEP_CACHE_STRIDE, BND>(o, f, h);
-        collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, k, w, n, m, c, o, f, h, wallx, heatx, prodx, pre);
+        gather_odd<L, S, NC, NS, LBM_STEP_CACHE_STRIDE, VAR>(o, f, h);
+        collide_scatter<L, S, NC, NS, COLL, parity, VAR>(a, k, w, n, m, c, o, f, h, wallx, heatx, prodx, pre);
       } else {
         pre();
       }
@@ -1340,9 +1385,9 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
       if (!(m & 1u)) continue;   // a node removed by deposition since the last list rebuild
       T f[NC][Q], h[NSD][QC];
       const int n = list_node(a, w);
-      const long long c = cell(e, n);
+      const long long c = R::cell(slot(e, n));
       gather_even<L, S, NC, NS>(a, c, f, h);
-      collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, k, w, n, m, c, O{a, c, m, nullptr}, f, h, wallx, heatx, prodx, []() {});
+      collide_scatter<L, S, NC, NS, COLL, parity, VAR>(a, k, w, n, m, c, O{a, c, m, nullptr}, f, h, wallx, heatx, prodx, []() {});
     }
   }
   // ---- wall-exchange monitor: one reduction per warp that saw a reactive link
@@ -1403,7 +1448,8 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
   __shared__ Args sa;
   __shared__ Coef<T> sk;
   using R = Rec<L, S, NC, NS>;
-  using O = OddCells<L, S, NC, NS, 1, BND>;
+  constexpr int VAR = BND ? kFull : kPlain;
+  using O = OddCells<L, S, NC, NS, 1, VAR>;
   extern __shared__ uint32_t slot_smem[];   // blockDim.x * Q words at odd parity (launcher)
   uint32_t* cache = slot_smem + threadIdx.x * L::Q;
   // blocks take chunks of consecutive tiles in turn (at most LBM_TILE_CHUNK, fewer where that would leave
@@ -1437,7 +1483,7 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
       have_next = false;
     }
     const Args& a = sa;
-    const uint32_t* map = BND ? a.slot : a.off;
+    const uint32_t* map = Entries<VAR>::map(a);
     T wallx = T(0), heatx = T(0), prodx = T(0);
     const unsigned int e = tile.first + threadIdx.x;
     const unsigned int count = a.fluid_count[0];
@@ -1481,16 +1527,16 @@ __global__ void __launch_bounds__(256, (NC == 1 && sizeof(typename Store<S>::T) 
       const unsigned int base = a.fluid_count[1];
       T f[NC][Q], h[NSD][QC];
       const int n = list_node(a, w);
-      const long long c = R::cell(e < base ? (long long)e : (long long)__ldg(a.slot + n));
+      const long long sn = e < base ? (long long)e : (long long)__ldg(a.slot + n), c = R::cell(sn);
       const O o{a, c, m, cache};
       if (parity) {
         // the plain variant addresses every flow link through its cache entry (wall_offsets)
-        if (!BND) wall_offsets<L, R, 1>(uint32_t(c) + uint32_t(kOffBias * R::FROW), m, cache);
-        gather_odd<L, S, NC, NS, 1, BND>(o, f, h);
+        if (!BND) wall_offsets<L, R, 1>(sn, m, cache);
+        gather_odd<L, S, NC, NS, 1, VAR>(o, f, h);
       } else {
         gather_even<L, S, NC, NS>(a, c, f, h);
       }
-      collide_scatter<L, S, NC, NS, COLL, parity, BND>(a, sk, w, n, m, c, o, f, h, wallx, heatx, prodx, pre);
+      collide_scatter<L, S, NC, NS, COLL, parity, VAR>(a, sk, w, n, m, c, o, f, h, wallx, heatx, prodx, pre);
     } else {
       pre();
     }
@@ -2202,10 +2248,10 @@ __device__ __forceinline__ unsigned int block_prefix(unsigned int b, unsigned in
 }
 
 // PRED 0 also assigns the new storage slots: fluid nodes take their list position, solid nodes
-// follow the fluid total in brick order (slot_new), and the byte offsets that go with them (off;
-// rec bytes per tile, elem per flow element).
+// follow the fluid total in brick order (slot_new), and the offsets that go with them (off; rec
+// bytes per tile of `tile` slots, elem per flow element).
 template <class L, int PRED>
-__global__ void __launch_bounds__(1024) k_list_write(const Args a, uint32_t* list, const uint32_t rec, const uint32_t elem) {
+__global__ void __launch_bounds__(1024) k_list_write(const Args a, uint32_t* list, const uint32_t rec, const uint32_t tile, const uint32_t elem) {
   __shared__ unsigned int wsum[32];
   const long long t = blockIdx.x * 1024ll + threadIdx.x;
   long long n;
@@ -2216,10 +2262,9 @@ __global__ void __launch_bounds__(1024) k_list_write(const Args a, uint32_t* lis
     if (n >= 0) {
       const unsigned int sl = f ? pos : a.fluid_count[0] + (vpos - pos);
       a.slot_new[n] = sl;
-      if (a.off_ok) {
-        const uint32_t tile = (uint32_t)tile_slots((int)elem);
-        a.off[n] = (sl / tile) * rec + (sl % tile + kOffBias * tile) * elem;
-      }
+      const unsigned long long o = (unsigned long long)(sl / tile) * rec + (sl % tile + kOffBias * tile) * elem;
+      if (a.off_ok) a.off[n] = (uint32_t)o;
+      else a.off64[n] = o;
     }
   }
   if (f) {

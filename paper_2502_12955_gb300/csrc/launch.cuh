@@ -155,7 +155,7 @@ struct Launchers {
     return (size_t)threads * L::Q * sizeof(uint32_t);
   }
 
-  template <int NC, int NS, int COLL, int PAR, bool BND>
+  template <int NC, int NS, int COLL, int PAR, int VAR>
   static cudaError_t step_p(const Args& a, cudaStream_t st) {
     const int threads = a.bx;
     static int cached_threads = -1, cached_blocks = 0;
@@ -163,7 +163,7 @@ struct Launchers {
       int dev = 0, sms = 0, occ = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step<L, S, NC, NS, COLL, PAR, BND>, threads, 0);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step<L, S, NC, NS, COLL, PAR, VAR>, threads, 0);
       cached_blocks = (occ > 0 ? occ : 1) * (sms > 0 ? sms : 1);
       cached_threads = threads;
     }
@@ -171,17 +171,17 @@ struct Launchers {
     unsigned int blocks = (unsigned int)(need < cached_blocks ? need : cached_blocks);
     if (blocks == 0) blocks = 1;
     Args b = a;
-    if (BND && NS > 1 && a.conjugate) blocks += b.solid_blocks = box_blocks(a);   // behind the step's own blocks
-    return launch_pdl(kEarly, k_step<L, S, NC, NS, COLL, PAR, BND>, blocks, threads, 0, st, b, coef(a));
+    if (VAR == kFull && NS > 1 && a.conjugate) blocks += b.solid_blocks = box_blocks(a);   // behind the step's own blocks
+    return launch_pdl(kEarly, k_step<L, S, NC, NS, COLL, PAR, VAR>, blocks, threads, 0, st, b, coef(a));
   }
-  // BND: a moving plate, a velocity inlet or the temperature-dependent reaction needs the full
-  // variant of the step kernel, and so does a domain too large for the plain variant's 32-bit
-  // byte offsets (4 GB of populations, 41 M nodes of D3Q19 + D3Q7 in FP32)
+  // a moving plate, a velocity inlet or the temperature-dependent reaction needs the full variant; the odd step of a
+  // domain with more than 4 GB of populations the wide one
   template <int NC, int NS, int COLL>
   static cudaError_t step_t(const Args& a, int parity, cudaStream_t st) {
-    if (a.moving_wall || a.flow_open_x || a.arrhenius || !a.off_ok)
-      return parity ? step_p<NC, NS, COLL, 1, true>(a, st) : step_p<NC, NS, COLL, 0, true>(a, st);
-    return parity ? step_p<NC, NS, COLL, 1, false>(a, st) : step_p<NC, NS, COLL, 0, false>(a, st);
+    if (a.moving_wall || a.flow_open_x || a.arrhenius)
+      return parity ? step_p<NC, NS, COLL, 1, kFull>(a, st) : step_p<NC, NS, COLL, 0, kFull>(a, st);
+    if (!parity) return step_p<NC, NS, COLL, 0, kPlain>(a, st);
+    return a.off_ok ? step_p<NC, NS, COLL, 1, kPlain>(a, st) : step_p<NC, NS, COLL, 1, kWide>(a, st);
   }
   template <int NC, int NS>
   static cudaError_t step_c(const Args& a, int parity, int coll, cudaStream_t st) {
@@ -352,12 +352,13 @@ struct Launchers {
       k_list_count<L, 0><<<bchunks, 1024, 0, st>>>(a);
       k_list_scan<<<1, 1024, 0, st>>>(a.block_counts, bchunks, a.fluid_count);
       k_list_scan<<<1, 1024, 0, st>>>(a.block_counts_v, bchunks, a.fluid_count + 2);
-      k_list_write<L, 0><<<bchunks, 1024, 0, st>>>(a, a.fluid_list, (uint32_t)rec_bytes(a), (uint32_t)sizeof(S));
+      k_list_write<L, 0><<<bchunks, 1024, 0, st>>>(a, a.fluid_list, (uint32_t)rec_bytes(a),
+                                                  (uint32_t)tile_slots((int)sizeof(S)), (uint32_t)sizeof(S));
     }
     if (which & 2) {
       k_list_count<L, 1><<<chunks, 1024, 0, st>>>(a);
       k_list_scan<<<1, 1024, 0, st>>>(a.block_counts, chunks, a.iface_count);
-      k_list_write<L, 1><<<chunks, 1024, 0, st>>>(a, a.iface_list, 0u, 0u);
+      k_list_write<L, 1><<<chunks, 1024, 0, st>>>(a, a.iface_list, 0u, 0u, 0u);
     }
     return cudaGetLastError();
   }

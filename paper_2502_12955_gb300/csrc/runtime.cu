@@ -592,6 +592,7 @@ lbm_status lbm_create(lbm_lattice lattice, int32_t nx, int32_t ny, int32_t nz, c
   DA(c->pop_alt, a.pop_bytes);
   DA(a.slot, N * 4);
   if (a.off_ok) DA(a.off, N * 4);
+  else DA(a.off64, N * 8);
   DA(a.slot_new, N * 4);
   if (a.sc_on)
     for (int s = 0; s < params->n_comp; ++s) DA(a.psi[s], P * c->ks->psi_bytes);
@@ -1344,9 +1345,9 @@ lbm_status ens_launch(lbm_ensemble* e, int parity, cudaStream_t st) {
   if (e->ntiles == 0) return LBM_OK;
   const lbm_params& p = e->m[0]->p;
   int bnd = 0;   // the boundary-rule kernel variant when any member has a moving plate or an inlet
-  // (or a domain too large for the plain variant's 32-bit wall offsets)
+  // (or, at odd steps, a domain too large for the plain variant's 32-bit offsets)
   for (size_t k = 0; k < e->m.size(); ++k)
-    bnd |= e->m[k]->a.moving_wall | e->m[k]->a.flow_open_x | e->m[k]->a.arrhenius | !e->m[k]->a.off_ok;
+    bnd |= e->m[k]->a.moving_wall | e->m[k]->a.flow_open_x | e->m[k]->a.arrhenius | (parity & !e->m[k]->a.off_ok);
   const cudaError_t r = e->ks->step_tiles(e->d_args, e->d_coefs, e->d_tiles, e->ntiles, p.n_comp, p.n_scal,
                                           p.collision, parity, bnd, e->threads, st);
   e->launches += 1;
