@@ -1658,8 +1658,28 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[K], unsigned int 
   }
 }
 
-// Monitors, one wave of blocks: population sums over the fluid list in the compute type
-// (deviations from the reference, so the sums stay accurate), bookkeeping sums over all nodes
+// Running sum of a thread over its nodes.  In FP32 the rounding error of every addition is kept (the two-sum of
+// Knuth, The Art of Computer Programming 2, 4.2.2), so that the number of nodes per thread costs no accuracy and no
+// FP64 operations; a sum that has left the finite numbers is its own result.
+template <class T>
+struct NodeSum {
+  T s = T(0), c = T(0);
+  __device__ __forceinline__ void add(T x) {
+    const T t = s + x, b = t - s;
+    c += (s - (t - b)) + (x - b);
+    s = t;
+  }
+  __device__ __forceinline__ double value() const { return isfinite(s) ? double(s) + double(c) : double(s); }
+};
+template <>
+struct NodeSum<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double x) { s += x; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+
+// Monitors, one wave of blocks: population sums over the fluid list, a node's in the compute type
+// (deviations from the reference, so they stay accurate), bookkeeping sums over all nodes
 // in FP64, per-block partials in FP64 (summed in fixed order by k_reduce_partials).  Bound by latency on small
 // domains (15 us at any size up to 512 x 512, 38 to 44 us when every warp reduced every value), else by DRAM.
 template <class L, class S, int NC, int NS>
@@ -1669,11 +1689,7 @@ __device__ __forceinline__ void monitor_block(const Args& a, const Coef<typename
   constexpr int Q = L::Q, QC = L::QC;
   const unsigned int tid = block * blockDim.x + threadIdx.x;
   const unsigned int nthr = blocks * blockDim.x;
-  T dm[NC > 0 ? NC : 1], mom[3] = {T(0), T(0), T(0)}, dsp[NS > 0 ? NS : 1];
-#pragma unroll
-  for (int s = 0; s < NC; ++s) dm[s] = T(0);
-#pragma unroll
-  for (int s = 0; s < NS; ++s) dsp[s] = T(0);
+  NodeSum<T> dm[NC > 0 ? NC : 1], mom[3], dsp[NS > 0 ? NS : 1];
   unsigned int nfluid = 0, nonfin = 0;
   const unsigned int count = a.fluid_count[0], base = a.fluid_count[1];
   for (unsigned int e = tid; e < count; e += nthr) {
@@ -1685,6 +1701,7 @@ __device__ __forceinline__ void monitor_block(const Args& a, const Coef<typename
     const Nbr nb = parity ? nbr_entry(a, n, w) : Nbr{};
     const long long cell = Rec<L, S, NC, NS>::cell(e < base ? (long long)e : (long long)a.slot[n]);
     bool bad = false;
+    T jn[3] = {T(0), T(0), T(0)};
 #pragma unroll
     for (int s = 0; s < NC; ++s) {
       T f[Q];
@@ -1693,13 +1710,15 @@ __device__ __forceinline__ void monitor_block(const Args& a, const Coef<typename
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
         r += f[i];
-        if (L::cx(i)) mom[0] += T(L::cx(i)) * f[i];
-        if (L::cy(i)) mom[1] += T(L::cy(i)) * f[i];
-        if (L::cz(i)) mom[2] += T(L::cz(i)) * f[i];
+        if (L::cx(i)) jn[0] += T(L::cx(i)) * f[i];
+        if (L::cy(i)) jn[1] += T(L::cy(i)) * f[i];
+        if (L::cz(i)) jn[2] += T(L::cz(i)) * f[i];
       }
       bad |= !isfinite(r);
-      dm[s] += r;
+      dm[s].add(r);
     }
+#pragma unroll
+    for (int q = 0; q < L::D; ++q) mom[q].add(jn[q]);
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
       T h[QC];
@@ -1708,16 +1727,16 @@ __device__ __forceinline__ void monitor_block(const Args& a, const Coef<typename
 #pragma unroll
       for (int j = 0; j < QC; ++j) c += h[j];
       bad |= !isfinite(c);
-      dsp[s] += c;
+      dsp[s].add(c);
     }
     nonfin += bad ? 1u : 0u;
   }
   double v[NMON];
 #pragma unroll
   for (int q = 0; q < NMON; ++q) v[q] = 0.0;
-  for (int s = 0; s < NC; ++s) v[M_MASS + s] = double(dm[s]) + double(k.rref[s]) * double(nfluid);
-  for (int c = 0; c < 3; ++c) v[M_MOM + c] = double(mom[c]);
-  for (int s = 0; s < NS; ++s) v[mon_spec(s)] = double(dsp[s]) + double(k.cref[s]) * double(nfluid);
+  for (int s = 0; s < NC; ++s) v[M_MASS + s] = dm[s].value() + double(k.rref[s]) * double(nfluid);
+  for (int c = 0; c < 3; ++c) v[M_MOM + c] = mom[c].value();
+  for (int s = 0; s < NS; ++s) v[mon_spec(s)] = dsp[s].value() + double(k.cref[s]) * double(nfluid);
   v[M_NFLUID] = double(nfluid);
   v[M_NONFIN] = double(nonfin);
   // bookkeeping over every node
@@ -1906,7 +1925,7 @@ __device__ __forceinline__ void resid_block(const Args& a, const Coef<typename S
   using T = typename Store<S>::T;
   T* snap = reinterpret_cast<T*>(a.snap);
   const long long P = a.pitch;
-  T du = T(0), uu = T(0), dc = T(0), cc = T(0);
+  NodeSum<T> du, uu, dc, cc;
   const unsigned int count = a.fluid_count[0], base = a.fluid_count[1];
   for (unsigned int e = block * blockDim.x + threadIdx.x; e < count; e += blocks * blockDim.x) {
     const uint32_t w = a.fluid_list[e];
@@ -1916,20 +1935,23 @@ __device__ __forceinline__ void resid_block(const Args& a, const Coef<typename S
     const long long sn = e < base ? (long long)e : (long long)a.slot[n];
     T rho[NC], u[3], C[NS > 0 ? NS : 1];
     node_macros<L, S, NC, NS>(a, k, n, nbr_entry(a, n, w), m, Rec<L, S, NC, NS>::cell(sn), parity, rho, u, C);
+    T dn = T(0), un = T(0);
     for (int c = 0; c < 3; ++c) {
       const T d = u[c] - snap[c * P + sn];
-      du += d * d;
-      uu += u[c] * u[c];
+      dn += d * d;
+      un += u[c] * u[c];
       snap[c * P + sn] = u[c];
     }
+    du.add(dn);
+    uu.add(un);
     if (NS > 0) {
       const T d = C[0] - snap[3 * P + sn];
-      dc += d * d;
-      cc += C[0] * C[0];
+      dc.add(d * d);
+      cc.add(C[0] * C[0]);
       snap[3 * P + sn] = C[0];
     }
   }
-  double v[4] = {double(du), double(uu), double(dc), double(cc)};
+  double v[4] = {du.value(), uu.value(), dc.value(), cc.value()};
   block_reduce_store<4>(v, 15u, a.partials + (long long)block * 4);
 }
 
