@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "kernels.cuh"
@@ -68,18 +69,35 @@ long long brick_positions(const Args& a) {
   return ((a.nx + B::X - 1) / B::X) * (long long)((a.ny + B::Y - 1) / B::Y) * ((a.nz + B::Z - 1) / B::Z) * B::V;
 }
 
+// SMs of the current device (queried once)
+inline int sm_count() {
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n > 0 ? n : 1;
+  }();
+  return sms;
+}
+
+// Blocks of one resident wave of a kernel, kept per block size: contexts of several block sizes, on several host
+// threads, each find their own.
+template <class K>
+int resident_blocks(std::atomic<int> (&cache)[9], K kernel, int threads, size_t smem) {
+  std::atomic<int>& c = cache[threads / 32];
+  int n = c.load(std::memory_order_relaxed);
+  if (n == 0) {
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem);
+    n = (occ > 0 ? occ : 1) * sm_count();
+    c.store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
 // blocks of 256 threads for one resident wave (4 per SM) of the reduction kernels, the most that the partial sums
 // have room for
-inline unsigned int wave_blocks() {
-  static unsigned int cached = 0;
-  if (!cached) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cached = (unsigned int)((sms > 0 ? sms : 1) * 4);
-  }
-  return cached;
-}
+inline unsigned int wave_blocks() { return 4u * (unsigned int)sm_count(); }
 
 // A reduction kernel over a small domain runs about four nodes per thread: the blocks past that only add partial
 // sums (a 128 x 128 ensemble member: 40 us for its monitors with 608 blocks).
@@ -158,17 +176,10 @@ struct Launchers {
   template <int NC, int NS, int COLL, int PAR, int VAR>
   static cudaError_t step_p(const Args& a, cudaStream_t st) {
     const int threads = a.bx;
-    static int cached_threads = -1, cached_blocks = 0;
-    if (cached_threads != threads) {
-      int dev = 0, sms = 0, occ = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step<L, S, NC, NS, COLL, PAR, VAR>, threads, 0);
-      cached_blocks = (occ > 0 ? occ : 1) * (sms > 0 ? sms : 1);
-      cached_threads = threads;
-    }
+    static std::atomic<int> cache[9];
+    const int wave = resident_blocks(cache, k_step<L, S, NC, NS, COLL, PAR, VAR>, threads, 0);
     long long need = (a.N + threads - 1) / threads;
-    unsigned int blocks = (unsigned int)(need < cached_blocks ? need : cached_blocks);
+    unsigned int blocks = (unsigned int)(need < wave ? need : wave);
     if (blocks == 0) blocks = 1;
     Args b = a;
     if (VAR == kFull && NS > 1 && a.conjugate) blocks += b.solid_blocks = box_blocks(a);   // behind the step's own blocks
@@ -211,17 +222,10 @@ struct Launchers {
   template <int NC, int NS, int PAR>
   static cudaError_t psi_p(const Args& a, cudaStream_t st) {
     const int threads = a.bx;
-    static int cached_threads = -1, cached_blocks = 0;
-    if (cached_threads != threads) {
-      int dev = 0, sms = 0, occ = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_psi<L, S, NC, NS, PAR>, threads, 0);
-      cached_blocks = (occ > 0 ? occ : 1) * (sms > 0 ? sms : 1);
-      cached_threads = threads;
-    }
+    static std::atomic<int> cache[9];
+    const int wave = resident_blocks(cache, k_psi<L, S, NC, NS, PAR>, threads, 0);
     const long long need = (a.N + threads - 1) / threads;
-    const unsigned int blocks = (unsigned int)(need < cached_blocks ? need : cached_blocks);
+    const unsigned int blocks = (unsigned int)(need < wave ? need : wave);
     return launch_pdl(kEarly, k_psi<L, S, NC, NS, PAR>, blocks > 0 ? blocks : 1, threads, 0, st, a, coef(a));
   }
   static cudaError_t psi(const Args& a, int parity, cudaStream_t st) {
@@ -370,12 +374,9 @@ struct Launchers {
   template <int NC, int NS, int COLL, int PAR, bool BND>
   static cudaError_t step_tiles_p(const Args* d_args, const void* d_coefs, const Tile* d_tiles, unsigned int ntiles,
                                   int threads, cudaStream_t st) {
-    int dev = 0, sms = 0, occ = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = slot_smem_bytes(PAR, threads);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step_tiles<L, S, NC, NS, COLL, PAR, BND>, threads, smem);
-    const unsigned int wave = (unsigned int)((occ > 0 ? occ : 1) * (sms > 0 ? sms : 1));
+    static std::atomic<int> cache[9];
+    const unsigned int wave = (unsigned int)resident_blocks(cache, k_step_tiles<L, S, NC, NS, COLL, PAR, BND>, threads, smem);
     const unsigned int blocks = ntiles < wave ? (ntiles > 0 ? ntiles : 1) : wave;
     // consecutive tiles per turn: about eight turns for every block, LBM_TILE_CHUNK tiles at most.  Fewer turns
     // leave the last one uneven: six 3D members (27 tiles per block) take 222 us per step in chunks of 8 and 212 us in
