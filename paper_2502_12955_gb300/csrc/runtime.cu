@@ -268,12 +268,14 @@ void fill_args(lbm_ctx* c) {
   int bx = p.block_x;
   if (bx == 0) {
     // the step kernel walks the fluid list: the block shape is not tied to nx.  256 threads, fewer on a domain
-    // whose blocks of that size would not reach every SM (152 on this GPU): 128 x 64 nodes in FP64 take
-    // 15.1 us per step as 32 blocks of 256 and 9.8 us as 128 blocks of 64 (16.0 us as 256 blocks of 32)
+    // whose blocks of that size would not reach every SM: 128 x 64 nodes in FP64 take
+    // 15.1 us per step as 32 blocks of 256 and 9.8 us as 128 blocks of 64 (16.0 us as 256 blocks of 32).
+    // The rule counts all nodes, since the block size is fixed before the geometry is known: a box of 40 % fluid
+    // needs 2.5 blocks of nodes per SM for its fluid to reach all of them with large blocks (block_x chooses otherwise).
     // FP64 arithmetic: 64 threads at every size.  Those kernels are bound by the FP64 units, and small blocks
     // share them out more evenly in the last wave (64^3 dissolution: 103.3 us per step with 256, 87.5 us with 64).
     bx = p.precision == LBM_FP64 ? 64 : 256;
-    while (bx > 64 && (c->N + bx - 1) / bx < 152) bx /= 2;
+    while (bx > 64 && (c->N + bx - 1) / bx < sm_count()) bx /= 2;
   }
   a.bx = bx;
   a.by = 1;
@@ -629,7 +631,7 @@ lbm_status lbm_create(lbm_lattice lattice, int32_t nx, int32_t ny, int32_t nz, c
   DA(a.err, 16);
   DA(a.inflow_row, 3 * rows * 8);
   DA(a.outflow_row, 3 * rows * 8);
-  // monitor partials: the monitor grid uses 128-thread blocks over x; the residual 256 over N
+  // partial sums of the monitors, also of the residual: a row per block of reduce_blocks, at most wave_blocks of them
   DA(a.partials, (long long)wave_blocks() * NMON * 8);
   DA(a.mon_out, (NMON + 8) * 8);
   DA(a.d_rho, 2 * N * 8);
