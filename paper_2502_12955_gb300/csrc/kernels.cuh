@@ -549,29 +549,12 @@ __device__ __forceinline__ void close_product(T* hp, uint32_t m, const Coef<T>& 
 
 // ---------------------------------------------------------- equilibria
 
-template <class L, class T>
-__device__ __forceinline__ T feq(int i, T rho, T ux, T uy, T uz) {
-  const T cu = T(L::cx(i)) * ux + T(L::cy(i)) * uy + T(L::cz(i)) * uz;
-  const T uu = ux * ux + uy * uy + uz * uz;
-  return T(L::w(i)) * rho * (T(1) + T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu);
-}
-
 // f_i^eq - w_i rref, given drho = rho - rref (Eq. 6 written as a deviation)
 template <class L, class T>
 __device__ __forceinline__ T feq_dev(int i, T rho, T drho, T ux, T uy, T uz) {
   const T cu = T(L::cx(i)) * ux + T(L::cy(i)) * uy + T(L::cz(i)) * uz;
   const T uu = ux * ux + uy * uy + uz * uz;
   return T(L::w(i)) * (drho + rho * (T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu));
-}
-
-// Guo forcing term (Eq. 1.21) with c_s^2 = 1/3
-template <class L, class T>
-__device__ __forceinline__ T guo(int i, T ux, T uy, T uz, T Fx, T Fy, T Fz) {
-  const T cx = T(L::cx(i)), cy = T(L::cy(i)), cz = T(L::cz(i));
-  const T cu = cx * ux + cy * uy + cz * uz;
-  const T cF = cx * Fx + cy * Fy + cz * Fz;
-  const T uF = ux * Fx + uy * Fy + uz * Fz;
-  return T(L::w(i)) * (T(3) * (cF - uF) + T(9) * cu * cF);
 }
 
 // -------------------------------------------------------- flip list append
