@@ -158,7 +158,10 @@ __global__ void __launch_bounds__(192, 4) k_conv3(const ConvSrc src, const bf16*
   uint64_t* accfree = done + 2;
   uint32_t* slot = reinterpret_cast<uint32_t*>(accfree + 2);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * p.nz;
+  // one index for all tiles: any proportions of the domain, where the y and z of a grid end at 65535
+  const unsigned tiles_x = (unsigned)(W + TX - 1) / TX, tiles_y = (unsigned)(H + TY - 1) / TY;
+  const unsigned row = blockIdx.x / tiles_x;
+  const int x0 = (int)(blockIdx.x - row * tiles_x) * TX, y0 = (int)(row % tiles_y) * TY, z0 = (int)(row / tiles_y) * p.nz;
   const int nz = min(p.nz, D - z0);
   if (threadIdx.x == 0) {
     for (int i = 0; i < 4; ++i) {
@@ -692,13 +695,13 @@ static bool conv_plan(ConvPlan* p, int C, int N, int D, int H, int W) {
       }
       p->smem = (unsigned)o.planes * plane + b + extra;
       if (p->smem > limit) continue;
-      const int tiles = ((W + TX - 1) / TX) * ((H + TY - 1) / TY);
+      const long long tiles = (long long)((W + TX - 1) / TX) * ((H + TY - 1) / TY);
       int per_sm = (int)(kSmemOne / p->smem);
       if (per_sm > 4) per_sm = 4;   // registers
       // accumulators of the CTAs of an SM share 512 TMEM columns
       while (per_sm > 1 && per_sm * pow2_cols(2 * N) > 512) --per_sm;
       const int slots = sm_count() * per_sm;
-      int zs = std::max(1, std::min(D, slots / tiles));
+      int zs = std::max(1, std::min(D, (int)(slots / tiles)));
       p->nz = o.seq ? 1 : (D + zs - 1) / zs;
       p->accs = p->nz > 1 ? 2 : 1;
       if (p->accs * N > 512) p->accs = 1;
@@ -773,7 +776,7 @@ static bool by_narrow(int C, F&& f) {
 static bool conv_args_ok(const void* xa, int Ca, int up, const void* xb, int Cb, int D, int H, int W) {
   if (!xa || Ca <= 0 || Cb < 0 || (Cb > 0 && !xb) || D <= 0 || H <= 0 || W <= 0) return false;
   if (up && ((D | H | W) & 1)) return false;
-  if ((long long)D * H * W >= (1ll << 31) || (H + TY - 1) / TY > 65535 || D > 65535) return false;
+  if ((long long)D * H * W >= (1ll << 31)) return false;
   if (Ca % 16 == 0 && Cb % 16 == 0) return true;
   return Ca <= 8 && Cb == 0 && !up;   // the narrow first layer
 }
@@ -844,10 +847,10 @@ lbm_status lbm_nn_conv3(const void* xa, int32_t Ca, int32_t up, const void* xb, 
     NN_CK(e);
   } else {
     ConvPlan p;
-    if (!conv_plan(&p, Ca + Cb, N, D, H, W)) return LBM_ERR_INVALID_ARG;
+    if (!conv_plan(&p, Ca + Cb, N, D, H, W) || (long long)tx * ty * ((D + p.nz - 1) / p.nz) >= (1ll << 31)) return LBM_ERR_INVALID_ARG;
     NN_CK(allow_smem(k_conv3, p.smem));
     const ConvSrc src{static_cast<const bf16*>(xa), static_cast<const bf16*>(xb), Ca, Cb, up ? 1 : 0};
-    k_conv3<<<dim3(tx, ty, (D + p.nz - 1) / p.nz), 192, p.smem, st>>>(src, static_cast<const bf16*>(wp), out, p, D, H, W, err);
+    k_conv3<<<(unsigned)tx * (unsigned)ty * (unsigned)((D + p.nz - 1) / p.nz), 192, p.smem, st>>>(src, static_cast<const bf16*>(wp), out, p, D, H, W, err);
   }
   NN_CK(cudaGetLastError());
   return LBM_OK;
