@@ -466,7 +466,8 @@ __global__ void __launch_bounds__(288, FIRST ? 1 : 2) k_wgrad(const ConvSrc src,
   unsigned char* sB = base + (size_t)p.ws * 16 * WBLOCK;
   const uint32_t bbytes = (uint32_t)(p.Co / 8) * WBLOCK;
   // per pair of 8-row chunks (16 channels of a tap): tap, part of the input (0 a, 1 a on the coarse grid, 2 b, -1 past
-  // 27 C), element offset from the voxel's own row (channel alone on the coarse grid)
+  // 27 C), element offset from the voxel's own row (channel alone on the coarse grid) in 64 bits: a plane of H W C
+  // elements may pass 2^31
   int4* table = reinterpret_cast<int4*>(sB + (size_t)p.nb * bbytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int C = p.C, Co = p.Co, ws = p.ws;
@@ -482,11 +483,10 @@ __global__ void __launch_bounds__(288, FIRST ? 1 : 2) k_wgrad(const ConvSrc src,
   }
   for (int i = threadIdx.x; i < 8 * nt; i += 288) {
     const int k = (t0 * 8 + i) * 16, tap = k / C, c = k % C;
-    const int shift = ((tap / 9 - 1) * H + (tap / 3) % 3 - 1) * W + tap % 3 - 1;
-    table[i] = k >= 27 * C ? make_int4(0, -1, 0, 0)
-               : c >= src.ca ? make_int4(tap, 2, shift * src.cb + c - src.ca, 0)
-               : src.up ? make_int4(tap, 1, c, 0)
-                        : make_int4(tap, 0, shift * src.ca + c, 0);
+    const long long shift = ((long long)(tap / 9 - 1) * H + (tap / 3) % 3 - 1) * W + tap % 3 - 1;
+    const int part = k >= 27 * C ? -1 : c >= src.ca ? 2 : src.up ? 1 : 0;
+    const long long off = part == 2 ? shift * src.cb + c - src.ca : part == 1 ? c : shift * src.ca + c;
+    table[i] = make_int4(part < 0 ? 0 : tap, part, (int)(unsigned)off, (int)(off >> 32));
   }
   if (warp == 0) tmem_alloc(&slot, (uint32_t)p.cols);
   tc_fence_before();
@@ -559,8 +559,9 @@ __global__ void __launch_bounds__(288, FIRST ? 1 : 2) k_wgrad(const ConvSrc src,
             const bool in = e.y >= 0 && ((mz >> e.x) & 1u);
             const bf16* q = src.a;
             if (in) {
-              if (e.y == 0) q = pa + e.z;
-              else if (e.y == 2) q = pb + e.z;
+              const long long off = (long long)e.w << 32 | (unsigned)e.z;
+              if (e.y == 0) q = pa + off;
+              else if (e.y == 2) q = pb + off;
               else
                 q = pa + ((long long)(((z + e.x / 9 - 1) >> 1) * (H >> 1) + ((y + (e.x / 3) % 3 - 1) >> 1)) * (W >> 1) +
                           ((x + e.x % 3 - 1) >> 1)) * src.ca + e.z;
