@@ -59,7 +59,9 @@ lbm_status lbm_nn_im2col_cv(const void* xT, void* colT, int32_t D, int32_t H, in
 lbm_status lbm_nn_transpose(const void* x, void* y, int64_t R, int32_t Cc, void* stream);
 /* out[i] = sum_z part[z * stride + i], i < n (FP32). */
 lbm_status lbm_nn_reduce_splits(const float* part, float* out, int64_t n, int32_t splits, int64_t stride, void* stream);
-/* dx = dy where y > 0, else 0 (gradient through y = relu(x)); n BF16 elements. */
+/* dx = dy where y > 0, else 0 (gradient through y = relu(x)); n BF16 elements.  The network takes it in
+   lbm_nn_relu_grad_bias; this pass, lbm_nn_colsum, lbm_nn_add and the backward pass of lbm_nn_pool2 are kept as the
+   separate steps which that one has to repeat. */
 lbm_status lbm_nn_relu_grad(const void* y, const void* dy, void* dx, int64_t n, void* stream);
 /* Gradient through y = relu(conv + b) with the bias gradient: dx = dy where y > 0, else 0; db[c] = sum_v
    dx[v][c] (FP32, overwritten).  With dskip, dy is the gradient of the 2x average pooling of y (coarse
@@ -68,7 +70,8 @@ lbm_status lbm_nn_relu_grad(const void* y, const void* dy, void* dx, int64_t n, 
 lbm_status lbm_nn_relu_grad_bias(const void* y, const void* dy, const void* dskip, void* dx, float* db, int32_t D, int32_t H,
                                  int32_t W, int32_t C, void* stream);
 /* 2x average pooling of in [D*H*W][C] into out [D/2*H/2*W/2][C] (D, H, W even), or with
-   backward = 1 its gradient: in = dL/dout (coarse), out = dL/din (fine, D*H*W). */
+   backward = 1 its gradient: in = dL/dout (coarse), out = dL/din (fine, D*H*W; kept for comparison, see
+   lbm_nn_relu_grad). */
 lbm_status lbm_nn_pool2(const void* in, void* out, int32_t D, int32_t H, int32_t W, int32_t C, int32_t backward,
                         void* stream);
 /* 2x nearest upsampling of in [D*H*W][C] (coarse sizes) into out [2D*2H*2W][C], or with
@@ -78,7 +81,7 @@ lbm_status lbm_nn_up2(const void* in, void* out, int32_t D, int32_t H, int32_t W
 /* out [V][Ca+Cb] = [a [V][Ca], b [V][Cb]]; backward = 1 splits out back into a and b. */
 lbm_status lbm_nn_concat(void* a, int32_t Ca, void* b, int32_t Cb, void* out, int64_t V, int32_t backward,
                          void* stream);
-/* out[c] = sum_v x[v][c] (bias gradient), FP32, overwritten. */
+/* out[c] = sum_v x[v][c] (bias gradient), FP32, overwritten.  Kept for comparison (see lbm_nn_relu_grad). */
 lbm_status lbm_nn_colsum(const void* x, float* out, int64_t V, int32_t C, void* stream);
 /* Head (1x1 convolution, FP32 weights w [Co][C], bias b [Co]): y [V][Co] FP32 from h [V][C]. */
 lbm_status lbm_nn_head_fwd(const void* h, const float* w, const float* b, float* y, int64_t V, int32_t C, int32_t Co,
@@ -126,7 +129,7 @@ int64_t lbm_nn_conv3_packed(int32_t Co, int32_t Ci);
 /* 1 if lbm_nn_conv3 and lbm_nn_conv3_wgrad take a layer of these channels, its input gradient included
    (shared and tensor memory hold its operands), else 0. */
 int32_t lbm_nn_conv3_fits(int32_t Ca, int32_t up, int32_t Cb, int32_t Co);
-/* y = a + b, n BF16 elements. */
+/* y = a + b, n BF16 elements.  Kept for comparison (see lbm_nn_relu_grad). */
 lbm_status lbm_nn_add(const void* a, const void* b, void* y, int64_t n, void* stream);
 /* y = BF16(x), n elements. */
 lbm_status lbm_nn_cast_bf16(const float* x, void* y, int64_t n, void* stream);

@@ -438,7 +438,9 @@ __global__ void __launch_bounds__(128, 3) k_conv3_first(const bf16* __restrict__
 // and 8-voxel K groups 128 bytes apart.  A CTA owns some of the 128-row tiles and one of the voxel ranges that the
 // split-K GEMM over im2col rows would take, adds the voxels in the same order, and writes FP32 partial sums
 // that k_wgrad_sum adds in split order: the same result bit for bit.
-// Bound by the gather: a 16 KB tile per 0.6 us and SM, 27 bytes per clock, wherever the tiles run (128^3: 48 -> 16
+// Bound by the gather, not by a bandwidth: a 16 KB tile per 0.6 us and SM is 13 bytes per clock, and no order of the
+// tiles changed it.  A tile is 32 copy instructions of a warp, each of sixteen 32-byte pieces from different rows with
+// their tap's test and address, with the copies of WLAG tiles in flight behind the one being issued (128^3: 48 -> 16
 // channels 1514 us, 16 -> 16 channels 621 us, the 5-channel input 534 us, from 3597 us with unpadded rows).
 struct WgradPlan {
   int C, Co;
@@ -713,7 +715,8 @@ static bool conv_plan(ConvPlan* p, int C, int N, int D, int H, int W) {
 }
 
 // Voxel ranges of the weight gradient: those of the split-K GEMM over im2col rows (K padded to 128, at most 64
-// splits, about four waves of tiles over 152 SMs), so that partial sums keep their boundaries.
+// splits, about four waves of tiles over 152 SMs: a constant of that rule, so that the boundaries of the partial sums, and
+// with them the results, do not depend on the device).
 static bool wgrad_plan(WgradPlan* p, int C, int Co, int D, int H, int W) {
   const long long V = (long long)D * H * W;
   if (Co % 16 || Co > 256 || V % 64 || V >= (1ll << 31) - 64) return false;

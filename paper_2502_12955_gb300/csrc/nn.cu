@@ -283,7 +283,8 @@ __global__ void k_reduce_splits(const float* __restrict__ part, float* __restric
   }
 }
 
-// dx = dy where y > 0, else 0 (gradient through y = relu(x))
+// dx = dy where y > 0, else 0 (gradient through y = relu(x)).  With k_colsum, k_add and k_pool2's backward pass one of
+// the separate steps that k_relu_grad_bias takes together and has to repeat; kept for that comparison.
 __global__ void k_relu_grad(const bf16* __restrict__ y, const bf16* __restrict__ dy, bf16* __restrict__ dx, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     dx[i] = __bfloat162float(y[i]) > 0.f ? dy[i] : __float2bfloat16_rn(0.f);
