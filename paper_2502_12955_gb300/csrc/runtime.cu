@@ -297,6 +297,9 @@ void fill_args(lbm_ctx* c) {
 int parity_of(long long step) { return int(step & 1); }
 
 constexpr long long kListRebuild = 1024;   // steps between sorted rebuilds of the fluid list
+#ifndef LBM_OFF32_BYTES
+#define LBM_OFF32_BYTES (1ll << 32)   // populations below this take 32-bit offsets (a test builds with 0)
+#endif
 #ifndef LBM_STEP_GRAPHS
 #define LBM_STEP_GRAPHS 1
 #endif
@@ -589,7 +592,7 @@ lbm_status lbm_create(lbm_lattice lattice, int32_t nx, int32_t ny, int32_t nz, c
   c->rec = c->ks->rec_bytes(a);
   const int tile = tile_slots((int)c->elem);
   a.pop_bytes = (N + tile - 1) / tile * c->rec;
-  a.off_ok = a.pop_bytes + tile * kOffBias * (long long)c->elem < (1ll << 32) ? 1 : 0;
+  a.off_ok = a.pop_bytes + tile * kOffBias * (long long)c->elem < LBM_OFF32_BYTES ? 1 : 0;
   DA(a.pop, a.pop_bytes);
   DA(c->pop_alt, a.pop_bytes);
   DA(a.slot, N * 4);
